@@ -320,6 +320,7 @@ def run_gw(args):
         torch.distributed.barrier()
     local_ms = ev0.elapsed_time(ev1)
     st = ctx.stats()
+    form = ctx.update_form()
     launches = int(st["kernel_launches"] - launches0)
     herk_ms = st["herk_ms_mean"]
     times = ctx.times()
@@ -444,20 +445,27 @@ def run_gw(args):
 
     peaks, peak_src = load_peaks()
     peak = float(peaks.get("bf16_tflops_sustained", 1700.0))     # FP16 dense = BF16 dense rate
-    achieved = flop_step / (herk_ms * 1e-3) / 1e12 if herk_ms > 0 else None
+    # the contraction as it is formed: over T (nc + nv) states in separable form, else over k pairs
+    rank = form["terms"] * (w.nv + w.nc) if form["terms"] else w.k
+    achieved = 4.0 * rank * w.nr * (w.nr + 1) / (herk_ms * 1e-3) / 1e12 if herk_ms > 0 else None
     # tensor-pipe work actually issued per 16-k chunk per tile: 3 MMAs of 2*128*256*16 and 6 of
     # 2*128*128*16, the same as 6 of N = 256; a CTA pair issues 6 of M = 256, N = 256
-    kpad = (w.k + 15) // 16 * 16
+    pair_kernel = args.herk_kernel == "pair" and not form["terms"]
     rows_per_tile = 256 if args.herk_kernel == "pair" else 128
-    tensor_flop = st["herk_tiles"] * (kpad // 16) * 6 * 2.0 * rows_per_tile * 256 * 16
-    traffic = herk_traffic(w.name, args.precision, (int(st["window_chunks"]), int(st["flush_windows"])),
-                           args.herk_kernel)
+    tensor_flop = st["herk_tiles"] * form["chunks"] * 6 * 2.0 * rows_per_tile * 256 * 16
+    traffic = None if form["terms"] else herk_traffic(
+        w.name, args.precision, (int(st["window_chunks"]), int(st["flush_windows"])), args.herk_kernel)
     roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                 "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
                 "kernel": ("herk16x2_kernel<fp16> (tcgen05 kind::f16 cta_group::2, CTA pairs, 256x128 tiles, "
-                           "promoted TMEM windows)" if args.herk_kernel == "pair" else
+                           "promoted TMEM windows)" if pair_kernel else
+                           "herk16p_kernel<fp16> (tcgen05 kind::f16, persistent, 128x128 tiles, promoted TMEM "
+                           f"windows, separable form of {form['terms']} terms)" if form["terms"] else
                            "herk16_kernel<fp16> (tcgen05 kind::f16, 128x128 tiles, promoted TMEM windows)"),
+                "contracted_rank": rank, "update_form": form,
+                "flop_note": "achieved counts 4 rank N_r (N_r + 1) of the contraction that ran; value counts the "
+                             "direct sum over pairs, rank k = nv nc",
                 "peak_source": f"{peak_src} bf16_tflops_sustained (FP16:BF16 nominal ratio 1)",
                 "tensor_pipe_frac": (tensor_flop / (herk_ms * 1e-3) / 1e12 / peak) if herk_ms > 0 else None,
                 "herk_ms": herk_ms}
@@ -479,7 +487,7 @@ def run_gw(args):
                 else "eps and eps^-1 (Cholesky) in FP64")
     prec_note = (f"{args.precision}: {part} hi+lo split, 3 products, FP32 accumulation (TMEM windows promoted to "
                  f"FP32); {inv_note}" if part else f"{args.precision}; {inv_note}")
-    f_gb = (w.k + 15) // 16 * 16 * ((w.nr + 255) // 256 * 256) * 8 / 1e9
+    f_gb = form["chunks"] * 16 * ((w.nr + 255) // 256 * 256) * 8 / 1e9
     p_gb = w.nr * w.nr * 8 / 1e9
     line = {"metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
@@ -665,7 +673,8 @@ def section_batch(args, steps):
            "warmup": args.warmup, "ms_per_step": ms, "s_per_pass": ms / 1e3, "tflops": flop / (ms * 1e-3) / 1e12,
            "herk_flop_per_step": flop, "gpu_launches": launches,
            "herk": {"ms": herk_ms, "achieved_tflops": flop / (herk_ms * 1e-3) / 1e12,
-                    "kernel": "herk16p_kernel (persistent, all instances)"},
+                    "kernel": "herk16p_kernel (persistent, all instances, each in its separable or pair form)",
+                    "flop_note": "direct sums over pairs"},
            "clocks": clk.summary()}
     b.close()
     for c in ctxs:

@@ -70,6 +70,18 @@ typedef enum gw_precision {
                            /* three-product split, short TMEM windows promoted to FP32 registers */
 } gw_precision;
 
+/*
+ * How the 16-bit modes form the update.  The sum over pairs is taken either pair by pair (k = nv nc) or,
+ * where that contracts less, in separable form: 2 / (E_c - E_v) = sum_{t < T} u_t(v) z_t(c) to a relative
+ * 2^-26 of every weight, so that
+ *     P(r,r') = -sum_t [sum_v u_t(v) conj(psi_v(r)) psi_v(r')] [sum_c z_t(c) psi_c(r) conj(psi_c(r'))],
+ * T (nv + nc) states instead of nv nc pairs (T is 8 to 13 for the gaps and band widths of Sec. 3).  The
+ * library decides from nv, nc and the energies alone; GW_BUF_FACTORS is there after an update in
+ * separable form.  Both forms
+ * agree to the error of the precision mode; in the separable form the mean loss of the tensor cores'
+ * truncating additions is multiplied back, and its error against FP64 is the smaller one.
+ */
+
 typedef enum gw_inv_method {
     GW_INV_CHOLESKY = 0,   /* FP64 blocked Cholesky eps = L L^H, then eps^-1 = L^-H L^-1        */
     GW_INV_NEWTON = 1,     /* FP64 Newton iteration X <- X (2I - eps X) of Sec. 5.1, from        */
@@ -186,12 +198,17 @@ typedef enum gw_buffer {
     GW_BUF_EPS = 3,      /* N_g x N_g complex128, eps                                           */
     GW_BUF_EPSINV = 4,   /* N_g x N_g complex128, eps^-1                                        */
     GW_BUF_WEIGHTS = 5,  /* [nv][nc] float, sqrt(2 / (E_c - E_v)) in Hartree^-1/2              */
-    GW_BUF_PSIT = 6      /* [N_r][nv + nc] complex64, the loaded states transposed (r major)     */
+    GW_BUF_PSIT = 6,     /* [N_r][nv + nc] complex64, the loaded states transposed (r major)     */
+    GW_BUF_FACTORS = 7   /* separable form of the last update: [T][16 ceil(nc/16) + 16 ceil(nv/16)] */
+                         /* float, the factors z_t of the unoccupied states (last state first), then */
+                         /* u_t, zero-padded, each scaled by a power of two; GW_E_NOT_READY pair by pair */
 } gw_buffer;
 
 /*
  * Return the device pointer and byte size of an internal buffer (GW_E_NOT_READY if it has not
- * been produced yet).  Pointers stay valid until the next gw_load_states or gw_destroy.
+ * been produced yet).  Pointers stay valid until the next gw_load_states or gw_destroy.  After an
+ * update in separable form, which has no pair densities, GW_BUF_F allocates and enqueues them on the
+ * context's stream when it is asked for.
  *
  * GW_BUF_F layout (precisions TF32X3 / TF32X1): float planes, k = v * nc + c padded with zeros
  * to a multiple of 8 (kpad), rows padded with zeros to a multiple of 256 (nr_pad).  For chunk
@@ -231,8 +248,9 @@ GW_API gw_status gw_reset_times(gw_ctx *ctx);
  * process, [1] = Newton iterations of the last GW_INV_NEWTON inverse (FP16X3 steps for
  * GW_INV_NEWTON_TC and gw_zinv_tc), [2] = mean rank-k update
  * time in ms over the timed calls since gw_reset_times, [3] = number of those calls, [4] = the
- * FP16 scale exponent e of the last 16-bit build, [5] = rank-k update tiles (CTA pairs for
- * GW_HERK_PAIR), [6] and [7] = the window and flush lengths of the 16-bit update.
+ * FP16 scale exponent e of the last 16-bit build (of the pair densities; of the unoccupied states in
+ * separable form), [5] = rank-k update tiles (256 x 128 for GW_HERK_PAIR), [6] and [7] = the window and
+ * flush lengths of the 16-bit update.
  */
 GW_API gw_status gw_get_stats(gw_ctx *ctx, double *stats8);
 
@@ -242,7 +260,7 @@ GW_API gw_status gw_get_stats(gw_ctx *ctx, double *stats8);
  * as gw_build_P (16-bit precisions) + gw_P_to_G + gw_eps_inv(GW_INV_CHOLESKY):
  *   - pair densities per instance;
  *   - ONE persistent launch of the rank-k update over the tiles of every instance (one CTA per SM
- *     walks a static tile list ordered by decreasing k), bit-identical to the per-instance kernel
+ *     walks a static tile list ordered by decreasing work), bit-identical to the per-instance kernel
  *     for the same window settings;
  *   - per-instance transforms, eps and FP64 inverse.
  * Results are read from each context (gw_get_buffer GW_BUF_PG / GW_BUF_EPSINV, or gw_eps_inv-style
@@ -390,7 +408,8 @@ GW_API gw_status gw_newton_tc_report(gw_ctx *ctx, double *out4);
  * Window length of the 16-bit rank-k update: the tensor core accumulates `window_chunks` chunks
  * of 16 k (1..64, default 3) in TMEM before they are added into FP32 registers, and every
  * `flush_windows` windows (1..4096, default 256) the registers are added into P.  Shorter windows
- * and flushes mean smaller accumulation error.
+ * and flushes mean smaller accumulation error.  In separable form the registers are multiplied out and
+ * added after every term, so flush_windows has no effect there.
  */
 GW_API gw_status gw_set_herk_window(gw_ctx *ctx, int window_chunks, int flush_windows);
 
@@ -401,7 +420,8 @@ GW_API gw_status gw_set_herk_window(gw_ctx *ctx, int window_chunks, int flush_wi
  *                   M = 256): each CTA holds 128 rows of A and half of B, 256 x 128 complex tiles;
  *                   the operand holds six 16-bit planes per k chunk (the Im planes also negated)
  *   GW_HERK_SINGLE  (default) one CTA per 128 x 128 complex tile, four planes per k chunk
- * Takes effect at the next gw_build_P; GW_E_INVALID for another value.
+ * Takes effect at the next gw_build_P; GW_E_INVALID for another value.  An update in separable form
+ * runs the persistent one-CTA kernel under either setting.
  */
 enum { GW_HERK_SINGLE = 0, GW_HERK_PAIR = 1 };
 GW_API gw_status gw_set_herk_kernel(gw_ctx *ctx, int kind);

@@ -558,6 +558,81 @@ void newton_tc_record(Ctx &c, int n)
         c.tc_report[i] = r[i];
 }
 
+// Separable form of the 16-bit rank-k update for the loaded energies: c.sep.T terms, 0 where the pair
+// form has less to contract.  A term costs its ceil(nc / 16) + ceil(nv / 16) chunks of 16 states and
+// about SEP_TERM_CHUNKS more for its shorter windows and for multiplying its sums out; the pair form
+// costs ceil(nv nc / 16).  Update, pair against separable form, 20^3 grid, W = 3 (us): nv x nc =
+// 8 x 300 (150 chunks against T = 8 times 20) 1389 / 1704, 20 x 64 (80; 9 x 6) 797 / 779, 14 x 200 (175;
+// 9 x 14) 1604 / 1443, 30 x 120 (225; 10 x 10) 2023 / 1329; the lines cross at 3 to 4.5 chunks a term.
+constexpr int SEP_TERM_CHUNKS = 4;
+
+void find_separable(Ctx &c)
+{
+    if (c.sep_known)
+        return;
+    const int ncc = (c.nc + HERK16_KC - 1) / HERK16_KC, nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
+    const int pair_chunks = (c.k + HERK16_KC - 1) / HERK16_KC;
+    const int most = (pair_chunks - 1) / (ncc + nvc + SEP_TERM_CHUNKS);
+    c.sep = most >= 1 ? sep_factors(c.E_h.data(), c.nv, c.nc, HERK16_KC, most) : SepFactors();
+    c.sep_known = true;
+}
+
+// The separable job of a context whose d_P and scale words exist: operand buffers, factors and job
+// table uploaded; the planes themselves are made by separable_planes.  `job` receives the job.
+gw_status prepare_separable(Ctx &c, HerkJob *job)
+{
+    HerkJob j = {};
+    j.T = c.sep.T;
+    j.ncc = (c.nc + HERK16_KC - 1) / HERK16_KC;
+    j.nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
+    const size_t chunk = plane16_block(1, 0, c.nr_pad / 128, HERK16_NPL, 0) * sizeof(uint16_t);
+    GW_TRY(ensure(c, c.d_sepA, c.cap_sepA, (size_t)j.T * (j.ncc + j.nvc) * chunk, "separable operand"));
+    GW_TRY(ensure(c, c.d_sepB, c.cap_sepB, (size_t)(j.ncc + j.nvc) * chunk, "separable operand"));
+    constexpr size_t head = 256;
+    static_assert(sizeof(HerkJob) <= head, "job record");
+    const size_t off_tab = head + (j.T * sizeof(float) + 255) / 256 * 256;
+    const size_t bytes = off_tab + c.sep.tab.size() * sizeof(float);
+    GW_TRY(ensure(c, c.d_sept, c.cap_sept, bytes, "separable factors"));
+    unsigned char *dev = static_cast<unsigned char *>(c.d_sept);
+    j.A = c.d_sepA;
+    j.B = c.d_sepB;
+    j.P = c.d_P;
+    j.scale_exp = reinterpret_cast<const int *>(c.d_small + 2);
+    j.term_scale = reinterpret_cast<const float *>(dev + head);
+    j.nr = c.nr;
+    j.nr_pad = c.nr_pad;
+    c.sep_host.assign(bytes, 0);
+    std::memcpy(c.sep_host.data(), &j, sizeof j);
+    std::memcpy(c.sep_host.data() + head, c.sep.scale.data(), j.T * sizeof(float));
+    std::memcpy(c.sep_host.data() + off_tab, c.sep.tab.data(), c.sep.tab.size() * sizeof(float));
+    GW_CUDA(cudaMemcpyAsync(dev, c.sep_host.data(), bytes, cudaMemcpyHostToDevice, c.stream), "separable factors");
+    c.sep_tab = reinterpret_cast<const float *>(dev + off_tab);
+    *job = j;
+    return GW_OK;
+}
+
+cudaError_t separable_planes(Ctx &c, const HerkJob &j, bool bf16, cudaStream_t s)
+{
+    return launch_sep_planes(c.d_psiT, c.sep_tab, j.T, c.nr, c.nb, c.nv, j.ncc, j.nvc, c.nr_pad, bf16, c.d_small,
+                             reinterpret_cast<int *>(c.d_small + 2), c.d_sepA, c.d_sepB, s);
+}
+
+// GW_BUF_F after a separable update, which has no pair densities: form them now.
+gw_status form_pair_planes(Ctx &c)
+{
+    const bool bf16 = c.F_prec == GW_PREC_BF16X3;
+    const int npl = c.last_herk_kernel == GW_HERK_PAIR ? HERK16_NPL_PAIR : HERK16_NPL;
+    GW_CUDA(cudaSetDevice(c.device), "set device");
+    c.F_bytes = (size_t)c.kpad * c.nr_pad * sizeof(uint16_t) * npl;
+    GW_TRY(ensure(c, c.d_F, c.cap.F, c.F_bytes, "pair-density operand"));
+    GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, bf16,
+                                  c.d_small, reinterpret_cast<int *>(c.d_small + 1),
+                                  reinterpret_cast<uint16_t *>(c.d_F), c.stream, npl),
+            "pair densities (16-bit)");
+    c.F_formed = true;
+    return GW_OK;
+}
+
 bool is_device_pointer(const void *p)
 {
     cudaPointerAttributes a;
@@ -582,6 +657,10 @@ void Ctx::release()
     dfree(d_E);
     dfree(d_sw);
     dfree(d_F);
+    dfree(d_sept);
+    dfree(d_sepA);
+    dfree(d_sepB);
+    dfree(d_sums);
     dfree(d_P);
     dfree(d_tiles);
     dfree(d_tiles_g);
@@ -798,7 +877,7 @@ gw_status gw_get_stats(gw_ctx *h, double *s8)
     s8[3] = c.times_n[1];
     int e = 0;
     if (c.d_small && (c.F_prec == GW_PREC_FP16X3 || c.F_prec == GW_PREC_BF16X3))
-        cudaMemcpy(&e, c.d_small + 1, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaMemcpy(&e, c.d_small + (c.F_formed ? 1 : 2), sizeof(int), cudaMemcpyDeviceToHost);
     s8[4] = e;
     s8[5] = c.n_tiles;
     s8[6] = c.last_W;
@@ -856,6 +935,7 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     GW_CUDA(cudaSetDevice(c.device), "set device");
     c.loaded = c.P_ready = c.PG_ready = c.eps_ready = false;
     c.q_pairs = false;
+    c.sep_known = false;
     c.n1 = n1;
     c.n2 = n2;
     c.n3 = n3;
@@ -898,9 +978,11 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     GW_CUDA(launch_transpose_states(src, nb, nr, c.d_psiT, s), "transpose states");
     GW_CUDA(cudaMemcpyAsync(c.d_E, Eh.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s), "copy energies");
     GW_CUDA(launch_weights(c.d_E, nv, nc, c.d_sw, s), "weights");
+    c.E_h = Eh;
+    if (nb <= 256)  // at most about 15 us on the host, behind the kernels above; larger sets in gw_build_P
+        find_separable(c);
     // Eh is a local: make sure the copy has consumed it before returning.
     GW_CUDA(cudaStreamSynchronize(s), "load sync");
-    c.E_h = Eh;
     c.loaded = true;
     return GW_OK;
 }
@@ -929,14 +1011,18 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     // CTA pairs take 256-row blocks of r: nr_pad is a multiple of 256 for every grid
     const bool pair = p16 && c.herk_kernel == GW_HERK_PAIR && c.nr_pad % 256 == 0;
     const int npl = pair ? HERK16_NPL_PAIR : HERK16_NPL;
-    size_t Fbytes;
+    if (p16)
+        find_separable(c);
+    const bool sep = p16 && c.sep.T > 0;
+    size_t Fbytes = 0;
     if (precision == GW_PREC_FP32_SIMT)
         Fbytes = (size_t)c.kpad * c.nr_pad * sizeof(float2);
     else if (p16)
         Fbytes = (size_t)c.kpad * c.nr_pad * 2 * npl;
     else
         Fbytes = (size_t)c.kpad * c.nr_pad * sizeof(float) * (precision == GW_PREC_TF32X3 ? 4 : 2);
-    GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
+    if (!sep)
+        GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
     if (!c.d_small)
         GW_CUDA(cudaMalloc(&c.d_small, 4 * sizeof(unsigned)), "scale words");
     c.F_bytes = Fbytes;
@@ -944,22 +1030,41 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     GW_TRY(ensure(c, c.d_P, c.cap.P, c.P_bytes, "P(r,r')"));
     c.P_ready = c.PG_ready = c.eps_ready = false;
 
-    const int tile_kind = pair ? 2 : p16 ? 1 : 0;
-    if (precision != GW_PREC_FP32_SIMT && (c.tiles_nr_pad != c.nr_pad || c.tiles_kind != tile_kind)) {
+    const int tile_kind = sep ? 3 : pair ? 2 : p16 ? 1 : 0;
+    if (sep && (c.tiles_nr_pad != c.nr_pad || c.tiles_kind != tile_kind)) {
+        std::vector<int4> t;
+        for (const int2 ij : herk_tiles(c.nr_pad, HERK16_T, HERK16_T))
+            t.push_back(make_int4(0, ij.x, ij.y, 0));
+        GW_TRY(ensure(c, c.d_tiles, c.cap.tiles, t.size() * sizeof(int4), "tile list"));
+        GW_CUDA(cudaMemcpy(c.d_tiles, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice), "tile upload");
+        c.n_tiles_run = static_cast<int>(t.size());
+        c.tiles_nr_pad = c.nr_pad;
+        c.tiles_kind = tile_kind;
+    } else if (precision != GW_PREC_FP32_SIMT && (c.tiles_nr_pad != c.nr_pad || c.tiles_kind != tile_kind)) {
         const auto t = pair  ? herk_pair_tiles(c.nr_pad)
                        : p16 ? herk_tiles(c.nr_pad, HERK16_T, HERK16_T)
                              : herk_tiles(c.nr_pad, HERK_BM, HERK_BN);
         GW_TRY(ensure(c, c.d_tiles, c.cap.tiles, t.size() * sizeof(int2), "tile list"));
         GW_CUDA(cudaMemcpy(c.d_tiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice), "tile upload");
-        c.n_tiles = static_cast<int>(t.size());
+        c.n_tiles_run = static_cast<int>(t.size());
         c.tiles_nr_pad = c.nr_pad;
         c.tiles_kind = tile_kind;
     }
+    c.n_tiles = sep && pair ? static_cast<int>(herk_pair_tiles(c.nr_pad).size()) : c.n_tiles_run;
     const uint64_t wait_ns = static_cast<uint64_t>(c.wait_limit_ms * 1e6);
     int *scale_exp = reinterpret_cast<int *>(c.d_small + 1);
 
+    HerkJob job = {};
+    const int grid_sep = std::min(c.n_tiles_run, sm_count(c.device));
+    if (sep) {
+        GW_TRY(ensure(c, c.d_sums, c.cap_sums, (size_t)grid_sep * HERK16P_SUMS, "running sums"));
+        GW_TRY(prepare_separable(c, &job));
+    }
+
     record(c, 0);
-    if (p16)
+    if (sep)
+        GW_CUDA(separable_planes(c, job, precision == GW_PREC_BF16X3, s), "separable operand planes");
+    else if (p16)
         GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad,
                                       precision == GW_PREC_BF16X3, c.d_small, scale_exp,
                                       reinterpret_cast<uint16_t *>(c.d_F), s, npl),
@@ -968,24 +1073,30 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
         GW_CUDA(launch_pair_density(c.d_psiT, c.d_sw, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, precision, c.d_F, s),
                 "pair densities");
     c.F_prec = precision;
+    c.F_formed = !sep;
     if (p16)
         c.last_herk_kernel = pair ? GW_HERK_PAIR : GW_HERK_SINGLE;
     record(c, 1);
     if (precision == GW_PREC_FP32_SIMT) {
         GW_CUDA(launch_herk_simt(reinterpret_cast<float2 *>(c.d_F), c.kpad, c.nr, c.nr_pad, c.d_P, s),
                 "rank-k update (CUDA cores)");
+    } else if (sep) {
+        GW_CUDA(launch_herk16p(static_cast<const HerkJob *>(c.d_sept), reinterpret_cast<const int4 *>(c.d_tiles),
+                               c.n_tiles_run, grid_sep, precision == GW_PREC_BF16X3, c.d_err, wait_ns, c.last_W,
+                               c.herk_L, c.d_sums, s),
+                "rank-k update (tcgen05, separable, 16-bit)");
     } else if (pair) {
         GW_CUDA(launch_herk16x2(reinterpret_cast<uint16_t *>(c.d_F), precision == GW_PREC_BF16X3, c.kpad, c.nr,
-                                c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
+                                c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
                                 c.herk_L, s),
                 "rank-k update (tcgen05 CTA pairs, 16-bit)");
     } else if (p16) {
         GW_CUDA(launch_herk16(reinterpret_cast<uint16_t *>(c.d_F), precision == GW_PREC_BF16X3, c.kpad, c.nr,
-                              c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W, c.herk_L,
-                              s),
+                              c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
+                              c.herk_L, s),
                 "rank-k update (tcgen05, 16-bit)");
     } else {
-        GW_CUDA(launch_herk_tc(c.d_F, precision, c.kpad, c.nr, c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, c.d_err, wait_ns,
+        GW_CUDA(launch_herk_tc(c.d_F, precision, c.kpad, c.nr, c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, c.d_err, wait_ns,
                                s),
                 "rank-k update (tcgen05, TF32)");
     }
@@ -1641,8 +1752,16 @@ gw_status gw_get_buffer(gw_ctx *h, int which, void **ptr, size_t *bytes)
     case GW_BUF_F:
         if (c.F_prec < 0 || !c.P_ready)
             return GW_E_NOT_READY;
+        if (!c.F_formed)
+            GW_TRY(form_pair_planes(c));
         *ptr = c.d_F;
         *bytes = c.F_bytes;
+        return GW_OK;
+    case GW_BUF_FACTORS:
+        if ((c.F_prec != GW_PREC_FP16X3 && c.F_prec != GW_PREC_BF16X3) || !c.P_ready || c.sep.T == 0)
+            return GW_E_NOT_READY;
+        *ptr = const_cast<float *>(c.sep_tab);
+        *bytes = c.sep.tab.size() * sizeof(float);
         return GW_OK;
     case GW_BUF_PG:
         if (!c.PG_ready)
@@ -1708,6 +1827,8 @@ struct gw_batch {
     cudaStream_t stream = nullptr;  // the batch's own non-blocking stream
     bool own_stream = false;
     HerkJob *d_jobs = nullptr;
+    std::vector<HerkJob> jobs;      // as uploaded
+    float4 *d_sums = nullptr;       // HERK16P_SUMS per CTA of the update
     int4 *d_tiles = nullptr;
     int n_tiles = 0, grid = 0;
     int W = 2, L = 256;
@@ -1773,18 +1894,22 @@ void drop_graph(gw_batch &b)
 // Allocate every buffer the pass needs (graph capture must not allocate) and build the plans.
 gw_status batch_prepare(gw_batch &b)
 {
-    const bool bf16 = b.precision == GW_PREC_BF16X3;
-    std::vector<HerkJob> jobs;
+    std::vector<HerkJob> &jobs = b.jobs;
+    jobs.clear();
     std::vector<int4> tiles;
     for (size_t i = 0; i < b.ctxs.size(); ++i) {
         Ctx &c = b.ctxs[i]->c;
         const int kpad = ((c.k + HERK16_KC - 1) / HERK16_KC) * HERK16_KC;
         c.kpad = kpad;
+        find_separable(c);
+        const bool sep = c.sep.T > 0;
         const size_t Fbytes = (size_t)kpad * c.nr_pad * 2 * HERK16_NPL;
-        GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
+        if (!sep)
+            GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
         if (!c.d_small)
             GW_CUDA(cudaMalloc(&c.d_small, 4 * sizeof(unsigned)), "scale words");
         c.F_bytes = Fbytes;
+        c.last_herk_kernel = GW_HERK_SINGLE;
         c.P_bytes = (size_t)c.nr * c.nr * sizeof(float2);
         GW_TRY(ensure(c, c.d_P, c.cap.P, c.P_bytes, "P(r,r')"));
         if (b.gcut[i] != c.gcut)
@@ -1808,14 +1933,28 @@ gw_status batch_prepare(gw_batch &b)
             const size_t work = (size_t)3 * ng * ng + (size_t)NB * ng + (size_t)nblk * NB * NB;
             GW_TRY(ensure(c, c.d_work, c.cap.work, work * sizeof(double2), "inverse workspace"));
         }
-        jobs.push_back({reinterpret_cast<const uint16_t *>(c.d_F), c.d_P, reinterpret_cast<const int *>(c.d_small + 1),
-                        c.nr, c.nr_pad, kpad, 0});
+        HerkJob job = {};
+        if (sep) {
+            GW_TRY(prepare_separable(c, &job));
+        } else {
+            job.A = job.B = reinterpret_cast<const uint16_t *>(c.d_F);
+            job.P = c.d_P;
+            job.scale_exp = reinterpret_cast<const int *>(c.d_small + 1);
+            job.nr = c.nr;
+            job.nr_pad = c.nr_pad;
+            job.T = 1;
+            job.ncc = kpad / HERK16_KC;
+        }
+        jobs.push_back(job);
         for (const int2 t : herk_tiles(c.nr_pad, HERK16_T, HERK16_T))
             tiles.push_back(make_int4((int)i, t.x, t.y, 0));
     }
     // longest tiles first: with the static round-robin schedule every CTA gets a similar load
     std::stable_sort(tiles.begin(), tiles.end(),
-                     [&](const int4 &a, const int4 &c2) { return jobs[a.x].kpad > jobs[c2.x].kpad; });
+                     [&](const int4 &a, const int4 &c2) {
+                         const HerkJob &x = jobs[a.x], &y = jobs[c2.x];
+                         return x.T * (x.ncc + x.nvc) > y.T * (y.ncc + y.nvc);
+                     });
     if (b.d_jobs)
         cudaFree(b.d_jobs);
     if (b.d_tiles)
@@ -1830,19 +1969,28 @@ gw_status batch_prepare(gw_batch &b)
     int sms = 0;
     GW_BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b.device), "SM count");
     b.grid = std::min(b.n_tiles, sms);
-    (void)bf16;
+    if (b.d_sums)
+        cudaFree(b.d_sums);
+    b.d_sums = nullptr;
+    GW_BCUDA(cudaMalloc(&b.d_sums, (size_t)b.grid * HERK16P_SUMS), "running sums");
     return GW_OK;
 }
 
 gw_status batch_pair_densities(gw_batch &b)
 {
-    for (gw_ctx *h : b.ctxs) {
-        Ctx &c = h->c;
-        GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad,
-                                      b.precision == GW_PREC_BF16X3, c.d_small, reinterpret_cast<int *>(c.d_small + 1),
-                                      reinterpret_cast<uint16_t *>(c.d_F), b.stream),
-                "pair densities (batch)");
+    const bool bf16 = b.precision == GW_PREC_BF16X3;
+    for (size_t i = 0; i < b.ctxs.size(); ++i) {
+        Ctx &c = b.ctxs[i]->c;
+        const bool sep = b.jobs[i].nvc > 0;
+        if (sep)
+            GW_CUDA(separable_planes(c, b.jobs[i], bf16, b.stream), "separable operand planes (batch)");
+        else
+            GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, bf16,
+                                          c.d_small, reinterpret_cast<int *>(c.d_small + 1),
+                                          reinterpret_cast<uint16_t *>(c.d_F), b.stream),
+                    "pair densities (batch)");
         c.F_prec = b.precision;
+        c.F_formed = !sep;
     }
     return GW_OK;
 }
@@ -1852,7 +2000,7 @@ gw_status batch_herk(gw_batch &b)
     const uint64_t wait_ns = static_cast<uint64_t>(b.ctxs[0]->c.wait_limit_ms * 1e6);
     GW_BCUDA(cudaEventRecord(b.e0, b.stream), "event");
     GW_BCUDA(launch_herk16p(b.d_jobs, b.d_tiles, b.n_tiles, b.grid, b.precision == GW_PREC_BF16X3, b.d_err, wait_ns,
-                            b.W, b.L, b.stream),
+                            b.W, b.L, b.d_sums, b.stream),
              "rank-k update (persistent, batch)");
     GW_BCUDA(cudaEventRecord(b.e1, b.stream), "event");
     return GW_OK;
@@ -1992,6 +2140,8 @@ gw_status gw_batch_destroy(gw_batch *b)
         cudaFree(b->d_jobs);
     if (b->d_tiles)
         cudaFree(b->d_tiles);
+    if (b->d_sums)
+        cudaFree(b->d_sums);
     if (b->d_err)
         cudaFree(b->d_err);
     if (b->e0)

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/gw.h"
+#include "sep_factors.h"
 
 namespace gw {
 
@@ -178,8 +179,20 @@ struct Ctx {
             scal, tcw, PGsum, coef, gidx, gtw, psig, ppw;
     } cap = {};
     int tiles_nr_pad = -1, tiles_kind = -1;
+    int n_tiles_run = 0;            // tiles in d_tiles (n_tiles is what gw_get_stats reports)
+    // separable rank-k update (sep_factors.h, k_herk16p.cu)
+    SepFactors sep;                 // factors of the loaded energies (T = 0: pair form)
+    bool sep_known = false;         // sep belongs to the loaded energies
+    std::vector<unsigned char> sep_host;  // the job, the term scales and the factors, as uploaded
+    void *d_sept = nullptr;         // their device copy
+    const float *sep_tab = nullptr; // the factors in it
+    uint16_t *d_sepA = nullptr, *d_sepB = nullptr;
+    float4 *d_sums = nullptr;       // HERK16P_SUMS per CTA
+    size_t cap_sept = 0, cap_sepA = 0, cap_sepB = 0, cap_sums = 0;
+    bool F_formed = false;          // d_F holds the planes of F_prec (false after a separable update)
     float sw_max = 0.f;             // max sqrt(2/(E_c - E_v)) (host, from the energies)
-    unsigned *d_small = nullptr;    // [0] |f| bound bits, [1] FP16 scale exponent
+    unsigned *d_small = nullptr;    // [0] |f| bound bits, [1] FP16 scale exponent; separable update: [0], [1]
+                                    // bounds and [2], [3] exponents of psi_c and psi_v
     int herk_W = 3, herk_L = 256;   // 6.5e-7 against FP64 at 24^3; see gw_set_herk_window
     int herk_kernel = GW_HERK_SINGLE; // r-space 16-bit update: one CTA per tile or CTA pairs
     std::vector<double> E_h;        // the loaded energies in Hartree (host copy)
@@ -285,17 +298,25 @@ cudaError_t launch_herk16x2(const uint16_t *F, bool bf16, int kpad, int nr, int 
 cudaError_t launch_planes16_from_c64(const float2 *M, int rows, int cols, long ld, int kpad, int cols_pad, bool bf16,
                                      unsigned *bound_bits, int *scale_exp, uint16_t *F, cudaStream_t s);
 
-// k_herk16p.cu: persistent multi-instance rank-k update.  One job per instance; tiles are
+// k_herk16p.cu: persistent rank-k update of one or many systems.  One job per system; tiles are
 // (job, 128-row block of r, 128-row block of r', 0) in the order CTAs take them (tile t goes to
-// CTA t mod grid).
+// CTA t mod grid).  Pair form: A = B = the pair densities' planes, T = 1, ncc = kpad / 16, nvc = 0.
+// Separable form: the planes of launch_sep_planes.
 struct HerkJob {
-    const uint16_t *F;
+    const uint16_t *A, *B;
     float2 *P;
-    const int *scale_exp;
-    int nr, nr_pad, kpad, pad;
+    const int *scale_exp;     // [0] exponent of the pair densities or of psi_c, [1] of psi_v
+    const float *term_scale;  // separable form: [T]
+    int nr, nr_pad, T, ncc, nvc;
 };
+constexpr size_t HERK16P_SUMS = 128 * 1024;  // running sums per CTA of the grid, in bytes
 cudaError_t launch_herk16p(const HerkJob *jobs, const int4 *tiles, int n_tiles, int grid, bool bf16, uint32_t *err,
-                           uint64_t wait_ns, int W, int L, cudaStream_t s);
+                           uint64_t wait_ns, int W, int L, float4 *sums, cudaStream_t s);
+// k_planes16.cu: its operands.  A: T (ncc + nvc) chunks, B: ncc + nvc chunks, both of nr_pad rows and
+// HERK16_NPL planes; tab [T][16 (ncc + nvc)] from sep_factors; bound_bits and scale_exp: two words each.
+cudaError_t launch_sep_planes(const float2 *psiT, const float *tab, int T, int nr, int nb, int nv, int ncc, int nvc,
+                              int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint16_t *A, uint16_t *B,
+                              cudaStream_t s);
 
 // k_mlp_tc.cu: tensor-core inference of the correction network (hidden width 256, n_in <= 16)
 // on CTA pairs; the weights go through launch_mlp_tile_weights into a buffer of

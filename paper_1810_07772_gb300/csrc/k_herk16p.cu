@@ -1,14 +1,42 @@
-// Persistent multi-instance variant of the 16-bit Hermitian rank-k update (Eq. Pstatic; the outer
-// product of Sec. 4.1) for a batch of independent systems of uneven size.
+// Persistent Hermitian rank-k update of one or many systems (Eq. Pstatic; the outer product of
+// Sec. 4.1) on the 16-bit tensor cores.  One CTA per SM walks a static list of (job, row block,
+// column block) tiles (CTA b takes tiles b, b + grid, b + 2 grid, ...; the host orders them by
+// decreasing work so the static schedule balances).
 //
-// One CTA per SM walks a static list of (instance, row block, column block) tiles (CTA b takes
-// tiles b, b + grid, b + 2 grid, ...; the host orders them by decreasing k so the static schedule
-// balances).  The arithmetic per tile is exactly that of herk16_kernel -- the FP16/BF16 hi/lo
-// split, W-chunk TMEM windows promoted to FP32 registers, flushes into the tile's region of P
-// every L windows -- so every instance's P equals the single-instance result bit for bit.
-// What changes is the control: mbarrier phases and the two TMEM window buffers carry across
-// tiles, and each tile's final sums go from registers straight to P, so the producer streams the
-// next tile's operands while the current tile is being written.
+// A job is a system in one of two forms.
+//  * Pair form (nvc = 0): P = -sum_k f_k(r) conj(f_k(r')) over all k = nv nc pair densities.  The
+//    arithmetic per tile is that of herk16_kernel -- the FP16 / BF16 hi/lo split, W-chunk TMEM windows
+//    promoted to FP32 registers, the registers added up every L windows -- bit for bit.
+//  * Separable form (nvc > 0): with 2 / (E_c - E_v) = sum_t u_t(v) z_t(c) (sep_factors.h) the sum over
+//    pairs splits, at every (r, r'), into products of two short sums,
+//        P(r, r') = -sum_t V_t(r, r') C_t(r, r'),
+//        C_t = sum_c z_t(c) psi_c(r) conj(psi_c(r')),   V_t = sum_v u_t(v) conj(psi_v(r)) psi_v(r'),
+//    so the tensor cores contract T (nc + nv) states instead of nv nc pairs: 352 chunks of 16 against
+//    960 at 24^3 (T = 11), 871 against 4000 at 36^3 with 64 / 1000 states.  Per term the C windows are
+//    promoted into registers as above, then each V window is multiplied into them element by element
+//    in FP32 and the products are added into the tile's sums.  The registers hold C_t (128 of the 168
+//    a thread can have), so the sums over t live in global memory: 128 KB per CTA, written and read by
+//    their own threads only (20 MB for the GPU, resident in L2), added with fire-and-forget vector
+//    reductions so no thread waits for a load.
+//
+// Measured on one GB300 (update alone, FP16X3, W = 3): 24^3, 32 x 480 states: 24.2 -> 9.44 ms (0.95 of
+// the sustained FP16 rate would be 6.9 ms for the issued MMAs; windows of 16 chunks take 8.0 ms, so the
+// window boundaries cost the most of what is left); 36^3, 64 x 1000, BF16X3, W = 16: 0.97 -> 0.19 s.
+//
+// Bound: the tensor pipe and the shared memory that feeds it, as herk16_kernel (32 KB staged and 84 KB
+// read per chunk).  Control: mbarrier phases and the two TMEM window buffers carry across tiles, so the
+// producer streams the next tile's operands while the current tile is being written.
+//
+// Truncation.  tcgen05 adds into TMEM with truncation, so a window of n chunks comes out smaller by a
+// nearly uniform factor, 1 - b n.  Measured in the separable form: b = 1.3e-7 to 1.8e-7 on P~ and the
+// diagonal of P, 0.5e-7 to 1.4e-7 on its other elements, the same on random and on band-structured
+// states.  A product of two windows carries both losses, so the separable form multiplies the mean loss
+// back (window_loss).  P~ against FP64 at 24^3, W = 3: 9.1e-7 without, 3.3e-7 with it, 6.5e-7 in the
+// pair form; off-diagonal elements of P at 16^3 2.6e-7 against 4.3e-7.
+//
+// The occupied planes are FP16 in either precision (they are 1/16 of the work), so with BF16 operands
+// only C_t carries the 8 + 8-bit split: both at 8 + 8 bits measured 5.7e-6 on the off-diagonal elements
+// of P against 4.5e-6 in the pair form; now 4.1e-6, and 1.4e-6 against 3.4e-6 on P~.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -19,8 +47,8 @@ namespace gw {
 
 namespace {
 
-constexpr int TM = 128, TN = 128, KC16 = HERK16_KC;
-constexpr uint32_t PL = TM * KC16 * 2;  // 4 KB: one plane of one 128-row block
+constexpr int TM = 128, TN = 128;
+constexpr uint32_t PL = TM * HERK16_KC * 2;  // 4 KB: one plane of one 128-row block
 constexpr uint32_t NPL = HERK16_NPL;
 // stage as in herk16_kernel: the A block's planes Im hi, Re hi, Im lo, Re lo (one bulk copy), then
 // the B block's in the same order, i.e. regions [Im | Re] of the
@@ -30,37 +58,80 @@ constexpr uint32_t STAGE_BYTES = 8 * PL;  // 32 KB
 constexpr int STAGES = 6;
 constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;
 constexpr uint32_t LBO = 128, SBO = 256;
-constexpr size_t SMEM = PIPE_BYTES + 256;
 constexpr int NPROMO_WARPS = 8;
 constexpr int PRODUCER_WARP = 8, MMA_WARP = 9;
 constexpr int NTHREADS = 320;
 constexpr uint64_t DRAIN_NS = 2000000000ull;
+// each promotion warp turns 32 rows x 16 columns of the result at a time, so that the rows of P are
+// written in 128-byte runs (a row pitch of 17 values: conflict-free both ways)
+constexpr int OUT_COLS = 16, OUT_PITCH = 17;
+constexpr uint32_t BAR_BYTES = 256;
+constexpr size_t SMEM = PIPE_BYTES + BAR_BYTES + NPROMO_WARPS * 32 * OUT_PITCH * sizeof(float2);
+static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
+constexpr int SUM_F4 = 32;  // float4 values per promotion thread: 64 complex sums
+static_assert(HERK16P_SUMS == (size_t)SUM_F4 * NPROMO_WARPS * 32 * sizeof(float4), "sums per CTA");
 
-__device__ __forceinline__ void named_bar(int id, int n)
+// A thread's own running sums in global memory: a plain store starts them, reductions add, and the
+// load at the tile's end bypasses L1, which may hold the previous tile's values.
+__device__ __forceinline__ void sums_add(float4 *p, float4 v, bool first)
 {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+    if (first)
+        asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z),
+                     "f"(v.w)
+                     : "memory");
+    else
+        asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y),
+                     "f"(v.z), "f"(v.w)
+                     : "memory");
 }
 
-// Named barrier that also ORs a predicate over the n participating threads, so a decision to stop
-// is the same in every warp (a warp leaving between two named barriers would strand the rest).
-__device__ __forceinline__ bool named_bar_or(int id, int n, bool pred)
+__device__ __forceinline__ float4 sums_load(const float4 *p)
 {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}\n"
-        : "=r"(r)
-        : "r"(pred ? 1u : 0u), "r"(id), "r"(n)
-        : "memory");
-    return r != 0;
+    float4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+
+// Position in the ring of stages: stage and phase parity of a chunk counter.
+struct Ring {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next()
+    {
+        if (++s == STAGES) {
+            s = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
+// Windows of a job: each term has nwc windows of W chunks over its ncc unoccupied (or pair) chunks, the
+// last one shorter, then nwv windows of wv chunks over its nvc occupied ones.
+struct Windows {
+    int nwc, nwv, wv;
+    __device__ __forceinline__ Windows(const HerkJob &j, int W)
+        : nwc((j.ncc + W - 1) / W), nwv((j.nvc + W - 1) / W), wv(nwv > 0 ? (j.nvc + nwv - 1) / nwv : 0)
+    {
+    }
+};
+
+// Mean relative loss of a sum over n chunks taken in windows of w chunks (the last one shorter).
+constexpr float LOSS_PER_CHUNK = 1.3e-7f;
+__device__ __forceinline__ float window_loss(int n, int w)
+{
+    if (n <= 0)
+        return 0.f;
+    const int full = n / w, rest = n - full * w;
+    return LOSS_PER_CHUNK * (float)(full * w * w + rest * rest) / (float)n;
 }
 
 template <bool BF16>
 __global__ void __launch_bounds__(NTHREADS, 1)
     herk16p_kernel(const HerkJob *__restrict__ jobs, const int4 *__restrict__ tiles, int n_tiles, uint32_t *err,
-                   uint64_t wait_ns, int W, int L)
+                   uint64_t wait_ns, int W, int L, float4 *__restrict__ sums)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + PIPE_BYTES);
@@ -74,6 +145,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     volatile long long *n_consumed = n_issued + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // With W < STAGES the commit to the empty barrier of a window's last chunk tells the promotion
+    // warps that the window is complete; longer windows have a commit of their own.
+    const bool own = W >= STAGES;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -100,93 +174,103 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     if (warp == PRODUCER_WARP) {
         if (lane == 0) {
             long long g = 0;  // chunks issued by this CTA over all its tiles
+            Ring ring;
             bool stop = false;
             for (int t = blockIdx.x; t < n_tiles && !stop; t += gridDim.x) {
                 const int4 tl = tiles[t];
                 const HerkJob jb = jobs[tl.x];
-                const int nkc = jb.kpad / KC16;
+                const int nch = jb.ncc + jb.nvc;
                 const int nblk = jb.nr_pad / TM;  // block layout: one 16 KB copy per operand block
-                for (int kc = 0; kc < nkc; ++kc, ++g) {
-                    const int s = (int)(g % STAGES);
-                    const uint32_t ph = (uint32_t)((g / STAGES) & 1);
-                    if (g >= STAGES && !mbar_wait(&empty[s], ph ^ 1, wait_ns)) {
-                        record_error(err, GW_E_TIMEOUT, SITE_HERK_PRODUCER, blockIdx.x);
-                        *abort_flag = 1;
-                        stop = true;
-                        break;
+                const size_t step = plane16_block(1, 0, nblk, NPL, 0);
+                const uint16_t *a = jb.A + plane16_block(0, tl.y, nblk, NPL, 0);
+                for (int term = 0; term < jb.T && !stop; ++term) {
+                    const uint16_t *b = jb.B + plane16_block(0, tl.z, nblk, NPL, 0);  // the same for every term
+                    for (int j = 0; j < nch; ++j, ++g, a += step, b += step, ring.next()) {
+                        if (g >= STAGES && !mbar_wait(&empty[ring.s], ring.ph ^ 1u, wait_ns)) {
+                            record_error(err, GW_E_TIMEOUT, SITE_HERK_PRODUCER, blockIdx.x);
+                            *abort_flag = 1;
+                            stop = true;
+                            break;
+                        }
+                        if (*abort_flag) {
+                            stop = true;
+                            break;
+                        }
+                        uint8_t *st = smem + ring.s * STAGE_BYTES;
+                        mbar_arrive_expect_tx(&full[ring.s], STAGE_BYTES);
+                        bulk_g2s(st, a, 4 * PL, &full[ring.s]);
+                        bulk_g2s(st + B_OFF, b, 4 * PL, &full[ring.s]);
+                        *n_issued = g + 1;
                     }
-                    if (*abort_flag) {
-                        stop = true;
-                        break;
-                    }
-                    uint8_t *st = smem + s * STAGE_BYTES;
-                    mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-                    bulk_g2s(st, jb.F + plane16_block(kc, tl.y, nblk, NPL, 0), 4 * PL, &full[s]);
-                    bulk_g2s(st + B_OFF, jb.F + plane16_block(kc, tl.z, nblk, NPL, 0), 4 * PL, &full[s]);
-                    *n_issued = g + 1;
                 }
             }
         }
         __syncwarp();
     } else if (warp == MMA_WARP) {
         if (lane == 0) {
-            constexpr uint32_t FMT = BF16 ? 1u : 0u;
-            constexpr uint32_t ID = mma_idesc(FMT, TM, 2 * TN, false);
-            constexpr uint32_t ID1 = mma_idesc(FMT, TM, TN, false), ID1N = mma_idesc(FMT, TM, TN, true);
+            constexpr uint32_t FMT = BF16 ? mma_idesc(1u, 0, 0, false) ^ mma_idesc(0u, 0, 0, false) : 0u;
             const uint32_t sbase = smem_u32(smem);
-            long long g = 0, gw = 0;  // chunks and windows consumed by this CTA
+            long long g = 0;
+            uint32_t gw = 0;  // windows issued by this CTA
+            Ring ring;
             bool ok = true;
-            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-                const int4 tl = tiles[t];
-                const int nkc = jobs[tl.x].kpad / KC16;
-                const int nwin = (nkc + W - 1) / W;
-                int kc = 0;
-                for (int win = 0; win < nwin && ok; ++win, ++gw) {
-                    const int b = (int)(gw & 1);
-                    if (gw >= 2 && !mbar_wait(&acce[b], (uint32_t)(((gw >> 1) - 1) & 1), wait_ns)) {
+            // one window of n chunks into TMEM buffer gw & 1; the formats' bits of the descriptors: fmt
+            auto window = [&](int n, uint32_t fmt) {
+                const int b = (int)(gw & 1u);
+                if (gw >= 2 && !mbar_wait(&acce[b], ((gw >> 1) - 1u) & 1u, wait_ns)) {
+                    record_error(err, GW_E_TIMEOUT, SITE_HERK_MMA, blockIdx.x);
+                    *abort_flag = 1;
+                    return false;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + b * 256;
+                const uint32_t ID = mma_idesc(0u, TM, 2 * TN, false) | fmt;
+                const uint32_t ID1 = mma_idesc(0u, TM, TN, false) | fmt, ID1N = mma_idesc(0u, TM, TN, true) | fmt;
+                for (int c = 0; c < n; ++c, ++g, ring.next()) {
+                    const int s = ring.s;
+                    if (!mbar_wait(&full[s], ring.ph, wait_ns)) {
                         record_error(err, GW_E_TIMEOUT, SITE_HERK_MMA, blockIdx.x);
                         *abort_flag = 1;
-                        ok = false;
-                        break;
+                        return false;
                     }
                     tc_fence_after();
-                    const uint32_t d = tmem + b * 256;
-                    const int kend = min(nkc, kc + W);
-                    for (int c = 0; kc < kend; ++kc, ++c, ++g) {
-                        const int s = (int)(g % STAGES);
-                        if (!mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1), wait_ns)) {
-                            record_error(err, GW_E_TIMEOUT, SITE_HERK_MMA, blockIdx.x);
-                            *abort_flag = 1;
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t st = sbase + s * STAGE_BYTES;
-                        const uint64_t a_ih = smem_desc(st, LBO, SBO), a_rh = smem_desc(st + PL, LBO, SBO);
-                        const uint64_t a_il = smem_desc(st + 2 * PL, LBO, SBO);
-                        const uint64_t a_rl = smem_desc(st + 3 * PL, LBO, SBO);
-                        const uint64_t b_ih = smem_desc(st + B_OFF, LBO, SBO);
-                        const uint64_t b_rh = smem_desc(st + B_OFF + PL, LBO, SBO);
-                        const uint64_t b_il = smem_desc(st + B_OFF + 2 * PL, LBO, SBO);
-                        const uint64_t b_rl = smem_desc(st + B_OFF + 3 * PL, LBO, SBO);
-                        const uint32_t acc = c > 0 ? 1u : 0u;
-                        mma_f16(d, a_ih, b_ih, ID, acc);       // Re += Ai Bi, Im += Ai Br
-                        mma_f16(d, a_ih, b_il, ID, 1);
-                        mma_f16(d, a_il, b_ih, ID, 1);
-                        mma_f16(d, a_rh, b_rh, ID1, 1);        // Re += Ar Br
-                        mma_f16(d, a_rh, b_rl, ID1, 1);
-                        mma_f16(d, a_rl, b_rh, ID1, 1);
-                        mma_f16(d + 128, a_rh, b_ih, ID1N, 1);  // Im -= Ar Bi
-                        mma_f16(d + 128, a_rh, b_il, ID1N, 1);
-                        mma_f16(d + 128, a_rl, b_ih, ID1N, 1);
-                        mma_commit(&empty[s]);
-                        *n_consumed = g + 1;
-                    }
-                    if (ok)
-                        mma_commit(&accf[b]);
+                    const uint32_t st = sbase + s * STAGE_BYTES;
+                    const uint64_t a_ih = smem_desc(st, LBO, SBO), a_rh = smem_desc(st + PL, LBO, SBO);
+                    const uint64_t a_il = smem_desc(st + 2 * PL, LBO, SBO);
+                    const uint64_t a_rl = smem_desc(st + 3 * PL, LBO, SBO);
+                    const uint64_t b_ih = smem_desc(st + B_OFF, LBO, SBO);
+                    const uint64_t b_rh = smem_desc(st + B_OFF + PL, LBO, SBO);
+                    const uint64_t b_il = smem_desc(st + B_OFF + 2 * PL, LBO, SBO);
+                    const uint64_t b_rl = smem_desc(st + B_OFF + 3 * PL, LBO, SBO);
+                    const uint32_t acc = c > 0 ? 1u : 0u;
+                    mma_f16(d, a_ih, b_ih, ID, acc);       // Re += Ai Bi, Im += Ai Br
+                    mma_f16(d, a_ih, b_il, ID, 1);
+                    mma_f16(d, a_il, b_ih, ID, 1);
+                    mma_f16(d, a_rh, b_rh, ID1, 1);        // Re += Ar Br
+                    mma_f16(d, a_rh, b_rl, ID1, 1);
+                    mma_f16(d, a_rl, b_rh, ID1, 1);
+                    mma_f16(d + 128, a_rh, b_ih, ID1N, 1);  // Im -= Ar Bi
+                    mma_f16(d + 128, a_rh, b_il, ID1N, 1);
+                    mma_f16(d + 128, a_rl, b_ih, ID1N, 1);
+                    mma_commit(&empty[s]);
+                    *n_consumed = g + 1;
+                }
+                if (own)
+                    mma_commit(&accf[b]);
+                ++gw;
+                return true;
+            };
+            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+                const HerkJob jb = jobs[tiles[t].x];
+                const Windows w(jb, W);
+                for (int term = 0; term < jb.T && ok; ++term) {
+                    for (int i = 0; i < w.nwc && ok; ++i)
+                        ok = window(min(W, jb.ncc - i * W), FMT);
+                    for (int i = 0; i < w.nwv && ok; ++i)
+                        ok = window(min(w.wv, jb.nvc - i * w.wv), 0u);
                 }
             }
-            mma_commit(done);
+            mma_commit(done);  // arrives once every MMA issued above has completed
         }
         __syncwarp();
     } else {
@@ -194,39 +278,58 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int q = warp & 3, h = warp >> 2;
         const int m = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
-        long long gw = 0;
+        float4 *my = sums + (size_t)blockIdx.x * (SUM_F4 * NPROMO_WARPS * 32) + threadIdx.x;  // stride 256
+        float2 *stage = reinterpret_cast<float2 *>(smem + PIPE_BYTES + BAR_BYTES) + warp * 32 * OUT_PITCH;
+        uint32_t gw = 0;
+        int at = 0;  // chunks seen, modulo 2 STAGES: stage and parity of the next chunk
         bool stop = false;
         float are[64], aim[64];
+        // Wait for the next window (n chunks); the outcome is the same in every lane, as the TMEM loads
+        // need.  The empty barrier of its last chunk cannot complete another phase before the window is
+        // promoted: the chunk STAGES later lies at least two windows on (the next window has at most
+        // W < STAGES chunks), and the MMAs of that window wait for this promotion.
+        auto ready = [&](int n) {
+            at += n;
+            at -= at >= 2 * STAGES ? (at / (2 * STAGES)) * (2 * STAGES) : 0;
+            const int last = at == 0 ? 2 * STAGES - 1 : at - 1;
+            uint64_t *bar = own ? &accf[gw & 1u] : &empty[last >= STAGES ? last - STAGES : last];
+            const uint32_t par = own ? (gw >> 1) & 1u : (last >= STAGES ? 1u : 0u);
+            if (!__all_sync(0xffffffffu, mbar_wait(bar, par, wait_ns))) {
+                if (lane == 0)
+                    record_error(err, GW_E_TIMEOUT, SITE_HERK_EPILOGUE, blockIdx.x);
+                *abort_flag = 1;
+                stop = true;
+                return false;
+            }
+            tc_fence_after();
+            return true;
+        };
+        auto release = [&]() {  // the window's TMEM buffer is free again
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&acce[gw & 1u]);
+            ++gw;
+        };
         for (int t = blockIdx.x; t < n_tiles && !stop; t += gridDim.x) {
             const int4 tl = tiles[t];
-            const HerkJob jb = jobs[tl.x];
-            const int nr = jb.nr;
-            float2 *P = jb.P;
-            const int r = tl.y * TM + m;
-            const int cbase = tl.z * TN + h * 64;
-            const int nkc = jb.kpad / KC16;
-            const int nwin = (nkc + W - 1) / W;
-            const int nseg = (nwin + L - 1) / L;
-            const bool vec_ok = (nr & 1) == 0;
-            int flushed = 0;
+            const HerkJob &jb = jobs[tl.x];  // fields are read as needed: the registers hold the sums
+            const bool sep = jb.nvc > 0;
+            const Windows w(jb, W);
+            // segments: the registers restart from zero in each (a fresh start rather than a conditional
+            // reset keeps all 128 sums in registers)
+            const int nseg = sep ? jb.T : (w.nwc + L - 1) / L;
             for (int seg = 0; seg < nseg && !stop; ++seg) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) {
                     are[i] = 0.f;
                     aim[i] = 0.f;
                 }
-                const int wend = min(nwin, (seg + 1) * L);
-                for (int win = seg * L; win < wend; ++win, ++gw) {
-                    const int b = (int)(gw & 1);
-                    if (!__all_sync(0xffffffffu, mbar_wait(&accf[b], (uint32_t)((gw >> 1) & 1), wait_ns))) {
-                        if (lane == 0)
-                            record_error(err, GW_E_TIMEOUT, SITE_HERK_EPILOGUE, blockIdx.x);
-                        *abort_flag = 1;
-                        stop = true;
+                const int w0 = sep ? 0 : seg * L, w1 = sep ? w.nwc : min(w.nwc, w0 + L);
+                for (int win = w0; win < w1; ++win) {
+                    if (!ready(min(W, jb.ncc - win * W)))
                         break;
-                    }
-                    tc_fence_after();
-                    const uint32_t base = tmem + lane_addr + b * 256 + h * 64;
+                    const uint32_t base = tmem + lane_addr + (gw & 1u) * 256 + h * 64;
 #pragma unroll
                     for (int c0 = 0; c0 < 64; c0 += 16) {
                         float v[16];
@@ -239,73 +342,78 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                         for (int i = 0; i < 16; ++i)
                             aim[c0 + i] += v[i];
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0)
-                        mbar_arrive(&acce[b]);
+                    release();
                 }
-                if (stop || seg + 1 == nseg)
+                if (stop)
                     break;
-                if (r < nr) {
-                    float2 *row = P + (size_t)r * nr + cbase;
-                    const int avail = nr - cbase;
-                    if (vec_ok && avail >= 64) {
-                        float4 *r4 = reinterpret_cast<float4 *>(row);
+                if (!sep) {
 #pragma unroll
-                        for (int g4 = 0; g4 < 8; ++g4) {
-                            float4 o[4];
+                    for (int i = 0; i < SUM_F4; ++i)
+                        sums_add(my + i * 256, make_float4(are[2 * i], aim[2 * i], are[2 * i + 1], aim[2 * i + 1]),
+                                 seg == 0);
+                    continue;
+                }
+                const float vs = jb.term_scale[seg] * ldexpf(1.0f, -2 * jb.scale_exp[1]);
+                for (int win = 0; win < w.nwv; ++win) {
+                    if (!ready(min(w.wv, jb.nvc - win * w.wv)))
+                        break;
+                    const uint32_t base = tmem + lane_addr + (gw & 1u) * 256 + h * 64;
+                    const bool first = seg == 0 && win == 0;
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                o[j] = flushed ? r4[g4 * 4 + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int c0 = 0; c0 < 64; c0 += 8) {
+                        float vr[8], vi[8];
+                        tmem_ld8x2(base + c0, base + 128 + c0, vr, vi);
+                        float4 o[4];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const int i = g4 * 8 + 2 * j;
-                                r4[g4 * 4 + j] = make_float4(o[j].x + are[i], o[j].y + aim[i], o[j].z + are[i + 1],
-                                                             o[j].w + aim[i + 1]);
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            const float x = vr[i] * vs, y = vi[i] * vs;
+                            const float pr = fmaf(x, are[c0 + i], -(y * aim[c0 + i]));
+                            const float pi = fmaf(x, aim[c0 + i], y * are[c0 + i]);
+                            (i & 1 ? o[i / 2].z : o[i / 2].x) = pr;
+                            (i & 1 ? o[i / 2].w : o[i / 2].y) = pi;
                         }
-                    } else {
 #pragma unroll
-                        for (int i = 0; i < 64; ++i)
-                            if (i < avail) {
-                                const float2 o = flushed ? row[i] : make_float2(0.f, 0.f);
-                                row[i] = make_float2(o.x + are[i], o.y + aim[i]);
-                            }
+                        for (int i = 0; i < 4; ++i)
+                            sums_add(my + (c0 / 2 + i) * 256, o[i], first);
                     }
+                    release();
                 }
-                flushed = 1;
             }
-            // every promotion warp has finished this tile's flushes before mirrors are written;
-            // the stop decision is reduced over all promotion threads so all warps take it
-            if (named_bar_or(1, NPROMO_WARPS * 32, stop || *abort_flag != 0))
+            if (stop)
                 break;
-            const float s2 = ldexpf(1.0f, -2 * (*jb.scale_exp));
-            if (flushed && r < nr) {
-                const float2 *row = P + (size_t)r * nr + cbase;
+            // the tile's sums -> P: entries c >= r (real diagonal) in 128-byte row runs through the
+            // warp's stage, their mirror P[c][r] = conj(P[r][c]) straight from the lanes, which hold
+            // consecutive r
+            const int nr = jb.nr, r0 = tl.y * TM + q * 32, r = r0 + lane, cbase = tl.z * TN + h * 64;
+            const float gain = sep ? 1.f + window_loss(jb.ncc, W) + window_loss(jb.nvc, w.wv) : 1.f;
+            const float s2 = -gain * ldexpf(1.0f, -2 * jb.scale_exp[0]);
+            float2 *P = jb.P;
+            for (int g0 = 0; g0 < 64; g0 += OUT_COLS) {
+                float2 x[OUT_COLS];
 #pragma unroll
-                for (int i = 0; i < 64; ++i)
-                    if (cbase + i < nr) {
-                        const float2 o = row[i];
-                        are[i] += o.x;
-                        aim[i] += o.y;
+                for (int i = 0; i < OUT_COLS / 2; ++i) {
+                    const float4 v = sums_load(my + (g0 / 2 + i) * 256);
+                    x[2 * i] = make_float2(v.x * s2, v.y * s2);
+                    x[2 * i + 1] = make_float2(v.z * s2, v.w * s2);
+                }
+#pragma unroll
+                for (int i = 0; i < OUT_COLS; ++i) {
+                    const int col = cbase + g0 + i;
+                    if (r < nr && col < nr && col > r)
+                        P[(size_t)col * nr + r] = make_float2(x[i].x, -x[i].y);
+                    stage[lane * OUT_PITCH + i] = x[i];
+                }
+                __syncwarp();
+#pragma unroll 4
+                for (int p = 0; p < 16; ++p) {
+                    const int row = 2 * p + (lane >> 4), i = lane & 15;
+                    const int rr = r0 + row, col = cbase + g0 + i;
+                    if (rr < nr && col < nr && col >= rr) {
+                        const float2 v = stage[row * OUT_PITCH + i];
+                        P[(size_t)rr * nr + col] = make_float2(v.x, col == rr ? 0.f : v.y);
                     }
-            }
-            named_bar(1, NPROMO_WARPS * 32);
-            if (r < nr) {
-                // direct entries c >= r (real diagonal) from this thread's row
-#pragma unroll
-                for (int i = 0; i < 64; ++i) {
-                    const int col = cbase + i;
-                    if (col < nr && col >= r)
-                        P[(size_t)r * nr + col] = make_float2(-are[i] * s2, col == r ? 0.f : -aim[i] * s2);
                 }
-                // mirrored entries P[c][r] = conj(P[r][c]) for c > r (lanes hold consecutive r)
-#pragma unroll
-                for (int i = 0; i < 64; ++i) {
-                    const int col = cbase + i;
-                    if (col < nr && col > r)
-                        P[(size_t)col * nr + r] = make_float2(-are[i] * s2, aim[i] * s2);
-                }
+                __syncwarp();
             }
         }
     }
@@ -332,22 +440,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 }  // namespace
 
 cudaError_t launch_herk16p(const HerkJob *jobs, const int4 *tiles, int n_tiles, int grid, bool bf16, uint32_t *err,
-                           uint64_t wait_ns, int W, int L, cudaStream_t s)
+                           uint64_t wait_ns, int W, int L, float4 *sums, cudaStream_t s)
 {
     if (n_tiles <= 0)
         return cudaSuccess;
-    cudaError_t e;
-    if (bf16) {
-        e = cudaFuncSetAttribute(herk16p_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-        if (e != cudaSuccess)
-            return e;
-        herk16p_kernel<true><<<grid, NTHREADS, SMEM, s>>>(jobs, tiles, n_tiles, err, wait_ns, W, L);
-    } else {
-        e = cudaFuncSetAttribute(herk16p_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-        if (e != cudaSuccess)
-            return e;
-        herk16p_kernel<false><<<grid, NTHREADS, SMEM, s>>>(jobs, tiles, n_tiles, err, wait_ns, W, L);
-    }
+    auto kernel = bf16 ? herk16p_kernel<true> : herk16p_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+    if (e != cudaSuccess)
+        return e;
+    kernel<<<grid, NTHREADS, SMEM, s>>>(jobs, tiles, n_tiles, err, wait_ns, W, L, sums);
     count_launches(1);
     return cudaGetLastError();
 }

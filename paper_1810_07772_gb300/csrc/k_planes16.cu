@@ -231,6 +231,114 @@ __global__ void __launch_bounds__(256) pair_density16_rows_kernel(const float2 *
     }
 }
 
+// Bits of max |psi_c| (bound_bits[0]) and max |psi_v| (bound_bits[1]): one warp per row of psiT.
+__global__ void state_bound_kernel(const float2 *__restrict__ psiT, int nr, int nb, int nv, unsigned *bound_bits)
+{
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    float mv = 0.f, mc = 0.f;
+    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < nr; r += gridDim.x * wpb)
+        for (int n = lane; n < nb; n += 32) {
+            const float2 z = psiT[(size_t)r * nb + n];
+            const float a = fmaxf(fabsf(z.x), fabsf(z.y));
+            if (n < nv)
+                mv = fmaxf(mv, a);
+            else
+                mc = fmaxf(mc, a);
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        mv = fmaxf(mv, __shfl_xor_sync(0xffffffffu, mv, o));
+        mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, o));
+    }
+    if (lane == 0) {
+        atomicMax(&bound_bits[0], __float_as_uint(mc));
+        atomicMax(&bound_bits[1], __float_as_uint(mv));
+    }
+}
+
+// Exponent e with bound 2^e in [2^13, 2^14) (0 for a zero or a non-finite bound).
+__device__ __forceinline__ int state_exp(unsigned bits)
+{
+    const float b = __uint_as_float(bits);
+    return !(b > 0.f) || !isfinite(b) ? 0 : max(-100, min(100, 13 - ilogbf(b)));
+}
+
+// Operand planes of the separable rank-k update (herk16p_kernel): chunk j < ncc holds 16 unoccupied
+// states psi_c (the last loaded state first), chunk ncc + i 16 conjugated occupied states, zero-padded.  B gets the states, A the
+// states times the factors of term t (tab[t][16 j + k], see sep_factors.h) as chunks t (ncc + nvc) + j.
+// The layout of work is that of pair_density16_rows_kernel: blockIdx.x is an 8-row group, a warp
+// takes a chunk and writes the group's 256 contiguous bytes of each plane.  BF16 concerns the
+// unoccupied chunks; the occupied ones are FP16 always (see herk16p_kernel).  Bound by the plane
+// writes, (T + 1)(nc + nv) N_r 8 bytes; at 24^3 (T = 11, 512 states) 0.68 GB where the pair
+// densities' planes take 1.70 GB.
+template <bool BF16>
+__global__ void __launch_bounds__(256)
+    sep_planes_kernel(const float2 *__restrict__ psiT, const float *__restrict__ tab, int T, int nr, int nb, int nv,
+                      int ncc, int nvc, int nr_pad, int staged, const unsigned *__restrict__ bound_bits,
+                      int *__restrict__ scale_exp, uint16_t *__restrict__ A, uint16_t *__restrict__ B)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    float2 *s_psi = reinterpret_cast<float2 *>(smem);  // [8][nb + PD_LDP_PAD] where it fits
+    const int grp = blockIdx.x, nblk = nr_pad / 128;
+    if (staged) {
+        const int ldp = nb + PD_LDP_PAD;
+        for (int t = threadIdx.x; t < 8 * nb; t += blockDim.x) {
+            const int rr = t / nb, n = t - rr * nb, r = grp * 8 + rr;
+            s_psi[rr * ldp + n] = r < nr ? psiT[(size_t)r * nb + n] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+    }
+    const int ec = BF16 ? 0 : state_exp(bound_bits[0]), ev = state_exp(bound_bits[1]);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        scale_exp[0] = ec;
+        scale_exp[1] = ev;
+    }
+    const float sc = ldexpf(1.0f, ec), sv = ldexpf(1.0f, ev);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rem = 4 * lane;  // element offset in the group's 128
+    const int r8 = (rem & 63) >> 3, kk0 = ((rem & 127) >> 6) * 8 + (rem & 7);
+    const bool live = grp * 8 + r8 < nr;
+    const float2 *row = staged ? s_psi + r8 * (nb + PD_LDP_PAD) : psiT + (size_t)(live ? grp * 8 + r8 : 0) * nb;
+    const int nch = ncc + nvc, ldu = nch * KC16;
+    const int nc = nb - nv;
+    for (int j = blockIdx.y * (blockDim.x >> 5) + warp; j < nch; j += gridDim.y * (blockDim.x >> 5)) {
+        const bool occ = j >= ncc;
+        float xr[4], xi[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int n = (occ ? (j - ncc) : j) * KC16 + kk0 + i;
+            float2 z = make_float2(0.f, 0.f);
+            if (live && n < (occ ? nv : nc))
+                z = row[occ ? n : nb - 1 - n];
+            xr[i] = z.x * (occ ? sv : sc);
+            xi[i] = occ ? -z.y * sv : z.y * sc;
+        }
+        const size_t off = (size_t)(grp & 15) * 128 + rem;
+        auto store = [&](uint16_t *F, int chunk, float4 w) {
+            uint32_t p[4][2];  // Re hi, Re lo, Im hi, Im lo
+            if (BF16 && !occ) {
+                split2<true>(xr[0] * w.x, xr[1] * w.y, p[0][0], p[1][0]);
+                split2<true>(xr[2] * w.z, xr[3] * w.w, p[0][1], p[1][1]);
+                split2<true>(xi[0] * w.x, xi[1] * w.y, p[2][0], p[3][0]);
+                split2<true>(xi[2] * w.z, xi[3] * w.w, p[2][1], p[3][1]);
+            } else {
+                split2<false>(xr[0] * w.x, xr[1] * w.y, p[0][0], p[1][0]);
+                split2<false>(xr[2] * w.z, xr[3] * w.w, p[0][1], p[1][1]);
+                split2<false>(xi[0] * w.x, xi[1] * w.y, p[2][0], p[3][0]);
+                split2<false>(xi[2] * w.z, xi[3] * w.w, p[2][1], p[3][1]);
+            }
+            uint16_t *dst = F + plane16_block(chunk, grp >> 4, nblk, NPL, 0) + off;
+            *reinterpret_cast<uint2 *>(dst + P4_RH * 2048) = make_uint2(p[0][0], p[0][1]);
+            *reinterpret_cast<uint2 *>(dst + P4_RL * 2048) = make_uint2(p[1][0], p[1][1]);
+            *reinterpret_cast<uint2 *>(dst + P4_IH * 2048) = make_uint2(p[2][0], p[2][1]);
+            *reinterpret_cast<uint2 *>(dst + P4_IL * 2048) = make_uint2(p[3][0], p[3][1]);
+        };
+        store(B, j, make_float4(1.f, 1.f, 1.f, 1.f));
+        const float4 *w4 = reinterpret_cast<const float4 *>(tab + (size_t)j * KC16 + kk0);  // kk0: 0, 4, 8 or 12
+        for (int t = 0; t < T; ++t)
+            store(A, t * nch + j, w4[(size_t)t * ldu / 4]);
+    }
+}
+
 // max |M[k][j]| over a complex64 matrix (rows x cols, row stride ld), as float bits.
 __global__ void absmax_c64_kernel(const float2 *__restrict__ M, int rows, int cols, long ld, unsigned *bound_bits)
 {
@@ -327,6 +435,31 @@ cudaError_t launch_pair_density16(const float2 *psiT, const float *sw, float sw_
         pair_density16_kernel<true><<<grid, 256, 0, s>>>(psiT, sw, nr, nb, nv, nc, kpad, nr_pad, npl, scale_exp, F);
     else
         pair_density16_kernel<false><<<grid, 256, 0, s>>>(psiT, sw, nr, nb, nv, nc, kpad, nr_pad, npl, scale_exp, F);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sep_planes(const float2 *psiT, const float *tab, int T, int nr, int nb, int nv, int ncc, int nvc,
+                              int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint16_t *A, uint16_t *B,
+                              cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(bound_bits, 0, 2 * sizeof(unsigned), s);
+    if (e != cudaSuccess)
+        return e;
+    state_bound_kernel<<<std::max(1, std::min((nr + 7) / 8, 152 * 16)), 256, 0, s>>>(psiT, nr, nb, nv, bound_bits);
+    count_launches(1);
+    size_t smem = (size_t)8 * (nb + PD_LDP_PAD) * sizeof(float2);
+    const int staged = smem <= 100 * 1024;
+    if (!staged)
+        smem = 0;
+    auto kernel = bf16 ? sep_planes_kernel<true> : sep_planes_kernel<false>;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    // parts of the chunks per row group: about four blocks per SM-resident slot, a chunk per warp at least
+    const int ngrp = nr_pad / 8, nch = ncc + nvc;
+    const int parts = std::max(1, std::min((nch + 7) / 8, (152 * 6 * 4 + ngrp - 1) / ngrp));
+    kernel<<<dim3(ngrp, parts), 256, smem, s>>>(psiT, tab, T, nr, nb, nv, ncc, nvc, nr_pad, staged, bound_bits,
+                                                scale_exp, A, B);
     count_launches(1);
     return cudaGetLastError();
 }

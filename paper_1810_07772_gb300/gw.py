@@ -24,7 +24,7 @@ HERK_KERNEL = {"single": 0, "pair": 1}
 TRANSFORM_KERNEL = {"two_kernel": 0, "fused": 1, "tables": 2}
 ZGEMM_MODE = {"fp16x3": 0, "slices": 1}
 GW_C64, GW_C128 = 0, 1
-BUF = {"P": 0, "F": 1, "PG": 2, "eps": 3, "epsinv": 4, "weights": 5, "psiT": 6}
+BUF = {"P": 0, "F": 1, "PG": 2, "eps": 3, "epsinv": 4, "weights": 5, "psiT": 6, "factors": 7}
 
 # Every symbol include/gw.h declares, with its ctypes signature.
 _c = ctypes
@@ -355,6 +355,18 @@ class Context:
         keys = ["kernel_launches", "newton_iters", "herk_ms_mean", "herk_calls", "fp16_scale_exp", "herk_tiles",
                 "window_chunks", "flush_windows"]
         return dict(zip(keys, list(d)))
+
+    def update_form(self):
+        """The last 16-bit build_P: terms of its separable form (0 = pair by pair) and the 16-wide chunks
+        of states or pairs contracted per tile."""
+        per_term = -(-self.nv // 16) + -(-self.nc // 16)
+        try:
+            terms = self.buffer("factors")[1] // (per_term * 16 * 4)
+        except GwError as e:
+            if e.status != GW_E_NOT_READY:
+                raise
+            terms = 0
+        return {"terms": terms, "chunks": terms * per_term if terms else -(-self.nv * self.nc // 16)}
 
     def set_herk_window(self, window_chunks, flush_windows):
         self._check(lib().gw_set_herk_window(self._h, int(window_chunks), int(flush_windows)))

@@ -1,0 +1,128 @@
+"""The separable form of the 16-bit rank-k update (gw_build_P where T (nv + nc) states are fewer than
+nv nc pairs) against the FP64 sum of Eq. (Pstatic), at the edges of its tiles and chunks.
+
+Bars as in test_gpu_parity: FP16X3 1e-6 relative at the default window, 2e-6 at any window; BF16X3
+1e-5 (the 8 + 8-bit split: 4.5e-6 measured in the pair form, which the separable form must not exceed by
+more than its spread)."""
+import numpy as np
+import pytest
+
+from oracle import gw_oracle as O
+from paper_1810_07772_gb300 import gw, inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+def build(dims, nv, nc, psi, E, prec="fp16x3", window=None, kind="single"):
+    nr = int(np.prod(dims))
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        ctx.set_herk_kernel(kind)
+        if window:
+            ctx.set_herk_window(*window)
+        P = torch.empty((nr, nr), dtype=torch.complex64, device="cuda:0")
+        ctx.build_P(prec, P_out=P)
+        ctx.sync()
+        return P, ctx.update_form()
+
+
+# exact multiples of 128 rows and 16 states; one state beyond a chunk on both sides; ragged rows with
+# a 1-row last block; several occupied chunks; fewer tiles than SMs and more
+CASES = [((8, 8, 8), 16, 208, 1), ((7, 9, 11), 33, 97, 2), ((3, 11, 27), 33, 160, 3), ((9, 10, 11), 70, 81, 4),
+         ((16, 16, 13), 24, 200, 5)]
+
+
+@pytest.mark.parametrize("dims,nv,nc,seed", CASES)
+@pytest.mark.parametrize("window", [None, (1, 1), (5, 256), (6, 256), (64, 4096)])
+def test_matches_fp64(dims, nv, nc, seed, window):
+    psi, E = inputs.make_states(0, nv, nc, seed, dims=dims)
+    P, form = build(dims, nv, nc, psi, E, window=window)
+    assert form["terms"] > 1 and form["chunks"] == form["terms"] * (-(-nv // 16) + -(-nc // 16))
+    ref = O.P_rspace(psi, E, nv)
+    P = P.cpu().numpy()
+    assert rel(P, ref) <= (1e-6 if window is None else 2e-6)
+    assert np.array_equal(P, P.conj().T) and not np.diag(P).imag.any()
+
+
+@pytest.mark.parametrize("window", [None, (16, 256)])
+def test_bf16(window):
+    dims, nv, nc = (7, 9, 11), 33, 97
+    psi, E = inputs.make_states(0, nv, nc, 2, dims=dims)
+    P, form = build(dims, nv, nc, psi, E, "bf16x3", window)
+    assert form["terms"] > 1 and rel(P.cpu().numpy(), O.P_rspace(psi, E, nv)) <= 1e-5
+
+
+def test_energies_in_any_order_and_degenerate():
+    """Unsorted energies and shells of equal ones; the states' amplitudes differ by orders of magnitude
+    (unnormalised input), which the per-set power-of-two scales must carry."""
+    dims, nv, nc = (7, 9, 11), 20, 110
+    rng = np.random.default_rng(9)
+    psi, _ = inputs.make_states(0, nv, nc, 6, dims=dims)
+    psi = psi * np.concatenate([np.full(nv, 1e-7), np.full(nc, 300.0)])[:, None]
+    E = np.concatenate([np.round(rng.uniform(-8, 0, nv)), 0.5 + np.round(rng.uniform(0, 12, nc))])
+    P, form = build(dims, nv, nc, psi, E)
+    assert form["terms"] > 1 and rel(P.cpu().numpy(), O.P_rspace(psi, E, nv)) <= 1e-6
+
+
+def test_kernel_setting_and_pair_densities_afterwards():
+    """GW_HERK_PAIR gives the same P; GW_BUF_F still holds the pair densities when it is asked for."""
+    from test_gpu_parity import _decode_16
+    dims, nv, nc = (8, 8, 8), 16, 208
+    psi, E = inputs.make_states(0, nv, nc, 1, dims=dims)
+    a, _ = build(dims, nv, nc, psi, E)
+    b, form = build(dims, nv, nc, psi, E, kind="pair")
+    assert torch.equal(a, b) and form["terms"] > 1
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        ctx.build_P("fp16x3")
+        ptr, nbytes = ctx.buffer("F")
+        torch.cuda.synchronize()
+        F = torch.as_tensor(gw.DeviceView(ptr, (nbytes,), "|u1"), device="cuda:0").cpu().numpy()
+        e = int(ctx.stats()["fp16_scale_exp"])
+        f, _ = _decode_16(F, ctx.dims8()[7], 512, nv * nc, bf16=False)
+    assert rel(f / 2.0 ** e, O.pair_density(psi, E, nv).T) < 1e-6
+
+
+def test_batch_of_both_forms_equals_single_instances():
+    """One launch over a separable, a pair-form and another separable instance, replayed from the graph
+    and after a change of window: bit for bit the single-instance P~."""
+    systems = [((9, 10, 11), 24, 200, 5, 71), ((8, 10, 12), 3, 30, 6, 73), ((12, 12, 12), 33, 97, 8, 72)]
+    loaded = []
+    for dims, nv, nc, gcut, seed in systems:
+        psi, E = inputs.make_states(0, nv, nc, seed, dims=dims)
+        loaded.append((torch.from_numpy(psi.astype(np.complex64)).cuda(), E))
+
+    def single(W):
+        out = []
+        for (dims, nv, nc, gcut, _), (psi, E) in zip(systems, loaded):
+            with gw.Context(0) as ctx:
+                ctx.load_states(psi, E, dims, nv)
+                ctx.set_herk_window(W, 256)
+                ctx.build_P("fp16x3")
+                form = ctx.update_form()["terms"]
+                ctx.P_to_G(gcut)
+                out.append((ctx.view("PG").clone(), form))
+        return out
+
+    ctxs = []
+    for (dims, nv, nc, gcut, _), (psi, E) in zip(systems, loaded):
+        ctx = gw.Context(0)
+        ctx.load_states(psi, E, dims, nv)
+        ctxs.append(ctx)
+    with gw.Batch(ctxs, [s[3] for s in systems]) as b:
+        for W in (2, 7):
+            b.set_window(W, 256)
+            ref = single(W)
+            assert [f > 0 for _, f in ref] == [True, False, True]
+            for _ in range(3):
+                b.run(use_graph=True)
+                for c, (PG, _) in zip(ctxs, ref):
+                    assert torch.equal(c.view("PG"), PG)
+    for c in ctxs:
+        c.close()
