@@ -243,6 +243,7 @@ gw_status upload_sqrt_v(Ctx &c)
 gw_status build_plan(Ctx &c, int gcut)
 {
     const int n[3] = {c.n1, c.n2, c.n3};
+    c.gcut = -1;  // no plan until this one is complete
     const auto g = sphere_vectors(n, gcut);
     const int ng = static_cast<int>(g.size());
     std::vector<int> m3vals;
@@ -936,6 +937,13 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     c.loaded = c.P_ready = c.PG_ready = c.eps_ready = false;
     c.q_pairs = false;
     c.sep_known = false;
+    // The sphere plan depends on the grid and the cut only (its sqrt(V) on the cell and q): states of
+    // another system, k-point or step on the same grid and cell keep it.  Building it takes the host 50 us
+    // at 12^3 and 130 us at 24^3, with the GPU idle.
+    if (c.gcut >= 0 && (n1 != c.n1 || n2 != c.n2 || n3 != c.n3 || cell_L != c.cell_L)) {
+        c.gcut = -1;
+        c.ng = 0;
+    }
     c.n1 = n1;
     c.n2 = n2;
     c.n3 = n3;
@@ -948,8 +956,6 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     c.kpad = ((c.k + HERK_KC - 1) / HERK_KC) * HERK_KC;
     c.sw_max = static_cast<float>(std::sqrt(2.0 / ((emin_c - emax_v) / HARTREE_EV)));
     c.nr_pad = ((nr + HERK_BN - 1) / HERK_BN) * HERK_BN;
-    c.gcut = -1;
-    c.ng = 0;
     const size_t n = (size_t)nb * nr;
     cudaStream_t s = c.stream;
     GW_TRY(ensure(c, c.d_psiT, c.cap.psiT, n * sizeof(float2), "transposed states"));
