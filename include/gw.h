@@ -89,12 +89,12 @@ typedef enum gw_inv_method {
     GW_INV_NEWTON_TC = 2   /* the Newton iteration of Sec. 5.1 on the 16-bit tensor cores, for a  */
                            /* Hermitian positive definite eps: FP16X3 steps from the Jacobi-scaled */
                            /* X0 = 2/(1+u) diag(eps)^-1 (u = max row sum of the scaled |eps|) to  */
-                           /* max |I - eps X| < 3e-5, then two                                     */
-                           /* refinements R = I - eps X, X <- X + X R with R exact to FP64 from   */
-                           /* integer slices (see gw_zgemm_tc); GW_E_NUMERIC if the residual      */
-                           /* before the last refinement exceeds 1e-8.  gw_eps_inv replays it     */
-                           /* from a CUDA graph with 8 FP16X3 steps queued; an eps that needs    */
-                           /* more is finished by the eager form (up to 16, host-checked)         */
+                           /* max |I - X eps| < 2e-4 and one more, then up to three refinements    */
+                           /* X <- X + R X with R = I - X eps exact to FP64 from integer slices;  */
+                           /* GW_E_NUMERIC if the residual before the last refinement exceeds     */
+                           /* 1e-8.  gw_eps_inv replays it from a CUDA graph with 8 FP16X3 steps   */
+                           /* queued; an eps that needs more is finished by the eager form (up to 16, */
+                           /* host-checked)                                                        */
 } gw_inv_method;
 
 typedef enum gw_dtype { GW_C64 = 0, GW_C128 = 1 } gw_dtype;

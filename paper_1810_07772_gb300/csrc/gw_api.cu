@@ -480,24 +480,26 @@ void drop_ns_graph(Ctx &c)
     c.ns_key = Ctx::NsKey{};
 }
 
+// Queue the copy of the inverse's scalars that newton_tc_record reads after the next synchronisation.
+gw_status queue_ns_report(Ctx &c, int n)
+{
+    if (!c.h_nsrep)
+        GW_CUDA(cudaMallocHost(&c.h_nsrep, ns_report_bytes()), "Newton report");
+    GW_CUDA(ns_report_copy(c.d_tcw, n, c.h_nsrep, c.stream), "Newton report");
+    return GW_OK;
+}
+
 // The tensor-core Newton inverse of A (n x n) into X.  With use_graph, every step is queued in its
-// graph-safe form (tables uploaded beforehand, device flags skip the unneeded steps, no host reads)
-// and captured once into a CUDA graph per (n, buffers, wait limit, stream), then replayed: the
+// graph-safe form (device words skip the unneeded steps, no host reads) and captured once into a CUDA graph per (n, buffers, wait limit, stream), then replayed: the
 // eager form stops queuing on host reads of the convergence flag, which leave the GPU idle.
 gw_status inverse_newton_tc(Ctx &c, const double2 *A, int n, double2 *X, bool use_graph = false)
 {
     const int nsm = sm_count(c.device);
-    GW_TRY(ensure(c, c.d_tcw, c.cap.tcw, ns_work_bytes(n, nsm), "tensor-core Newton workspace"));
-    GW_TRY(ensure(c, c.d_scal, c.cap.scal, 4 * sizeof(double), "Newton scalars"));
+    GW_TRY(ensure(c, c.d_tcw, c.cap.tcw, ns_work_bytes(n), "tensor-core Newton workspace"));
     const uint64_t wait_ns = static_cast<uint64_t>(c.wait_limit_ms * 1e6);
     if (!use_graph) {
-        // the eager form uploads the tables of order n into the workspace: a graph captured for
-        // another order would then read tables of the wrong layout
-        if (c.ns_exec && c.ns_key.n != n)
-            drop_ns_graph(c);
-        GW_CUDA(ns_inverse_enqueue(A, n, X, c.d_tcw, c.d_scal, c.d_err, wait_ns, nsm, c.stream),
-                "tensor-core Newton inverse");
-        return GW_OK;
+        GW_CUDA(ns_inverse_enqueue(A, n, X, c.d_tcw, c.d_err, wait_ns, nsm, c.stream), "tensor-core Newton inverse");
+        return queue_ns_report(c, n);
     }
     Ctx::NsKey key;
     key.n = n;
@@ -509,7 +511,6 @@ gw_status inverse_newton_tc(Ctx &c, const double2 *A, int n, double2 *X, bool us
     key.s = c.stream;
     if (!c.ns_exec || !(key == c.ns_key)) {
         drop_ns_graph(c);
-        GW_CUDA(ns_prepare(c.d_tcw, n, nsm, c.stream), "Newton tables");
         // captured on a private stream (the caller's may be the legacy default stream, which
         // cannot be captured); the graph is then launched on the caller's stream
         if (!c.ns_cap_stream)
@@ -522,8 +523,8 @@ gw_status inverse_newton_tc(Ctx &c, const double2 *A, int n, double2 *X, bool us
         // the graph queues NS_GRAPH_STEPS FP16X3 steps (every queued step costs a launch even when
         // its flag makes it return at once); an eps that needs more is finished by the eager form
         // (gw_eps_inv retries on the NS_DETAIL_CAP status)
-        const cudaError_t eq = ns_inverse_enqueue(A, n, X, c.d_tcw, c.d_scal, c.d_err, wait_ns, nsm,
-                                                  c.ns_cap_stream, true, NS_GRAPH_STEPS);
+        const cudaError_t eq = ns_inverse_enqueue(A, n, X, c.d_tcw, c.d_err, wait_ns, nsm, c.ns_cap_stream, true,
+                                                  NS_GRAPH_STEPS);
         g_launches.store(counted);  // captured launches run at replay time, where they are counted
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(c.ns_cap_stream, &g);
@@ -544,19 +545,15 @@ gw_status inverse_newton_tc(Ctx &c, const double2 *A, int n, double2 *X, bool us
     }
     GW_CUDA(cudaGraphLaunch(c.ns_exec, c.stream), "Newton graph launch");
     count_launches(static_cast<int>(c.ns_graph_kernels));
-    return GW_OK;
+    return queue_ns_report(c, n);
 }
 
-// Report of the last tensor-core Newton inverse of order n (after the stream has been
-// synchronised): FP16X3 steps, residual after phase 1, last measured residual, refinements.
-void newton_tc_record(Ctx &c, int n)
+// Report of the last tensor-core Newton inverse (after the stream has been synchronised): FP16X3
+// steps, residual after phase 1, last measured residual, refinements.
+void newton_tc_record(Ctx &c)
 {
-    double r[4] = {-1, -1, -1, -1};
-    if (ns_report(c.d_tcw, n, sm_count(c.device), r) != cudaSuccess)
-        cudaGetLastError();
-    c.newton_iters = static_cast<int>(r[0]);
-    for (int i = 0; i < 4; ++i)
-        c.tc_report[i] = r[i];
+    ns_report(c.h_nsrep, c.tc_report);
+    c.newton_iters = static_cast<int>(c.tc_report[0]);
 }
 
 // Separable form of the 16-bit rank-k update for the loaded energies: c.sep.T terms, 0 where the pair
@@ -679,6 +676,9 @@ void Ctx::release()
     if (ns_cap_stream)
         cudaStreamDestroy(ns_cap_stream);
     ns_cap_stream = nullptr;
+    if (h_nsrep)
+        cudaFreeHost(h_nsrep);
+    h_nsrep = nullptr;
     dfree(d_scal);
     dfree(d_tcw);
     dfree(d_csw);
@@ -1515,7 +1515,7 @@ gw_status gw_eps_inv(gw_ctx *h, int method, void *eps_out, void *epsinv_out)
     }
     resolve_times(c);
     if (method == GW_INV_NEWTON_TC)
-        newton_tc_record(c, ng);
+        newton_tc_record(c);
     c.eps_ready = st == GW_OK;
     return st;
 }
@@ -1721,7 +1721,7 @@ gw_status gw_zinv_tc(gw_ctx *h, int n, const void *A, void *X)
     GW_CUDA(cudaSetDevice(c.device), "set device");
     GW_TRY(inverse_newton_tc(c, static_cast<const double2 *>(A), n, static_cast<double2 *>(X)));
     const gw_status st = read_device_status(c);
-    newton_tc_record(c, n);
+    newton_tc_record(c);
     return st;
 }
 
@@ -1931,10 +1931,7 @@ gw_status batch_prepare(gw_batch &b)
         GW_TRY(ensure(c, c.d_eps, c.cap.eps, (size_t)ng * ng * sizeof(double2), "eps"));
         GW_TRY(ensure(c, c.d_epsinv, c.cap.epsinv, (size_t)ng * ng * sizeof(double2), "eps^-1"));
         if (b.inv_method == GW_INV_NEWTON_TC) {
-            const int nsm = sm_count(c.device);
-            GW_TRY(ensure(c, c.d_tcw, c.cap.tcw, ns_work_bytes(ng, nsm), "tensor-core Newton workspace"));
-            GW_TRY(ensure(c, c.d_scal, c.cap.scal, 4 * sizeof(double), "Newton scalars"));
-            GW_CUDA(ns_prepare(c.d_tcw, ng, nsm, b.stream), "Newton tables");
+            GW_TRY(ensure(c, c.d_tcw, c.cap.tcw, ns_work_bytes(ng), "tensor-core Newton workspace"));
         } else {
             const size_t work = (size_t)3 * ng * ng + (size_t)NB * ng + (size_t)nblk * NB * NB;
             GW_TRY(ensure(c, c.d_work, c.cap.work, work * sizeof(double2), "inverse workspace"));
@@ -2028,8 +2025,7 @@ gw_status batch_enqueue(gw_batch &b)
         GW_CUDA(launch_eps_build(c.d_PG, c.d_sv, ng, c.d_eps, s), "eps build");
         if (b.inv_method == GW_INV_NEWTON_TC) {
             const uint64_t wait_ns = static_cast<uint64_t>(c.wait_limit_ms * 1e6);
-            GW_CUDA(ns_inverse_enqueue(c.d_eps, ng, c.d_epsinv, c.d_tcw, c.d_scal, c.d_err, wait_ns,
-                                       sm_count(c.device), s, true),
+            GW_CUDA(ns_inverse_enqueue(c.d_eps, ng, c.d_epsinv, c.d_tcw, c.d_err, wait_ns, sm_count(c.device), s, true),
                     "tensor-core Newton inverse");
         } else {
             GW_TRY(inverse_cholesky(c, s));

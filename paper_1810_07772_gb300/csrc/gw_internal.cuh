@@ -143,6 +143,7 @@ struct Ctx {
     void *d_tcw = nullptr;          // workspace of the tensor-core Newton iteration / gw_zgemm_tc
     bool eps_ready = false;
     int newton_iters = 0;
+    void *h_nsrep = nullptr;        // pinned: its scalars (ns_report_copy)
     double tc_report[4] = {-1, -1, -1, -1};  // last tensor-core Newton inverse (gw_newton_tc_report)
     // gw_eps_inv's tensor-core inverse as a captured CUDA graph, valid for the key below
     cudaGraph_t ns_graph = nullptr;
@@ -422,13 +423,12 @@ cudaError_t launch_row_abs_sum_max(const double2 *A, int n, double *out, cudaStr
 struct ZPlan {
     int mode = 0;  // 0 = FP16X3 split, 1 = integer slices (FP64 accuracy)
     int M = 0, N = 0, K = 0, Mpad = 0, Npad = 0, nkc = 0, ntiles = 0, nslots = 0, npairs = 0;
-    int ns = 0;   // slices of B (and the pairs t + u < ns); FP16X3: 2 (hi, lo)
-    int nsA = 0;  // slices held in the A planes (>= ns; the refinement reuses eps's nine)
+    int ns = 0;  // slices of either operand (and the pairs t + u < ns); FP16X3: 2 (hi, lo)
     std::vector<int2> host_pairs;
     std::vector<int> host_slots, host_wexp;
     int2 *d_pairs = nullptr;
     int *d_slots = nullptr, *d_wexp = nullptr;
-    void build(int mode, int M, int N, int K, int nsm, int slices = 0, int slicesA = 0);
+    void build(int mode, int M, int N, int K, int nsm);
     size_t table_bytes() const;
     size_t planes_bytes(bool a_operand) const;
     size_t T_bytes() const;
@@ -462,16 +462,19 @@ cudaError_t launch_states_from_g(const float2 *coef, int nb, int npw, const int 
 cudaError_t launch_kweight(float2 *PG, const float2 *sum, size_t n, float w, bool acc, cudaStream_t s);
 cudaError_t zgemm_enqueue(ZPlan &p, const double2 *A, long lda, const double2 *B, long ldb, double2 *C, void *work,
                           uint32_t *err, uint64_t wait_ns, cudaStream_t s);
-size_t ns_work_bytes(int N, int nsm);
-cudaError_t ns_report(const void *work, int N, int nsm, double *out4);
-cudaError_t ns_prepare(void *work, int N, int nsm, cudaStream_t s);
+// k_newton.cu
+size_t ns_work_bytes(int N);
+// ns_report_copy queues a copy of the scalars of the inverse last run on `work` into `host` (ns_report_bytes
+// long); ns_report reads them once it has arrived.
+size_t ns_report_bytes();
+cudaError_t ns_report_copy(const void *work, int N, void *host, cudaStream_t s);
+void ns_report(const void *host, double *out4);
 // max_steps: FP16X3 Newton steps queued in the graph-safe form (at most 16, the eager form's limit).
 // A last residual above the acceptance bar is GW_E_NUMERIC at SITE_NS with detail NS_DETAIL_CAP
 // when phase 1 had not converged within its steps (the eager form, with more steps, may), else 0.
 constexpr int NS_GRAPH_STEPS = 8;   // the typical eps needs 5-6 from the Jacobi-scaled start
 constexpr uint32_t NS_DETAIL_CAP = 1;
-cudaError_t ns_inverse_enqueue(const double2 *A, int N, double2 *Xout, void *work, double *rowsum, uint32_t *err,
-                               uint64_t wait_ns, int nsm, cudaStream_t s, bool graph_safe = false,
-                               int max_steps = 16);
+cudaError_t ns_inverse_enqueue(const double2 *A, int N, double2 *Xout, void *work, uint32_t *err, uint64_t wait_ns,
+                               int nsm, cudaStream_t s, bool graph_safe = false, int max_steps = 16);
 
 }  // namespace gw

@@ -1,28 +1,12 @@
-// Complex GEMM C = A B on the 16-bit tensor cores from sliced FP64 operands, and the Newton
-// iteration X <- X (2I - eps X) of Sec. 5.1 for eps^-1 built on it.
+// Complex GEMM C = A B on the 16-bit tensor cores from sliced FP64 operands (gw_zgemm_tc).
 //
-// FP64 runs at about 1 TFLOP/s on this GPU and FP16 tensor MMAs at about 2 PFLOP/s, so the
-// inverse is carried by the tensor cores:
-//  * Phase 1: Newton iterations whose products use the FP16X3 split (22 significant bits), until
-//    max |I - eps X| < 3e-5, from the Jacobi-scaled start X0 = 2 / (1 + u) D^-1: D = diag(eps)
-//    (through rs_i = 1 / sqrt(eps_ii) in FP32, D^-1 = diag(rs^2)) and
-//    u = max_i rs_i sum_j |eps_ij| rs_j >= lambda_max(D^-1/2 eps D^-1/2).  eps X0 is similar to
-//    2 / (1 + u) D^-1/2 eps D^-1/2, whose eigenvalues lie in (0, 2) for a Hermitian positive
-//    definite eps, and the error e = I - eps X squares each step.  Scaling the rows and columns of
-//    eps by a positive diagonal leaves the scaled matrix, and so the step count, unchanged.  A
-//    diagonal entry that is not positive and finite falls back to X0 = 2 / (1 + u) I with the
-//    plain row-sum bound u = max_i sum_j |eps_ij|.
-//  * Phase 2: up to three refinement steps R = I - eps X, X <- X + X R.  R is computed to FP64 accuracy
-//    from integer slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// FP64 runs at about 1 TFLOP/s on this GPU and FP16 tensor MMAs at about 2 PFLOP/s.  Two splits:
+//  * FP16X3 (22 significant bits): hi*hi + hi*lo + lo*hi accumulated in FP32;
+//  * integer slices, to FP64 accuracy (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
 //    Algorithms 59, 2012): every entry scaled into [-1, 1] is a sum of slices a_t 2^(-6(t+1))
 //    with integer a_0 in [-64, 64] and a_t in [-32, 32] (t >= 1); nine slices keep 54 bits.  The
 //    slice products a_t b_u are exact in FP16 and their sums over one work slot stay below 2^24,
-//    so the FP32 tensor-core accumulation is exact; the slots are scaled by 2^(-6(t+u+2)) and
-//    added in FP64.  X R only needs the relative accuracy of the FP16X3 split, because R is small.
-//    Each refinement squares the residual (plus the FP16X3 error of X R, ~4e-6 |R|); once a
-//    measured residual is <= 1e-9 its correction is the last one (the result then sits near 4e-15).
-//    If three refinements end with a last measured residual above 1e-8 (or a non-finite one), the
-//    inverse is reported as GW_E_NUMERIC.
+//    so the FP32 tensor-core accumulation is exact; the slots are shifted and added in 128-bit integers.
 //
 // Operand planes (K-major, 8-row x 16-byte core matrices, as in the rank-k update): element
 // (r, k) of plane p sits at 16-bit offset ((kc Rpad/128 + r/128) NP + p) 2048 + ((r%128)/8) 128 +
@@ -68,14 +52,10 @@ constexpr uint64_t DRAIN_NS = 2000000000ull;
 
 constexpr int MODE_FP16X3 = 0, MODE_SLICES = 1;
 constexpr int OZ_SLICES = 9;
-constexpr double NS_TOL = 3e-5;     // phase 1 stops below this max |I - eps X|
-constexpr double NS_LAST = 1e-9;    // a refinement whose residual is below this is the last one
-constexpr double NS_ACCEPT = 1e-8;  // largest residual before the last correction
-constexpr int NS_MAX = 16, NS_REFINE = 3;
 
 // Scale exponent e of a matrix from the bits of max(|Re|, |Im|): m (1 + 2^-20) < 2^e, so a max
 // taken in FP32 (relative error 2^-24) still bounds every entry (0 for an all-zero or non-finite
-// matrix; a non-finite residual is caught by the final check).
+// matrix).
 __device__ __forceinline__ int exp_of(const unsigned long long *w)
 {
     const double m = __longlong_as_double((long long)*w);
@@ -147,11 +127,8 @@ __global__ void zmaxabs_kernel(const double2 *__restrict__ M, int rows, int cols
 //           the rest, |a_0| <= 64; so x 2^-e = sum_t a_t 2^(-6 (t + 1)) up to 2^(-6 ns - 1).
 __global__ void __launch_bounds__(512) zslice_kernel(const double2 *__restrict__ M, long ld, int rows, int K,
                                                      int transpose, int Rpad, int mode, int ns, int npl,
-                                                     const unsigned long long *maxw, uint16_t *__restrict__ planes,
-                                                     const int *skip)
+                                                     const unsigned long long *maxw, uint16_t *__restrict__ planes)
 {
-    if (skip && *skip)
-        return;
     __shared__ double2 tile[16][129];
     const int kc = blockIdx.x, rb = blockIdx.y;
     const int k0 = kc * 16, r0 = rb * 128;
@@ -228,12 +205,10 @@ template <bool F3>  // true: FP16X3 slots, one stage per chunk with the pairs (0
 __global__ void __launch_bounds__(ZTHREADS, 2)
     zgemm16_kernel(const uint16_t *__restrict__ Ap, int npA, int Mpad, const uint16_t *__restrict__ Bp, int npB,
                    int Npad, const int2 *__restrict__ pairs, const ZSlot *__restrict__ slots, int ntj,
-                   float2 *__restrict__ T, uint32_t *err, uint64_t wait_ns, const int *skip)
+                   float2 *__restrict__ T, uint32_t *err, uint64_t wait_ns)
 {
     constexpr uint32_t SB = F3 ? ZSTAGE3 : ZSTAGE;
     constexpr int NST = F3 ? ZSTAGES3 : ZSTAGES;
-    if (skip && *skip)
-        return;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + ZPIPE);
     uint64_t *empty = full + NST;
@@ -400,121 +375,20 @@ __global__ void __launch_bounds__(ZTHREADS, 2)
     }
 }
 
-// Words of the scalar area (unsigned long long each), zeroed at the start of an inverse.
-enum NsWord : int {
-    W_EPS = 0,   // max of eps
-    W_X,         // max of the current X
-    W_XN,        // max of the X being written (moved to W_X by the last block)
-    W_Z,         // max of the current Z (2I - eps X) or R
-    W_ZN,
-    W_DEVN,      // max |out - ref I| being accumulated
-    W_RES0,      // residual max |I - eps X| measured by refinement 1 (after phase 1)
-    W_RLAST,     // residual measured by the last refinement that ran
-    W_NREF,      // refinements that ran
-    W_ITERS,     // Newton iterations of phase 1
-    W_COUNT,     // completed blocks of the running combine
-    W_DISCARD,   // deviations nobody reads
-    W_U,         // row-sum bound of lambda_max
-    W_UJ,        // the same bound of the Jacobi-scaled matrix
-    W_RS2,       // max rs_i^2 (the largest entry of X0 / alpha)
-    W_DBAD,      // nonzero: a diagonal entry is not positive and finite (identity start)
-    W_TOTAL
-};
-static_assert(W_TOTAL <= 64, "scalar area");
-
-// What the last block of a combine does with the deviation d = max |out - ref I|.
-enum DevUse : int {
-    DEV_STORE = 0,   // words[dev_to] = d
-    DEV_PHASE1 = 1,  // d < tol: set flags[0] (phase 1 done) and store the iteration count
-    DEV_REFINE = 2,  // words[dev_to] = W_RLAST = d, ++W_NREF; d <= tol: set flags[iter + 1 ..]
-};
-
-// Block and grid reduction of a combine's two maxima (max(|Re|, |Im|) of out into
-// words[acc_max]; deviation into W_DEVN); the last block to finish moves acc_max -> fin_max and
-// acts on the deviation as `use` says.
-__device__ void combine_tail(float best, float dev, unsigned long long *words, int acc_max, int fin_max, int dev_to,
-                             int use, double tol, int iter, int *flags)
-{
-    __shared__ float red[2][32];
-    __shared__ bool last;
-    for (int o = 16; o > 0; o >>= 1) {
-        best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-        dev = fmaxf(dev, __shfl_xor_sync(0xffffffffu, dev, o));
-    }
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-        red[0][warp] = best;
-        red[1][warp] = dev;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {  // one atomic per block and word: same-address atomics serialise
-        for (int w = 1; w < nw; ++w) {
-            best = fmaxf(best, red[0][w]);
-            dev = fmaxf(dev, red[1][w]);
-        }
-        atomicMax(&words[acc_max], (unsigned long long)__double_as_longlong((double)best));
-        atomicMax(&words[W_DEVN], (unsigned long long)__double_as_longlong((double)dev));
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        last = atomicAdd(&words[W_COUNT], 1ull) == (unsigned long long)gridDim.x * gridDim.y - 1;
-    __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        volatile unsigned long long *vw = words;
-        vw[fin_max] = vw[acc_max];
-        vw[acc_max] = 0ull;
-        const unsigned long long d = vw[W_DEVN];
-        const double dv = __longlong_as_double((long long)d);
-        vw[W_DEVN] = 0ull;
-        vw[W_COUNT] = 0ull;
-        if (use == DEV_STORE) {
-            vw[dev_to] = d;
-        } else if (use == DEV_PHASE1) {
-            if (dv < tol) {
-                flags[0] = 1;
-                vw[W_ITERS] = (unsigned long long)iter;
-            }
-        } else {
-            vw[dev_to] = d;
-            vw[W_RLAST] = d;
-            vw[W_NREF] = vw[W_NREF] + 1ull;
-            if (dv <= tol)
-                for (int j = iter + 1; j <= NS_REFINE; ++j)
-                    reinterpret_cast<volatile int *>(flags)[j] = 1;
-        }
-    }
-}
-
-__device__ __forceinline__ float finite_or_inf(float d)
-{
-    return d <= 3.0e38f ? d : __int_as_float(0x7f800000);  // NaN or inf: +inf, which fmaxf keeps
-}
-
-// FP16X3 products: out = cI I + cC 2^(eA + eB - 28) sum_slot T[slot] + cD D, the K-range slots
-// summed in FP32 (their own rounding is below the split's 2^-22), the rest in FP64.
+// FP16X3 products: out = 2^(eA + eB - 28) sum_slot T[slot], the K-range slots summed in FP32 (their own
+// rounding is below the split's 2^-22).
 __global__ void zcombine16_kernel(const float2 *__restrict__ T, int nslots, int Mpad, int Npad,
-                                  const unsigned long long *wA, const unsigned long long *wB, int M, int N, double cI,
-                                  double cC, const double2 *D, double cD, double2 *out, double ref,
-                                  unsigned long long *words, int acc_max, int fin_max, int dev_to, int use, double tol,
-                                  int iter, const int *skip, int *flags)
+                                  const unsigned long long *wA, const unsigned long long *wB, int M, int N,
+                                  double2 *__restrict__ out)
 {
-    if (skip && *skip)
-        return;
-    // FP64 runs at 1/64 of the FP32 rate here, so the product part stays in FP32 (it carries the
-    // split's 22 bits only) and each entry takes one conversion plus the FP64 terms it needs
     __shared__ float s_sc;
     if (threadIdx.x == 0)
-        s_sc = (float)(cC * ldexp(1.0, exp_of(wA) + exp_of(wB) - 28));
+        s_sc = (float)ldexp(1.0, exp_of(wA) + exp_of(wB) - 28);
     __syncthreads();
     const float sc = s_sc;
-    const float cIf = (float)cI, cIref = (float)(cI - ref), cDf = (float)cD;
-    float best = 0.f, dev = 0.f;
     const size_t plane = (size_t)Mpad * Npad;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     for (int r = blockIdx.y; r < M && c < N; r += gridDim.y) {
-        const size_t i = (size_t)r * N + c;
         const float2 *t = T + (size_t)r * Npad + c;
         float sr = 0.f, si = 0.f;
         for (int s = 0; s < nslots; ++s) {
@@ -522,27 +396,8 @@ __global__ void zcombine16_kernel(const float2 *__restrict__ T, int nslots, int 
             sr += v.x;
             si += v.y;
         }
-        const float pr = sr * sc, pi = si * sc;  // the product term, exact scaling by 2^k
-        double xr = (double)pr, xi = (double)pi;
-        float fr = pr, fi = pi, dr = pr;
-        if (r == c) {
-            xr += cI;
-            fr += cIf;
-            dr += cIref;
-        }
-        if (D) {
-            const double2 d = D[i];
-            xr = fma(cD, d.x, xr);
-            xi = fma(cD, d.y, xi);
-            fr += cDf * (float)d.x;
-            fi += cDf * (float)d.y;
-            dr = fr - (r == c ? (float)ref : 0.f);
-        }
-        out[i] = make_double2(xr, xi);
-        best = fmaxf(best, fmaxf(fabsf(fr), fabsf(fi)));
-        dev = fmaxf(dev, finite_or_inf(sqrtf(dr * dr + fi * fi)));
+        out[(size_t)r * N + c] = make_double2((double)(sr * sc), (double)(si * sc));
     }
-    combine_tail(best, dev, words, acc_max, fin_max, dev_to, use, tol, iter, flags);
 }
 
 // Exact 128-bit integer -> double (one rounding in each half; the halves do not cancel).
@@ -557,35 +412,22 @@ __device__ __forceinline__ double i128_to_double(__int128 a)
 
 // Integer-slice products: every slot tile is an exact integer below 2^24 with weight
 // 2^(wexp - 60 + 60) = 2^(-6(d + 2)); sum_slot T 2^(wexp + 60) is added up exactly in 128-bit
-// integers, so out = sign (2^(eA + eB - 60) (that sum)) (+ I when identity = 1, added in the same
-// integer units, which keeps I - eps X exact) is rounded once.
+// integers, so out = 2^(eA + eB - 60) (that sum) is rounded once.
 __global__ void zcombine_int_kernel(const float2 *__restrict__ T, int nslots, const int *__restrict__ wexp, int Mpad,
                                     int Npad, const unsigned long long *wA, const unsigned long long *wB, int M, int N,
-                                    int identity, int negate, double2 *out, double ref, unsigned long long *words,
-                                    int acc_max, int fin_max, int dev_to, int use, double tol, int iter,
-                                    const int *skip, int *flags)
+                                    double2 *__restrict__ out)
 {
-    if (skip && *skip)
-        return;
     __shared__ int shift[256];
-    __shared__ int s_eab;
     __shared__ double s_sc;
     for (int s = threadIdx.x; s < nslots && s < 256; s += blockDim.x)
         shift[s] = wexp[s] + 60;  // 6 (8 - d) in [0, 48]
-    if (threadIdx.x == 0) {
-        s_eab = exp_of(wA) + exp_of(wB);
-        s_sc = ldexp(1.0, s_eab - 60);
-    }
+    if (threadIdx.x == 0)
+        s_sc = ldexp(1.0, exp_of(wA) + exp_of(wB) - 60);
     __syncthreads();
-    const int eab = s_eab;
-    const int ish = 60 - eab;  // I in units of 2^(eab - 60)
-    const bool exact_i = ish >= 0 && ish <= 120;
     const double sc = s_sc;
-    float best = 0.f, dev = 0.f;
     const size_t plane = (size_t)Mpad * Npad;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     for (int r = blockIdx.y; r < M && c < N; r += gridDim.y) {
-        const size_t i = (size_t)r * N + c;
         const float2 *t = T + (size_t)r * Npad + c;
         __int128 ar = 0, ai = 0;
         for (int s = 0; s < nslots; ++s) {
@@ -593,95 +435,8 @@ __global__ void zcombine_int_kernel(const float2 *__restrict__ T, int nslots, co
             ar += (__int128)__float2int_rn(v.x) << shift[s];
             ai += (__int128)__float2int_rn(v.y) << shift[s];
         }
-        if (negate) {
-            ar = -ar;
-            ai = -ai;
-        }
-        const bool diag = identity && r == c;
-        if (diag && exact_i)
-            ar += (__int128)1 << ish;
-        double xr = i128_to_double(ar) * sc, xi = i128_to_double(ai) * sc;
-        if (diag && !exact_i)
-            xr += 1.0;
-        out[i] = make_double2(xr, xi);
-        const float fr = (float)xr, fi = (float)xi;
-        best = fmaxf(best, fmaxf(fabsf(fr), fabsf(fi)));
-        const float dr = r == c ? (float)(xr - ref) : fr;
-        dev = fmaxf(dev, finite_or_inf(sqrtf(dr * dr + fi * fi)));
+        out[(size_t)r * N + c] = make_double2(i128_to_double(ar) * sc, i128_to_double(ai) * sc);
     }
-    combine_tail(best, dev, words, acc_max, fin_max, dev_to, use, tol, iter, flags);
-}
-
-// rs_i = 1 / sqrt(Re a_ii) (FP32 reciprocal square root, widened) for the Jacobi-scaled start;
-// words[W_RS2] = max rs_i^2, words[W_DBAD] set where a diagonal entry gives no positive finite rs.
-__global__ void jacobi_rs_kernel(const double2 *__restrict__ A, int n, double *__restrict__ rs,
-                                 unsigned long long *words)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double d = A[(size_t)i * n + i].x;
-        const double r = (d > 0.0 && d < 1e30) ? (double)rsqrtf((float)d) : 0.0;
-        if (r > 0.0 && isfinite(r)) {
-            rs[i] = r;
-            atomicMax(&words[W_RS2], (unsigned long long)__double_as_longlong(r * r));
-        } else {
-            rs[i] = 0.0;
-            atomicOr(&words[W_DBAD], 1ull);
-        }
-    }
-}
-
-// u = max_i sum_j (|Re a_ij| + |Im a_ij|) >= max_i sum_j |a_ij| >= lambda_max, one warp per row,
-// into words[W_U], and the same bound of diag(rs) A diag(rs) into words[W_UJ] (the bits of
-// non-negative doubles; zero beforehand).
-__global__ void row_sum_bound_kernel(const double2 *__restrict__ A, int n, const double *__restrict__ rs,
-                                     unsigned long long *words)
-{
-    const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * warps + (threadIdx.x >> 5); i < n; i += gridDim.x * warps) {
-        double s = 0.0, sj = 0.0;
-        for (int j = lane; j < n; j += 32) {
-            const double2 a = A[(size_t)i * n + j];
-            const double m = fabs(a.x) + fabs(a.y);
-            s += m;
-            sj += m * rs[j];
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, o);
-            sj += __shfl_xor_sync(0xffffffffu, sj, o);
-        }
-        if (lane == 0) {
-            atomicMax(&words[W_U], (unsigned long long)__double_as_longlong(s));
-            atomicMax(&words[W_UJ], (unsigned long long)__double_as_longlong(sj * rs[i]));
-        }
-    }
-}
-
-// X0 = c diag(rs)^2 with c = 2 / (1 + u_J) (the Jacobi-scaled start), or c I with c = 2 / (1 + u)
-// when words[W_DBAD] is set; both bounds from row_sum_bound_kernel.
-__global__ void ns_init_kernel(double2 *X, int N, const double *__restrict__ rs, unsigned long long *words,
-                               int *flags)
-{
-    const bool jac = words[W_DBAD] == 0;
-    const double c = 2.0 / (1.0 + __longlong_as_double((long long)words[jac ? W_UJ : W_U]));
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    for (int r = blockIdx.y; r < N && col < N; r += gridDim.y)
-        X[(size_t)r * N + col] = make_double2(r == col ? (jac ? c * rs[r] * rs[r] : c) : 0.0, 0.0);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-        const double xmax = jac ? c * __longlong_as_double((long long)words[W_RS2]) : c;
-        words[W_X] = (unsigned long long)__double_as_longlong(fabs(xmax));
-        words[W_ITERS] = (unsigned long long)NS_MAX;
-        for (int j = 0; j <= NS_REFINE + 1; ++j)
-            flags[j] = 0;
-    }
-}
-
-// flags[0]: phase 1 converged.  A failure after a phase 1 that ran out of steps is told apart
-// (NS_DETAIL_CAP): the eager form, with more steps, may still converge.
-__global__ void ns_final_kernel(const unsigned long long *words, const int *flags, uint32_t *err)
-{
-    const double r = __longlong_as_double((long long)words[W_RLAST]);
-    if (!(r <= NS_ACCEPT))
-        record_error(err, GW_E_NUMERIC, SITE_NS, flags[0] ? 0u : NS_DETAIL_CAP);
 }
 
 // Grid of the element-wise kernels over an M x N matrix: x covers the columns in 256-thread blocks,
@@ -706,7 +461,7 @@ int round_up(int x, int m)
 // K range split so that tiles x slots fills the GPU); slices = the pairs (t, u) with t + u <= 8,
 // grouped by t + u into slots whose exact-sum bound sum 2 m_t m_u K_range stays below 2^24
 // (m_0 = 64, m_t = 32) and that hold at most five pairs.
-void ZPlan::build(int mode_, int M_, int N_, int K_, int nsm, int slices, int slicesA)
+void ZPlan::build(int mode_, int M_, int N_, int K_, int nsm)
 {
     mode = mode_;
     M = M_;
@@ -716,8 +471,7 @@ void ZPlan::build(int mode_, int M_, int N_, int K_, int nsm, int slices, int sl
     Npad = round_up(std::max(N, 1), ZT);
     nkc = round_up(std::max(K, 1), 16) / 16;
     ntiles = (Mpad / ZT) * (Npad / ZT);
-    ns = mode == MODE_FP16X3 ? 2 : std::max(1, std::min(OZ_SLICES, slices > 0 ? slices : OZ_SLICES));
-    nsA = std::max(ns, slicesA > 0 ? std::min(OZ_SLICES, slicesA) : ns);  // planes in the A operand
+    ns = mode == MODE_FP16X3 ? 2 : OZ_SLICES;
     std::vector<int2> pr;
     std::vector<int> sl, we;  // slot: p0, p1, kc0, kc1
     auto add_slot = [&](int p0, int p1, int kc0, int kc1, int w) {
@@ -772,7 +526,7 @@ size_t ZPlan::table_bytes() const
 size_t ZPlan::planes_bytes(bool a_operand) const
 {
     const int npl = 2;  // Re, Im per slice for both operands
-    return (size_t)nkc * (a_operand ? nsA : ns) * npl * (a_operand ? Mpad : Npad) * 16 * sizeof(uint16_t);
+    return (size_t)nkc * ns * npl * (a_operand ? Mpad : Npad) * 16 * sizeof(uint16_t);
 }
 
 size_t ZPlan::T_bytes() const
@@ -804,56 +558,40 @@ cudaError_t launch_zmaxabs(const double2 *M, int rows, int cols, long ld, unsign
 }
 
 cudaError_t launch_zslice(const ZPlan &p, bool a_operand, const double2 *Mx, long ld, const unsigned long long *maxw,
-                          uint16_t *planes, const int *skip, cudaStream_t s)
+                          uint16_t *planes, cudaStream_t s)
 {
     const int rows = a_operand ? p.M : p.N, Rpad = a_operand ? p.Mpad : p.Npad;
-    zslice_kernel<<<dim3(p.nkc, Rpad / ZT), 512, 0, s>>>(Mx, ld, rows, p.K, a_operand ? 0 : 1, Rpad, p.mode,
-                                                         a_operand ? p.nsA : p.ns,
-                                                         2, maxw, planes, skip);
+    zslice_kernel<<<dim3(p.nkc, Rpad / ZT), 512, 0, s>>>(Mx, ld, rows, p.K, a_operand ? 0 : 1, Rpad, p.mode, p.ns, 2,
+                                                         maxw, planes);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_zgemm16(const ZPlan &p, const uint16_t *Ap, const uint16_t *Bp, float2 *T, uint32_t *err,
-                           uint64_t wait_ns, const int *skip, cudaStream_t s)
+                           uint64_t wait_ns, cudaStream_t s)
 {
-    const bool f3 = p.mode == MODE_FP16X3;
-    cudaError_t e = f3 ? cudaFuncSetAttribute(zgemm16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)ZSMEM)
-                       : cudaFuncSetAttribute(zgemm16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)ZSMEM);
+    auto kernel = p.mode == MODE_FP16X3 ? zgemm16_kernel<true> : zgemm16_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ZSMEM);
     if (e != cudaSuccess)
         return e;
-    dim3 grid(p.ntiles, p.nslots);
-    if (f3)
-        zgemm16_kernel<true><<<grid, ZTHREADS, ZSMEM, s>>>(Ap, 2 * p.nsA, p.Mpad, Bp, 2 * p.ns, p.Npad, p.d_pairs,
-                                                           reinterpret_cast<const ZSlot *>(p.d_slots), p.Npad / ZT,
-                                                           T, err, wait_ns, skip);
-    else
-        zgemm16_kernel<false><<<grid, ZTHREADS, ZSMEM, s>>>(Ap, 2 * p.nsA, p.Mpad, Bp, 2 * p.ns, p.Npad, p.d_pairs,
-                                                            reinterpret_cast<const ZSlot *>(p.d_slots), p.Npad / ZT,
-                                                            T, err, wait_ns, skip);
+    kernel<<<dim3(p.ntiles, p.nslots), ZTHREADS, ZSMEM, s>>>(Ap, 2 * p.ns, p.Mpad, Bp, 2 * p.ns, p.Npad, p.d_pairs,
+                                                             reinterpret_cast<const ZSlot *>(p.d_slots), p.Npad / ZT, T,
+                                                             err, wait_ns);
     count_launches(1);
     return cudaGetLastError();
 }
 
-// out = cI I + cC (A B) + cD D from the slot tiles of plan p.  With integer slices only
-// cI in {0, 1}, cC = +-1 and no D are taken (the exact forms the inverse needs).
+// out = A B from the slot tiles of plan p.
 cudaError_t launch_zcombine(const ZPlan &p, const float2 *T, const unsigned long long *wA,
-                            const unsigned long long *wB, double cI, double cC, const double2 *D, double cD,
-                            double2 *out, double ref, unsigned long long *words, int acc_max, int fin_max, int dev_to,
-                            int use, double tol, int iter, const int *skip, int *flags, cudaStream_t s)
+                            const unsigned long long *wB, double2 *out, cudaStream_t s)
 {
     const dim3 grid(grid2d(p.M, p.N));
     if (p.mode == MODE_FP16X3) {
-        zcombine16_kernel<<<grid, 256, 0, s>>>(T, p.nslots, p.Mpad, p.Npad, wA, wB, p.M, p.N, cI, cC, D, cD, out, ref,
-                                               words, acc_max, fin_max, dev_to, use, tol, iter, skip, flags);
+        zcombine16_kernel<<<grid, 256, 0, s>>>(T, p.nslots, p.Mpad, p.Npad, wA, wB, p.M, p.N, out);
     } else {
-        if (D || (cI != 0.0 && cI != 1.0) || (cC != 1.0 && cC != -1.0) || p.nslots > 256)
+        if (p.nslots > 256)
             return cudaErrorInvalidValue;
-        zcombine_int_kernel<<<grid, 256, 0, s>>>(T, p.nslots, p.d_wexp, p.Mpad, p.Npad, wA, wB, p.M, p.N,
-                                                 cI == 1.0 ? 1 : 0, cC < 0 ? 1 : 0, out, ref, words, acc_max, fin_max,
-                                                 dev_to, use, tol, iter, skip, flags);
+        zcombine_int_kernel<<<grid, 256, 0, s>>>(T, p.nslots, p.d_wexp, p.Mpad, p.Npad, wA, wB, p.M, p.N, out);
     }
     count_launches(1);
     return cudaGetLastError();
@@ -915,220 +653,18 @@ cudaError_t zgemm_enqueue(ZPlan &p, const double2 *A, long lda, const double2 *B
         return e;
     if ((e = cudaMemsetAsync(words, 0, 64 * 8, s)) != cudaSuccess)
         return e;
-    // words[0], [1]: max of A and B; [2]: max of C (unused), [3]: scratch
+    // words[0], [1]: max of A and B
     if ((e = launch_zmaxabs(A, p.M, p.K, lda, &words[0], s)) != cudaSuccess)
         return e;
     if ((e = launch_zmaxabs(B, p.K, p.N, ldb, &words[1], s)) != cudaSuccess)
         return e;
-    if ((e = launch_zslice(p, true, A, lda, &words[0], Ap, nullptr, s)) != cudaSuccess)
+    if ((e = launch_zslice(p, true, A, lda, &words[0], Ap, s)) != cudaSuccess)
         return e;
-    if ((e = launch_zslice(p, false, B, ldb, &words[1], Bp, nullptr, s)) != cudaSuccess)
+    if ((e = launch_zslice(p, false, B, ldb, &words[1], Bp, s)) != cudaSuccess)
         return e;
-    if ((e = launch_zgemm16(p, Ap, Bp, T, err, wait_ns, nullptr, s)) != cudaSuccess)
+    if ((e = launch_zgemm16(p, Ap, Bp, T, err, wait_ns, s)) != cudaSuccess)
         return e;
-    // C = 2^(eA + eB) sum_slot 2^wexp T; words[0] and [1] are W_EPS and W_X, untouched here
-    return launch_zcombine(p, T, &words[0], &words[1], 0.0, 1.0, nullptr, 0.0, C, 0.0, words, W_ZN, W_Z,
-                           W_DISCARD, DEV_STORE, 0.0, 0, nullptr, nullptr, s);
-}
-
-namespace {
-struct NsWork {
-    uint16_t *A16, *AOZ, *XA16, *XB16, *ZB16, *XBOZ;
-    float2 *T;
-    double2 *X, *Z;
-    unsigned long long *words;
-    int *skip;
-    void *tab16, *taboz, *taboz7;
-};
-
-// The first refinement only has to bring max |I - eps X| from the FP16X3 floor (~1e-6) to where
-// the second can finish, so its residual uses seven slices (2^-42 relative, 28 slice pairs) of X
-// against the nine of eps; the second uses nine (45 pairs).
-constexpr int NS_SLICES_FIRST = 7;
-
-void ns_plans(int N, int nsm, ZPlan &p16, ZPlan &poz, ZPlan &poz7)
-{
-    p16.build(MODE_FP16X3, N, N, N, nsm);
-    poz.build(MODE_SLICES, N, N, N, nsm);
-    poz7.build(MODE_SLICES, N, N, N, nsm, NS_SLICES_FIRST, OZ_SLICES);
-}
-
-NsWork carve_ns(const ZPlan &p16, const ZPlan &poz, const ZPlan &poz7, int N, Carver &c)
-{
-    NsWork w;
-    const size_t nn = (size_t)N * N;
-    w.A16 = static_cast<uint16_t *>(c.take(p16.planes_bytes(true)));
-    w.AOZ = static_cast<uint16_t *>(c.take(poz.planes_bytes(true)));
-    w.XA16 = static_cast<uint16_t *>(c.take(p16.planes_bytes(true)));
-    w.XB16 = static_cast<uint16_t *>(c.take(p16.planes_bytes(false)));
-    w.ZB16 = static_cast<uint16_t *>(c.take(p16.planes_bytes(false)));
-    w.XBOZ = static_cast<uint16_t *>(c.take(poz.planes_bytes(false)));
-    w.T = static_cast<float2 *>(c.take(std::max(p16.T_bytes(), std::max(poz.T_bytes(), poz7.T_bytes()))));
-    w.X = static_cast<double2 *>(c.take(nn * sizeof(double2)));
-    w.Z = static_cast<double2 *>(c.take(nn * sizeof(double2)));
-    w.words = static_cast<unsigned long long *>(c.take(64 * 8));
-    w.skip = static_cast<int *>(c.take(64));
-    w.tab16 = c.take(p16.table_bytes());
-    w.taboz = c.take(poz.table_bytes());
-    w.taboz7 = c.take(poz7.table_bytes());
-    return w;
-}
-}  // namespace
-
-// eps^-1 by the tensor-core Newton iteration (header comment).  A is eps (N x N, device).
-size_t ns_work_bytes(int N, int nsm)
-{
-    ZPlan p16, poz, poz7;
-    ns_plans(N, nsm, p16, poz, poz7);
-    Carver c(nullptr);
-    carve_ns(p16, poz, poz7, N, c);
-    return c.used;
-}
-
-// Report of the last inverse run on workspace `work` (synchronous read after the stream is idle):
-// out[0] FP16X3 steps of phase 1, [1] residual max |I - eps X| after phase 1, [2] the last measured
-// residual, [3] refinements that ran.
-cudaError_t ns_report(const void *work, int N, int nsm, double *out4)
-{
-    ZPlan p16, poz, poz7;
-    ns_plans(N, nsm, p16, poz, poz7);
-    Carver c(const_cast<void *>(work));
-    const NsWork w = carve_ns(p16, poz, poz7, N, c);
-    unsigned long long h[W_TOTAL];
-    const cudaError_t e = cudaMemcpy(h, w.words, sizeof h, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess)
-        return e;
-    out4[0] = (double)h[W_ITERS];
-    out4[1] = __builtin_bit_cast(double, h[W_RES0]);
-    out4[2] = __builtin_bit_cast(double, h[W_RLAST]);
-    out4[3] = (double)h[W_NREF];
-    return cudaSuccess;
-}
-
-namespace {
-// Host read of a device flag (waits for the stream); a failed read counts as "not set".
-bool flag_set(const int *d_flag, cudaStream_t s)
-{
-    int h = 0;
-    if (cudaMemcpyAsync(&h, d_flag, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return h != 0;
-}
-}  // namespace
-
-// Upload the slot tables of order N into the workspace (done inside ns_inverse_enqueue unless
-// the caller did it beforehand, as a captured CUDA graph needs: no pageable copies in capture).
-cudaError_t ns_prepare(void *work, int N, int nsm, cudaStream_t s)
-{
-    ZPlan p16, poz, poz7;
-    ns_plans(N, nsm, p16, poz, poz7);
-    Carver cv(work);
-    const NsWork nw = carve_ns(p16, poz, poz7, N, cv);
-    cudaError_t e = p16.upload(nw.tab16, s);
-    if (e == cudaSuccess)
-        e = poz.upload(nw.taboz, s);
-    if (e == cudaSuccess)
-        e = poz7.upload(nw.taboz7, s);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(s);  // the host tables are locals
-    return e;
-}
-
-// The kernels of every step check the device flags, so the result does not depend on the host
-// reads below: they only stop queuing steps that would return at once (after phase-1 steps 3, 5,
-// 7, ... and before the third refinement), at the price of one stream synchronisation each.
-// With graph_safe the tables must have been uploaded by ns_prepare and every step is queued (no
-// host reads, no pageable copies), so the whole inverse can be captured into a CUDA graph.
-cudaError_t ns_inverse_enqueue(const double2 *A, int N, double2 *Xout, void *work, double *rowsum, uint32_t *err,
-                               uint64_t wait_ns, int nsm, cudaStream_t s, bool graph_safe, int max_steps)
-{
-    max_steps = std::max(1, std::min(max_steps, NS_MAX));
-    ZPlan p16, poz, poz7;
-    ns_plans(N, nsm, p16, poz, poz7);
-    Carver cv(work);
-    const NsWork nw = carve_ns(p16, poz, poz7, N, cv);
-    uint16_t *A16 = nw.A16, *AOZ = nw.AOZ, *XA16 = nw.XA16, *XB16 = nw.XB16, *ZB16 = nw.ZB16, *XBOZ = nw.XBOZ;
-    float2 *T = nw.T;
-    double2 *X = nw.X, *Z = nw.Z;
-    unsigned long long *words = nw.words;
-    int *skip = nw.skip;
-    void *tab16 = nw.tab16, *taboz = nw.taboz, *taboz7 = nw.taboz7;
-    const size_t nn = (size_t)N * N;
-    cudaError_t e;
-#define NS_TRY(x)                      \
-    do {                               \
-        if ((e = (x)) != cudaSuccess)  \
-            return e;                  \
-    } while (0)
-    if (graph_safe) {  // the device pointers of the tables, uploaded earlier by ns_prepare
-        p16.d_pairs = static_cast<int2 *>(tab16);
-        p16.d_slots = reinterpret_cast<int *>(static_cast<uint8_t *>(tab16) + p16.host_pairs.size() * sizeof(int2));
-        p16.d_wexp = p16.d_slots + p16.host_slots.size();
-        poz.d_pairs = static_cast<int2 *>(taboz);
-        poz.d_slots = reinterpret_cast<int *>(static_cast<uint8_t *>(taboz) + poz.host_pairs.size() * sizeof(int2));
-        poz.d_wexp = poz.d_slots + poz.host_slots.size();
-        poz7.d_pairs = static_cast<int2 *>(taboz7);
-        poz7.d_slots =
-            reinterpret_cast<int *>(static_cast<uint8_t *>(taboz7) + poz7.host_pairs.size() * sizeof(int2));
-        poz7.d_wexp = poz7.d_slots + poz7.host_slots.size();
-    } else {
-        NS_TRY(p16.upload(tab16, s));
-        NS_TRY(poz.upload(taboz, s));
-        NS_TRY(poz7.upload(taboz7, s));
-    }
-    NS_TRY(cudaMemsetAsync(words, 0, 64 * 8, s));
-    // eps: its max, both slicings, and the row-sum bound for X0
-    NS_TRY(launch_zmaxabs(A, N, N, N, &words[W_EPS], s));
-    NS_TRY(launch_zslice(p16, true, A, N, &words[W_EPS], A16, nullptr, s));
-    NS_TRY(launch_zslice(poz, true, A, N, &words[W_EPS], AOZ, nullptr, s));
-    (void)rowsum;
-    double *rs = reinterpret_cast<double *>(Z);  // scratch: Z is first written by phase 1
-    jacobi_rs_kernel<<<std::max(1, std::min(152 * 4, (N + 255) / 256)), 256, 0, s>>>(A, N, rs, words);
-    row_sum_bound_kernel<<<std::max(1, std::min(152 * 4, (N + 7) / 8)), 256, 0, s>>>(A, N, rs, words);
-    count_launches(2);
-    ns_init_kernel<<<grid2d(N, N), 256, 0, s>>>(X, N, rs, words, skip);  // skip[0]: phase 1, [1 + j]: refinement j
-    count_launches(1);
-    NS_TRY(cudaGetLastError());
-    // phase 1: X <- X (2I - eps X) with FP16X3 products, stopped on device below NS_TOL
-    for (int it = 0; it < max_steps; ++it) {
-        NS_TRY(launch_zslice(p16, false, X, N, &words[W_X], XB16, skip, s));
-        NS_TRY(launch_zgemm16(p16, A16, XB16, T, err, wait_ns, skip, s));
-        // Z = 2I - eps X; deviation |Z - I| = |I - eps X|
-        NS_TRY(launch_zcombine(p16, T, &words[W_EPS], &words[W_X], 2.0, -1.0, nullptr, 0.0, Z, 1.0, words, W_ZN, W_Z,
-                               W_DISCARD, DEV_PHASE1, NS_TOL, it, skip, skip, s));
-        NS_TRY(launch_zslice(p16, true, X, N, &words[W_X], XA16, skip, s));
-        NS_TRY(launch_zslice(p16, false, Z, N, &words[W_Z], ZB16, skip, s));
-        NS_TRY(launch_zgemm16(p16, XA16, ZB16, T, err, wait_ns, skip, s));
-        NS_TRY(launch_zcombine(p16, T, &words[W_X], &words[W_Z], 0.0, 1.0, nullptr, 0.0, X, 0.0, words, W_XN, W_X,
-                               W_DISCARD, DEV_STORE, 0.0, it, skip, nullptr, s));
-        if (!graph_safe && it >= 3 && (it & 1) && flag_set(skip, s))
-            break;
-    }
-    // phase 2: R = I - eps X to FP64 accuracy (integer slices), X <- X + X R (FP16X3); refinement
-    // j runs unless an earlier one measured a residual <= NS_LAST (flag skip[1 + j])
-    for (int j = 0; j < NS_REFINE; ++j) {
-        const int *sk = skip + 1 + j;
-        if (!graph_safe && j == 2 && flag_set(sk, s))
-            break;
-        const ZPlan &pr = j == 0 ? poz7 : poz;
-        NS_TRY(launch_zslice(pr, false, X, N, &words[W_X], XBOZ, sk, s));
-        NS_TRY(launch_zslice(p16, true, X, N, &words[W_X], XA16, sk, s));
-        NS_TRY(launch_zgemm16(pr, AOZ, XBOZ, T, err, wait_ns, sk, s));
-        NS_TRY(launch_zcombine(pr, T, &words[W_EPS], &words[W_X], 1.0, -1.0, nullptr, 0.0, Z, 0.0, words, W_ZN, W_Z,
-                               j == 0 ? W_RES0 : W_DISCARD, DEV_REFINE, NS_LAST, j, sk, skip + 1, s));
-        NS_TRY(launch_zslice(p16, false, Z, N, &words[W_Z], ZB16, sk, s));
-        NS_TRY(launch_zgemm16(p16, XA16, ZB16, T, err, wait_ns, sk, s));
-        NS_TRY(launch_zcombine(p16, T, &words[W_X], &words[W_Z], 0.0, 1.0, X, 1.0, X, 0.0, words, W_XN, W_X,
-                               W_DISCARD, DEV_STORE, 0.0, j, sk, nullptr, s));
-    }
-    NS_TRY(cudaMemcpyAsync(Xout, X, nn * sizeof(double2), cudaMemcpyDeviceToDevice, s));
-    ns_final_kernel<<<1, 1, 0, s>>>(words, skip, err);
-    count_launches(1);
-#undef NS_TRY
-    return cudaGetLastError();
+    return launch_zcombine(p, T, &words[0], &words[1], C, s);
 }
 
 }  // namespace gw
