@@ -19,20 +19,19 @@
 //    their own threads only (20 MB for the GPU, resident in L2), added with fire-and-forget vector
 //    reductions so no thread waits for a load.
 //
-// Measured on one GB300 (update alone, FP16X3, W = 3): 24^3, 32 x 480 states: 24.2 -> 9.44 ms (0.95 of
-// the sustained FP16 rate would be 6.9 ms for the issued MMAs; windows of 16 chunks take 8.0 ms, so the
-// window boundaries cost the most of what is left); 36^3, 64 x 1000, BF16X3, W = 16: 0.97 -> 0.19 s.
+// Measured on one GB300 (update alone, FP16X3, W = 3): 24^3, 32 x 480 states: 24.2 -> 8.48 ms (0.95 of
+// the sustained FP16 rate would be 6.9 ms for the issued MMAs); 36^3, 64 x 1000, BF16X3, W = 16: 0.97 ->
+// 0.19 s.
 //
 // Bound: the tensor pipe and the shared memory that feeds it, as herk16_kernel (32 KB staged and 84 KB
 // read per chunk).  Control: mbarrier phases and the two TMEM window buffers carry across tiles, so the
 // producer streams the next tile's operands while the current tile is being written.
 //
-// Truncation.  tcgen05 adds into TMEM with truncation, so a window of n chunks comes out smaller by a
-// nearly uniform factor, 1 - b n.  Measured in the separable form: b = 1.3e-7 to 1.8e-7 on P~ and the
-// diagonal of P, 0.5e-7 to 1.4e-7 on its other elements, the same on random and on band-structured
-// states.  A product of two windows carries both losses, so the separable form multiplies the mean loss
-// back (window_loss).  P~ against FP64 at 24^3, W = 3: 9.1e-7 without, 3.3e-7 with it, 6.5e-7 in the
-// pair form; off-diagonal elements of P at 16^3 2.6e-7 against 4.3e-7.
+// Truncation.  tcgen05 adds into TMEM with truncation, so a window comes out smaller by a nearly uniform
+// factor.  Measured in the separable form, for windows of n chunks together (C and V): 1.0e-7 + 1.5e-7 n on
+// the diagonal of P, where every term has one sign, 3.0e-7 + 0.3e-7 n on its other elements, the same on
+// random and on band-structured states.  The separable form multiplies these mean losses back (loss_gain),
+// which leaves its errors below those of the pair form even at windows of twice the length (Windows).
 //
 // The occupied planes are FP16 in either precision (they are 1/16 of the work), so with BF16 operands
 // only C_t carries the 8 + 8-bit split: both at 8 + 8 bits measured 5.7e-6 on the off-diagonal elements
@@ -54,9 +53,13 @@ constexpr uint32_t NPL = HERK16_NPL;
 // the B block's in the same order, i.e. regions [Im | Re] of the
 // hi part and of the lo part, so one N = 256 MMA from A = Im fills the Re and Im columns of a window
 constexpr uint32_t B_OFF = 4 * PL;
-constexpr uint32_t STAGE_BYTES = 8 * PL;  // 32 KB
-constexpr int STAGES = 6;
-constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;
+constexpr uint32_t CHUNK_BYTES = 8 * PL;  // 32 KB
+// Two chunks per pipeline stage (a stage holds chunks of one window only): half the barrier round trips and
+// commits.  Measured at 24^3 with windows of six chunks, one / two / three chunks a stage: 8.73 / 8.48 /
+// 8.80 ms; with windows of 32, 8.30 / 8.11 / 8.21 ms.
+constexpr int CPS = 2, STAGES = 3;
+constexpr uint32_t STAGE_BYTES = CPS * CHUNK_BYTES;
+constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;  // 192 KB
 constexpr uint32_t LBO = 128, SBO = 256;
 constexpr int NPROMO_WARPS = 8;
 constexpr int PRODUCER_WARP = 8, MMA_WARP = 9;
@@ -95,7 +98,7 @@ __device__ __forceinline__ float4 sums_load(const float4 *p)
     return v;
 }
 
-// Position in the ring of stages: stage and phase parity of a chunk counter.
+// Position in the ring of stages: stage and phase parity of a stage counter.
 struct Ring {
     int s = 0;
     uint32_t ph = 0;
@@ -108,24 +111,37 @@ struct Ring {
     }
 };
 
-// Windows of a job: each term has nwc windows of W chunks over its ncc unoccupied (or pair) chunks, the
-// last one shorter, then nwv windows of wv chunks over its nvc occupied ones.
+// Windows of a job: each term has nwc windows of wc chunks over its ncc unoccupied (or pair) chunks, the
+// last one shorter, then nwv windows of wv chunks over its nvc occupied ones.  The separable form takes
+// windows of 2 W chunks: with the mean loss multiplied back its errors still lie below those of the pair
+// form at W (16^3, 16 / 200 states, FP16X3, off-diagonal P, separable against pair:
+// 2.2e-7 / 2.8e-7 at W = 1, 3.3e-7 / 4.3e-7 at 3, 5.4e-7 / 9.4e-7 at 8; P~ at 24^3: 1.1e-7 / 2.9e-7, 2.2e-7 /
+// 6.5e-7, 4.4e-7 / 1.6e-6), and the boundaries, about 0.3 us each, halve: 9.43 -> 8.48 ms at 24^3, W = 3.
 struct Windows {
-    int nwc, nwv, wv;
+    int wc, nwc, nwv, wv;
     __device__ __forceinline__ Windows(const HerkJob &j, int W)
-        : nwc((j.ncc + W - 1) / W), nwv((j.nvc + W - 1) / W), wv(nwv > 0 ? (j.nvc + nwv - 1) / nwv : 0)
     {
+        wc = j.nvc > 0 ? 2 * W : W;
+        nwc = (j.ncc + wc - 1) / wc;
+        nwv = (j.nvc + 2 * W - 1) / (2 * W);
+        wv = nwv > 0 ? (j.nvc + nwv - 1) / nwv : 0;
     }
 };
 
-// Mean relative loss of a sum over n chunks taken in windows of w chunks (the last one shorter).
-constexpr float LOSS_PER_CHUNK = 1.3e-7f;
-__device__ __forceinline__ float window_loss(int n, int w)
+// Mean chunks per window of a sum over n chunks taken in windows of w (the last one shorter).
+__device__ __forceinline__ float mean_window(int n, int w)
 {
     if (n <= 0)
         return 0.f;
     const int full = n / w, rest = n - full * w;
-    return LOSS_PER_CHUNK * (float)(full * w * w + rest * rest) / (float)n;
+    return (float)(full * w * w + rest * rest) / (float)n;
+}
+
+// Factor that undoes the mean truncation loss of a product of two sums over windows of n chunks together
+// (header comment): sums of terms of one sign lose most, so the diagonal has its own.
+__device__ __forceinline__ float loss_gain(float n, bool diagonal)
+{
+    return diagonal ? 1.f + (1.0e-7f + 1.5e-7f * n) : 1.f + (3.0e-7f + 0.3e-7f * n);
 }
 
 template <bool BF16>
@@ -145,9 +161,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     volatile long long *n_consumed = n_issued + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // With W < STAGES the commit to the empty barrier of a window's last chunk tells the promotion
-    // warps that the window is complete; longer windows have a commit of their own.
-    const bool own = W >= STAGES;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -173,35 +186,42 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
     if (warp == PRODUCER_WARP) {
         if (lane == 0) {
-            long long g = 0;  // chunks issued by this CTA over all its tiles
+            long long g = 0;  // stages issued by this CTA over all its tiles
             Ring ring;
-            bool stop = false;
-            for (int t = blockIdx.x; t < n_tiles && !stop; t += gridDim.x) {
+            bool ok = true;
+            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
                 const int4 tl = tiles[t];
                 const HerkJob jb = jobs[tl.x];
-                const int nch = jb.ncc + jb.nvc;
+                const Windows w(jb, W);
                 const int nblk = jb.nr_pad / TM;  // block layout: one 16 KB copy per operand block
                 const size_t step = plane16_block(1, 0, nblk, NPL, 0);
-                const uint16_t *a = jb.A + plane16_block(0, tl.y, nblk, NPL, 0);
-                for (int term = 0; term < jb.T && !stop; ++term) {
-                    const uint16_t *b = jb.B + plane16_block(0, tl.z, nblk, NPL, 0);  // the same for every term
-                    for (int j = 0; j < nch; ++j, ++g, a += step, b += step, ring.next()) {
+                const uint16_t *a = jb.A + plane16_block(0, tl.y, nblk, NPL, 0), *b = nullptr;
+                auto window = [&](int n) {
+                    for (int c = 0; c < n; c += CPS, ++g, ring.next()) {
                         if (g >= STAGES && !mbar_wait(&empty[ring.s], ring.ph ^ 1u, wait_ns)) {
                             record_error(err, GW_E_TIMEOUT, SITE_HERK_PRODUCER, blockIdx.x);
                             *abort_flag = 1;
-                            stop = true;
-                            break;
+                            return false;
                         }
-                        if (*abort_flag) {
-                            stop = true;
-                            break;
-                        }
+                        if (*abort_flag)
+                            return false;
                         uint8_t *st = smem + ring.s * STAGE_BYTES;
-                        mbar_arrive_expect_tx(&full[ring.s], STAGE_BYTES);
-                        bulk_g2s(st, a, 4 * PL, &full[ring.s]);
-                        bulk_g2s(st + B_OFF, b, 4 * PL, &full[ring.s]);
+                        const int m = min(CPS, n - c);
+                        mbar_arrive_expect_tx(&full[ring.s], m * CHUNK_BYTES);
+                        for (int j = 0; j < m; ++j, a += step, b += step, st += CHUNK_BYTES) {
+                            bulk_g2s(st, a, 4 * PL, &full[ring.s]);
+                            bulk_g2s(st + B_OFF, b, 4 * PL, &full[ring.s]);
+                        }
                         *n_issued = g + 1;
                     }
+                    return true;
+                };
+                for (int term = 0; term < jb.T && ok; ++term) {
+                    b = jb.B + plane16_block(0, tl.z, nblk, NPL, 0);  // the same for every term
+                    for (int i = 0; i < w.nwc && ok; ++i)
+                        ok = window(min(w.wc, jb.ncc - i * w.wc));
+                    for (int i = 0; i < w.nwv && ok; ++i)
+                        ok = window(min(w.wv, jb.nvc - i * w.wv));
                 }
             }
         }
@@ -226,15 +246,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 const uint32_t d = tmem + b * 256;
                 const uint32_t ID = mma_idesc(0u, TM, 2 * TN, false) | fmt;
                 const uint32_t ID1 = mma_idesc(0u, TM, TN, false) | fmt, ID1N = mma_idesc(0u, TM, TN, true) | fmt;
-                for (int c = 0; c < n; ++c, ++g, ring.next()) {
+                for (int c = 0; c < n; ++c) {
                     const int s = ring.s;
-                    if (!mbar_wait(&full[s], ring.ph, wait_ns)) {
-                        record_error(err, GW_E_TIMEOUT, SITE_HERK_MMA, blockIdx.x);
-                        *abort_flag = 1;
-                        return false;
+                    if (c % CPS == 0) {
+                        if (!mbar_wait(&full[s], ring.ph, wait_ns)) {
+                            record_error(err, GW_E_TIMEOUT, SITE_HERK_MMA, blockIdx.x);
+                            *abort_flag = 1;
+                            return false;
+                        }
+                        tc_fence_after();
                     }
-                    tc_fence_after();
-                    const uint32_t st = sbase + s * STAGE_BYTES;
+                    const uint32_t st = sbase + s * STAGE_BYTES + (c % CPS) * CHUNK_BYTES;
                     const uint64_t a_ih = smem_desc(st, LBO, SBO), a_rh = smem_desc(st + PL, LBO, SBO);
                     const uint64_t a_il = smem_desc(st + 2 * PL, LBO, SBO);
                     const uint64_t a_rl = smem_desc(st + 3 * PL, LBO, SBO);
@@ -252,11 +274,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     mma_f16(d + 128, a_rh, b_ih, ID1N, 1);  // Im -= Ar Bi
                     mma_f16(d + 128, a_rh, b_il, ID1N, 1);
                     mma_f16(d + 128, a_rl, b_ih, ID1N, 1);
-                    mma_commit(&empty[s]);
-                    *n_consumed = g + 1;
+                    if (c % CPS == CPS - 1 || c == n - 1) {
+                        mma_commit(&empty[s]);
+                        *n_consumed = ++g;
+                        ring.next();
+                    }
                 }
-                if (own)
-                    mma_commit(&accf[b]);
+                mma_commit(&accf[b]);
                 ++gw;
                 return true;
             };
@@ -265,7 +289,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 const Windows w(jb, W);
                 for (int term = 0; term < jb.T && ok; ++term) {
                     for (int i = 0; i < w.nwc && ok; ++i)
-                        ok = window(min(W, jb.ncc - i * W), FMT);
+                        ok = window(min(w.wc, jb.ncc - i * w.wc), FMT);
                     for (int i = 0; i < w.nwv && ok; ++i)
                         ok = window(min(w.wv, jb.nvc - i * w.wv), 0u);
                 }
@@ -276,25 +300,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     } else {
         // ---------------- promotion warps 0..7
         const int q = warp & 3, h = warp >> 2;
-        const int m = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         float4 *my = sums + (size_t)blockIdx.x * (SUM_F4 * NPROMO_WARPS * 32) + threadIdx.x;  // stride 256
         float2 *stage = reinterpret_cast<float2 *>(smem + PIPE_BYTES + BAR_BYTES) + warp * 32 * OUT_PITCH;
         uint32_t gw = 0;
-        int at = 0;  // chunks seen, modulo 2 STAGES: stage and parity of the next chunk
         bool stop = false;
         float are[64], aim[64];
-        // Wait for the next window (n chunks); the outcome is the same in every lane, as the TMEM loads
-        // need.  The empty barrier of its last chunk cannot complete another phase before the window is
-        // promoted: the chunk STAGES later lies at least two windows on (the next window has at most
-        // W < STAGES chunks), and the MMAs of that window wait for this promotion.
-        auto ready = [&](int n) {
-            at += n;
-            at -= at >= 2 * STAGES ? (at / (2 * STAGES)) * (2 * STAGES) : 0;
-            const int last = at == 0 ? 2 * STAGES - 1 : at - 1;
-            uint64_t *bar = own ? &accf[gw & 1u] : &empty[last >= STAGES ? last - STAGES : last];
-            const uint32_t par = own ? (gw >> 1) & 1u : (last >= STAGES ? 1u : 0u);
-            if (!__all_sync(0xffffffffu, mbar_wait(bar, par, wait_ns))) {
+        // Wait for the next window; the outcome is the same in every lane, as the TMEM loads need.
+        auto ready = [&]() {
+            if (!__all_sync(0xffffffffu, mbar_wait(&accf[gw & 1u], (gw >> 1) & 1u, wait_ns))) {
                 if (lane == 0)
                     record_error(err, GW_E_TIMEOUT, SITE_HERK_EPILOGUE, blockIdx.x);
                 *abort_flag = 1;
@@ -327,7 +341,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 }
                 const int w0 = sep ? 0 : seg * L, w1 = sep ? w.nwc : min(w.nwc, w0 + L);
                 for (int win = w0; win < w1; ++win) {
-                    if (!ready(min(W, jb.ncc - win * W)))
+                    if (!ready())
                         break;
                     const uint32_t base = tmem + lane_addr + (gw & 1u) * 256 + h * 64;
 #pragma unroll
@@ -355,7 +369,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 }
                 const float vs = jb.term_scale[seg] * ldexpf(1.0f, -2 * jb.scale_exp[1]);
                 for (int win = 0; win < w.nwv; ++win) {
-                    if (!ready(min(w.wv, jb.nvc - win * w.wv)))
+                    if (!ready())
                         break;
                     const uint32_t base = tmem + lane_addr + (gw & 1u) * 256 + h * 64;
                     const bool first = seg == 0 && win == 0;
@@ -385,16 +399,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // warp's stage, their mirror P[c][r] = conj(P[r][c]) straight from the lanes, which hold
             // consecutive r
             const int nr = jb.nr, r0 = tl.y * TM + q * 32, r = r0 + lane, cbase = tl.z * TN + h * 64;
-            const float gain = sep ? 1.f + window_loss(jb.ncc, W) + window_loss(jb.nvc, w.wv) : 1.f;
-            const float s2 = -gain * ldexpf(1.0f, -2 * jb.scale_exp[0]);
+            const float nw = mean_window(jb.ncc, w.wc) + mean_window(jb.nvc, w.wv);
+            const float s1 = -ldexpf(1.0f, -2 * jb.scale_exp[0]);
+            const float s2 = sep ? s1 * loss_gain(nw, false) : s1, sd = sep ? s1 * loss_gain(nw, true) : s1;
             float2 *P = jb.P;
             for (int g0 = 0; g0 < 64; g0 += OUT_COLS) {
                 float2 x[OUT_COLS];
 #pragma unroll
                 for (int i = 0; i < OUT_COLS / 2; ++i) {
                     const float4 v = sums_load(my + (g0 / 2 + i) * 256);
-                    x[2 * i] = make_float2(v.x * s2, v.y * s2);
-                    x[2 * i + 1] = make_float2(v.z * s2, v.w * s2);
+                    const int col = cbase + g0 + 2 * i;
+                    x[2 * i] = make_float2(v.x * (col == r ? sd : s2), v.y * s2);
+                    x[2 * i + 1] = make_float2(v.z * (col + 1 == r ? sd : s2), v.w * s2);
                 }
 #pragma unroll
                 for (int i = 0; i < OUT_COLS; ++i) {
