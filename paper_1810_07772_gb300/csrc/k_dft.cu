@@ -633,20 +633,46 @@ __global__ void __launch_bounds__(P12_WARPS * 32)
 using twiddle::kcos;
 using twiddle::ksin;
 
+// Both parts of a complex value in one instruction (rounded as the two scalar operations would be): half the
+// issue slots of the sums; 24^3 plain rows 326 -> 295 us (6.2 TB/s with the workspace), stage 3 69 -> 63 us.
+__device__ __forceinline__ unsigned long long f2_bits(float2 a)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+
+__device__ __forceinline__ float2 bits_f2(unsigned long long r)
+{
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return bits_f2(r);
+}
+
+__device__ __forceinline__ float2 fma2(float2 a, float c, float2 b)  // a c + b
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(make_float2(c, c))), "l"(f2_bits(b)));
+    return bits_f2(r);
+}
+
 // One term j of the paired sums of output m: A += s_j cos, B += t_j sin (s_j in x[j], t_j in
 // x[N - j]); a zero constant drops its FMAs.
 template <int N, int M, int J>
 __device__ __forceinline__ void pterm(const float2 (&x)[N], float2 &A, float2 &B)
 {
     constexpr float c = kcos<N, M * J>, s = ksin<N, M * J>;
-    if constexpr (c != 0.f) {
-        A.x = fmaf(x[J].x, c, A.x);
-        A.y = fmaf(x[J].y, c, A.y);
-    }
-    if constexpr (s != 0.f) {
-        B.x = fmaf(x[N - J].x, s, B.x);
-        B.y = fmaf(x[N - J].y, s, B.y);
-    }
+    if constexpr (c != 0.f)
+        A = fma2(x[J], c, A);
+    if constexpr (s != 0.f)
+        B = fma2(x[N - J], s, B);
 }
 
 // A = x_0 + (-1)^M x_{N/2} + sum_{0<j<N/2} s_j cos(2 pi M j / N),  B = sum_{0<j<N/2} t_j sin(2 pi M j / N)
@@ -657,8 +683,7 @@ __device__ __forceinline__ void paired_sums(const float2 (&x)[N], float2 &A, flo
     A = x[0];
     if constexpr (N % 2 == 0) {
         constexpr float sg = (M & 1) ? -1.f : 1.f;
-        A.x = fmaf(sg, x[N / 2].x, A.x);
-        A.y = fmaf(sg, x[N / 2].y, A.y);
+        A = fma2(x[N / 2], sg, A);
     }
     B = make_float2(0.f, 0.f);
     (pterm<N, M, J + 1>(x, A, B), ...);
@@ -671,8 +696,8 @@ __device__ __forceinline__ void pair_fold(float2 (&x)[N])
 #pragma unroll
     for (int j = 1; j <= (N - 1) / 2; ++j) {
         const float2 u = x[j], v = x[N - j];
-        x[j] = make_float2(u.x + v.x, u.y + v.y);
-        x[N - j] = make_float2(u.x - v.x, u.y - v.y);
+        x[j] = add2(u, v);
+        x[N - j] = fma2(v, -1.f, u);
     }
 }
 
@@ -725,10 +750,8 @@ __device__ __forceinline__ void paired_sums2(const float2 (&x)[N], float2 &A, fl
     C = x[0];
     if constexpr (N % 2 == 0) {
         constexpr float sa = (Ma & 1) ? -1.f : 1.f, sb = (Mb & 1) ? -1.f : 1.f;
-        A.x = fmaf(sa, x[N / 2].x, A.x);
-        A.y = fmaf(sa, x[N / 2].y, A.y);
-        C.x = fmaf(sb, x[N / 2].x, C.x);
-        C.y = fmaf(sb, x[N / 2].y, C.y);
+        A = fma2(x[N / 2], sa, A);
+        C = fma2(x[N / 2], sb, C);
     }
     B = make_float2(0.f, 0.f);
     D = B;
@@ -811,20 +834,109 @@ __host__ __device__ inline size_t p12c_smem(int N, int c3, bool async = false)
 
 constexpr int P12C_MAX_C3 = 16;  // stage 2 runs two planes side by side, one per half-warp
 
-// A warp takes two tasks (planes) at a time: stage 1 of each (a lane per line), then stage 2 of
-// both together, lanes 0-15 on the first plane's columns and lanes 16-31 on the second's, so a
-// sphere with c3 <= 16 keeps twice as many lanes busy in stage 2 as one plane would.
+// Stage 1 of one plane (a lane per line j2): a1t[M + m3][j2] = sum_j3 x[j2][j3] e(+-m3 j3 / N), the line
+// read into registers by line(j2, x).
+template <int N, class Line>
+__device__ __forceinline__ void p12c_stage1(int lane, int M, float sgn, float2 *a1t, Line line)
+{
+    constexpr int H = (N - 1) / 2, LDA = N | 1;
+    for (int j2 = lane; j2 < N; j2 += 32) {
+        float2 x[N];
+        line(j2, x);
+        pair_fold<N>(x);
+        float2 a0 = x[0];
+#pragma unroll
+        for (int j = 1; j <= H; ++j) {  // the m3 = 0 sum, in the order of the table form
+            a0 = add2(a0, x[j]);
+        }
+        float2 *col = a1t + j2;
+        if constexpr (N % 2 == 0)
+            col[M * LDA] = make_float2(a0.x + x[N / 2].x, a0.y + x[N / 2].y);
+        else
+            col[M * LDA] = a0;
+        stage1_all2<N>(x, M, sgn, col, LDA, std::make_integer_sequence<int, (H + 1) / 2>{});
+    }
+    __syncwarp();
+}
+
+// One line of a staged plane, N values at ls.
+template <int N>
+__device__ __forceinline__ void line_read(const float2 *ls, float2 (&x)[N])
+{
+    if constexpr (N % 2 == 0) {
+#pragma unroll
+        for (int j = 0; j < N; j += 2) {
+            const float4 v = *reinterpret_cast<const float4 *>(ls + j);
+            x[j] = make_float2(v.x, v.y);
+            x[j + 1] = make_float2(v.z, v.w);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            x[j] = ls[j];
+    }
+}
+
+// Stage 2 of two planes: ys[d] = sum_j2 a1t[i3][j2] e(+-m2 j2 / N) for the disk points
+// d = (m2, m3(i3)), lanes 0-15 on the first plane's columns and lanes 16-31 on the second's, so a sphere
+// with c3 <= 16 keeps twice as many lanes busy as one plane would; written over the plane's a1t once
+// every lane holds its column, then each plane's cd values to dA and dB (dB null: one plane only).
+template <int N>
+__device__ __forceinline__ void p12c_stage2(int lane, int c3, int cd, int k2, float sgn, const int2 *dtab, float2 *a1t0,
+                                            float2 *a1t1, float2 *dA, float2 *dB)
+{
+    constexpr int H = (N - 1) / 2, LDA = N | 1;
+    const int half = lane >> 4, i3 = lane & 15;
+    float2 *a1t = half ? a1t1 : a1t0;
+    const bool act = i3 < c3 && (half == 0 || dB);
+    float2 y[N];
+    if (act) {
+        const float2 *cs = a1t + i3 * LDA;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            y[j] = cs[j];
+    }
+    __syncwarp();
+    if (act) {
+        pair_fold<N>(y);
+        stage2_all2<N>(y, k2, sgn, dtab + i3 * (H + 1), a1t, std::make_integer_sequence<int, H / 2 + 1>{});
+    }
+    __syncwarp();
+    for (int t = lane; t < cd; t += 32)
+        dA[t] = a1t0[t];
+    if (dB)
+        for (int t = lane; t < cd; t += 32)
+            dB[t] = a1t1[t];
+    __syncwarp();  // a1t is rewritten by the next pair
+}
+
+// dtab[i3][m2] = (disk index of (m2, m3), of (-m2, m3)), -1 where the disk has none
+template <int N>
+__device__ __forceinline__ void p12c_table(int2 *dtab, int c3, int np2, const int4 *g_pair2)
+{
+    constexpr int H = (N - 1) / 2;
+    for (int t = threadIdx.x; t < c3 * (H + 1); t += blockDim.x)
+        dtab[t] = make_int2(-1, -1);
+    __syncthreads();
+    for (int t = threadIdx.x; t < np2; t += blockDim.x) {
+        const int4 pr = g_pair2[t];  // (i3, m2 >= 0, disk index of m2, of -m2 or -1)
+        dtab[pr.x * (H + 1) + pr.y] = make_int2(pr.z, pr.w);
+    }
+    __syncthreads();
+}
+
+// A warp takes two tasks (planes) at a time: stage 1 of each, then stage 2 of both together.
 //
-// ASYNC (plain rows, even N, 16-byte aligned rows): the planes arrive by cp.async into two buffers
-// per warp, the next pair's first plane issued once this pair's first plane has been read and its
-// second plane once the second has been read, so the copies run behind the other plane's stage 1
-// and stage 2 instead of stalling the warp; 7 warps per CTA keep two CTAs per SM.
-template <int N, bool PAIR, bool ASYNC = false>  // two CTAs per SM (shared memory allows two at every compiled N)
+// ASYNC (even N, 16-byte aligned rows): the planes arrive by cp.async into two buffers per warp, the
+// next pair's first plane issued once this pair's first plane has been read and its second plane once
+// the second has been read, so the copies run behind the other plane's stage 1 and stage 2 instead of
+// stalling the warp; 7 warps per CTA keep two CTAs per SM.
+template <int N, bool ASYNC>  // two CTAs per SM (shared memory allows two at every compiled N)
 __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
     dft_plane12c_kernel(const float2 *__restrict__ X, long long ldx, int rows, int n1, int M, int cd, int np2, int k2,
-                        const int4 *__restrict__ g_pair2, float sgn, float2 *__restrict__ Y2, PairSrc ps)
+                        const int4 *__restrict__ g_pair2, float sgn, float2 *__restrict__ Y2)
 {
-    static_assert(!ASYNC || (!PAIR && N % 2 == 0), "the asynchronous form takes plain rows of even N");
+    static_assert(!ASYNC || N % 2 == 0, "the asynchronous form takes rows of even N");
     constexpr int NWARPS = ASYNC ? P12A_WARPS : P12_WARPS;
     constexpr int H = (N - 1) / 2;
     constexpr int SP = p12_pitch(N);
@@ -834,135 +946,24 @@ __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
     const int c3 = 2 * M + 1;
     int2 *dtab = reinterpret_cast<int2 *>(smem);  // [c3][H + 1]
     float2 *wbase = reinterpret_cast<float2 *>(smem + align16(sizeof(int2) * (size_t)c3 * (H + 1)));
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int t = tid; t < c3 * (H + 1); t += blockDim.x)
-        dtab[t] = make_int2(-1, -1);
-    __syncthreads();
-    for (int t = tid; t < np2; t += blockDim.x) {
-        const int4 pr = g_pair2[t];  // (i3, m2 >= 0, disk index of m2, of -m2 or -1)
-        dtab[pr.x * (H + 1) + pr.y] = make_int2(pr.z, pr.w);
-    }
-    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    p12c_table<N>(dtab, c3, np2, g_pair2);
     float2 *pl = wbase + (size_t)warp * p12c_warp_floats2(N, c3, ASYNC);  // [N][SP]
     float2 *pl2 = pl + (ASYNC ? N * SP : 0);                               // ASYNC: the second buffer
     float2 *a1t0 = pl2 + N * SP;                                           // [c3][LDA], first plane
     float2 *a1t1 = a1t0 + c3 * LDA;                                        // [c3][LDA], second plane
-    const bool vec = (N % 2 == 0) && (ldx % 2 == 0) && ((reinterpret_cast<size_t>(X) & 15) == 0);
-    // task -> (row, j1): plain rows row-major, pair rows j1-major (the warps of a CTA share psi_v);
-    // 32-bit arithmetic (the launcher keeps rows n1 below 2^31)
+    // task -> (row, j1), row-major; 32-bit arithmetic (the launcher keeps rows n1 below 2^31)
     const unsigned ntasks = (unsigned)rows * (unsigned)n1, npairs = (ntasks + 1) / 2;
-    auto locate = [&](unsigned task, long long &row, int &j1) {
-        if (PAIR) {
-            const unsigned q = task / (unsigned)rows;
-            j1 = (int)q;
-            row = (long long)(task - q * (unsigned)rows);
-        } else {
-            const unsigned q = task / (unsigned)n1;
-            row = (long long)q;
-            j1 = (int)(task - q * (unsigned)n1);
-        }
+    auto source = [&](unsigned task) {
+        const unsigned row = task / (unsigned)n1;
+        return X + (long long)row * ldx + (size_t)(task - row * (unsigned)n1) * plane;
     };
-    // one plane into pl (pair densities formed on the way)
-    auto load_plane = [&](long long row, int j1) {
-        const float2 *src, *srcv = nullptr;
-        float w = 0.f;
-        if (PAIR) {
-            const int kk = (int)row, v = kk / ps.nc;
-            src = X + (size_t)(ps.c0 + kk - v * ps.nc) * ldx + (size_t)j1 * plane;
-            srcv = X + (size_t)v * ldx + (size_t)j1 * plane;
-            w = ps.sw[kk];
-        } else {
-            src = X + row * ldx + (size_t)j1 * plane;
-        }
-        if (N % 2 == 0 && vec) {
-            constexpr int QR = N / 2;  // 16-byte words per line
-            const float4 *s4 = reinterpret_cast<const float4 *>(src);
-            const float4 *v4 = reinterpret_cast<const float4 *>(srcv);
-            constexpr int UNR = PAIR ? 4 : 8;  // loads in flight per lane (pair rows load two values)
-#pragma unroll UNR
-            for (int q = lane; q < N * QR; q += 32) {
-                const int j2 = q / QR, c = q - j2 * QR;
-                float4 x = __ldg(s4 + q);
-                if (PAIR) {
-                    const float4 a = __ldg(v4 + q);
-                    const float2 lo = pair_or_x<PAIR>(make_float2(a.x, a.y), make_float2(x.x, x.y), w);
-                    const float2 hi = pair_or_x<PAIR>(make_float2(a.z, a.w), make_float2(x.z, x.w), w);
-                    x = make_float4(lo.x, lo.y, hi.x, hi.y);
-                }
-                *reinterpret_cast<float4 *>(pl + j2 * SP + 2 * c) = x;
-            }
-        } else {
-#pragma unroll 8
-            for (int q = lane; q < plane; q += 32) {
-                const int j2 = q / N, j3 = q - j2 * N;
-                const float2 xs = __ldg(src + q);
-                pl[j2 * SP + j3] = PAIR ? pair_or_x<true>(__ldg(srcv + q), xs, w) : xs;
-            }
-        }
-        __syncwarp();
-    };
-    // stage 1 of the plane in buffer b: a1t[M + m3][j2] = sum_j3 x[j2][j3] e(+-m3 j3 / N)
     auto stage1 = [&](const float2 *b, float2 *a1t) {
-        for (int j2 = lane; j2 < N; j2 += 32) {
-            float2 x[N];
-            const float2 *ls = b + j2 * SP;
-            if constexpr (N % 2 == 0) {
-#pragma unroll
-                for (int j = 0; j < N; j += 2) {
-                    const float4 v = *reinterpret_cast<const float4 *>(ls + j);
-                    x[j] = make_float2(v.x, v.y);
-                    x[j + 1] = make_float2(v.z, v.w);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    x[j] = ls[j];
-            }
-            pair_fold<N>(x);
-            float2 a0 = x[0];
-#pragma unroll
-            for (int j = 1; j <= H; ++j) {  // the m3 = 0 sum, in the order of the table form
-                a0.x += x[j].x;
-                a0.y += x[j].y;
-            }
-            float2 *col = a1t + j2;
-            if constexpr (N % 2 == 0)
-                col[M * LDA] = make_float2(a0.x + x[N / 2].x, a0.y + x[N / 2].y);
-            else
-                col[M * LDA] = a0;
-            stage1_all2<N>(x, M, sgn, col, LDA, std::make_integer_sequence<int, (H + 1) / 2>{});
-        }
-        __syncwarp();  // the buffer is rewritten by a later plane
+        p12c_stage1<N>(lane, M, sgn, a1t, [&](int j2, float2(&x)[N]) { line_read<N>(b + j2 * SP, x); });
     };
-    // stage 2 of a pair: ys[d] = sum_j2 a1t[i3][j2] e(+-m2 j2 / N) for the disk points
-    // d = (m2, m3(i3)), written over the plane's a1t once every lane holds its column; then both
-    // planes' cd values to the workspace
-    auto stage2 = [&](long long rowA, int j1A, long long rowB, int j1B, bool hasB) {
-        const int half = lane >> 4, i3 = lane & 15;
-        float2 *a1t = half ? a1t1 : a1t0;
-        const bool act = i3 < c3 && (half == 0 || hasB);
-        float2 y[N];
-        if (act) {
-            const float2 *cs = a1t + i3 * LDA;
-#pragma unroll
-            for (int j = 0; j < N; ++j)
-                y[j] = cs[j];
-        }
-        __syncwarp();
-        if (act) {
-            pair_fold<N>(y);
-            stage2_all2<N>(y, k2, sgn, dtab + i3 * (H + 1), a1t, std::make_integer_sequence<int, H / 2 + 1>{});
-        }
-        __syncwarp();
-        float2 *dA = Y2 + (rowA * n1 + j1A) * cd;
-        for (int t = lane; t < cd; t += 32)
-            dA[t] = a1t0[t];
-        if (hasB) {
-            float2 *dB = Y2 + (rowB * n1 + j1B) * cd;
-            for (int t = lane; t < cd; t += 32)
-                dB[t] = a1t1[t];
-        }
-        __syncwarp();  // a1t is rewritten by the next pair
+    auto stage2 = [&](unsigned tA, bool hasB) {
+        float2 *d = Y2 + (size_t)tA * cd;  // task order is row-major
+        p12c_stage2<N>(lane, c3, cd, k2, sgn, dtab, a1t0, a1t1, d, hasB ? d + cd : nullptr);
     };
     const unsigned ustride = gridDim.x * NWARPS;
     if constexpr (ASYNC) {
@@ -970,10 +971,7 @@ __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
         // t is past the end, so that every wait below sees the same count of groups)
         auto issue = [&](unsigned t, float2 *b) {
             if (t < ntasks) {
-                long long row;
-                int j1;
-                locate(t, row, j1);
-                const float2 *src = X + row * ldx + (size_t)j1 * plane;
+                const float2 *src = source(t);
                 constexpr int QR = N / 2;
 #pragma unroll 4
                 for (int q = lane; q < N * QR; q += 32) {
@@ -987,13 +985,8 @@ __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
         issue(2 * u, pl);
         issue(2 * u + 1, pl2);
         for (; u < npairs; u += ustride) {
-            const unsigned tA = 2 * u, tB = tA + 1, nA = 2 * (u + ustride);
-            const bool hasB = tB < ntasks;
-            long long rowA, rowB = 0;
-            int j1A, j1B = 0;
-            locate(tA, rowA, j1A);
-            if (hasB)
-                locate(tB, rowB, j1B);
+            const unsigned tA = 2 * u, nA = 2 * (u + ustride);
+            const bool hasB = tA + 1 < ntasks;
             cp_async_wait<1>();  // groups in flight: this pair's A and B; A is in
             __syncwarp();
             stage1(pl, a1t0);
@@ -1003,25 +996,150 @@ __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
             if (hasB)
                 stage1(pl2, a1t1);
             issue(nA + 1 < 2 * npairs ? nA + 1 : ntasks, pl2);  // the next pair's B
-            stage2(rowA, j1A, rowB, j1B, hasB);
+            stage2(tA, hasB);
         }
         cp_async_wait<0>();
     } else {
+        const bool vec = (N % 2 == 0) && (ldx % 2 == 0) && ((reinterpret_cast<size_t>(X) & 15) == 0);
+        auto load_plane = [&](unsigned t) {
+            const float2 *src = source(t);
+            if (N % 2 == 0 && vec) {
+                constexpr int QR = N / 2;  // 16-byte words per line
+                const float4 *s4 = reinterpret_cast<const float4 *>(src);
+#pragma unroll 8
+                for (int q = lane; q < N * QR; q += 32) {
+                    const int j2 = q / QR, c = q - j2 * QR;
+                    *reinterpret_cast<float4 *>(pl + j2 * SP + 2 * c) = __ldg(s4 + q);
+                }
+            } else {
+#pragma unroll 8
+                for (int q = lane; q < plane; q += 32) {
+                    const int j2 = q / N, j3 = q - j2 * N;
+                    pl[j2 * SP + j3] = __ldg(src + q);
+                }
+            }
+            __syncwarp();
+        };
         for (unsigned u = blockIdx.x * NWARPS + warp; u < npairs; u += ustride) {
-            const unsigned tA = 2 * u, tB = tA + 1;
-            const bool hasB = tB < ntasks;
-            long long rowA, rowB = 0;
-            int j1A, j1B = 0;
-            locate(tA, rowA, j1A);
-            load_plane(rowA, j1A);
+            const unsigned tA = 2 * u;
+            const bool hasB = tA + 1 < ntasks;
+            load_plane(tA);
             stage1(pl, a1t0);
             if (hasB) {
-                locate(tB, rowB, j1B);
-                load_plane(rowB, j1B);
+                load_plane(tA + 1);
                 stage1(pl, a1t1);
             }
-            stage2(rowA, j1A, rowB, j1B, hasB);
+            stage2(tA, hasB);
         }
+    }
+}
+
+// Pair-density rows.  A CTA takes, at one j1, the planes of TV occupied and TC unoccupied states into
+// shared memory and transforms the TV TC products, two tasks a warp at a time: the line of the product,
+// conj(psi_v) psi_c w, is formed in registers as stage 1 reads it (the FP32 operations of
+// pair_density_tiled_kernel).  Ten planes are copied for 24 tasks, where a plane of psi_c per task, staged by
+// the warp that used it, cost 3.4 GB of L2 loads at 24^3 with 32 / 480 states (454 us; now 393).  Bound: issue
+// slots and the dependences of 12 warps an SM.  6 warps a CTA keep the folded line, the accumulators and
+// the constant pairs in 168 registers; 7 and 8 warps (128 registers) took 455 and 416 us, one CTA of 16
+// warps with the next tile's planes copied ahead 447 us.
+constexpr int P12P_WARPS = 6, P12P_PLANES = 4 + P12P_WARPS, P12P_TV = 4;
+
+struct PairTile {
+    int tv, tc;
+};
+
+// Dynamic shared memory of a CTA with `planes` staged planes, and the tile that fits two CTAs an SM.
+__host__ __device__ inline size_t p12p_smem(int N, int c3, int planes)
+{
+    return align16(sizeof(int2) * (size_t)c3 * ((N - 1) / 2 + 1)) +
+           sizeof(float2) * ((size_t)planes * N * p12_pitch(N) + (size_t)P12P_WARPS * 2 * c3 * (N | 1));
+}
+
+static PairTile pair_tile(int N, int c3, int nv, int nc)
+{
+    int planes = P12P_PLANES;
+    while (planes > 2 && p12p_smem(N, c3, planes) > 112 * 1024)
+        --planes;
+    const int tv = std::min({nv, P12P_TV, planes / 2});
+    return {tv, std::min(nc, planes - tv)};
+}
+
+template <int N>
+__global__ void __launch_bounds__(P12P_WARPS * 32, 2)
+    dft_pairs12c_kernel(const float2 *__restrict__ psi, long long ldx, int n1, int M, int cd, int np2, int k2,
+                        const int4 *__restrict__ g_pair2, float sgn, float2 *__restrict__ Y2, PairSrc ps, PairTile tl)
+{
+    constexpr int H = (N - 1) / 2;
+    constexpr int SP = p12_pitch(N);
+    constexpr int LDA = N | 1;
+    constexpr int plane = N * N;
+    extern __shared__ __align__(16) uint8_t smem[];
+    const int c3 = 2 * M + 1;
+    int2 *dtab = reinterpret_cast<int2 *>(smem);  // [c3][H + 1]
+    float2 *planes = reinterpret_cast<float2 *>(smem + align16(sizeof(int2) * (size_t)c3 * (H + 1)));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    p12c_table<N>(dtab, c3, np2, g_pair2);
+    float2 *a1t0 = planes + (size_t)(tl.tv + tl.tc) * N * SP + (size_t)warp * 2 * c3 * LDA;  // [c3][LDA] each
+    float2 *a1t1 = a1t0 + c3 * LDA;
+    const bool vec = (N % 2 == 0) && (ldx % 2 == 0) && ((reinterpret_cast<size_t>(psi) & 15) == 0);
+    const unsigned nvb = (ps.nv + tl.tv - 1) / tl.tv, ncb = (ps.nc + tl.tc - 1) / tl.tc, ntiles = nvb * ncb * n1;
+    for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const unsigned vb = t % nvb, r = t / nvb, cb = r % ncb;
+        const int j1 = (int)(r / ncb), v0 = (int)vb * tl.tv, c0 = (int)cb * tl.tc;
+        const int nvt = min(tl.tv, ps.nv - v0), nct = min(tl.tc, ps.nc - c0);
+        for (int p = warp; p < nvt + nct; p += P12P_WARPS) {
+            const int b = p < nvt ? v0 + p : ps.c0 + c0 + p - nvt;
+            const float2 *src = psi + b * ldx + (size_t)j1 * plane;
+            float2 *dst = planes + (size_t)p * N * SP;
+            if (N % 2 == 0 && vec) {
+                constexpr int QR = N / 2;
+#pragma unroll 4
+                for (int q = lane; q < N * QR; q += 32) {
+                    const int j2 = q / QR, c = q - j2 * QR;
+                    cp_async16(dst + j2 * SP + 2 * c, src + 2 * q);
+                }
+            } else {
+#pragma unroll 4
+                for (int q = lane; q < plane; q += 32) {
+                    const int j2 = q / N, j3 = q - j2 * N;
+                    cp_async8(dst + j2 * SP + j3, src + q);
+                }
+            }
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+        auto stage1 = [&](int task, float2 *a1t) {  // returns the task's row of Y2
+            const int v = task / nct, c = task - v * nct;
+            const long long row = (long long)(v0 + v) * ps.nc + c0 + c;
+            const float w = ps.sw[row];
+            const float2 *pv = planes + (size_t)v * N * SP, *pc = planes + (size_t)(nvt + c) * N * SP;
+            p12c_stage1<N>(lane, M, sgn, a1t, [&](int j2, float2(&x)[N]) {
+                const float2 *lv = pv + j2 * SP, *lc = pc + j2 * SP;
+                if constexpr (N % 2 == 0) {
+#pragma unroll
+                    for (int j = 0; j < N; j += 2) {
+                        const float4 a = *reinterpret_cast<const float4 *>(lv + j);
+                        const float4 b = *reinterpret_cast<const float4 *>(lc + j);
+                        x[j] = pair_or_x<true>(make_float2(a.x, a.y), make_float2(b.x, b.y), w);
+                        x[j + 1] = pair_or_x<true>(make_float2(a.z, a.w), make_float2(b.z, b.w), w);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        x[j] = pair_or_x<true>(lv[j], lc[j], w);
+                }
+            });
+            return Y2 + (row * n1 + j1) * cd;
+        };
+        const int nt = nvt * nct;
+        for (int u = 2 * warp; u < nt; u += 2 * P12P_WARPS) {
+            float2 *dA = stage1(u, a1t0), *dB = nullptr;
+            if (u + 1 < nt)
+                dB = stage1(u + 1, a1t1);
+            p12c_stage2<N>(lane, c3, cd, k2, sgn, dtab, a1t0, a1t1, dA, dB);
+        }
+        __syncthreads();  // the planes are rewritten by the next tile
     }
 }
 
@@ -1334,36 +1452,47 @@ static cudaError_t launch_p12_t(int grid, size_t smem, const float2 *X, long lon
     return cudaGetLastError();
 }
 
-template <int N, bool PAIR, bool ASYNC>
+template <int N, bool ASYNC>
 static cudaError_t launch_p12c_t(int grid, const float2 *X, long long ldx, int rows, const DftPlan &p, float sgn,
-                                 float2 *work, PairSrc ps, cudaStream_t s)
+                                 float2 *work, cudaStream_t s)
 {
     const size_t smem = p12c_smem(N, p.c3, ASYNC);
-    cudaError_t e = cudaFuncSetAttribute(dft_plane12c_kernel<N, PAIR, ASYNC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(dft_plane12c_kernel<N, ASYNC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
-    dft_plane12c_kernel<N, PAIR, ASYNC><<<grid, (ASYNC ? P12A_WARPS : P12_WARPS) * 32, smem, s>>>(
-        X, ldx, rows, p.n[0], p.sym3, p.cd, p.np2, p.k2, p.pair2, sgn, work, ps);
+    dft_plane12c_kernel<N, ASYNC><<<grid, (ASYNC ? P12A_WARPS : P12_WARPS) * 32, smem, s>>>(
+        X, ldx, rows, p.n[0], p.sym3, p.cd, p.np2, p.k2, p.pair2, sgn, work);
     return cudaGetLastError();
 }
 
-// Plain rows of even N on 16-byte boundaries take the asynchronous form.
+// Pair rows have their own kernel; plain rows of even N on 16-byte boundaries take the asynchronous form.
 template <int N>
 static cudaError_t launch_p12c(int grid, const float2 *X, long long ldx, int rows, const DftPlan &p, float sgn,
                                float2 *work, const PairSrc *ps, cudaStream_t s)
 {
-    if (ps)
-        return launch_p12c_t<N, true, false>(grid, X, ldx, rows, p, sgn, work, *ps, s);
+    if (ps) {
+        const PairTile tl = pair_tile(N, p.c3, ps->nv, ps->nc);
+        const size_t smem = p12p_smem(N, p.c3, tl.tv + tl.tc);
+        const cudaError_t e =
+            cudaFuncSetAttribute(dft_pairs12c_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess)
+            return e;
+        // at most rows n1 tiles, which the caller keeps below 2^31
+        const long long nt = (long long)((ps->nv + tl.tv - 1) / tl.tv) * ((ps->nc + tl.tc - 1) / tl.tc) * p.n[0];
+        dft_pairs12c_kernel<N><<<(int)std::min<long long>(nt, 152LL * 2), P12P_WARPS * 32, smem, s>>>(
+            X, ldx, p.n[0], p.sym3, p.cd, p.np2, p.k2, p.pair2, sgn, work, *ps, tl);
+        return cudaGetLastError();
+    }
     if constexpr (N % 2 == 0) {
         if (ldx % 2 == 0 && (reinterpret_cast<size_t>(X) & 15) == 0 &&
             p12c_smem(N, p.c3, true) <= DFT_SMEM_MAX) {
             const long long ntasks = (long long)rows * p.n[0];
             const int ga = (int)std::min<long long>((ntasks + P12A_WARPS - 1) / P12A_WARPS, 152LL * 16);
-            return launch_p12c_t<N, false, true>(ga, X, ldx, rows, p, sgn, work, PairSrc{nullptr, 0, 1, 0}, s);
+            return launch_p12c_t<N, true>(ga, X, ldx, rows, p, sgn, work, s);
         }
     }
-    return launch_p12c_t<N, false, false>(grid, X, ldx, rows, p, sgn, work, PairSrc{nullptr, 0, 1, 0}, s);
+    return launch_p12c_t<N, false>(grid, X, ldx, rows, p, sgn, work, s);
 }
 
 template <int N1>
