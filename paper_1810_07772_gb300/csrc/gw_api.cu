@@ -1557,10 +1557,14 @@ gw_status gw_load_states_g(gw_ctx *h, int n1, int n2, int n3, double cell_L, int
     std::vector<int> idx(npw);
     std::vector<char> seen(nr, 0);
     const int nn[3] = {n1, n2, n3};
+    StateAxes ax = {{n1, n2, n3}, {0, 0, 0}, {0, 0, 0}};
     for (int p = 0; p < npw; ++p) {
         int j[3];
-        for (int a = 0; a < 3; ++a)
+        for (int a = 0; a < 3; ++a) {
             j[a] = ((gvec_psi[3 * p + a] % nn[a]) + nn[a]) % nn[a];
+            ax.m[a] += !(ax.mask[a] >> j[a] & 1);
+            ax.mask[a] |= 1ull << j[a];
+        }
         const int lin = (j[0] * n2 + j[1]) * n3 + j[2];
         if (seen[lin])
             return fail(c, GW_E_INVALID, "plane wave %d (%d, %d, %d) aliases an earlier one on the %d x %d x %d grid",
@@ -1579,7 +1583,8 @@ gw_status gw_load_states_g(gw_ctx *h, int n1, int n2, int n3, double cell_L, int
     const size_t ncoef = (size_t)nb * npw, n = (size_t)nb * nr;
     GW_TRY(ensure(c, c.d_gidx, c.cap.gidx, npw * sizeof(int), "plane-wave indices"));
     GW_TRY(ensure(c, c.d_gtw, c.cap.gtw, tw.size() * sizeof(float2), "axis twiddles"));
-    GW_TRY(ensure(c, c.d_psig, c.cap.psig, n * sizeof(float2), "state transform workspace"));
+    if (!states_fused(ax))
+        GW_TRY(ensure(c, c.d_psig, c.cap.psig, n * sizeof(float2), "state transform workspace"));
     GW_TRY(ensure(c, c.d_psi, c.cap.psi, n * sizeof(float2), "state staging"));
     GW_CUDA(cudaMemcpyAsync(c.d_gidx, idx.data(), npw * sizeof(int), cudaMemcpyHostToDevice, s), "copy indices");
     GW_CUDA(cudaMemcpyAsync(c.d_gtw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, s),
@@ -1604,7 +1609,7 @@ gw_status gw_load_states_g(gw_ctx *h, int n1, int n2, int n3, double cell_L, int
         }
         coef64 = c.d_coef;
     }
-    GW_CUDA(launch_states_from_g(coef64, nb, npw, c.d_gidx, n1, n2, n3, c.d_gtw, c.d_psig, c.d_psi, s),
+    GW_CUDA(launch_states_from_g(coef64, nb, npw, c.d_gidx, ax, c.d_gtw, c.d_psig, c.d_psi, s),
             "states to the grid");
     // host vectors idx and tw are read by the copies above: finish them before they go out of scope
     GW_CUDA(cudaStreamSynchronize(s), "transform sync");

@@ -457,7 +457,12 @@ cudaError_t closure_enqueue(const float2 *psiT, int nr, int nb, int nv, const do
                             const int *gvec_dev, int ng, const float2 *Ph, float2 *out, void *work,
                             cudaStream_t s);
 // k_states.cu
-cudaError_t launch_states_from_g(const float2 *coef, int nb, int npw, const int *idx, int n1, int n2, int n3,
+struct StateAxes {
+    int n[3], m[3];               // grid points and used Miller indices (modulo n) of each axis
+    unsigned long long mask[3];   // the used indices
+};
+bool states_fused(const StateAxes &ax);
+cudaError_t launch_states_from_g(const float2 *coef, int nb, int npw, const int *idx, const StateAxes &ax,
                                  const float2 *tw, float2 *work, float2 *out, cudaStream_t s);
 cudaError_t launch_kweight(float2 *PG, const float2 *sum, size_t n, float w, bool acc, cudaStream_t s);
 cudaError_t zgemm_enqueue(ZPlan &p, const double2 *A, long lda, const double2 *B, long ldb, double2 *C, void *work,
