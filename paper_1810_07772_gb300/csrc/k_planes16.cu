@@ -339,16 +339,36 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// max |M[k][j]| over a complex64 matrix (rows x cols, row stride ld), as float bits.
+// max |M[k][j]| over a complex64 matrix (rows x cols, row stride ld), as float bits; the root is monotonic, so
+// it is taken of the largest square.  VEC: contiguous rows (ld = cols) on a 16-byte boundary, two values a
+// load.  At 15360 x 691 (85 MB): 32 us with a 64-bit division and a root per value, now 26 (mostly HBM: the
+// transform before it leaves L2 full of its own writes).
+template <bool VEC>
 __global__ void absmax_c64_kernel(const float2 *__restrict__ M, int rows, int cols, long ld, unsigned *bound_bits)
 {
     float best = 0.f;
-    const size_t total = (size_t)rows * cols;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int k = static_cast<int>(i / cols), j = static_cast<int>(i - (size_t)k * cols);
-        const float2 z = M[(size_t)k * ld + j];
-        best = fmaxf(best, sqrtf(z.x * z.x + z.y * z.y));
+    const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        const size_t total = (size_t)rows * cols, pairs = total / 2;
+        const float4 *v = reinterpret_cast<const float4 *>(M);
+#pragma unroll 4
+        for (size_t i = tid; i < pairs; i += nt) {
+            const float4 z = v[i];
+            best = fmaxf(best, fmaxf(z.x * z.x + z.y * z.y, z.z * z.z + z.w * z.w));
+        }
+        if (tid == 0 && (total & 1)) {
+            const float2 z = M[total - 1];
+            best = fmaxf(best, z.x * z.x + z.y * z.y);
+        }
+    } else {
+        const int warps = (int)(nt >> 5);
+        for (int k = (int)(tid >> 5); k < rows; k += warps)
+            for (int j = threadIdx.x & 31; j < cols; j += 32) {
+                const float2 z = M[(size_t)k * ld + j];
+                best = fmaxf(best, z.x * z.x + z.y * z.y);
+            }
     }
+    best = sqrtf(best);
     for (int o = 16; o > 0; o >>= 1)
         best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
     if ((threadIdx.x & 31) == 0)
@@ -358,30 +378,45 @@ __global__ void absmax_c64_kernel(const float2 *__restrict__ M, int rows, int co
 // The 16-bit hi/lo planes of a complex64 matrix M[k][j] (k < rows, j < cols), in the operand
 // layout of herk16_kernel with the column index j in the place of r: row k of M is one "pair
 // density" of the rank-k update, scaled by 2^scale_exp and split as pair_density16_kernel does.
+// A thread takes eight consecutive k of one j, which are 16 contiguous bytes of each plane; the lanes of
+// a warp are on consecutive j, so each of the eight loads is one contiguous run.  At 15360 x 691: a value
+// per thread with 2-byte stores took 43 us, now 28.
 template <bool BF16>
-__global__ void planes16_from_c64_kernel(const float2 *__restrict__ M, int rows, int cols, long ld, int kpad,
-                                         int cols_pad, const int *__restrict__ scale_exp, uint16_t *__restrict__ F)
+__global__ void __launch_bounds__(256)
+    planes16_from_c64_kernel(const float2 *__restrict__ M, int rows, int cols, long ld, int kpad, int cols_pad,
+                             const int *__restrict__ scale_exp, uint16_t *__restrict__ F)
 {
     const float s = ldexpf(1.0f, *scale_exp);
-    const size_t per_chunk = (size_t)cols_pad * KC16;
-    const size_t total = (size_t)(kpad / KC16) * per_chunk;
+    const size_t total = (size_t)(kpad / 8) * cols_pad;  // cols_pad is a multiple of 128
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t kc = i / per_chunk;
-        const int rem = static_cast<int>(i - kc * per_chunk);
-        const int j = (rem >> 7) * 8 + ((rem & 63) >> 3);
-        const int k = static_cast<int>(kc) * KC16 + ((rem & 127) >> 6) * 8 + (rem & 7);
-        float fr = 0.f, fi = 0.f;
-        if (j < cols && k < rows) {
-            const float2 z = M[(size_t)k * ld + j];
-            fr = z.x * s;
-            fi = z.y * s;
+        const int kg = (int)(i / cols_pad), j = (int)(i - (size_t)kg * cols_pad), k0 = kg * 8;
+        float2 z[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            z[e] = j < cols && k0 + e < rows ? M[(size_t)(k0 + e) * ld + j] : make_float2(0.f, 0.f);
+        uint32_t w[4][4];  // planes x words of two values
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            uint16_t h[4][2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float fr = z[e + u].x * s, fi = z[e + u].y * s;
+                const uint16_t rh = to16<BF16>(fr), ih = to16<BF16>(fi);
+                h[P4_RH][u] = rh;
+                h[P4_RL][u] = to16<BF16>(fr - from16<BF16>(rh));
+                h[P4_IH][u] = ih;
+                h[P4_IL][u] = to16<BF16>(fi - from16<BF16>(ih));
+            }
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+                w[p][e / 2] = h[p][0] | ((uint32_t)h[p][1] << 16);
         }
-        const uint16_t rh = to16<BF16>(fr), ih = to16<BF16>(fi), il = to16<BF16>(fi - from16<BF16>(ih));
-        uint16_t *base = F + plane16_block((int)kc, rem >> 11, cols_pad / 128, NPL, 0) + (rem & 2047);
-        base[P4_RH * 2048] = rh;
-        base[P4_RL * 2048] = to16<BF16>(fr - from16<BF16>(rh));
-        base[P4_IH * 2048] = ih;
-        base[P4_IL * 2048] = il;
+        const int jr = j & 127;
+        uint16_t *base = F + plane16_block(kg >> 1, j >> 7, cols_pad / 128, NPL, 0) + (jr >> 3) * 128 + (kg & 1) * 64 +
+                         (jr & 7) * 8;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            *reinterpret_cast<uint4 *>(base + p * 2048) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
     }
 }
 
@@ -470,11 +505,14 @@ cudaError_t launch_planes16_from_c64(const float2 *M, int rows, int cols, long l
     cudaError_t e = cudaMemsetAsync(bound_bits, 0, sizeof(unsigned), s);
     if (e != cudaSuccess)
         return e;
-    absmax_c64_kernel<<<grid_for((size_t)rows * cols), 256, 0, s>>>(M, rows, cols, ld, bound_bits);
+    if (ld == cols && (reinterpret_cast<uintptr_t>(M) & 15) == 0)
+        absmax_c64_kernel<true><<<grid_for((size_t)rows * cols / 8), 256, 0, s>>>(M, rows, cols, ld, bound_bits);
+    else
+        absmax_c64_kernel<false><<<grid_for((size_t)rows * 32), 256, 0, s>>>(M, rows, cols, ld, bound_bits);
     count_launches(1);
     scale_exp_kernel<<<1, 1, 0, s>>>(bound_bits, 1.0f, bf16 ? 1 : 0, scale_exp);
     count_launches(1);
-    const size_t total = (size_t)kpad * cols_pad;
+    const size_t total = (size_t)kpad * cols_pad / 8;
     if (bf16)
         planes16_from_c64_kernel<true><<<grid_for(total), 256, 0, s>>>(M, rows, cols, ld, kpad, cols_pad, scale_exp, F);
     else
