@@ -516,11 +516,11 @@ GW_API gw_status gw_mlp_num_params(int n_in, int hidden, size_t *n);
  *   max_batch  largest batch of gw_mlp_grad / gw_mlp_train_step, and the chunk of gw_mlp_forward;
  *              1..2^22
  *   stream     cudaStream_t for every call on the handle (NULL = legacy default stream)
- * Device memory: 5 P floats, P halves, 5 max_batch x hidden floats, a split-K workspace of
- * 64 x hidden x (hidden + 1) floats, and the tensor-core operands of training at 6 bytes a value
- * (three BF16 parts): 6 x (7 hidden + 144) bytes per row of max_batch (activations and deltas in
- * two orientations; the inputs padded to 16 and 128) plus five weight matrices; gw_mlp_infer adds
- * 272 KB of tiled weights. */
+ * Device memory: 5 P floats, P halves, 3 max_batch x hidden floats, the partial sums of the gradient
+ * (at most 64 x hidden x (2 hidden + n_in) floats and 3 (hidden + 1) per 16 rows of max_batch), and the
+ * tensor-core operands of training at 6 bytes a value (three BF16 parts): 6 x (8 hidden + 144) bytes per row of
+ * max_batch (activations and deltas in two orientations; the inputs padded to 16 and 128) plus five weight
+ * matrices; gw_mlp_infer adds 272 KB of tiled weights. */
 GW_API gw_status gw_mlp_create(gw_mlp **out, int device, int n_in, int hidden, int max_batch, void *stream);
 GW_API gw_status gw_mlp_destroy(gw_mlp *m);
 GW_API gw_status gw_mlp_last_error(gw_mlp *m, char *buf, size_t n);

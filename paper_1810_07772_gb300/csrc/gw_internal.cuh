@@ -329,32 +329,59 @@ cudaError_t launch_mlp_tc_forward(const float *X, long n, int n_in, const uint8_
                                   const float *b2, const float *b3, const __half *W4, const float *b4, float *Y,
                                   int num_sms, uint32_t *err, uint64_t wait_ns, cudaStream_t s);
 
-// k_mlp_train.cu: tensor-core products of the correction network's training step.  Operands in the
-// three-part BF16 block layout (mlp_pack3_bytes(rows, k) bytes); launch_mlp_pack3 writes an FP32
-// matrix S [R][C] (rows gathered by `rows` if given) as rowop (rows R, k = C) and/or colop (rows
-// C, k = R) and, if colsum is given, the column sums of each 128-row tile to colsum[ceil(R/128)][C].
-// launch_mlp_gemm3: C(m, n) = sum_k A(m, k) B(n, k) (M x N, K), epi 0 = partial products of up to
-// `splits` slices of K at C + z * zstride, 1 = tanh(acc + bias[n]), 2 = acc * (1 - H(m, n)^2);
-// the slice count used goes to *slices_used.
-// launch_mlp_gemm3 with epi 1 or 2 also writes its result (M x N) to rowop (rows M, k = N), colop
-// (rows N, k = M) and its column sums per 128-row tile to colsum, where given.
+// k_mlp_train.cu: the kernels of the correction network's training step.  Operands are in the three-part BF16
+// block layout (mlp_pack3_bytes(rows, k) bytes): "rowop" has the matrix's rows as rows and its columns as k,
+// "colop" its columns as rows and its rows as k.
+// launch_mlp_pack_x: the inputs X[rows ? rows[r] : r] (R x C) as rowop and, where given, colop (its rows beyond C
+// are never written: clear it once).
+// launch_mlp_gemm3: C(m, n) = sum_k A(m, k) B(n, k) (M x N, K) of up to three jobs; epi 0 = partial products of
+// `slices` slices of K (mlp_gemm3_slices) at C + z M N, 1 = tanh(acc + bias[n]), 2 = acc * (1 - H(m, n)^2).  With
+// epi 1 or 2 the result also goes to rowop, colop and its column sums per 128-row tile to colsum, where given, and
+// C may be null.
+// launch_mlp_out_train: the output layer, loss and deltas of layer 3; csum and part have mlp_out_parts(batch) rows.
 // launch_mlp_pack_weights: W1 (hidden x n_in), W2, W3 (hidden x hidden) at w + off[l] into row[l]
 // (rows = outputs) and W2, W3 into col[0], col[1] (rows = inputs), element by element (the
 // padding of these buffers is never written: clear them once).
+// launch_mlp_finish: the gradient from its partial sums and, with adam, the parameters' step and weight operands.
 struct MlpWeightPack {
     uint8_t *row[3];
     uint8_t *col[2];
     long off[3];
     int hidden, n_in;
 };
+struct MlpGemmJob {
+    const uint8_t *A, *B;
+    int M, N, K, slices, kcs, ctas;  // ctas is filled in by the launch, slices and kcs too unless epi = 0
+    float *C;
+    const float *bias, *H;
+    uint8_t *rowop, *colop;
+    float *colsum;
+};
+struct MlpGemmJobs {
+    int n;
+    MlpGemmJob job[3];
+};
+struct MlpFinish {
+    const float *part[3], *csum[3], *out_part;  // slices of dW_l, column sums of D_l, [dW4 | db4 | loss]
+    int n_part[3], n_csum[3], n_out, nb_w;      // how many of each; nb_w is filled in by the launch
+    long off_b[3], off_out;
+    float *grad;                                // written without adam
+    float *loss;                                // loss_scale times the summed squares is added to it (may be null)
+    float loss_scale;
+    float *theta, *w32, *m, *v;
+    __half *theta16;
+    float lr, b1, b2, c1, c2, eps;
+};
 size_t mlp_pack3_bytes(int rows, int k);
+int mlp_gemm3_slices(int K, int splits, int *kcs);
+int mlp_out_parts(int batch);
+cudaError_t launch_mlp_pack_x(const float *X, const int *rows, int R, int C, uint8_t *rowop, uint8_t *colop,
+                              cudaStream_t s);
 cudaError_t launch_mlp_pack_weights(const float *w, const MlpWeightPack &p, int num_sms, cudaStream_t s);
-cudaError_t launch_mlp_pack3(const float *S, long ld, const int *rows, int R, int C, uint8_t *rowop, uint8_t *colop,
-                             float *colsum, cudaStream_t s);
-cudaError_t launch_mlp_gemm3(int epi, const uint8_t *A, int M, const uint8_t *B, int N, int K, int splits, float *C,
-                             long ldc, long zstride, const float *bias, const float *H, long ldh, uint8_t *rowop,
-                             uint8_t *colop, float *colsum, uint32_t *err, uint64_t wait_ns, cudaStream_t s,
-                             int *slices_used);
+cudaError_t launch_mlp_gemm3(int epi, MlpGemmJobs jobs, int num_sms, uint32_t *err, uint64_t wait_ns, cudaStream_t s);
+cudaError_t launch_mlp_out_train(const float *H2, int Hd, const __half *W4, const float *b4, int batch, const float *T,
+                                 const int *trow, uint8_t *rowop, uint8_t *colop, float *csum, float *part, cudaStream_t s);
+cudaError_t launch_mlp_finish(MlpFinish f, const MlpWeightPack &p, bool adam, int num_sms, cudaStream_t s);
 
 // k_dft_fused.cu: the whole sphere transform of a row in one kernel (planes streamed by bulk
 // copies, stages j1 -> m1, j2 -> m2, j3 -> m3 in shared memory), for grids whose planes and rows

@@ -11,7 +11,7 @@
 //                                accuracy; bias + tanh and tanh' in the epilogues; the weight
 //                                gradients over slices of the batch, added in a fixed order);
 //                                the 2-wide output layer, the loss, the deltas of layer 3 and
-//                                the output layer's gradient in one kernel (a warp per row, sums
+//                                the output layer's gradient in one kernel (16 rows per block, sums
 //                                per block added in a fixed order); the weights are the
 //                                FP16-rounded ones
 //   loss                         L = (1 / (2B)) sum (y - t)^2 and dL/dy = (y - t) / B
@@ -217,68 +217,13 @@ __global__ void __launch_bounds__(128) apply_kernel(float2 *PG, int ng, const fl
     }
 }
 
-// gW[e] = sum_z part[z * stride + e] (e < n_w) and, from blocks past the first nb_w,
-// gb[o] = sum_rb csum[rb * out + o] (o < out, rb < nrb): both in a fixed order
-__global__ void __launch_bounds__(256) grad_finish_kernel(const float *part, int S, long stride, long n_w, int nb_w,
-                                                          float *gW, const float *csum, int nrb, int out, float *gb)
-{
-    if ((int)blockIdx.x < nb_w) {
-        for (long e = blockIdx.x * 256L + threadIdx.x; e < n_w; e += (long)nb_w * 256) {
-            float acc = 0.f;
-            for (int z = 0; z < S; ++z)
-                acc += part[z * stride + e];
-            gW[e] = acc;
-        }
-        return;
-    }
-    const int o = ((int)blockIdx.x - nb_w) * 256 + threadIdx.x;
-    if (o < out) {
-        float acc = 0.f;
-        for (int rb = 0; rb < nrb; ++rb)
-            acc += csum[(long)rb * out + o];
-        gb[o] = acc;
-    }
-}
-
-// The 2-wide output layer, OUT_ROWS rows per block (8 warps, a warp per row at a time): y = W4 h + b4
-// (h = H2[b], W4 FP16) into Y.  With targets T (row trow[b] if given) also D4[b] = (y - t) / B,
-// loss += |y - t|^2 / (2B), the deltas of layer 3, D[b][n] = (D4[b] W4)[n] (1 - h[n]^2), and the
-// block's share of the output layer's gradient, part[block] = [sum_b D4[b] h^T (2 x Hd) | sum_b D4[b]]
-// (2 Hd + 2 values; each warp sums its rows in shared memory, the warps are then added in order).
+// The 2-wide output layer, OUT_ROWS rows per block (8 warps, a warp per row at a time): Y[b] = W4 h + b4
+// (h = H2[b], W4 FP16).
 constexpr int OUT_ROWS = 16;
-// out[e] = sum_s part[s * G + e] for one e per block: strided partial sums, then a tree, both in a
-// fixed order
-__global__ void __launch_bounds__(256) sum_parts_tree_kernel(const float *part, int S, long G, float *out)
-{
-    __shared__ float red[256];
-    const long e = blockIdx.x;
-    float acc = 0.f;
-    for (int z = threadIdx.x; z < S; z += 256)
-        acc += part[z * G + e];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        out[e] = red[0];
-}
-
 __global__ void __launch_bounds__(256) out_layer_kernel(const float *H2, int Hd, const __half *W4, const float *b4,
-                                                        int batch, float *Y, const float *T, const int *trow,
-                                                        float invB, float *D4, float *D, float *loss, float *part)
+                                                        int batch, float *Y)
 {
-    extern __shared__ float gsh[];  // [8 warps][2 Hd + 2]
-    __shared__ float red[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = 2 * Hd + 2;
-    float *g = gsh + warp * G;
-    if (T)
-        for (int e = lane; e < G; e += 32)
-            g[e] = 0.f;
-    __syncwarp();
-    float l2 = 0.f, s0 = 0.f, s1 = 0.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int rr = warp; rr < OUT_ROWS; rr += 8) {
         const int b = blockIdx.x * OUT_ROWS + rr;
         if (b >= batch)
@@ -295,68 +240,10 @@ __global__ void __launch_bounds__(256) out_layer_kernel(const float *H2, int Hd,
             y0 += __shfl_xor_sync(0xffffffffu, y0, o);
             y1 += __shfl_xor_sync(0xffffffffu, y1, o);
         }
-        y0 += b4[0];
-        y1 += b4[1];
         if (lane == 0) {
-            Y[2 * (long)b] = y0;
-            Y[2 * (long)b + 1] = y1;
+            Y[2 * (long)b] = y0 + b4[0];
+            Y[2 * (long)b + 1] = y1 + b4[1];
         }
-        if (T) {
-            const long r = trow ? trow[b] : b;
-            const float e0 = y0 - T[2 * r], e1 = y1 - T[2 * r + 1];
-            const float d0 = e0 * invB, d1 = e1 * invB;
-            if (lane == 0) {
-                D4[2 * (long)b] = d0;
-                D4[2 * (long)b + 1] = d1;
-            }
-            l2 += e0 * e0 + e1 * e1;
-            s0 += d0;
-            s1 += d1;
-            for (int n = lane; n < Hd; n += 32) {
-                const float hv = h[n];
-                const float w0 = __half2float(W4[n]), w1 = __half2float(W4[Hd + n]);
-                D[(long)b * Hd + n] = (d0 * w0 + d1 * w1) * (1.f - hv * hv);
-                g[n] += d0 * hv;
-                g[Hd + n] += d1 * hv;
-            }
-        }
-    }
-    if (!T)
-        return;
-    if (lane == 0) {
-        g[2 * Hd] = s0;
-        g[2 * Hd + 1] = s1;
-        red[warp] = l2;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < G; e += 256) {
-        float acc = 0.f;
-        for (int w = 0; w < 8; ++w)
-            acc += gsh[w * G + e];
-        part[(long)blockIdx.x * G + e] = acc;
-    }
-    if (threadIdx.x == 0 && loss) {
-        float t = 0.f;
-        for (int w = 0; w < 8; ++w)
-            t += red[w];
-        atomicAdd(loss, 0.5f * invB * t);
-    }
-}
-
-__global__ void adam_kernel(float *theta, __half *theta16, float *w32, const float *g, float *m, float *v, long P,
-                            float lr, float b1, float b2, float c1, float c2, float eps)
-{
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < P; i += (long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float t = theta[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-        theta[i] = t;
-        const __half t16 = __float2half_rn(t);
-        theta16[i] = t16;
-        w32[i] = __half2float(t16);
     }
 }
 
@@ -381,15 +268,18 @@ struct gw_mlp {
     cudaStream_t stream = nullptr;
     float *theta = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     __half *theta16 = nullptr;
-    float *H[3] = {}, *Da = nullptr, *Db = nullptr, *D4 = nullptr, *Y = nullptr, *part = nullptr;
+    float *H[3] = {};
     // tensor-core products: the FP16-rounded parameters as FP32, and the operands in the
     // three-part BF16 block layout: X, H0, H1 as layer inputs (row) and weight-gradient operands
-    // (col), the deltas (row: two, a product reads one and writes the other; col), W1..W3 (row)
+    // (col), the deltas of layers 2 and 3 (row: pD[l - 1]) and of all three (col; pDc[0] is pD[1]), W1..W3 (row)
     // and W2, W3 transposed (col)
     float *w32 = nullptr;
-    uint8_t *pX = nullptr, *pXc = nullptr, *pH[2] = {}, *pHc[2] = {}, *pD[2] = {}, *pDc = nullptr;
+    uint8_t *pX = nullptr, *pXc = nullptr, *pH[2] = {}, *pHc[2] = {}, *pD[2] = {}, *pDc[3] = {};
     uint8_t *pW[3] = {}, *pWc[2] = {};
-    float *csum = nullptr;  // column sums of the deltas per 128-row tile (bias gradients)
+    // sums of the gradient: slices of dW_l (at most `splits`), column sums of the deltas (db_l), the blocks'
+    // shares of [dW4 | db4 | loss]
+    float *part = nullptr, *csum[3] = {}, *out_part = nullptr;
+    int splits = 1;
     bool wpacked = false;
     long step = 0;
     // tensor-core inference: W1, W2, W3 in the operand layout (valid while tiled == true); d_err:
@@ -442,12 +332,8 @@ long num_params(int n_in, int hidden)
 
 constexpr uint64_t TC_WAIT_NS = 2000000000ull;
 
-// W1..W3 as the B operands of the forward products (rows = outputs) and W2, W3 transposed for the
-// products back through them (rows = inputs), from the FP16-rounded weights
-cudaError_t pack_weights(gw_mlp *m)
+gw::MlpWeightPack weight_pack(const gw_mlp *m)
 {
-    if (m->wpacked)
-        return cudaSuccess;
     gw::MlpWeightPack p{};
     for (int l = 0; l < 3; ++l) {
         p.row[l] = m->pW[l];
@@ -457,10 +343,24 @@ cudaError_t pack_weights(gw_mlp *m)
     p.col[1] = m->pWc[1];
     p.hidden = m->hidden;
     p.n_in = m->n_in;
-    const cudaError_t e = gw::launch_mlp_pack_weights(m->w32, p, m->num_sms, m->stream);
+    return p;
+}
+
+// W1..W3 as the B operands of the forward products (rows = outputs) and W2, W3 transposed for the
+// products back through them (rows = inputs), from the FP16-rounded weights
+cudaError_t pack_weights(gw_mlp *m)
+{
+    if (m->wpacked)
+        return cudaSuccess;
+    const cudaError_t e = gw::launch_mlp_pack_weights(m->w32, weight_pack(m), m->num_sms, m->stream);
     if (e == cudaSuccess)
         m->wpacked = true;
     return e;
+}
+
+cudaError_t gemm3(gw_mlp *m, int epi, const gw::MlpGemmJobs &jobs)
+{
+    return gw::launch_mlp_gemm3(epi, jobs, m->num_sms, m->d_err, TC_WAIT_NS, m->stream);
 }
 
 // Forward of `batch` rows of X (gathered by rows if given) into H[0..2] and Yout.  keep: also
@@ -471,89 +371,81 @@ cudaError_t forward_batch(gw_mlp *m, const float *X, const int *rows, int batch,
     const int Hd = m->hidden;
     cudaError_t e = pack_weights(m);
     if (e == cudaSuccess)
-        e = gw::launch_mlp_pack3(X, m->n_in, rows, batch, m->n_in, m->pX, keep ? m->pXc : nullptr, nullptr,
-                                 m->stream);
-    const uint8_t *Ain = m->pX;
-    int K = m->n_in;
+        e = gw::launch_mlp_pack_x(X, rows, batch, m->n_in, m->pX, keep ? m->pXc : nullptr, m->stream);
     // each layer also writes its output as the next layer's operand and, for the backward pass, as
     // the operand of a weight gradient
     for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
-        e = gw::launch_mlp_gemm3(1, Ain, batch, m->pW[l], Hd, K, 1, m->H[l], Hd, 0, m->theta + m->off_b[l], nullptr, 0,
-                                 l < 2 ? m->pH[l] : nullptr, keep && l < 2 ? m->pHc[l] : nullptr, nullptr, m->d_err,
-                                 TC_WAIT_NS, m->stream, nullptr);
-        if (l < 2) {
-            Ain = m->pH[l];
-            K = Hd;
-        }
+        gw::MlpGemmJobs jobs{1, {}};
+        gw::MlpGemmJob &j = jobs.job[0];
+        j.A = l == 0 ? m->pX : m->pH[l - 1];
+        j.B = m->pW[l];
+        j.M = batch;
+        j.N = Hd;
+        j.K = l == 0 ? m->n_in : Hd;
+        j.C = m->H[l];
+        j.bias = m->theta + m->off_b[l];
+        j.rowop = l < 2 ? m->pH[l] : nullptr;
+        j.colop = keep && l < 2 ? m->pHc[l] : nullptr;
+        e = gemm3(m, 1, jobs);
     }
     if (e != cudaSuccess || !Yout)
         return e;
     // the 2-wide output layer
     out_layer_kernel<<<(batch + OUT_ROWS - 1) / OUT_ROWS, 256, 0, m->stream>>>(
-        m->H[2], Hd, m->theta16 + m->off_w[3], m->theta + m->off_b[3], batch, Yout, nullptr, nullptr, 0.f, nullptr,
-        nullptr, nullptr, nullptr);
+        m->H[2], Hd, m->theta16 + m->off_w[3], m->theta + m->off_b[3], batch, Yout);
     gw::count_launches(1);
     return cudaGetLastError();
 }
 
-// Loss and the gradient of every parameter into m->grad.
-cudaError_t loss_grad(gw_mlp *m, const float *X, const float *T, const int *rows, int batch, float *loss)
+// Loss, and the partial sums of every parameter's gradient, which f then describes.
+cudaError_t loss_grad(gw_mlp *m, const float *X, const float *T, const int *rows, int batch, float *loss,
+                      gw::MlpFinish &f)
 {
     const int Hd = m->hidden;
     cudaError_t e = forward_batch(m, X, rows, batch, nullptr, true);
-    if (e != cudaSuccess)
-        return e;
-    // output layer, loss, its deltas D4 = (y - t) / B, those of layer 3, D = (D4 W4) (1 - H2^2), and
-    // per-block partial sums of dW4, db4, then added over the blocks (W4 and b4 are adjacent)
-    const int nob = (batch + OUT_ROWS - 1) / OUT_ROWS;
-    const size_t osh = (size_t)8 * (2 * Hd + 2) * sizeof(float);
-    if ((e = cudaFuncSetAttribute(out_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osh)) !=
-        cudaSuccess)
-        return e;
-    out_layer_kernel<<<nob, 256, osh, m->stream>>>(m->H[2], Hd, m->theta16 + m->off_w[3], m->theta + m->off_b[3],
-                                                    batch, m->Y, T, rows, 1.f / batch, m->D4, m->Da, loss, m->part);
-    gw::count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return e;
-    sum_parts_tree_kernel<<<2 * Hd + 2, 256, 0, m->stream>>>(m->part, nob, 2L * Hd + 2, m->grad + m->off_w[3]);
-    gw::count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return e;
-    // hidden layers l = 2, 1, 0 (weights W_{l+1}): dW = D^T (layer input), db = the column sums of D,
-    // and the deltas of layer l - 1, (D W_{l+1}) (1 - H_{l-1}^2), which the product writes as the
-    // operands of the next steps (row, col) with their column sums
-    if ((e = gw::launch_mlp_pack3(m->Da, Hd, nullptr, batch, Hd, m->pD[0], m->pDc, m->csum, m->stream)) !=
-        cudaSuccess)
-        return e;
-    float *D = m->Da;
-    int cur = 0;
-    for (int l = 2; l >= 0; --l) {
-        const int in = l > 0 ? Hd : m->n_in;
-        const int tiles = ((Hd + 127) / 128) * ((in + 127) / 128);
-        int S = 1;
-        if ((e = gw::launch_mlp_gemm3(0, m->pDc, Hd, l > 0 ? m->pHc[l - 1] : m->pXc, in, batch,
-                                      std::max(1, std::min(SPLIT_MAX, m->num_sms / tiles)), m->part, in,
-                                      (long)Hd * in, nullptr, nullptr, 0, nullptr, nullptr, nullptr, m->d_err,
-                                      TC_WAIT_NS, m->stream, &S)) != cudaSuccess)
-            return e;
-        const long nw = (long)Hd * in;
-        const int nbw = (int)std::min<long>((nw + 255) / 256, 4L * m->num_sms);
-        grad_finish_kernel<<<nbw + (Hd + 255) / 256, 256, 0, m->stream>>>(
-            m->part, S, nw, nw, nbw, m->grad + m->off_w[l], m->csum, (batch + 127) / 128, Hd, m->grad + m->off_b[l]);
-        gw::count_launches(1);
-        if ((e = cudaGetLastError()) != cudaSuccess)
-            return e;
-        if (l > 0) {
-            float *Dn = D == m->Da ? m->Db : m->Da;
-            if ((e = gw::launch_mlp_gemm3(2, m->pD[cur], batch, m->pWc[l - 1], Hd, Hd, 1, Dn, Hd, 0, nullptr,
-                                          m->H[l - 1], Hd, l > 1 ? m->pD[1 - cur] : nullptr, m->pDc, m->csum, m->d_err,
-                                          TC_WAIT_NS, m->stream, nullptr)) != cudaSuccess)
-                return e;
-            D = Dn;
-            cur = 1 - cur;
-        }
+    // output layer, loss, the deltas of layer 3 and the shares of dW4, db4
+    if (e == cudaSuccess)
+        e = gw::launch_mlp_out_train(m->H[2], Hd, m->theta16 + m->off_w[3], m->theta + m->off_b[3], batch, T, rows,
+                                     m->pD[1], m->pDc[2], m->csum[2], m->out_part, m->stream);
+    // the deltas of layers 2 and 1, (D W_{l+1}) (1 - H_{l-1}^2), as the operands of the next steps
+    for (int l = 2; l > 0 && e == cudaSuccess; --l) {
+        gw::MlpGemmJobs jobs{1, {}};
+        gw::MlpGemmJob &j = jobs.job[0];
+        j.A = m->pD[l - 1];
+        j.B = m->pWc[l - 1];
+        j.M = batch;
+        j.N = j.K = Hd;
+        j.H = m->H[l - 1];
+        j.rowop = l > 1 ? m->pD[l - 2] : nullptr;
+        j.colop = m->pDc[l - 1];
+        j.colsum = m->csum[l - 1];
+        e = gemm3(m, 2, jobs);
     }
-    return cudaSuccess;
+    // dW_l = D_l^T (layer input), all three in slices of the batch
+    gw::MlpGemmJobs jobs{3, {}};
+    float *part = m->part;
+    for (int l = 0; l < 3; ++l) {
+        gw::MlpGemmJob &j = jobs.job[l];
+        j.A = m->pDc[l];
+        j.B = l == 0 ? m->pXc : m->pHc[l - 1];
+        j.M = Hd;
+        j.N = l == 0 ? m->n_in : Hd;
+        j.K = batch;
+        j.slices = gw::mlp_gemm3_slices(batch, m->splits, &j.kcs);
+        j.C = part;
+        f.part[l] = part;
+        f.n_part[l] = j.slices;
+        f.csum[l] = m->csum[l];
+        f.n_csum[l] = l == 2 ? gw::mlp_out_parts(batch) : (batch + 127) / 128;
+        f.off_b[l] = m->off_b[l];
+        part += (size_t)m->splits * j.M * j.N;
+    }
+    f.out_part = m->out_part;
+    f.loss = loss;
+    f.loss_scale = 0.5f / batch;
+    f.n_out = gw::mlp_out_parts(batch);
+    f.off_out = m->off_w[3];
+    return e == cudaSuccess ? gemm3(m, 0, jobs) : e;
 }
 
 gw_status check_mlp(gw_mlp *m)
@@ -574,17 +466,23 @@ namespace {
 gw_status train_step(gw_mlp *m, const float *X, const float *T, const int *rows, int batch, double lr, double beta1,
                      double beta2, double adam_eps, float *loss_accum)
 {
-    MLP_CUDA(loss_grad(m, X, T, rows, batch, loss_accum), "gw_mlp_train_step");
+    gw::MlpFinish f{};
+    MLP_CUDA(loss_grad(m, X, T, rows, batch, loss_accum, f), "gw_mlp_train_step");
     m->step += 1;
     m->tiled = false;
-    m->wpacked = false;
-    const double c1 = 1.0 / (1.0 - std::pow(beta1, (double)m->step));
-    const double c2 = 1.0 / (1.0 - std::pow(beta2, (double)m->step));
-    adam_kernel<<<(int)std::min<long>((m->P + 255) / 256, 4L * m->num_sms), 256, 0, m->stream>>>(
-        m->theta, m->theta16, m->w32, m->grad, m->m, m->v, m->P, (float)lr, (float)beta1, (float)beta2, (float)c1,
-        (float)c2, (float)adam_eps);
-    gw::count_launches(1);
-    MLP_CUDA(cudaGetLastError(), "gw_mlp_train_step adam");
+    f.theta = m->theta;
+    f.theta16 = m->theta16;
+    f.w32 = m->w32;
+    f.m = m->m;
+    f.v = m->v;
+    f.lr = (float)lr;
+    f.b1 = (float)beta1;
+    f.b2 = (float)beta2;
+    f.c1 = (float)(1.0 / (1.0 - std::pow(beta1, (double)m->step)));
+    f.c2 = (float)(1.0 / (1.0 - std::pow(beta2, (double)m->step)));
+    f.eps = (float)adam_eps;
+    // writes the weight operands of the next step as well
+    MLP_CUDA(gw::launch_mlp_finish(f, weight_pack(m), true, m->num_sms, m->stream), "gw_mlp_train_step adam");
     return GW_OK;
 }
 
@@ -674,21 +572,26 @@ gw_status gw_mlp_create(gw_mlp **out, int device, int n_in, int hidden, int max_
         return cleanup(GW_E_CUDA);
     }
     const size_t P = (size_t)m->P, act = (size_t)max_batch * hidden;
-    const size_t part = std::max((size_t)SPLIT_MAX * hidden * (std::max(hidden, n_in) + 1),
-                                 (size_t)((max_batch + 15) / 16) * (2 * hidden + 2));  // + output-layer partials
+    // slices of the batch in the weight gradients: their tiles fill the GPU once
+    const int tiles = (hidden + 127) / 128 * (2 * ((hidden + 127) / 128) + 1);
+    m->splits = std::max(1, std::min(SPLIT_MAX, m->num_sms / tiles));
+    const size_t part = (size_t)m->splits * hidden * (2 * hidden + n_in);
+    const size_t nout = gw::mlp_out_parts(max_batch), nrb = (max_batch + 127) / 128;
     float **fbufs[] = {&m->theta, &m->grad, &m->m, &m->v, &m->w32};
     for (float **p : fbufs)
         if (cudaMalloc(p, P * sizeof(float)) != cudaSuccess)
             return cleanup(GW_E_NOMEM);
     if (cudaMalloc(&m->theta16, P * sizeof(__half)) != cudaSuccess)
         return cleanup(GW_E_NOMEM);
-    float **abufs[] = {&m->H[0], &m->H[1], &m->H[2], &m->Da, &m->Db};
+    float **abufs[] = {&m->H[0], &m->H[1], &m->H[2]};
     for (float **p : abufs)
         if (cudaMalloc(p, act * sizeof(float)) != cudaSuccess)
             return cleanup(GW_E_NOMEM);
-    if (cudaMalloc(&m->D4, (size_t)max_batch * NOUT * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&m->Y, (size_t)max_batch * NOUT * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&m->part, part * sizeof(float)) != cudaSuccess)
+    if (cudaMalloc(&m->part, part * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&m->csum[0], nrb * hidden * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&m->csum[1], nrb * hidden * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&m->csum[2], nout * hidden * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&m->out_part, nout * (2 * hidden + 3) * sizeof(float)) != cudaSuccess)
         return cleanup(GW_E_NOMEM);
     // operands of the tensor-core products (sizes: rows x k of each)
     struct {
@@ -696,19 +599,26 @@ gw_status gw_mlp_create(gw_mlp **out, int device, int n_in, int hidden, int max_
         int rows, k;
     } packs[] = {{&m->pX, max_batch, n_in},      {&m->pXc, n_in, max_batch},      {&m->pH[0], max_batch, hidden},
                  {&m->pH[1], max_batch, hidden}, {&m->pHc[0], hidden, max_batch}, {&m->pHc[1], hidden, max_batch},
-                 {&m->pD[0], max_batch, hidden}, {&m->pD[1], max_batch, hidden},  {&m->pDc, hidden, max_batch},
+                 {&m->pD[0], max_batch, hidden}, {&m->pDc[1], hidden, max_batch}, {&m->pDc[2], hidden, max_batch},
                  {&m->pW[0], hidden, n_in},
                  {&m->pW[1], hidden, hidden},    {&m->pW[2], hidden, hidden},     {&m->pWc[0], hidden, hidden},
                  {&m->pWc[1], hidden, hidden}};
     for (auto &pk : packs)
         if (cudaMalloc(pk.p, gw::mlp_pack3_bytes(pk.rows, pk.k)) != cudaSuccess)
             return cleanup(GW_E_NOMEM);
+    // layer 3's row deltas have been read when the transposed deltas of layer 1 are written: one buffer
+    if (cudaMalloc(&m->pD[1], std::max(gw::mlp_pack3_bytes(max_batch, hidden),
+                                       gw::mlp_pack3_bytes(hidden, max_batch))) != cudaSuccess)
+        return cleanup(GW_E_NOMEM);
+    m->pDc[0] = m->pD[1];
     // the weights' padding is never written: clear their buffers once
     for (uint8_t *w : {m->pW[0], m->pW[1], m->pW[2], m->pWc[0], m->pWc[1]})
         if (cudaMemsetAsync(w, 0, gw::mlp_pack3_bytes(hidden, w == m->pW[0] ? n_in : hidden), m->stream) != cudaSuccess)
             return cleanup(GW_E_CUDA);
-    if (cudaMalloc(&m->d_err, sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&m->csum, (size_t)((max_batch + 127) / 128) * hidden * sizeof(float)) != cudaSuccess)
+    // nor are the rows of the transposed inputs beyond n_in
+    if (cudaMemsetAsync(m->pXc, 0, gw::mlp_pack3_bytes(n_in, max_batch), m->stream) != cudaSuccess)
+        return cleanup(GW_E_CUDA);
+    if (cudaMalloc(&m->d_err, sizeof(uint32_t)) != cudaSuccess)
         return cleanup(GW_E_NOMEM);
     if (cudaMemsetAsync(m->theta, 0, P * sizeof(float), m->stream) != cudaSuccess ||
         cudaMemsetAsync(m->theta16, 0, P * sizeof(__half), m->stream) != cudaSuccess ||
@@ -732,10 +642,10 @@ gw_status gw_mlp_destroy(gw_mlp *m)
         cudaStreamSynchronize(m->stream);
     else
         cudaDeviceSynchronize();
-    void *ptrs[] = {m->theta, m->grad,   m->m,      m->v,      m->theta16, m->w32,  m->H[0],  m->H[1],
-                    m->H[2],  m->Da,     m->Db,     m->D4,     m->Y,       m->part, m->pX,    m->pXc,
-                    m->pH[0], m->pH[1],  m->pHc[0], m->pHc[1], m->pD[0],   m->pD[1], m->pDc,  m->pW[0], m->pW[1],
-                    m->pW[2], m->pWc[0], m->pWc[1], m->csum,   m->Wt,      m->d_err};
+    void *ptrs[] = {m->theta, m->grad,  m->m,      m->v,      m->theta16, m->w32,    m->H[0],   m->H[1],
+                    m->H[2],  m->part,  m->csum[0], m->csum[1], m->csum[2], m->out_part, m->pX,   m->pXc,
+                    m->pH[0], m->pH[1], m->pHc[0], m->pHc[1], m->pD[0],   m->pD[1],  m->pDc[1],
+                    m->pDc[2], m->pW[0], m->pW[1], m->pW[2],  m->pWc[0],  m->pWc[1], m->Wt,     m->d_err};
     for (void *p : ptrs)
         if (p)
             cudaFree(p);
@@ -846,7 +756,10 @@ gw_status gw_mlp_grad(gw_mlp *m, const float *X, const float *T, const int *rows
     if (!X || !T || !grad || !loss || batch < 1 || batch > m->max_batch)
         return mfail(m, GW_E_INVALID, "gw_mlp_grad: null pointer or batch outside [1, max_batch]");
     MLP_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), m->stream), "gw_mlp_grad loss reset");
-    MLP_CUDA(loss_grad(m, X, T, rows, batch, loss), "gw_mlp_grad");
+    gw::MlpFinish f{};
+    MLP_CUDA(loss_grad(m, X, T, rows, batch, loss, f), "gw_mlp_grad");
+    f.grad = m->grad;
+    MLP_CUDA(gw::launch_mlp_finish(f, weight_pack(m), false, m->num_sms, m->stream), "gw_mlp_grad sums");
     MLP_CUDA(cudaMemcpyAsync(grad, m->grad, (size_t)m->P * sizeof(float), cudaMemcpyDeviceToDevice, m->stream),
              "gw_mlp_grad copy");
     return GW_OK;
