@@ -420,25 +420,16 @@ cudaError_t launch_hermitize(float2 *A, int n, cudaStream_t s);  // A <- (A + A^
 // k_eps.cu
 cudaError_t launch_eps_build(const float2 *PG, const double *sv, int ng, double2 *eps, cudaStream_t s);
 // C = alpha * op(A) * op(B) + beta * C, complex128 row-major; op: 0 = N, 1 = conj-transpose.
-// flags: ZG_B_LOWER  op(B)[k][j] = 0 for k < j (skip those k);  ZG_A_UPPER  op(A)[i][k] = 0 for
-// k < i;  ZG_C_LOWER  compute and store only C[i][j] with j <= i;  ZG_C_MIRROR  with ZG_C_LOWER,
-// also store C[j][i] = conj(C[i][j]) (beta must be 0);  ZG_A_LOWER  op(A)[i][k] = 0 for k > i.
-enum { ZG_B_LOWER = 1, ZG_A_UPPER = 2, ZG_C_LOWER = 4, ZG_C_MIRROR = 8, ZG_A_LOWER = 16 };
 cudaError_t launch_zgemm(int M, int N, int K, double2 alpha, const double2 *A, int lda, int opA,
-                         const double2 *B, int ldb, int opB, double2 beta, double2 *C, int ldc, cudaStream_t s,
-                         int flags = 0);
+                         const double2 *B, int ldb, int opB, double2 beta, double2 *C, int ldc, cudaStream_t s);
 // The same for `batch` independent products; problem z uses A + z sA, B + z sB, C + z sC.
 cudaError_t launch_zgemm_batched(int M, int N, int K, double2 alpha, const double2 *A, int lda, int opA, long sA,
                                  const double2 *B, int ldb, int opB, long sB, double2 beta, double2 *C, int ldc,
-                                 long sC, int batch, cudaStream_t s, int flags = 0);
-cudaError_t launch_chol_diag(double2 *A, int lda, int n, double2 *Linv, int ldl, int pivot0, uint32_t *err,
-                             cudaStream_t s);
+                                 long sC, int batch, cudaStream_t s);
 // Enqueue eps^-1 = (L L^H)^-1 in FP64 (Cholesky, recursive-doubling triangular inverse, Y^H Y).
 // Workspace: A, Y, T of N^2 complex128 each, W of 32 N, Dinv of ceil(N/32) 32^2.
 cudaError_t chol_inverse_enqueue(const double2 *eps, int N, double2 *epsinv, double2 *A, double2 *Y, double2 *T,
                                  double2 *W, double2 *Dinv, uint32_t *err, cudaStream_t s);
-cudaError_t launch_copy_block(const double2 *src, int lds, double2 *dst, int ldd, int rows, int cols,
-                              cudaStream_t s);
 cudaError_t launch_set_identity(double2 *A, int lda, int n, double scale, cudaStream_t s);
 cudaError_t launch_two_minus(double2 *T, int n, cudaStream_t s);  // T <- 2I - T
 cudaError_t launch_scaled_adjoint(const double2 *A, int n, const double *d_den, double2 *X, cudaStream_t s);

@@ -451,12 +451,12 @@ cudaError_t gram(const double2 *X, const double2 *Y, int ng, int ld, int b, doub
     const int kc = 16, nparts = (ng + kc - 1) / kc;
     const double2 one = make_double2(1, 0), zero = make_double2(0, 0);
     cudaError_t e = launch_zgemm_batched(b, b, kc, one, X, ld, 1, (long)kc * ld, Y, ld, 0, (long)kc * ld, zero, parts,
-                                         b, (long)b * b, nparts - 1, s, 0);
+                                         b, (long)b * b, nparts - 1, s);
     if (e != cudaSuccess)
         return e;
     const int last = ng - (nparts - 1) * kc;  // the ragged last part
     e = launch_zgemm(b, b, last, one, X + (size_t)(nparts - 1) * kc * ld, ld, 1, Y + (size_t)(nparts - 1) * kc * ld,
-                     ld, 0, zero, parts + (size_t)(nparts - 1) * b * b, b, s, 0);
+                     ld, 0, zero, parts + (size_t)(nparts - 1) * b * b, b, s);
     if (e != cudaSuccess)
         return e;
     sum_parts64_kernel<<<blocks_for((size_t)b * b), 256, 0, s>>>(parts, nparts, b * b, C);
@@ -471,12 +471,12 @@ cudaError_t prod_ksplit(const double2 *A, const double2 *X, int ng, int b, doubl
     const int kc = 64, nparts = (ng + kc - 1) / kc;
     const double2 one = make_double2(1, 0), zero = make_double2(0, 0);
     cudaError_t e = launch_zgemm_batched(ng, b, kc, one, A, ng, 0, kc, X, b, 0, (long)kc * b, zero, parts, b,
-                                         (long)ng * b, nparts - 1, s, 0);
+                                         (long)ng * b, nparts - 1, s);
     if (e != cudaSuccess)
         return e;
     const int last = ng - (nparts - 1) * kc;
     e = launch_zgemm(ng, b, last, one, A + (size_t)(nparts - 1) * kc, ng, 0, X + (size_t)(nparts - 1) * kc * b, b, 0,
-                     zero, parts + (size_t)(nparts - 1) * ng * b, b, s, 0);
+                     zero, parts + (size_t)(nparts - 1) * ng * b, b, s);
     if (e != cudaSuccess)
         return e;
     sum_parts64_kernel<<<blocks_for((size_t)ng * b), 256, 0, s>>>(parts, nparts, ng * b, Y);
@@ -658,7 +658,7 @@ cudaError_t pp_iterate(PPWork &w, int ng, int b, int nmodes, double tol, int max
                 return e;
             chol_inv_small_kernel<<<1, 256, small_smem(b), s>>>(w.G, b, w.U, w.flag);
             count_launches(1);
-            if ((e = launch_zgemm(ng, b, b, one, w.X, b, 0, w.U, b, 0, zero, w.T, b, s, 0)) != cudaSuccess)
+            if ((e = launch_zgemm(ng, b, b, one, w.X, b, 0, w.U, b, 0, zero, w.T, b, s)) != cudaSuccess)
                 return e;
             std::swap(w.X, w.T);
         }
@@ -675,10 +675,10 @@ cudaError_t pp_iterate(PPWork &w, int ng, int b, int nmodes, double tol, int max
             return e;
         jacobi_small_kernel<<<1, 256, small_smem(b), s>>>(w.G, b, 30, w.theta, w.U);
         count_launches(1);
-        if ((e = launch_zgemm(ng, b, b, one, w.X, b, 0, w.U, b, 0, zero, w.T, b, s, 0)) != cudaSuccess)
+        if ((e = launch_zgemm(ng, b, b, one, w.X, b, 0, w.U, b, 0, zero, w.T, b, s)) != cudaSuccess)
             return e;
         std::swap(w.X, w.T);
-        if ((e = launch_zgemm(ng, b, b, one, w.Y, b, 0, w.U, b, 0, zero, w.T, b, s, 0)) != cudaSuccess)
+        if ((e = launch_zgemm(ng, b, b, one, w.Y, b, 0, w.U, b, 0, zero, w.T, b, s)) != cudaSuccess)
             return e;
         std::swap(w.Y, w.T);
         resid_kernel<<<b, 256, 0, s>>>(w.X, w.Y, ng, b, w.theta, w.res);
@@ -716,7 +716,7 @@ cudaError_t pp_eval(const PPWork &w, int ng, int b, int nuse, double omega, doub
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
-    return launch_zgemm(ng, ng, nuse, one, w.T, nuse, 0, w.X, b, 1, zero, Sout, ng, s, 0);
+    return launch_zgemm(ng, ng, nuse, one, w.T, nuse, 0, w.X, b, 1, zero, Sout, ng, s);
 }
 
 }  // namespace gw
