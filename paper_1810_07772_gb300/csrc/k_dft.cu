@@ -1143,6 +1143,218 @@ __global__ void __launch_bounds__(P12P_WARPS * 32, 2)
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Stages 1 and 2 for any plane size, for spheres at q = 0 (m3 values -M..M, disk symmetric in m2).  A warp takes a
+// plane at a time, as in dft_plane12_kernel, with the same paired sums in the same order, but a lane
+// makes four outputs m of a line (stage 1) or column (stage 2) at once: per term it reads one folded pair and four
+// twiddles (broadcast) for 16 FMAs, where the generic table form read two values for every four.  A line per lane
+// would leave 32 - n2 lanes idle, so the items are (line, four outputs) pairs.  Row transforms of P, against the
+// row-block kernel (above 4096 rows) or the generic table form: 19 x 21 x 17, 439 -> 264 us; 22 x 25 x 23, 1.47 -> 0.72 ms;
+// 28^3, 5.46 -> 2.65; 40 x 38 x 37, 32 -> 23; 22 x 25 x 23 with 800 pair rows, 105 -> 63 us.
+constexpr int PG_WARPS = 8;
+
+struct PlaneG {
+    int h3, h2, mp3, mp2, ld3, lda;     // pairs per line and column; outputs padded to fours; pitches
+    size_t tw2, dtab, warps, per_warp;  // offsets in float2, and of one warp's buffers
+    __host__ __device__ PlaneG(int n2, int n3, int M, int k2)
+    {
+        h3 = (n3 - 1) / 2;
+        h2 = (n2 - 1) / 2;
+        mp3 = (M + 3) / 4 * 4;
+        mp2 = (k2 + 4) / 4 * 4;
+        ld3 = n3 | 1;
+        lda = n2 | 1;
+        tw2 = (size_t)(h3 + 1) * mp3;
+        dtab = tw2 + (size_t)(h2 + 1) * mp2;
+        warps = dtab + (size_t)(2 * M + 1) * mp2;
+        per_warp = (size_t)n2 * ld3 + (size_t)(2 * M + 1) * lda;
+    }
+};
+
+// A[e] +- i B[e] of NE outputs from a folded line: A = x_0 + (-1)^m x_{n/2} + sum s_j cos, B = sum t_j sin, with
+// x_j = s_j, x_{n-j} = t_j at p[j], p[n - j].  ODD: the first of the outputs is odd.
+template <int NE, bool ODD>
+__device__ __forceinline__ void folded_sums(const float2 *p, int n, int h, const float2 *tw, int mp, float2 (&A)[NE],
+                                            float2 (&B)[NE])
+{
+    const float2 x0 = p[0];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+        A[e] = x0;
+        B[e] = make_float2(0.f, 0.f);
+    }
+    if ((n & 1) == 0) {
+        const float2 mid = p[n / 2];
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const float sg = ((e + (ODD ? 1 : 0)) & 1) ? -1.f : 1.f;
+            A[e].x = fmaf(sg, mid.x, A[e].x);
+            A[e].y = fmaf(sg, mid.y, A[e].y);
+        }
+    }
+    for (int j = 1; j <= h; ++j) {
+        const float2 s = p[j], t = p[n - j];
+#pragma unroll
+        for (int e = 0; e < NE; e += 2) {
+            const float4 w = *reinterpret_cast<const float4 *>(tw + j * mp + e);
+            A[e].x = fmaf(s.x, w.x, A[e].x);
+            A[e].y = fmaf(s.y, w.x, A[e].y);
+            B[e].x = fmaf(t.x, w.y, B[e].x);
+            B[e].y = fmaf(t.y, w.y, B[e].y);
+            A[e + 1].x = fmaf(s.x, w.z, A[e + 1].x);
+            A[e + 1].y = fmaf(s.y, w.z, A[e + 1].y);
+            B[e + 1].x = fmaf(t.x, w.w, B[e + 1].x);
+            B[e + 1].y = fmaf(t.y, w.w, B[e + 1].y);
+        }
+    }
+}
+
+// x_j, x_{n-j} -> x_j + x_{n-j}, x_j - x_{n-j} for 0 < j <= h, of `lines` lines `pitch` apart (a warp).
+__device__ __forceinline__ void fold_lines(float2 *x, int pitch, int lines, int n, int h, int lane)
+{
+    int j = 1 + lane / lines, l = lane - lane / lines * lines;
+    const int dj = 32 / lines, dl = 32 - dj * lines;
+    while (j <= h) {
+        float2 *p = x + l * pitch;
+        const float2 u = p[j], v = p[n - j];
+        p[j] = make_float2(u.x + v.x, u.y + v.y);
+        p[n - j] = make_float2(u.x - v.x, u.y - v.y);
+        j += dj;
+        l += dl;
+        if (l >= lines) {
+            l -= lines;
+            ++j;
+        }
+    }
+}
+
+// Stage 2 of a plane: the disk values of the folded columns a1, NE outputs m2 an item, into ys.
+template <int NE>
+__device__ __forceinline__ void planeg_stage2(const PlaneG &L, const float2 *a1, const float2 *tw2, const int2 *dtab,
+                                              int n2, int c3, int lane, float2 *ys)
+{
+    for (int q = lane; q < c3 * (L.mp2 / NE); q += 32) {
+        const int mb = q / c3, i3 = q - mb * c3;
+        float2 A[NE], B[NE];
+        folded_sums<NE, false>(a1 + i3 * L.lda, n2, L.h2, tw2 + NE * mb, L.mp2, A, B);
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int2 d = dtab[i3 * L.mp2 + NE * mb + e];
+            if (d.x >= 0)
+                ys[d.x] = make_float2(A[e].x - B[e].y, A[e].y + B[e].x);
+            if (d.y >= 0)
+                ys[d.y] = make_float2(A[e].x + B[e].y, A[e].y - B[e].x);
+        }
+    }
+}
+
+template <bool PAIR>
+__global__ void __launch_bounds__(PG_WARPS * 32, 3)
+    dft_planeg_kernel(const float2 *__restrict__ X, long long ldx, int rows, int n1, int n2, int n3, int M, int cd,
+                      int np2, int k2, const int4 *__restrict__ g_pair2, const float2 *__restrict__ g_tw,
+                      float2 *__restrict__ Y2, PairSrc ps)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    const PlaneG L(n2, n3, M, k2);
+    float2 *tw3 = reinterpret_cast<float2 *>(smem), *tw2 = tw3 + L.tw2;  // [j][m], m = 1.. and m = 0..
+    int2 *dtab = reinterpret_cast<int2 *>(tw3 + L.dtab);                 // [i3][m2]: disk index of +m2, of -m2
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, c3 = 2 * M + 1;
+    for (int t = tid; t < (L.h3 + 1) * L.mp3; t += blockDim.x) {
+        const int j = t / L.mp3, m = 1 + t - j * L.mp3;
+        tw3[t] = m <= M ? g_tw[n1 + n2 + m * j % n3] : make_float2(0.f, 0.f);
+    }
+    for (int t = tid; t < (L.h2 + 1) * L.mp2; t += blockDim.x) {
+        const int j = t / L.mp2, m = t - j * L.mp2;
+        tw2[t] = m <= k2 ? g_tw[n1 + m * j % n2] : make_float2(0.f, 0.f);
+    }
+    for (int t = tid; t < c3 * L.mp2; t += blockDim.x)
+        dtab[t] = make_int2(-1, -1);
+    __syncthreads();
+    for (int t = tid; t < np2; t += blockDim.x) {
+        const int4 pr = g_pair2[t];  // (i3, m2 >= 0, disk index of m2, of -m2 or -1)
+        dtab[pr.x * L.mp2 + pr.y] = make_int2(pr.z, pr.w);
+    }
+    __syncthreads();
+    float2 *xp = tw3 + L.warps + warp * L.per_warp;  // [n2][ld3]: the plane, later the disk values
+    float2 *a1 = xp + n2 * L.ld3;                    // [c3][lda]: stage 1's outputs
+    const int plane = n2 * n3, nwarps = blockDim.x >> 5, dj2 = 32 / n3, dj3 = 32 - dj2 * n3;
+    // 32-bit arithmetic (the launcher keeps rows n1 below 2^31)
+    const unsigned ntasks = (unsigned)rows * (unsigned)n1;
+    for (unsigned task = blockIdx.x * nwarps + warp; task < ntasks; task += gridDim.x * nwarps) {
+        unsigned row, j1;  // pair rows j1-major, so that the warps of a CTA share psi_v
+        if (PAIR) {
+            j1 = task / (unsigned)rows;
+            row = task - j1 * (unsigned)rows;
+        } else {
+            row = task / (unsigned)n1;
+            j1 = task - row * (unsigned)n1;
+        }
+        const float2 *src, *srcv = nullptr;
+        float w = 0.f;
+        if (PAIR) {
+            const int v = (int)row / ps.nc;
+            src = X + (size_t)(ps.c0 + (int)row - v * ps.nc) * ldx + (size_t)j1 * plane;
+            srcv = X + (size_t)v * ldx + (size_t)j1 * plane;
+            w = ps.sw[row];
+        } else {
+            src = X + row * ldx + (size_t)j1 * plane;
+        }
+        int j2 = lane / n3, j3 = lane - j2 * n3;
+#pragma unroll 4
+        for (int q = lane; q < plane; q += 32) {
+            const float2 x = __ldg(src + q);
+            xp[j2 * L.ld3 + j3] = PAIR ? pair_or_x<true>(__ldg(srcv + q), x, w) : x;
+            j2 += dj2;
+            j3 += dj3;
+            if (j3 >= n3) {
+                j3 -= n3;
+                ++j2;
+            }
+        }
+        __syncwarp();
+        fold_lines(xp, L.ld3, n2, n3, L.h3, lane);
+        __syncwarp();
+        // stage 1: a1[M + m3][j2] = sum_j3 x[j2][j3] e(m3 j3 / n3)
+        for (int q = lane; q < n2 * (1 + L.mp3 / 4); q += 32) {
+            const int mb = q / n2, l = q - mb * n2;
+            const float2 *x = xp + l * L.ld3;
+            if (mb == L.mp3 / 4) {  // m3 = 0
+                float2 a0 = x[0];
+                for (int j = 1; j <= L.h3; ++j) {
+                    a0.x += x[j].x;
+                    a0.y += x[j].y;
+                }
+                const float2 mid = (n3 & 1) ? make_float2(0.f, 0.f) : x[n3 / 2];
+                a1[M * L.lda + l] = make_float2(a0.x + mid.x, a0.y + mid.y);
+                continue;
+            }
+            float2 A[4], B[4];
+            folded_sums<4, true>(x, n3, L.h3, tw3 + 4 * mb, L.mp3, A, B);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int m = 1 + 4 * mb + e;
+                if (m <= M) {
+                    a1[(M + m) * L.lda + l] = make_float2(A[e].x - B[e].y, A[e].y + B[e].x);
+                    a1[(M - m) * L.lda + l] = make_float2(A[e].x + B[e].y, A[e].y - B[e].x);
+                }
+            }
+        }
+        __syncwarp();
+        fold_lines(a1, L.lda, c3, n2, L.h2, lane);
+        __syncwarp();
+        // stage 2, into the plane's buffer; two outputs an item where four leave half the lanes idle
+        if (c3 * (L.mp2 / 4) > 16)
+            planeg_stage2<4>(L, a1, tw2, dtab, n2, c3, lane, xp);
+        else
+            planeg_stage2<2>(L, a1, tw2, dtab, n2, c3, lane, xp);
+        __syncwarp();
+        float2 *dst = Y2 + ((size_t)row * n1 + j1) * cd;
+        for (int t = lane; t < cd; t += 32)
+            dst[t] = xp[t];
+        __syncwarp();  // the buffers are rewritten by the next task
+    }
+}
+
 // Stage 3 with sphere pairs (np1 > 0): y(+-m1, d) = A +- i B from the sums of
 // ys[j1][d] + ys[n1 - j1][d] (times the cosine) and ys[j1][d] - ys[n1 - j1][d] (times the sine),
 // formed while the row is loaded; tw1m[m1][j1] = e(m1 j1 / n1), m1 <= k1, rows of p3_ld1 (odd).
@@ -1428,9 +1640,23 @@ bool p12_compiled(int n3)
     }
 }
 
+// The any-size plane kernel: n3 without a compiled stage 1, spheres at q = 0, and at least one warp's buffers in a
+// CTA's shared memory.  A compiled n3 keeps a line in registers and is faster even where n2 differs (15 x 18 x 20:
+// 125 us against 177; 31 x 29 x 30: 2.88 ms against 3.97).  Planes below 13 x 14 leave most lanes idle in stage 2
+// and stay with the table form: row transforms at 11 x 10 x 13, 31 us there against 35; 13^3, 52 and 52; 14^3, 69
+// against 63.
+static int planeg_warps(const DftPlan &p)
+{
+    if (p12_compiled(p.n[2]) || p.n[1] * p.n[2] < 13 * 14 || p.sym3 < 0 || p.c3 != 2 * p.sym3 + 1 || p.np2 <= 0 || 2 * p.k2 >= p.n[1] || 2 * p.sym3 >= p.n[2])
+        return 0;
+    const PlaneG L(p.n[1], p.n[2], p.sym3, p.k2);
+    const size_t avail = DFT_SMEM_MAX / sizeof(float2);
+    return avail <= L.warps ? 0 : (int)std::min<size_t>(PG_WARPS, (avail - L.warps) / L.per_warp);
+}
+
 size_t dft_work_bytes(const DftPlan &p, int rows)
 {
-    const int r = p12_compiled(p.n[2]) ? rows : std::min(rows, WS_MAX_ROWS_GENERIC);
+    const int r = p12_compiled(p.n[2]) || planeg_warps(p) > 0 ? rows : std::min(rows, WS_MAX_ROWS_GENERIC);
     return (size_t)r * p.n[0] * p.cd * sizeof(float2);
 }
 
@@ -1521,6 +1747,23 @@ static bool p12c_applies(const DftPlan &p)
            p.c3 <= P12C_MAX_C3 && p.k2 <= (N - 1) / 2 && p12c_smem(N, p.c3) <= DFT_SMEM_MAX;
 }
 
+template <bool PAIR>
+static cudaError_t launch_planeg(int nwarps, const float2 *X, long long ldx, int rows, const DftPlan &p,
+                                 const float2 *tw, float2 *work, PairSrc ps, cudaStream_t s)
+{
+    const PlaneG L(p.n[1], p.n[2], p.sym3, p.k2);
+    const size_t smem = (L.warps + nwarps * L.per_warp) * sizeof(float2);
+    const cudaError_t e =
+        cudaFuncSetAttribute(dft_planeg_kernel<PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    const long long ntasks = (long long)rows * p.n[0];
+    const int grid = (int)std::min<long long>((ntasks + nwarps - 1) / nwarps, 152LL * 16);
+    dft_planeg_kernel<PAIR><<<grid, nwarps * 32, smem, s>>>(X, ldx, rows, p.n[0], p.n[1], p.n[2], p.sym3, p.cd, p.np2,
+                                                            p.k2, p.pair2, tw, work, ps);
+    return cudaGetLastError();
+}
+
 template <int N3>
 static cudaError_t launch_p12(int grid, size_t smem, const float2 *X, long long ldx, int rows, const DftPlan &p,
                               const float2 *tw, float2 *work, const PairSrc *ps, cudaStream_t s)
@@ -1538,7 +1781,8 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
 {
     if (rows <= 0)
         return cudaSuccess;
-    if ((!p12_compiled(p.n[2]) && rows > WS_MAX_ROWS_GENERIC) || !work)
+    const int pgw = const_twiddles && (long long)rows * p.n[0] < (1LL << 31) ? planeg_warps(p) : 0;
+    if ((!p12_compiled(p.n[2]) && pgw == 0 && rows > WS_MAX_ROWS_GENERIC) || !work)
         return ps ? cudaErrorNotSupported : launch_dft_rows(X, ldx, rows, Y, ldy, p, s, negative_exponent);
     const float2 *tw = negative_exponent ? p.twc : p.tw;
     const size_t sm12 = p12_smem(p.n, p.c3, p.cd, p.np2, p.k2, !p12_compiled(p.n[2]));
@@ -1546,7 +1790,7 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
     const size_t sm3 = paired3 ? p3_smem_paired(p.n[0], p.cd, p.np1, p.k1, p.ng)
                                : sizeof(float2) * ((size_t)p.n[0] * p.cd + p.n[0]) + sizeof(int) * 2 * p.ng;
     const bool cst = const_twiddles && p12c_applies(p) && (long long)rows * p.n[0] < (1LL << 31);
-    if ((!cst && sm12 > DFT_SMEM_MAX) || sm3 > DFT_SMEM_MAX)
+    if ((!cst && pgw == 0 && sm12 > DFT_SMEM_MAX) || sm3 > DFT_SMEM_MAX)
         return ps ? cudaErrorNotSupported : launch_dft_rows(X, ldx, rows, Y, ldy, p, s, negative_exponent);
     cudaError_t e = paired3 ? cudaFuncSetAttribute(dft_stage3_paired_kernel,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)
@@ -1567,6 +1811,9 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
         case 27: e = launch_p12c<27>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         default: e = cudaErrorNotSupported; break;
         }
+    } else if (pgw > 0) {
+        e = ps ? launch_planeg<true>(pgw, X, ldx, rows, p, tw, work, *ps, s)
+               : launch_planeg<false>(pgw, X, ldx, rows, p, tw, work, PairSrc{nullptr, 0, 1, 0}, s);
     } else switch (p.n[2]) {
     case 12: e = launch_p12<12>(g12, sm12, X, ldx, rows, p, tw, work, ps, s); break;
     case 16: e = launch_p12<16>(g12, sm12, X, ldx, rows, p, tw, work, ps, s); break;
