@@ -980,8 +980,7 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
         }
         src = c.d_psi;
     }
-    GW_CUDA(launch_check_finite(src, n, c.d_err, s), "check states");
-    GW_CUDA(launch_transpose_states(src, nb, nr, c.d_psiT, s), "transpose states");
+    GW_CUDA(launch_transpose_states(src, nb, nr, c.d_psiT, s, c.d_err), "transpose and check states");
     GW_CUDA(cudaMemcpyAsync(c.d_E, Eh.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s), "copy energies");
     GW_CUDA(launch_weights(c.d_E, nv, nc, c.d_sw, s), "weights");
     c.E_h = Eh;

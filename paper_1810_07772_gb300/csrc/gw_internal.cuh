@@ -233,9 +233,10 @@ void count_launches(int n);
 // ---- launchers (each returns cudaGetLastError() of its launches) ----
 
 // k_pair.cu
-cudaError_t launch_transpose_states(const float2 *psi, int nb, int nr, float2 *psiT, cudaStream_t s);
+// err (if given): GW_E_INVALID at SITE_INPUT for a value that is not finite
+cudaError_t launch_transpose_states(const float2 *psi, int nb, int nr, float2 *psiT, cudaStream_t s,
+                                    uint32_t *err = nullptr);
 cudaError_t launch_c128_to_c64(const double2 *in, size_t n, float2 *out, cudaStream_t s);
-cudaError_t launch_check_finite(const float2 *x, size_t n, uint32_t *err, cudaStream_t s);
 cudaError_t launch_weights(const double *E, int nv, int nc, float *sw, cudaStream_t s);
 // prec: 0 = TF32X3 planes, 2 = TF32X1 planes, 3 = plain complex64 [kpad][nr_pad]
 // Plain complex64 pair densities f [rows][nr_pad] (rows >= nv nc; extra rows and columns zero),
