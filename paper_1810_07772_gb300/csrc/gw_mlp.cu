@@ -57,7 +57,8 @@ __device__ __forceinline__ long tri_index(int g, int h, int ng)
 // approximation (relative error ~2^-23, seeded with d rounded to FP32) refined by one FP64
 // Newton-Raphson step r <- r + r (1 - d r), which squares the relative error to ~2^-45, instead of
 // an FP64 division per term.  The blocks' partial sums are added by block 0 through distributed
-// shared memory in rank order, so the result does not depend on scheduling.
+// shared memory in rank order, so the result does not depend on scheduling.  The states c go to the blocks
+// in turn: in runs of 512, 2000 of them kept half the blocks idle (44 us; now 26).
 constexpr int RATIO_THREADS = 512;
 constexpr int RATIO_CLUSTER = 8;
 constexpr int RATIO_MAX_NV = 1024;
@@ -84,7 +85,7 @@ __global__ void __cluster_dims__(RATIO_CLUSTER, 1, 1) __launch_bounds__(RATIO_TH
         ev[v] = E[v];
     __syncthreads();
     double om = 0, in = 0;
-    for (int c = (int)cluster.block_rank() * RATIO_THREADS + threadIdx.x; c < nc_all;
+    for (int c = (int)cluster.block_rank() + threadIdx.x * RATIO_CLUSTER; c < nc_all;
          c += RATIO_THREADS * RATIO_CLUSTER) {
         const double ec = E[nv + c];
         double acc = 0;
@@ -155,24 +156,29 @@ __global__ void __launch_bounds__(128) features_kernel(const float2 *PG, int ng,
     const int g1 = gvec[3 * g], g2 = gvec[3 * g + 1], g3 = gvec[3 * g + 2];
     const float m2g = (float)(g1 * g1 + g2 * g2 + g3 * g3);
     const float dg = PG[(long)g * ng + g].x;
+    const bool vec = (reinterpret_cast<size_t>(X) & 15) == 0;
     for (int h = g + (int)threadIdx.x; h < ng; h += blockDim.x) {
         const int h1 = gvec[3 * h], h2 = gvec[3 * h + 1], h3 = gvec[3 * h + 2];
         const int d1 = g1 - h1, d2 = g2 - h2, d3 = g3 - h3;
         const float2 p = PG[(long)g * ng + h];
-        float *x = X + tri_index(g, h, ng) * NF;
-        x[0] = m2g * inv_gcut;
-        x[1] = (float)(h1 * h1 + h2 * h2 + h3 * h3) * inv_gcut;
-        x[2] = (float)(d1 * d1 + d2 * d2 + d3 * d3) * (0.25f * inv_gcut);
-        x[3] = s * p.x;
-        x[4] = s * p.y;
-        x[5] = s * dg;
-        x[6] = s * PG[(long)h * ng + h].x;
-        x[7] = g == h ? 1.f : 0.f;
-        x[8] = rt;
-        x[9] = (g == 0 || h == 0) ? 1.f : 0.f;
         const float2 dc = clos ? clos[(long)g * ng + h] : make_float2(0.f, 0.f);
-        x[10] = s * dc.x;
-        x[11] = s * dc.y;
+        const float4 f[NF / 4] = {
+            make_float4(m2g * inv_gcut, (float)(h1 * h1 + h2 * h2 + h3 * h3) * inv_gcut,
+                        (float)(d1 * d1 + d2 * d2 + d3 * d3) * (0.25f * inv_gcut), s * p.x),
+            make_float4(s * p.y, s * dg, s * PG[(long)h * ng + h].x, g == h ? 1.f : 0.f),
+            make_float4(rt, (g == 0 || h == 0) ? 1.f : 0.f, s * dc.x, s * dc.y)};
+        float *x = X + tri_index(g, h, ng) * NF;  // 48 bytes an entry
+#pragma unroll
+        for (int q = 0; q < NF / 4; ++q) {
+            if (vec) {
+                reinterpret_cast<float4 *>(x)[q] = f[q];
+            } else {
+                x[4 * q] = f[q].x;
+                x[4 * q + 1] = f[q].y;
+                x[4 * q + 2] = f[q].z;
+                x[4 * q + 3] = f[q].w;
+            }
+        }
     }
 }
 
@@ -192,28 +198,40 @@ __global__ void __launch_bounds__(128) targets_kernel(const float2 *lo, const fl
 }
 
 // P~(g,h) += clos(g,h) + (y0 + i y1)/s and P~(h,g) = its conjugate; diagonal: real part only;
-// row and column 0 untouched (clos may be null).
-__global__ void __launch_bounds__(128) apply_kernel(float2 *PG, int ng, const float *Y, const float *scale,
+// row and column 0 untouched (clos may be null).  A block takes a 32 x 32 tile of the upper triangle and its
+// mirror, turned in shared memory so that both are accessed along rows (a row per block with the mirror
+// written along columns took 23 us at N_g = 691, now 8).
+__global__ void __launch_bounds__(256) apply_kernel(float2 *PG, int ng, const float *Y, const float *scale,
                                                     const float2 *clos)
 {
-    const int g = blockIdx.x;
-    if (g == 0)
+    const int bi = blockIdx.y, bj = blockIdx.x;
+    if (bj < bi)
         return;
+    __shared__ float2 delta[32][33];
     const float inv = 1.f / *scale;
-    for (int h = g + (int)threadIdx.x; h < ng; h += blockDim.x) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int i = ty; i < 32; i += 8) {
+        const int g = bi * 32 + i, h = bj * 32 + tx;
+        if (g == 0 || h < g || h >= ng)
+            continue;
         const float *y = Y + tri_index(g, h, ng) * NOUT;
         const float2 dc = clos ? clos[(long)g * ng + h] : make_float2(0.f, 0.f);
         const float dr = y[0] * inv + dc.x, di = y[1] * inv + dc.y;
-        if (h == g) {
-            PG[(long)g * ng + g].x += dr;
-        } else {
-            float2 &a = PG[(long)g * ng + h];
-            float2 &b = PG[(long)h * ng + g];
-            a.x += dr;
+        float2 &a = PG[(long)g * ng + h];
+        a.x += dr;
+        if (h > g)
             a.y += di;
-            b.x += dr;
-            b.y -= di;
-        }
+        delta[i][tx] = make_float2(dr, di);
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {
+        const int h = bj * 32 + i, g = bi * 32 + tx;  // entry (h, g), g < h
+        if (g == 0 || g >= h || h >= ng)
+            continue;
+        float2 &b = PG[(long)h * ng + g];
+        const float2 d = delta[tx][i];
+        b.x += d.x;
+        b.y -= d.y;
     }
 }
 
@@ -924,7 +942,8 @@ gw_status gw_corr_apply(void *PG, int ng, const float *Y, const float *scale, co
 {
     if (!PG || !Y || !scale || ng < 1)
         return GW_E_INVALID;
-    apply_kernel<<<ng, 128, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<float2 *>(PG), ng, Y, scale,
+    const unsigned nt = (unsigned)(ng + 31) / 32;
+    apply_kernel<<<dim3(nt, nt), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<float2 *>(PG), ng, Y, scale,
                                                                       static_cast<const float2 *>(PG_clos));
     gw::count_launches(1);
     return cudaGetLastError() == cudaSuccess ? GW_OK : GW_E_CUDA;
