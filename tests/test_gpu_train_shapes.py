@@ -59,3 +59,36 @@ def test_two_steps_follow_the_gradients(n_in, hid, B):
     # the step's operands are those the gradient was taken with: equal up to FP32 rounding of the update (an entry
     # whose gradient is near the sums' rounding error may move differently by a fraction of lr)
     assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref - th)
+
+
+def _order_keys(seed, n):
+    """SplitMix64's output of the documented keys of the first pass."""
+    u = np.uint64
+    z = np.array([seed], dtype=u) * u(0x9E3779B97F4A7C15) + np.array([1], dtype=u) * u(0xD1B54A32D192ED03)
+    z = z + np.arange(n, dtype=u)
+    z = (z ^ (z >> u(30))) * u(0xBF58476D1CE4E5B9)
+    z = (z ^ (z >> u(27))) * u(0x94D049BB133111EB)
+    return z ^ (z >> u(31))
+
+
+@pytest.mark.parametrize("n,seed", [(400000, 7), (1000, 1)])
+def test_pass_order_with_equal_upper_halves(n, seed):
+    """400000 rows: some twenty pairs of keys share their upper 32 bits, which is all the sort compares; their order
+    decides the order of the sums, so the parameters agree bit for bit only if it is that of the whole keys."""
+    n_in, hid, batch = 3, 16, n // 4
+    keys = _order_keys(seed, n)
+    order = np.argsort(keys, kind="stable").astype(np.int32)
+    up = keys[order] >> np.uint64(32)
+    assert (np.count_nonzero(up[1:] == up[:-1]) > 0) == (n > 100000)
+    rng = np.random.default_rng(n)
+    X = torch.from_numpy(rng.standard_normal((n, n_in)).astype(np.float32)).to(DEV)
+    T = torch.from_numpy(rng.standard_normal((n, 2)).astype(np.float32)).to(DEV)
+    rows = torch.from_numpy(order).to(DEV)
+    th = inputs.mlp_init(n_in, hid, 3).astype(np.float32)
+    with gw.Mlp(n_in, hid, max_batch=batch, device=0) as a, gw.Mlp(n_in, hid, max_batch=batch, device=0) as b:
+        a.set_params(th)
+        b.set_params(th)
+        a.train_corr(X, T, 1, batch, 1e-3, lr_final=1e-3, seed=seed, diag_repeat=1, diag_feature=-1)
+        for t in range(4):
+            b.train_step(X, T, rows[t * batch:(t + 1) * batch], 1e-3)
+        assert np.array_equal(a.get_params(), b.get_params())
