@@ -446,8 +446,8 @@ def run_gw(args):
     peaks, peak_src = load_peaks()
     peak = float(peaks.get("bf16_tflops_sustained", 1700.0))     # FP16 dense = BF16 dense rate
     # the contraction as it is formed: over T (nc + nv) states in separable form, else over k pairs
-    rank = form["terms"] * (w.nv + w.nc) if form["terms"] else w.k
-    achieved = 4.0 * rank * w.nr * (w.nr + 1) / (herk_ms * 1e-3) / 1e12 if herk_ms > 0 else None
+    contracted = form["terms"] * (w.nv + w.nc) if form["terms"] else w.k
+    achieved = 4.0 * contracted * w.nr * (w.nr + 1) / (herk_ms * 1e-3) / 1e12 if herk_ms > 0 else None
     # tensor-pipe work actually issued per 16-k chunk per tile: 3 MMAs of 2*128*256*16 and 6 of
     # 2*128*128*16, the same as 6 of N = 256; a CTA pair issues 6 of M = 256, N = 256
     pair_kernel = args.herk_kernel == "pair" and not form["terms"]
@@ -463,7 +463,7 @@ def run_gw(args):
                            "herk16p_kernel<fp16> (tcgen05 kind::f16, persistent, 128x128 tiles, promoted TMEM "
                            f"windows, separable form of {form['terms']} terms)" if form["terms"] else
                            "herk16_kernel<fp16> (tcgen05 kind::f16, 128x128 tiles, promoted TMEM windows)"),
-                "contracted_rank": rank, "update_form": form,
+                "contracted_rank": contracted, "update_form": form,
                 "flop_note": "achieved counts 4 rank N_r (N_r + 1) of the contraction that ran; value counts the "
                              "direct sum over pairs, rank k = nv nc",
                 "peak_source": f"{peak_src} bf16_tflops_sustained (FP16:BF16 nominal ratio 1)",
