@@ -238,20 +238,37 @@ __global__ void __launch_bounds__(256) apply_kernel(float2 *PG, int ng, const fl
 // The 2-wide output layer, OUT_ROWS rows per block (8 warps, a warp per row at a time): Y[b] = W4 h + b4
 // (h = H2[b], W4 FP16).
 constexpr int OUT_ROWS = 16;
-__global__ void __launch_bounds__(256) out_layer_kernel(const float *H2, int Hd, const __half *W4, const float *b4,
-                                                        int batch, float *Y)
+__global__ void __launch_bounds__(256) out_layer_kernel(const float *__restrict__ H2, int Hd,
+                                                        const __half *__restrict__ W4, const float *__restrict__ b4,
+                                                        int batch, float *__restrict__ Y)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float c0 = b4[0], c1 = b4[1];
     for (int rr = warp; rr < OUT_ROWS; rr += 8) {
         const int b = blockIdx.x * OUT_ROWS + rr;
         if (b >= batch)
             break;
         const float *h = H2 + (long)b * Hd;
         float y0 = 0.f, y1 = 0.f;
-        for (int n = lane; n < Hd; n += 32) {
-            const float hv = h[n];
-            y0 = fmaf(__half2float(W4[n]), hv, y0);
-            y1 = fmaf(__half2float(W4[Hd + n]), hv, y1);
+        if (Hd % 4 == 0) {  // every row of H2 and W4 starts on a multiple of four values
+#pragma unroll 2
+            for (int n = 4 * lane; n < Hd; n += 128) {
+                const float4 hv = *reinterpret_cast<const float4 *>(h + n);
+                const uint2 a = *reinterpret_cast<const uint2 *>(W4 + n);
+                const uint2 b = *reinterpret_cast<const uint2 *>(W4 + Hd + n);
+                const float2 a0 = __half22float2(*reinterpret_cast<const __half2 *>(&a.x));
+                const float2 a1 = __half22float2(*reinterpret_cast<const __half2 *>(&a.y));
+                const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&b.x));
+                const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&b.y));
+                y0 = fmaf(a1.y, hv.w, fmaf(a1.x, hv.z, fmaf(a0.y, hv.y, fmaf(a0.x, hv.x, y0))));
+                y1 = fmaf(b1.y, hv.w, fmaf(b1.x, hv.z, fmaf(b0.y, hv.y, fmaf(b0.x, hv.x, y1))));
+            }
+        } else {
+            for (int n = lane; n < Hd; n += 32) {
+                const float hv = h[n];
+                y0 = fmaf(__half2float(W4[n]), hv, y0);
+                y1 = fmaf(__half2float(W4[Hd + n]), hv, y1);
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -259,8 +276,8 @@ __global__ void __launch_bounds__(256) out_layer_kernel(const float *H2, int Hd,
             y1 += __shfl_xor_sync(0xffffffffu, y1, o);
         }
         if (lane == 0) {
-            Y[2 * (long)b] = y0 + b4[0];
-            Y[2 * (long)b + 1] = y1 + b4[1];
+            Y[2 * (long)b] = y0 + c0;
+            Y[2 * (long)b + 1] = y1 + c1;
         }
     }
 }

@@ -159,9 +159,16 @@ __global__ void __launch_bounds__(256) out_train_kernel(const float *__restrict_
     __shared__ float d4[OUT_ROWS][2], l2[OUT_ROWS];
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31, b0 = blockIdx.x * OUT_ROWS;
     const int nkc = (Hd + 15) / 16, pitch = 16 * nkc + 1, nrb = (batch + TR - 1) / TR;
+    const float c0 = b4[0], c1 = b4[1];
+#pragma unroll
     for (int r = warp; r < OUT_ROWS; r += 8) {
         const int b = b0 + r;
-        float y0 = 0.f, y1 = 0.f;
+        float y0 = 0.f, y1 = 0.f, t0 = 0.f, t1 = 0.f;
+        if (b < batch) {  // before the products: two dependent loads
+            const long q = trow ? trow[b] : b;
+            t0 = T[2 * q];
+            t1 = T[2 * q + 1];
+        }
         for (int n = lane; n < 16 * nkc; n += 32) {
             const float hv = b < batch && n < Hd ? H2[(long)b * Hd + n] : 0.f;
             hs[r * pitch + n] = hv;
@@ -178,9 +185,8 @@ __global__ void __launch_bounds__(256) out_train_kernel(const float *__restrict_
         if (lane == 0) {
             float e0 = 0.f, e1 = 0.f;
             if (b < batch) {
-                const long q = trow ? trow[b] : b;
-                e0 = y0 + b4[0] - T[2 * q];
-                e1 = y1 + b4[1] - T[2 * q + 1];
+                e0 = y0 + c0 - t0;
+                e1 = y1 + c1 - t1;
             }
             d4[r][0] = e0 * invB;
             d4[r][1] = e1 * invB;
