@@ -309,6 +309,7 @@ __global__ void hermitize_kernel(float2 *__restrict__ A, int n)
 // a1[j2] - a1[n2 - j2] are formed in place once per column, and one lane makes both outputs of
 // a pair.  Sums run in another order than in dft_rows_kernel; both are FP32 sums of the same
 // terms.
+constexpr size_t DFT_SMEM_MAX = 220 * 1024;
 constexpr int P12_WARPS = 8;
 
 // Per warp: a1 [n2][c3] and, for the generic stage 1 only, the plane [n2][n3 + 1] (rows padded:
@@ -819,7 +820,10 @@ __device__ __forceinline__ void stage2_all2(const float2 (&y)[N], int k2, float 
 // [c3][N | 1] of two planes (an odd pitch: lanes on different columns read different banks), each
 // reused for that plane's cd outputs; an even count of float2 so the next warp's plane stays
 // 16-byte aligned.
-constexpr int P12A_WARPS = 7;  // the asynchronous form: two CTAs of 7 warps fit an SM's shared memory
+// Warps of the asynchronous form: two CTAs of 7 fit an SM's shared memory (and a line the registers of 14 warps) up
+// to N = 27; above it one CTA of as many warps as its shared memory holds at 15 columns.
+__host__ __device__ constexpr int p12a_warps(int N) { return N <= 27 ? 7 : N <= 30 ? 9 : N <= 32 ? 8 : 7; }
+__host__ __device__ constexpr int p12_ctas(int N) { return N <= 27 ? 2 : 1; }
 
 __host__ __device__ inline size_t p12c_warp_floats2(int N, int c3, bool async = false)
 {
@@ -829,7 +833,7 @@ __host__ __device__ inline size_t p12c_warp_floats2(int N, int c3, bool async = 
 __host__ __device__ inline size_t p12c_smem(int N, int c3, bool async = false)
 {
     return align16(sizeof(int2) * (size_t)c3 * ((N - 1) / 2 + 1)) +
-           (async ? P12A_WARPS : P12_WARPS) * p12c_warp_floats2(N, c3, async) * sizeof(float2);
+           (async ? p12a_warps(N) : P12_WARPS) * p12c_warp_floats2(N, c3, async) * sizeof(float2);
 }
 
 constexpr int P12C_MAX_C3 = 16;  // stage 2 runs two planes side by side, one per half-warp
@@ -931,13 +935,13 @@ __device__ __forceinline__ void p12c_table(int2 *dtab, int c3, int np2, const in
 // next pair's first plane issued once this pair's first plane has been read and its second plane once
 // the second has been read, so the copies run behind the other plane's stage 1 and stage 2 instead of
 // stalling the warp; 7 warps per CTA keep two CTAs per SM.
-template <int N, bool ASYNC>  // two CTAs per SM (shared memory allows two at every compiled N)
-__global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
+template <int N, bool ASYNC>
+__global__ void __launch_bounds__((ASYNC ? p12a_warps(N) : P12_WARPS) * 32, p12_ctas(N))
     dft_plane12c_kernel(const float2 *__restrict__ X, long long ldx, int rows, int n1, int M, int cd, int np2, int k2,
                         const int4 *__restrict__ g_pair2, float sgn, float2 *__restrict__ Y2)
 {
     static_assert(!ASYNC || N % 2 == 0, "the asynchronous form takes rows of even N");
-    constexpr int NWARPS = ASYNC ? P12A_WARPS : P12_WARPS;
+    constexpr int NWARPS = ASYNC ? p12a_warps(N) : P12_WARPS;
     constexpr int H = (N - 1) / 2;
     constexpr int SP = p12_pitch(N);
     constexpr int LDA = N | 1;
@@ -1042,30 +1046,31 @@ __global__ void __launch_bounds__((ASYNC ? P12A_WARPS : P12_WARPS) * 32, 2)
 // slots and the dependences of 12 warps an SM.  6 warps a CTA keep the folded line, the accumulators and
 // the constant pairs in 168 registers; 7 and 8 warps (128 registers) took 455 and 416 us, one CTA of 16
 // warps with the next tile's planes copied ahead 447 us.
-constexpr int P12P_WARPS = 6, P12P_PLANES = 4 + P12P_WARPS, P12P_TV = 4;
+constexpr int P12P_TV = 4;
+__host__ __device__ constexpr int p12p_warps(int N) { return N <= 27 ? 6 : 10; }
 
 struct PairTile {
     int tv, tc;
 };
 
-// Dynamic shared memory of a CTA with `planes` staged planes, and the tile that fits two CTAs an SM.
+// Dynamic shared memory of a CTA with `planes` staged planes, and the tile that fits two CTAs an SM (one above N = 27).
 __host__ __device__ inline size_t p12p_smem(int N, int c3, int planes)
 {
     return align16(sizeof(int2) * (size_t)c3 * ((N - 1) / 2 + 1)) +
-           sizeof(float2) * ((size_t)planes * N * p12_pitch(N) + (size_t)P12P_WARPS * 2 * c3 * (N | 1));
+           sizeof(float2) * ((size_t)planes * N * p12_pitch(N) + (size_t)p12p_warps(N) * 2 * c3 * (N | 1));
 }
 
 static PairTile pair_tile(int N, int c3, int nv, int nc)
 {
-    int planes = P12P_PLANES;
-    while (planes > 2 && p12p_smem(N, c3, planes) > 112 * 1024)
+    int planes = P12P_TV + p12p_warps(N);
+    while (planes > 2 && p12p_smem(N, c3, planes) > (p12_ctas(N) == 2 ? 112 * 1024 : DFT_SMEM_MAX))
         --planes;
     const int tv = std::min({nv, P12P_TV, planes / 2});
     return {tv, std::min(nc, planes - tv)};
 }
 
 template <int N>
-__global__ void __launch_bounds__(P12P_WARPS * 32, 2)
+__global__ void __launch_bounds__(p12p_warps(N) * 32, p12_ctas(N))
     dft_pairs12c_kernel(const float2 *__restrict__ psi, long long ldx, int n1, int M, int cd, int np2, int k2,
                         const int4 *__restrict__ g_pair2, float sgn, float2 *__restrict__ Y2, PairSrc ps, PairTile tl)
 {
@@ -1087,7 +1092,7 @@ __global__ void __launch_bounds__(P12P_WARPS * 32, 2)
         const unsigned vb = t % nvb, r = t / nvb, cb = r % ncb;
         const int j1 = (int)(r / ncb), v0 = (int)vb * tl.tv, c0 = (int)cb * tl.tc;
         const int nvt = min(tl.tv, ps.nv - v0), nct = min(tl.tc, ps.nc - c0);
-        for (int p = warp; p < nvt + nct; p += P12P_WARPS) {
+        for (int p = warp; p < nvt + nct; p += p12p_warps(N)) {
             const int b = p < nvt ? v0 + p : ps.c0 + c0 + p - nvt;
             const float2 *src = psi + b * ldx + (size_t)j1 * plane;
             float2 *dst = planes + (size_t)p * N * SP;
@@ -1133,7 +1138,7 @@ __global__ void __launch_bounds__(P12P_WARPS * 32, 2)
             return Y2 + (row * n1 + j1) * cd;
         };
         const int nt = nvt * nct;
-        for (int u = 2 * warp; u < nt; u += 2 * P12P_WARPS) {
+        for (int u = 2 * warp; u < nt; u += 2 * p12p_warps(N)) {
             float2 *dA = stage1(u, a1t0), *dB = nullptr;
             if (u + 1 < nt)
                 dB = stage1(u + 1, a1t1);
@@ -1452,7 +1457,7 @@ __global__ void __launch_bounds__(256)
     cp_async_wait<0>();
 }
 
-// Stage 3 with constant twiddles (n1 a compiled size up to 27, sphere pairs present): a thread per
+// Stage 3 with constant twiddles (n1 a compiled size, sphere pairs present): a thread per
 // disk point d.  It reads its n1 values ys[j1][d] (consecutive threads on consecutive d, so no
 // bank conflicts), forms the pairs over j1 in registers and makes the outputs (+-m1, d) for
 // m1 = 0..k1 with the twiddles as compile-time constants (the same sums, in the same order, as
@@ -1571,7 +1576,6 @@ __global__ void __launch_bounds__(256)
 }
 
 constexpr size_t DFT_SMEM_TARGET = 56 * 1024;  // four CTAs per SM
-constexpr size_t DFT_SMEM_MAX = 220 * 1024;
 
 int rows_per_cta(const DftPlan &p)
 {
@@ -1687,7 +1691,7 @@ static cudaError_t launch_p12c_t(int grid, const float2 *X, long long ldx, int r
         cudaFuncSetAttribute(dft_plane12c_kernel<N, ASYNC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
-    dft_plane12c_kernel<N, ASYNC><<<grid, (ASYNC ? P12A_WARPS : P12_WARPS) * 32, smem, s>>>(
+    dft_plane12c_kernel<N, ASYNC><<<grid, (ASYNC ? p12a_warps(N) : P12_WARPS) * 32, smem, s>>>(
         X, ldx, rows, p.n[0], p.sym3, p.cd, p.np2, p.k2, p.pair2, sgn, work);
     return cudaGetLastError();
 }
@@ -1706,7 +1710,7 @@ static cudaError_t launch_p12c(int grid, const float2 *X, long long ldx, int row
             return e;
         // at most rows n1 tiles, which the caller keeps below 2^31
         const long long nt = (long long)((ps->nv + tl.tv - 1) / tl.tv) * ((ps->nc + tl.tc - 1) / tl.tc) * p.n[0];
-        dft_pairs12c_kernel<N><<<(int)std::min<long long>(nt, 152LL * 2), P12P_WARPS * 32, smem, s>>>(
+        dft_pairs12c_kernel<N><<<(int)std::min<long long>(nt, 152LL * p12_ctas(N)), p12p_warps(N) * 32, smem, s>>>(
             X, ldx, p.n[0], p.sym3, p.cd, p.np2, p.k2, p.pair2, sgn, work, *ps, tl);
         return cudaGetLastError();
     }
@@ -1714,7 +1718,7 @@ static cudaError_t launch_p12c(int grid, const float2 *X, long long ldx, int row
         if (ldx % 2 == 0 && (reinterpret_cast<size_t>(X) & 15) == 0 &&
             p12c_smem(N, p.c3, true) <= DFT_SMEM_MAX) {
             const long long ntasks = (long long)rows * p.n[0];
-            const int ga = (int)std::min<long long>((ntasks + P12A_WARPS - 1) / P12A_WARPS, 152LL * 16);
+            const int ga = (int)std::min<long long>((ntasks + p12a_warps(N) - 1) / p12a_warps(N), 152LL * 16);
             return launch_p12c_t<N, true>(ga, X, ldx, rows, p, sgn, work, s);
         }
     }
@@ -1732,12 +1736,13 @@ static cudaError_t launch_p3c(int grid, int nthr, size_t smem, const float2 *wor
     return cudaGetLastError();
 }
 
-// The constant-twiddle stages 1 and 2 serve square planes with N <= 27 (larger lines would not fit
-// two CTAs' registers per SM) and spheres whose m3 values are -M..M, M <= 7, with a disk symmetric
-// in m2 (every sphere at q = 0).
+// The constant-twiddle stages 1 and 2 serve square planes of the sizes below and spheres whose m3 values are
+// -M..M, M <= 7, with a disk symmetric in m2 (every sphere at q = 0).  Above N = 27 a line leaves room for one CTA per SM
+// only, and still takes half the table form's time: row transforms of P at 30^3, 2.87 -> 1.45 ms; 32^3, 4.10 -> 1.97;
+// 36^3, 13.8 -> 4.9; 300 pair rows at 32^3, 75 -> 54 us.
 static bool p12c_compiled(int N)
 {
-    return N == 12 || N == 16 || N == 18 || N == 20 || N == 24 || N == 27;
+    return N == 12 || N == 16 || N == 18 || N == 20 || N == 24 || N == 27 || N == 30 || N == 32 || N == 36;
 }
 
 static bool p12c_applies(const DftPlan &p)
@@ -1809,6 +1814,9 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
         case 20: e = launch_p12c<20>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 24: e = launch_p12c<24>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 27: e = launch_p12c<27>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 30: e = launch_p12c<30>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 32: e = launch_p12c<32>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 36: e = launch_p12c<36>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         default: e = cudaErrorNotSupported; break;
         }
     } else if (pgw > 0) {
@@ -1844,6 +1852,9 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
         case 20: e = launch_p3c<20>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 24: e = launch_p3c<24>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 27: e = launch_p3c<27>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 30: e = launch_p3c<30>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 32: e = launch_p3c<32>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 36: e = launch_p3c<36>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         default: e = cudaErrorNotSupported; break;
         }
         count_launches(2);

@@ -1,0 +1,35 @@
+"""Constant-twiddle planes of 30 x 30, 32 x 32 and 36 x 36 points (one CTA per SM) and stage 3 of those lengths, against the
+table form: the widest sphere (15 columns), few and many pair rows, an odd number of planes, and n1 alone at the size."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1810_07772_gb300 import gw
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("dims,gcut,nv,nc", [
+    ((15, 30, 30), 49, 2, 5), ((15, 32, 32), 49, 1, 3), ((15, 36, 36), 49, 3, 9),
+    ((3, 36, 36), 1, 5, 7), ((5, 30, 30), 4, 9, 21), ((7, 32, 32), 9, 4, 6),
+    ((30, 12, 12), 25, 2, 5), ((32, 16, 16), 30, 2, 5), ((36, 18, 18), 30, 2, 5),
+])
+def test_constant_form_matches_tables(dims, gcut, nv, nc):
+    rng = np.random.default_rng(sum(dims))
+    nr = int(np.prod(dims))
+    psi = (rng.standard_normal((nv + nc, nr)) + 1j * rng.standard_normal((nv + nc, nr))) / np.sqrt(2 * nr)
+    E = np.concatenate([np.linspace(-5, -1, nv), np.linspace(1, 9, nc)])
+    out = {}
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(DEV), E, dims, nv)
+        for kind in ("two_kernel", "tables"):
+            ctx.set_transform_kernel(kind)
+            ctx.build_P("fp16x3")
+            ctx.P_to_G(gcut)
+            r = ctx.view("PG").cpu().numpy()
+            ctx.build_PG(gcut)
+            out[kind] = (r, ctx.view("PG").cpu().numpy())
+    # the same FP32 sums in the same order; the twiddles differ only in the exact zeros
+    for a, b in zip(out["two_kernel"], out["tables"]):
+        assert np.linalg.norm(a - b) <= 1e-7 * np.linalg.norm(b)
