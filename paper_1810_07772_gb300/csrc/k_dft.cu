@@ -836,7 +836,7 @@ __host__ __device__ inline size_t p12c_smem(int N, int c3, bool async = false)
            (async ? p12a_warps(N) : P12_WARPS) * p12c_warp_floats2(N, c3, async) * sizeof(float2);
 }
 
-constexpr int P12C_MAX_C3 = 16;  // stage 2 runs two planes side by side, one per half-warp
+constexpr int P12C_MAX_C3 = 16;  // stage 2 runs two planes side by side, one per half-warp; so outputs m <= 7 only
 
 // Stage 1 of one plane (a lane per line j2): a1t[M + m3][j2] = sum_j3 x[j2][j3] e(+-m3 j3 / N), the line
 // read into registers by line(j2, x).
@@ -858,7 +858,7 @@ __device__ __forceinline__ void p12c_stage1(int lane, int M, float sgn, float2 *
             col[M * LDA] = make_float2(a0.x + x[N / 2].x, a0.y + x[N / 2].y);
         else
             col[M * LDA] = a0;
-        stage1_all2<N>(x, M, sgn, col, LDA, std::make_integer_sequence<int, (H + 1) / 2>{});
+        stage1_all2<N>(x, M, sgn, col, LDA, std::make_integer_sequence<int, (H + 1) / 2 < 4 ? (H + 1) / 2 : 4>{});
     }
     __syncwarp();
 }
@@ -903,7 +903,8 @@ __device__ __forceinline__ void p12c_stage2(int lane, int c3, int cd, int k2, fl
     __syncwarp();
     if (act) {
         pair_fold<N>(y);
-        stage2_all2<N>(y, k2, sgn, dtab + i3 * (H + 1), a1t, std::make_integer_sequence<int, H / 2 + 1>{});
+        stage2_all2<N>(y, k2, sgn, dtab + i3 * (H + 1), a1t,
+                       std::make_integer_sequence<int, H / 2 + 1 < 4 ? H / 2 + 1 : 4>{});
     }
     __syncwarp();
     for (int t = lane; t < cd; t += 32)
@@ -1739,17 +1740,23 @@ static cudaError_t launch_p3c(int grid, int nthr, size_t smem, const float2 *wor
 // The constant-twiddle stages 1 and 2 serve square planes of the sizes below and spheres whose m3 values are
 // -M..M, M <= 7, with a disk symmetric in m2 (every sphere at q = 0).  Above N = 27 a line leaves room for one CTA per SM
 // only, and still takes half the table form's time: row transforms of P at 30^3, 2.87 -> 1.45 ms; 32^3, 4.10 -> 1.97;
-// 36^3, 13.8 -> 4.9; 300 pair rows at 32^3, 75 -> 54 us.
+// 36^3, 13.8 -> 4.9; 360 pair rows at 32^3, 75 -> 54 us.  Against the any-size kernel: 15^3, 97 -> 57 us; 21^3, 474 -> 248;
+// 25^3, 1.38 -> 0.63 ms; 28^3, 2.74 -> 1.00.
 static bool p12c_compiled(int N)
 {
-    return N == 12 || N == 16 || N == 18 || N == 20 || N == 24 || N == 27 || N == 30 || N == 32 || N == 36;
+    switch (N) {
+    case 12: case 15: case 16: case 18: case 20: case 21: case 24: case 25: case 27: case 28: case 30: case 32: case 36:
+        return true;
+    default:
+        return false;
+    }
 }
 
 static bool p12c_applies(const DftPlan &p)
 {
     const int N = p.n[2];
     return p.n[1] == N && p12c_compiled(N) && p.sym3 >= 0 && p.c3 == 2 * p.sym3 + 1 && p.np2 > 0 &&
-           p.c3 <= P12C_MAX_C3 && p.k2 <= (N - 1) / 2 && p12c_smem(N, p.c3) <= DFT_SMEM_MAX;
+           p.c3 <= P12C_MAX_C3 && p.k2 <= std::min(7, (N - 1) / 2) && p12c_smem(N, p.c3) <= DFT_SMEM_MAX;
 }
 
 template <bool PAIR>
@@ -1809,11 +1816,15 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
     if (cst) {
         switch (p.n[2]) {
         case 12: e = launch_p12c<12>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 15: e = launch_p12c<15>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 16: e = launch_p12c<16>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 18: e = launch_p12c<18>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 20: e = launch_p12c<20>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 21: e = launch_p12c<21>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 24: e = launch_p12c<24>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 25: e = launch_p12c<25>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 27: e = launch_p12c<27>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
+        case 28: e = launch_p12c<28>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 30: e = launch_p12c<30>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 32: e = launch_p12c<32>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
         case 36: e = launch_p12c<36>(g12, X, ldx, rows, p, sgn, work, ps, s); break;
@@ -1847,11 +1858,15 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
         const int g3c = (int)std::min<long long>((rows + R - 1) / R, 152LL * per_sm);
         switch (p.n[0]) {
         case 12: e = launch_p3c<12>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 15: e = launch_p3c<15>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 16: e = launch_p3c<16>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 18: e = launch_p3c<18>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 20: e = launch_p3c<20>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 21: e = launch_p3c<21>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 24: e = launch_p3c<24>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 25: e = launch_p3c<25>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 27: e = launch_p3c<27>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
+        case 28: e = launch_p3c<28>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 30: e = launch_p3c<30>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 32: e = launch_p3c<32>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
         case 36: e = launch_p3c<36>(g3c, nthr, sm, work, rows, p, sgn, Y, ldy, s); break;
