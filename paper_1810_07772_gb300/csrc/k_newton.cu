@@ -373,7 +373,7 @@ static_assert(GSMEM <= 227 * 1024, "shared memory of one CTA");
 constexpr int GTHREADS = 320;  // warps 0..7 send the partial tile, warp 8 copies, warp 9 MMAs; all finish it
 constexpr int G_COPY = 8, G_MMA = 9;
 constexpr int MODE_Y = 0, MODE_X = 1, MODE_D = 2;
-constexpr float LOSS_PER_CHUNK = 1.3e-7f;  // mean truncation loss of the TMEM sums (see k_herk16p.cu)
+constexpr float LOSS_PER_CHUNK = 1.3e-7f;  // mean relative truncation loss of a TMEM sum, per 16-k chunk
 
 // C = P Q^H over all k, one 128 x 128 tile per cluster of C CTAs, each taking a part of k, in two TMEM
 // sums (half the truncation of one).  CTA `rank` finishes rows [rank 128/C, ...) of the tile: every CTA
