@@ -449,9 +449,9 @@ def run_gw(args):
     contracted = form["terms"] * (w.nv + w.nc) if form["terms"] else w.k
     achieved = 4.0 * contracted * w.nr * (w.nr + 1) / (herk_ms * 1e-3) / 1e12 if herk_ms > 0 else None
     # tensor-pipe work actually issued per 16-k chunk per tile: 3 MMAs of 2*128*256*16 and 6 of
-    # 2*128*128*16, the same as 6 of N = 256; a CTA pair issues 6 of M = 256, N = 256
+    # 2*128*128*16, the same as 6 of N = 256; a CTA pair issues 6 of M = 256, N = 256 (pair form only)
     pair_kernel = args.herk_kernel == "pair" and not form["terms"]
-    rows_per_tile = 256 if args.herk_kernel == "pair" else 128
+    rows_per_tile = 256 if pair_kernel else 128
     tensor_flop = st["herk_tiles"] * form["chunks"] * 6 * 2.0 * rows_per_tile * 256 * 16
     traffic = None if form["terms"] else herk_traffic(
         w.name, args.precision, (int(st["window_chunks"]), int(st["flush_windows"])), args.herk_kernel)

@@ -249,8 +249,8 @@ GW_API gw_status gw_reset_times(gw_ctx *ctx);
  * GW_INV_NEWTON_TC and gw_zinv_tc), [2] = mean rank-k update
  * time in ms over the timed calls since gw_reset_times, [3] = number of those calls, [4] = the
  * FP16 scale exponent e of the last 16-bit build (of the pair densities; of the unoccupied states in
- * separable form), [5] = rank-k update tiles (256 x 128 for GW_HERK_PAIR), [6] and [7] = the window and
- * flush lengths of the 16-bit update.
+ * separable form), [5] = tiles of the last rank-k update (256 x 128 where GW_HERK_PAIR ran), [6] and [7] =
+ * the window and flush lengths of the 16-bit update.
  */
 GW_API gw_status gw_get_stats(gw_ctx *ctx, double *stats8);
 
@@ -420,10 +420,12 @@ GW_API gw_status gw_set_herk_window(gw_ctx *ctx, int window_chunks, int flush_wi
  *                   M = 256): each CTA holds 128 rows of A and half of B, 256 x 128 complex tiles;
  *                   the operand holds six 16-bit planes per k chunk (the Im planes also negated)
  *   GW_HERK_SINGLE  (default) one CTA per 128 x 128 complex tile, four planes per k chunk
- * Takes effect at the next gw_build_P; GW_E_INVALID for another value.  An update in separable form
- * runs the persistent one-CTA kernel under either setting.
+ * An update in separable form runs the persistent one-CTA kernel under either setting.
+ *   GW_HERK_BY_PAIRS added to either: no separable form, every update is taken pair by pair
+ * Takes effect at the next gw_build_P (and the next gw_batch_create, which always runs the persistent
+ * kernel); GW_E_INVALID for another value.
  */
-enum { GW_HERK_SINGLE = 0, GW_HERK_PAIR = 1 };
+enum { GW_HERK_SINGLE = 0, GW_HERK_PAIR = 1, GW_HERK_BY_PAIRS = 2 };
 GW_API gw_status gw_set_herk_kernel(gw_ctx *ctx, int kind);
 
 /*

@@ -557,7 +557,7 @@ void newton_tc_record(Ctx &c)
 }
 
 // Separable form of the 16-bit rank-k update for the loaded energies: c.sep.T terms, 0 where the pair
-// form has less to contract.  A term costs its ceil(nc / 16) + ceil(nv / 16) chunks of 16 states and
+// form has less to contract (or was asked for, see separable).  A term costs its ceil(nc / 16) + ceil(nv / 16) chunks of 16 states and
 // about SEP_TERM_CHUNKS more for its shorter windows and for multiplying its sums out; the pair form
 // costs ceil(nv nc / 16).  Update, pair against separable form, 20^3 grid, W = 3 (us): nv x nc =
 // 8 x 300 (150 chunks against T = 8 times 20) 1389 / 1704, 20 x 64 (80; 9 x 6) 797 / 779, 14 x 200 (175;
@@ -573,6 +573,11 @@ void find_separable(Ctx &c)
     const int most = (pair_chunks - 1) / (ncc + nvc + SEP_TERM_CHUNKS);
     c.sep = most >= 1 ? sep_factors(c.E_h.data(), c.nv, c.nc, HERK16_KC, most) : SepFactors();
     c.sep_known = true;
+}
+
+bool separable(const Ctx &c)
+{
+    return !c.by_pairs && c.sep.T > 0;
 }
 
 // The separable job of a context whose d_P and scale words exist: operand buffers, factors and job
@@ -619,13 +624,12 @@ cudaError_t separable_planes(Ctx &c, const HerkJob &j, bool bf16, cudaStream_t s
 gw_status form_pair_planes(Ctx &c)
 {
     const bool bf16 = c.F_prec == GW_PREC_BF16X3;
-    const int npl = c.last_herk_kernel == GW_HERK_PAIR ? HERK16_NPL_PAIR : HERK16_NPL;
     GW_CUDA(cudaSetDevice(c.device), "set device");
-    c.F_bytes = (size_t)c.kpad * c.nr_pad * sizeof(uint16_t) * npl;
+    c.F_bytes = (size_t)c.kpad * c.nr_pad * sizeof(uint16_t) * c.F_npl;
     GW_TRY(ensure(c, c.d_F, c.cap.F, c.F_bytes, "pair-density operand"));
     GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, bf16,
                                   c.d_small, reinterpret_cast<int *>(c.d_small + 1),
-                                  reinterpret_cast<uint16_t *>(c.d_F), c.stream, npl),
+                                  reinterpret_cast<uint16_t *>(c.d_F), c.stream, c.F_npl),
             "pair densities (16-bit)");
     c.F_formed = true;
     return GW_OK;
@@ -829,9 +833,10 @@ gw_status gw_set_herk_window(gw_ctx *h, int window_chunks, int flush_windows)
 
 gw_status gw_set_herk_kernel(gw_ctx *h, int kind)
 {
-    if (!h || (kind != GW_HERK_SINGLE && kind != GW_HERK_PAIR))
+    if (!h || kind < 0 || kind > (GW_HERK_PAIR | GW_HERK_BY_PAIRS))
         return GW_E_INVALID;
-    h->c.herk_kernel = kind;
+    h->c.herk_kernel = kind & ~GW_HERK_BY_PAIRS;
+    h->c.by_pairs = (kind & GW_HERK_BY_PAIRS) != 0;
     return GW_OK;
 }
 
@@ -1018,7 +1023,7 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     const int npl = pair ? HERK16_NPL_PAIR : HERK16_NPL;
     if (p16)
         find_separable(c);
-    const bool sep = p16 && c.sep.T > 0;
+    const bool sep = p16 && separable(c);
     size_t Fbytes = 0;
     if (precision == GW_PREC_FP32_SIMT)
         Fbytes = (size_t)c.kpad * c.nr_pad * sizeof(float2);
@@ -1042,7 +1047,7 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
             t.push_back(make_int4(0, ij.x, ij.y, 0));
         GW_TRY(ensure(c, c.d_tiles, c.cap.tiles, t.size() * sizeof(int4), "tile list"));
         GW_CUDA(cudaMemcpy(c.d_tiles, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice), "tile upload");
-        c.n_tiles_run = static_cast<int>(t.size());
+        c.n_tiles = static_cast<int>(t.size());
         c.tiles_nr_pad = c.nr_pad;
         c.tiles_kind = tile_kind;
     } else if (precision != GW_PREC_FP32_SIMT && (c.tiles_nr_pad != c.nr_pad || c.tiles_kind != tile_kind)) {
@@ -1051,16 +1056,15 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
                              : herk_tiles(c.nr_pad, HERK_BM, HERK_BN);
         GW_TRY(ensure(c, c.d_tiles, c.cap.tiles, t.size() * sizeof(int2), "tile list"));
         GW_CUDA(cudaMemcpy(c.d_tiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice), "tile upload");
-        c.n_tiles_run = static_cast<int>(t.size());
+        c.n_tiles = static_cast<int>(t.size());
         c.tiles_nr_pad = c.nr_pad;
         c.tiles_kind = tile_kind;
     }
-    c.n_tiles = sep && pair ? static_cast<int>(herk_pair_tiles(c.nr_pad).size()) : c.n_tiles_run;
     const uint64_t wait_ns = static_cast<uint64_t>(c.wait_limit_ms * 1e6);
     int *scale_exp = reinterpret_cast<int *>(c.d_small + 1);
 
     HerkJob job = {};
-    const int grid_sep = std::min(c.n_tiles_run, sm_count(c.device));
+    const int grid_sep = std::min(c.n_tiles, sm_count(c.device));
     if (sep) {
         GW_TRY(ensure(c, c.d_sums, c.cap_sums, (size_t)grid_sep * HERK16P_SUMS, "running sums"));
         GW_TRY(prepare_separable(c, &job));
@@ -1079,29 +1083,30 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
                 "pair densities");
     c.F_prec = precision;
     c.F_formed = !sep;
+    c.last_terms = sep ? c.sep.T : 0;
     if (p16)
-        c.last_herk_kernel = pair ? GW_HERK_PAIR : GW_HERK_SINGLE;
+        c.F_npl = npl;
     record(c, 1);
     if (precision == GW_PREC_FP32_SIMT) {
         GW_CUDA(launch_herk_simt(reinterpret_cast<float2 *>(c.d_F), c.kpad, c.nr, c.nr_pad, c.d_P, s),
                 "rank-k update (CUDA cores)");
     } else if (sep) {
         GW_CUDA(launch_herk16p(static_cast<const HerkJob *>(c.d_sept), reinterpret_cast<const int4 *>(c.d_tiles),
-                               c.n_tiles_run, grid_sep, precision == GW_PREC_BF16X3, c.d_err, wait_ns, c.last_W,
+                               c.n_tiles, grid_sep, precision == GW_PREC_BF16X3, c.d_err, wait_ns, c.last_W,
                                c.herk_L, c.d_sums, s),
                 "rank-k update (tcgen05, separable, 16-bit)");
     } else if (pair) {
         GW_CUDA(launch_herk16x2(reinterpret_cast<uint16_t *>(c.d_F), precision == GW_PREC_BF16X3, c.kpad, c.nr,
-                                c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
+                                c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
                                 c.herk_L, s),
                 "rank-k update (tcgen05 CTA pairs, 16-bit)");
     } else if (p16) {
         GW_CUDA(launch_herk16(reinterpret_cast<uint16_t *>(c.d_F), precision == GW_PREC_BF16X3, c.kpad, c.nr,
-                              c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W,
-                              c.herk_L, s),
+                              c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, scale_exp, c.d_err, wait_ns, c.last_W, c.herk_L,
+                              s),
                 "rank-k update (tcgen05, 16-bit)");
     } else {
-        GW_CUDA(launch_herk_tc(c.d_F, precision, c.kpad, c.nr, c.nr_pad, c.d_tiles, c.n_tiles_run, c.d_P, c.d_err, wait_ns,
+        GW_CUDA(launch_herk_tc(c.d_F, precision, c.kpad, c.nr, c.nr_pad, c.d_tiles, c.n_tiles, c.d_P, c.d_err, wait_ns,
                                s),
                 "rank-k update (tcgen05, TF32)");
     }
@@ -1768,7 +1773,7 @@ gw_status gw_get_buffer(gw_ctx *h, int which, void **ptr, size_t *bytes)
         *bytes = c.F_bytes;
         return GW_OK;
     case GW_BUF_FACTORS:
-        if ((c.F_prec != GW_PREC_FP16X3 && c.F_prec != GW_PREC_BF16X3) || !c.P_ready || c.sep.T == 0)
+        if ((c.F_prec != GW_PREC_FP16X3 && c.F_prec != GW_PREC_BF16X3) || !c.P_ready || c.last_terms == 0)
             return GW_E_NOT_READY;
         *ptr = const_cast<float *>(c.sep_tab);
         *bytes = c.sep.tab.size() * sizeof(float);
@@ -1912,14 +1917,14 @@ gw_status batch_prepare(gw_batch &b)
         const int kpad = ((c.k + HERK16_KC - 1) / HERK16_KC) * HERK16_KC;
         c.kpad = kpad;
         find_separable(c);
-        const bool sep = c.sep.T > 0;
+        const bool sep = separable(c);
         const size_t Fbytes = (size_t)kpad * c.nr_pad * 2 * HERK16_NPL;
         if (!sep)
             GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
         if (!c.d_small)
             GW_CUDA(cudaMalloc(&c.d_small, 4 * sizeof(unsigned)), "scale words");
         c.F_bytes = Fbytes;
-        c.last_herk_kernel = GW_HERK_SINGLE;
+        c.F_npl = HERK16_NPL;
         c.P_bytes = (size_t)c.nr * c.nr * sizeof(float2);
         GW_TRY(ensure(c, c.d_P, c.cap.P, c.P_bytes, "P(r,r')"));
         if (b.gcut[i] != c.gcut)
@@ -1998,6 +2003,7 @@ gw_status batch_pair_densities(gw_batch &b)
                     "pair densities (batch)");
         c.F_prec = b.precision;
         c.F_formed = !sep;
+        c.last_terms = sep ? b.jobs[i].T : 0;
     }
     return GW_OK;
 }

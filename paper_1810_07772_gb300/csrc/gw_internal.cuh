@@ -109,7 +109,7 @@ struct Ctx {
     size_t P_bytes = 0;
     bool P_ready = false;
     int2 *d_tiles = nullptr;        // HERK tile list
-    int n_tiles = 0, tiles_rb = 0;
+    int n_tiles = 0;                // tiles in d_tiles, those of the last update
     int2 *d_tiles_g = nullptr;      // tile list of the N_g x N_g update (g-space route)
     int n_tiles_g = 0, tiles_g_pad = -1;
     float2 *d_PG_parts = nullptr;   // split-k partials of the N_g x N_g update
@@ -180,7 +180,6 @@ struct Ctx {
             scal, tcw, PGsum, coef, gidx, gtw, psig, ppw;
     } cap = {};
     int tiles_nr_pad = -1, tiles_kind = -1;
-    int n_tiles_run = 0;            // tiles in d_tiles (n_tiles is what gw_get_stats reports)
     // separable rank-k update (sep_factors.h, k_herk16p.cu)
     SepFactors sep;                 // factors of the loaded energies (T = 0: pair form)
     bool sep_known = false;         // sep belongs to the loaded energies
@@ -190,12 +189,15 @@ struct Ctx {
     uint16_t *d_sepA = nullptr, *d_sepB = nullptr;
     float4 *d_sums = nullptr;       // HERK16P_SUMS per CTA
     size_t cap_sept = 0, cap_sepA = 0, cap_sepB = 0, cap_sums = 0;
+    int last_terms = 0;             // terms of the last update's separable form (0: pair by pair)
     bool F_formed = false;          // d_F holds the planes of F_prec (false after a separable update)
+    int F_npl = 0;                  // 16-bit planes per block of d_F: the kernel setting at the last 16-bit update
     float sw_max = 0.f;             // max sqrt(2/(E_c - E_v)) (host, from the energies)
     unsigned *d_small = nullptr;    // [0] |f| bound bits, [1] FP16 scale exponent; separable update: [0], [1]
                                     // bounds and [2], [3] exponents of psi_c and psi_v
     int herk_W = 3, herk_L = 256;   // 6.5e-7 against FP64 at 24^3; see gw_set_herk_window
     int herk_kernel = GW_HERK_SINGLE; // r-space 16-bit update: one CTA per tile or CTA pairs
+    bool by_pairs = false;            // always pair by pair (GW_HERK_BY_PAIRS)
     std::vector<double> E_h;        // the loaded energies in Hartree (host copy)
     float *d_csw = nullptr;         // closure pair weights [nv][nb], then [nv][nv] for the occupied pairs
     float2 *d_Qc = nullptr;         // closure matrix elements when built from gw_build_PG's transforms
@@ -219,7 +221,6 @@ struct Ctx {
     int cgvec_gen = -1;
     int plan_gen = 0;               // incremented by every plan build
     size_t cap_csw = 0, cap_cw = 0, cap_cgvec = 0, cap_cwork = 0;
-    int last_herk_kernel = -1;      // the kernel of the last 16-bit r-space update
     double err_target = 0.0;        // > 0: the window comes from gw_set_error_target's rule
     int last_W = 3;                 // the window of the last 16-bit rank-k update
     uint32_t last_status = 0;       // the device status word read by the last synchronising call

@@ -21,6 +21,7 @@ GW_OK, GW_E_INVALID, GW_E_NOMEM, GW_E_CUDA, GW_E_NOT_READY, GW_E_NUMERIC, GW_E_T
 PRECISION = {"tf32x3": 0, "bf16x3": 1, "tf32x1": 2, "fp32_simt": 3, "fp16x3": 4}
 INV_METHOD = {"cholesky": 0, "newton": 1, "newton_tc": 2}
 HERK_KERNEL = {"single": 0, "pair": 1}
+GW_HERK_BY_PAIRS = 2
 TRANSFORM_KERNEL = {"two_kernel": 0, "fused": 1, "tables": 2}
 ZGEMM_MODE = {"fp16x3": 0, "slices": 1}
 GW_C64, GW_C128 = 0, 1
@@ -404,10 +405,11 @@ class Context:
         self._check(lib().gw_set_transform_kernel(self._h, TRANSFORM_KERNEL[kind] if isinstance(kind, str)
                                                   else int(kind)))
 
-    def set_herk_kernel(self, kind):
+    def set_herk_kernel(self, kind, by_pairs=False):
         """Kernel of the 16-bit r-space update: "single" (one CTA per tile, the default) or "pair"
-        (CTA pairs sharing 2-SM MMAs) (gw_set_herk_kernel)."""
-        self._check(lib().gw_set_herk_kernel(self._h, HERK_KERNEL[kind] if isinstance(kind, str) else int(kind)))
+        (CTA pairs sharing 2-SM MMAs); by_pairs: never in separable form (gw_set_herk_kernel)."""
+        k = HERK_KERNEL[kind] if isinstance(kind, str) else int(kind)
+        self._check(lib().gw_set_herk_kernel(self._h, k | (GW_HERK_BY_PAIRS if by_pairs else 0)))
 
     def set_error_target(self, target):
         """P~ error target of the 16-bit update; the window follows from it (gw_set_error_target)."""

@@ -1,5 +1,6 @@
 """The rank-k update on CTA pairs (GW_HERK_PAIR: 2-SM tensor-core MMAs, 256 x 128 complex tiles)
-against the one-CTA kernel and the FP64 oracle.
+against the one-CTA kernel and the FP64 oracle, both pair by pair (GW_HERK_BY_PAIRS: the separable form has
+a kernel of its own).
 
 Both kernels issue the same products in the same order for every element of P (per 16-k chunk:
 Ai Bi and Ai Br, hi*hi + hi*lo + lo*hi, then Ar Br and -Ar Bi), so P must agree bit for bit;
@@ -23,12 +24,13 @@ def rel(a, b):
 
 def build(ctx, kind, prec, window=None):
     nr = int(np.prod(ctx.dims))
-    ctx.set_herk_kernel(kind)
+    ctx.set_herk_kernel(kind, by_pairs=True)
     if window:
         ctx.set_herk_window(*window)
     P = torch.empty((nr, nr), dtype=torch.complex64, device="cuda:0")
     ctx.build_P(prec, P_out=P)
     ctx.sync()
+    assert ctx.update_form()["terms"] == 0
     return P
 
 

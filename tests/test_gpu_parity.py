@@ -310,11 +310,12 @@ def test_non_finite_state_is_reported():
         assert e.value.status == gw.GW_E_INVALID
 
 
-@pytest.mark.parametrize("prec", ["fp16x3", "tf32x3"])
-def test_wait_limit_expires_cleanly_and_context_recovers(prec):
+@pytest.mark.parametrize("prec,by_pairs", [("fp16x3", False), ("fp16x3", True), ("tf32x3", False)])
+def test_wait_limit_expires_cleanly_and_context_recovers(prec, by_pairs):
     """A wait limit far below the kernel's run time makes the rank-k update's waits run out:
     the kernel records GW_E_TIMEOUT and returns early; the context stays usable and the next
-    call with the default limit reproduces the earlier result bit for bit."""
+    call with the default limit reproduces the earlier result bit for bit.  FP16X3: the separable form's
+    kernel and the pair form's."""
     dims = (16, 16, 16)
     nv, nc = 16, 512                      # k = 8192: each tile's main loop lasts about a millisecond
     psi, E = inputs.make_states(16, nv, nc, 41)
@@ -323,8 +324,10 @@ def test_wait_limit_expires_cleanly_and_context_recovers(prec):
     with gw.Context(0) as ctx:
         ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(dev), E, dims, nv)
         P1 = torch.empty((nr, nr), dtype=torch.complex64, device=dev)
+        ctx.set_herk_kernel("single", by_pairs)
         ctx.build_P(prec, P_out=P1)
         ctx.sync()
+        assert (ctx.update_form()["terms"] > 0) == (prec == "fp16x3" and not by_pairs)
         ctx.set_wait_limit(1e-6)
         ctx.build_P(prec)
         with pytest.raises(gw.GwError) as e:

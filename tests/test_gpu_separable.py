@@ -19,11 +19,11 @@ def rel(a, b):
     return float(np.linalg.norm(a - b) / np.linalg.norm(b))
 
 
-def build(dims, nv, nc, psi, E, prec="fp16x3", window=None, kind="single"):
+def build(dims, nv, nc, psi, E, prec="fp16x3", window=None, kind="single", by_pairs=False):
     nr = int(np.prod(dims))
     with gw.Context(0) as ctx:
         ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
-        ctx.set_herk_kernel(kind)
+        ctx.set_herk_kernel(kind, by_pairs)
         if window:
             ctx.set_herk_window(*window)
         P = torch.empty((nr, nr), dtype=torch.complex64, device="cuda:0")
@@ -70,22 +70,44 @@ def test_energies_in_any_order_and_degenerate():
     assert form["terms"] > 1 and rel(P.cpu().numpy(), O.P_rspace(psi, E, nv)) <= 1e-6
 
 
-def test_kernel_setting_and_pair_densities_afterwards():
-    """GW_HERK_PAIR gives the same P; GW_BUF_F still holds the pair densities when it is asked for."""
-    from test_gpu_parity import _decode_16
+def test_by_pairs():
+    """GW_HERK_BY_PAIRS takes the other kernel: FP32 sums of the same numbers in another order, each within
+    1e-6 of FP64; the factors are there after the separable form only, and a bad value is refused."""
     dims, nv, nc = (8, 8, 8), 16, 208
     psi, E = inputs.make_states(0, nv, nc, 1, dims=dims)
-    a, _ = build(dims, nv, nc, psi, E)
-    b, form = build(dims, nv, nc, psi, E, kind="pair")
-    assert torch.equal(a, b) and form["terms"] > 1
+    a, fa = build(dims, nv, nc, psi, E)
+    b, fb = build(dims, nv, nc, psi, E, by_pairs=True)
+    assert fa["terms"] > 1 and fb == {"terms": 0, "chunks": nv * nc // 16}
+    assert not torch.equal(a, b) and rel(a.cpu().numpy(), b.cpu().numpy()) <= 2e-6
     with gw.Context(0) as ctx:
         ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
         ctx.build_P("fp16x3")
+        ctx.set_herk_kernel("single", by_pairs=True)
+        assert ctx.update_form()["terms"] == fa["terms"]  # the form of the last update, not of the next
+        ctx.build_P("fp16x3")
+        assert ctx.update_form()["terms"] == 0
+        with pytest.raises(gw.GwError) as e:
+            ctx.set_herk_kernel(4)
+        assert e.value.status == gw.GW_E_INVALID
+
+
+@pytest.mark.parametrize("kind,npl", [("single", 4), ("pair", 6)])
+def test_kernel_setting_and_pair_densities_afterwards(kind, npl):
+    """GW_HERK_PAIR leaves the kernel of the separable form as it is (128 x 128 tiles are reported); GW_BUF_F
+    still holds the pair densities, in the layout of the setting, when it is asked for."""
+    from test_gpu_parity import _decode_16
+    dims, nv, nc = (8, 8, 8), 16, 208
+    psi, E = inputs.make_states(0, nv, nc, 1, dims=dims)
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        ctx.set_herk_kernel(kind)
+        ctx.build_P("fp16x3")
+        assert ctx.update_form()["terms"] > 1 and ctx.stats()["herk_tiles"] == 10
         ptr, nbytes = ctx.buffer("F")
         torch.cuda.synchronize()
         F = torch.as_tensor(gw.DeviceView(ptr, (nbytes,), "|u1"), device="cuda:0").cpu().numpy()
         e = int(ctx.stats()["fp16_scale_exp"])
-        f, _ = _decode_16(F, ctx.dims8()[7], 512, nv * nc, bf16=False)
+        f, _ = _decode_16(F, ctx.dims8()[7], 512, nv * nc, bf16=False, npl=npl)
     assert rel(f / 2.0 ** e, O.pair_density(psi, E, nv).T) < 1e-6
 
 
