@@ -349,9 +349,10 @@ __global__ void __launch_bounds__(256) ns_init_kernel(const double2 *__restrict_
                     const double2 z = A[(size_t)r * N + k];
                     a = make_float2((float)z.x, (float)z.y);
                 }
-                const float f = xr * (jac ? c * rs[k] * rs[k] : c);
-                re[i] = (r == k ? 2.f * xr : 0.f) - f * a.x;
-                im[i] = -f * a.y;
+                // (X0 a) X0: the product of two entries of X0 can overflow
+                const float xk = jac ? c * rs[k] * rs[k] : c;
+                re[i] = (r == k ? 2.f * xr : 0.f) - xr * a.x * xk;
+                im[i] = -(xr * a.y) * xk;
                 best = fmaxf(best, fmaxf(fabsf(re[i]), fabsf(im[i])));
             }
             re[i] *= sc;
@@ -937,8 +938,9 @@ __global__ void __launch_bounds__(RTHREADS, 1)
 
 // R_0 = I - sum (j = 0) or R_j = R_(j-1) - sum (j > 0) of the slots' integers: R64, R's FP16X3 planes and
 // max |R_j|.  The integers are added modulo 2^64 in units of 2^(e - width); R_0 is far below 2^(e - 1) after a
-// phase 1 that converged, and an FP32 sum of the same slots tells where it is not (the residual is then
-// reported as infinite, which fails the final check).  Thread: one row, eight columns.
+// phase 1 that converged, and an FP32 sum of the same slots tells where it is not: the entry of R_0 is then
+// NaN and stays so in every later residual, whose maximum (infinite) fails the final check.  Thread: one row,
+// eight columns.
 __global__ void __launch_bounds__(256)
     ns_combine_kernel(const int4 *__restrict__ T, const __grid_constant__ Groups grp, int N, int nb, int nkc, int j,
                       int max_steps, double2 *__restrict__ R64, uint16_t *__restrict__ R16, Words *w)
@@ -996,13 +998,13 @@ __global__ void __launch_bounds__(256)
         if (gi >= N || gj >= N)
             continue;
         double xr, xi;
-        bool bad = false;
         if (j == 0) {
             const unsigned long long one = gi == gj && ish >= 0 && ish < 64 ? 1ull << ish : 0ull;
             const float one_f = gi == gj ? ldexpf(1.0f, -(ea + eb)) : 0.f;
             xr = (double)(long long)(one - (unsigned long long)sr[i]) * unit;
             xi = (double)(long long)(0ull - (unsigned long long)si[i]) * unit;
-            bad = !(fabsf(one_f - fr[i]) < 0.4f) || !(fabsf(fi[i]) < 0.4f) || ish < 0 || (gi == gj && ish >= 64);
+            if (!(fabsf(one_f - fr[i]) < 0.4f) || !(fabsf(fi[i]) < 0.4f) || ish < 0 || (gi == gj && ish >= 64))
+                xr = __longlong_as_double(0x7ff8000000000000ll);
         } else {
             const double2 r = R64[(size_t)gi * N + gj];
             xr = r.x - (double)sr[i] * unit;
@@ -1011,7 +1013,7 @@ __global__ void __launch_bounds__(256)
         R64[(size_t)gi * N + gj] = make_double2(xr, xi);
         re[i] = (float)xr;
         im[i] = (float)xi;
-        best = fmaxf(best, bad ? __int_as_float(0x7f800000) : finite_or_inf(sqrtf(re[i] * re[i] + im[i] * im[i])));
+        best = fmaxf(best, finite_or_inf(sqrtf(re[i] * re[i] + im[i] * im[i])));
         re[i] *= so;
         im[i] *= so;
     }
@@ -1021,7 +1023,8 @@ __global__ void __launch_bounds__(256)
     block_max(best, &w->mr[j]);
 }
 
-// Xout = X64 + the last dX, and the verdict.  A failure after a phase 1 that ran out of steps is told
+// Xout = X64 + the last dX, and the verdict: the last residual is small (each is exact for the X64 it was
+// taken of) and the last dX, which no residual has seen, finite.  A failure after a phase 1 that ran out of steps is told
 // apart (NS_DETAIL_CAP): the eager form, with more steps, may still converge.
 __global__ void ns_final_kernel(const double2 *__restrict__ X64, const double2 *__restrict__ D, size_t n,
                                 double2 *__restrict__ Xout, const Words *w, uint32_t *err)
@@ -1034,7 +1037,7 @@ __global__ void ns_final_kernel(const double2 *__restrict__ X64, const double2 *
         int last = 0;
         while (last + 1 < NS_REFINE && !refine_over(w, last + 1))
             ++last;
-        if (!(bits_f(w->mr[last]) <= (float)NS_ACCEPT))
+        if (!(bits_f(w->mr[last]) <= (float)NS_ACCEPT) || !isfinite(bits_f(w->md[last])))
             record_error(err, GW_E_NUMERIC, SITE_NS, w->done ? 0u : NS_DETAIL_CAP);
     }
 }

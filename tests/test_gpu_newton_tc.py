@@ -271,3 +271,22 @@ def test_eps_inv_refuses_a_stream_under_capture():
             ctx.eps_inv("newton_tc", epsinv_out=again)
         s.synchronize()
         assert torch.equal(again, ref)
+
+
+@pytest.mark.parametrize("n", [93, 400])
+@pytest.mark.parametrize("scale", [1e-40, 1e-36, 1e-30, 1e-25, 1e-20, 1e20, 1e30, 1e36, 1e40])
+def test_matrices_of_any_scale(n, scale):
+    """A well-conditioned matrix times 1e-30 .. 1e30 has its inverse to 1e-10 (its FP32 corrections lose bits
+    at the large end); beyond, where FP32 planes and scales run out, the call may refuse, but a status of
+    OK always comes with the inverse."""
+    rng = np.random.default_rng(n)
+    B = crand(rng, n, n // 2) / np.sqrt(n)
+    C = np.eye(n) + 0.5 * (B @ B.conj().T)
+    C = 0.5 * (C + C.conj().T)
+    with gw.Context(0) as ctx:
+        try:
+            X = ctx.zinv_tc(dev(C * scale)).cpu().numpy()
+        except gw.GwError as e:
+            assert e.status == gw.GW_E_NUMERIC and not 1e-31 < scale < 1e31
+            return
+    assert np.max(np.abs(np.eye(n) - (X * scale) @ C)) <= 1e-10
