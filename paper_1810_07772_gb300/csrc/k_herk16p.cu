@@ -137,6 +137,18 @@ __device__ __forceinline__ float mean_window(int n, int w)
     return (float)(full * w * w + rest * rest) / (float)n;
 }
 
+// The scales of the operands, 2^ec and 2^ev, come out of P = -sum_t V_t C_t 2^(-2 ec - 2 ev).  V is
+// brought down to the size of its terms, so that the products with C stay in range, and the rest is
+// applied to the sums in two factors, each a normal FP32 value.
+constexpr int V_SHIFT = -28;
+
+__device__ __forceinline__ void unscale(int ec, int ev, float &a, float &b)
+{
+    const int e = max(-252, min(252, -2 * ec - 2 * ev - V_SHIFT)), h = e / 2;
+    a = ldexpf(1.0f, h);
+    b = ldexpf(1.0f, e - h);
+}
+
 // Factor that undoes the mean truncation loss of a product of two sums over windows of n chunks together
 // (header comment): sums of terms of one sign lose most, so the diagonal has its own.
 __device__ __forceinline__ float loss_gain(float n, bool diagonal)
@@ -367,7 +379,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                                  seg == 0);
                     continue;
                 }
-                const float vs = jb.term_scale[seg] * ldexpf(1.0f, -2 * jb.scale_exp[1]);
+                const float vs = jb.term_scale[seg] * ldexpf(1.0f, V_SHIFT);
                 for (int win = 0; win < w.nwv; ++win) {
                     if (!ready())
                         break;
@@ -400,7 +412,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // consecutive r
             const int nr = jb.nr, r0 = tl.y * TM + q * 32, r = r0 + lane, cbase = tl.z * TN + h * 64;
             const float nw = mean_window(jb.ncc, w.wc) + mean_window(jb.nvc, w.wv);
-            const float s1 = -ldexpf(1.0f, -2 * jb.scale_exp[0]);
+            float s0 = 1.f, s1 = -ldexpf(1.0f, -2 * jb.scale_exp[0]);
+            if (sep) {
+                unscale(jb.scale_exp[0], jb.scale_exp[1], s0, s1);
+                s1 = -s1;
+            }
             const float s2 = sep ? s1 * loss_gain(nw, false) : s1, sd = sep ? s1 * loss_gain(nw, true) : s1;
             float2 *P = jb.P;
             for (int g0 = 0; g0 < 64; g0 += OUT_COLS) {
@@ -409,8 +425,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 for (int i = 0; i < OUT_COLS / 2; ++i) {
                     const float4 v = sums_load(my + (g0 / 2 + i) * 256);
                     const int col = cbase + g0 + 2 * i;
-                    x[2 * i] = make_float2(v.x * (col == r ? sd : s2), v.y * s2);
-                    x[2 * i + 1] = make_float2(v.z * (col + 1 == r ? sd : s2), v.w * s2);
+                    x[2 * i] = make_float2(v.x * (col == r ? sd : s2) * s0, v.y * s2 * s0);
+                    x[2 * i + 1] = make_float2(v.z * (col + 1 == r ? sd : s2) * s0, v.w * s2 * s0);
                 }
 #pragma unroll
                 for (int i = 0; i < OUT_COLS; ++i) {

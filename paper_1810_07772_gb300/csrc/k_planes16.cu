@@ -255,11 +255,12 @@ __global__ void state_bound_kernel(const float2 *__restrict__ psiT, int nr, int 
     }
 }
 
-// Exponent e with bound 2^e in [2^13, 2^14) (0 for a zero or a non-finite bound).
+// Exponent e with bound 2^e in [2^13, 2^14) (0 for a zero or a non-finite bound); 2^e and 2^-e are normal
+// FP32 values.
 __device__ __forceinline__ int state_exp(unsigned bits)
 {
     const float b = __uint_as_float(bits);
-    return !(b > 0.f) || !isfinite(b) ? 0 : max(-100, min(100, 13 - ilogbf(b)));
+    return !(b > 0.f) || !isfinite(b) ? 0 : max(-126, min(126, 13 - ilogbf(b)));
 }
 
 // Operand planes of the separable rank-k update (herk16p_kernel): chunk j < ncc holds 16 unoccupied
@@ -267,7 +268,9 @@ __device__ __forceinline__ int state_exp(unsigned bits)
 // states times the factors of term t (tab[t][16 j + k], see sep_factors.h) as chunks t (ncc + nvc) + j.
 // The layout of work is that of pair_density16_rows_kernel: blockIdx.x is an 8-row group, a warp
 // takes a chunk and writes the group's 256 contiguous bytes of each plane.  BF16 concerns the
-// unoccupied chunks; the occupied ones are FP16 always (see herk16p_kernel).  Bound by the plane
+// unoccupied chunks; the occupied ones are FP16 always (see herk16p_kernel).  Both sets are scaled by
+// a power of two of their own in either precision: the sums C_t and V_t of unscaled states would leave
+// FP32's range where their products, the weighted sums over pairs, do not.  Bound by the plane
 // writes, (T + 1)(nc + nv) N_r 8 bytes; at 24^3 (T = 11, 512 states) 0.68 GB where the pair
 // densities' planes take 1.70 GB.
 template <bool BF16>
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(256)
         }
         __syncthreads();
     }
-    const int ec = BF16 ? 0 : state_exp(bound_bits[0]), ev = state_exp(bound_bits[1]);
+    const int ec = state_exp(bound_bits[0]), ev = state_exp(bound_bits[1]);
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         scale_exp[0] = ec;
         scale_exp[1] = ev;

@@ -70,6 +70,20 @@ def test_energies_in_any_order_and_degenerate():
     assert form["terms"] > 1 and rel(P.cpu().numpy(), O.P_rspace(psi, E, nv)) <= 1e-6
 
 
+@pytest.mark.parametrize("prec,bar", [("fp16x3", 1e-6), ("bf16x3", 1e-5)])
+@pytest.mark.parametrize("ev,ec", [(60, -60), (-60, 60), (-100, 100), (100, -100), (30, 30), (-20, -30), (0, 55), (-55, 0)])
+def test_states_of_any_scale(prec, bar, ev, ec):
+    """Occupied states times 2^ev, unoccupied ones times 2^ec: P is 2^(2 ev + 2 ec) times that of the unit states,
+    an FP32 value, and only powers of two change on the way."""
+    dims, nv, nc = (7, 9, 11), 20, 110
+    psi, E = inputs.make_states(0, nv, nc, 6, dims=dims)
+    scale = np.concatenate([np.full(nv, 2.0 ** ev), np.full(nc, 2.0 ** ec)])[:, None]
+    P, form = build(dims, nv, nc, psi.astype(np.complex64).astype(np.complex128) * scale, E, prec)
+    assert form["terms"] > 1
+    P = P.cpu().numpy().astype(np.complex128) * 2.0 ** (-2 * ev - 2 * ec)
+    assert rel(P, O.P_rspace(psi, E, nv)) <= bar
+
+
 def test_by_pairs():
     """GW_HERK_BY_PAIRS takes the other kernel: FP32 sums of the same numbers in another order, each within
     1e-6 of FP64; the factors are there after the separable form only, and a bad value is refused."""
