@@ -19,23 +19,34 @@
 //    their own threads only (20 MB for the GPU, resident in L2), added with fire-and-forget vector
 //    reductions so no thread waits for a load.
 //
-// Measured on one GB300 (update alone, FP16X3, W = 3): 24^3, 32 x 480 states: 24.2 -> 8.48 ms (0.95 of
+// Measured on one GB300 (update alone, FP16X3, W = 3): 24^3, 32 x 480 states: 24.2 -> 9.3 ms (0.95 of
 // the sustained FP16 rate would be 6.9 ms for the issued MMAs); 36^3, 64 x 1000, BF16X3, W = 16: 0.97 ->
-// 0.19 s.
+// 0.20 s.
 //
 // Bound: the tensor pipe and the shared memory that feeds it, as herk16_kernel (32 KB staged and 84 KB
 // read per chunk).  Control: mbarrier phases and the two TMEM window buffers carry across tiles, so the
 // producer streams the next tile's operands while the current tile is being written.
 //
-// Truncation.  tcgen05 adds into TMEM with truncation, so a window comes out smaller by a nearly uniform
-// factor.  Measured in the separable form, for windows of n chunks together (C and V): 1.0e-7 + 1.5e-7 n on
-// the diagonal of P, where every term has one sign, 3.0e-7 + 0.3e-7 n on its other elements, the same on
-// random and on band-structured states.  The separable form multiplies these mean losses back (loss_gain),
-// which leaves its errors below those of the pair form even at windows of twice the length (Windows).
+// Truncation.  tcgen05 adds into TMEM with truncation, so a window comes out smaller, and the product of two
+// windowed sums loses twice.  How much depends on the states: elements of P whose terms have one sign
+// lose most.  Measured loss, in 1e-7, for windows of n chunks together (C and V), FP16X3:
+//                                n = 2          4         17 or 18     40 to 55
+//   diagonal                 2.4 ..  4.8    3.8 .. 8.4    16 .. 40    49 .. 110
+//   next to it               2.3 ..  5.4    3.7 .. 8.9    16 .. 22    48 ..  50
+//   far from it              2.3 ..  3.2    3.7 .. 5.3     7 .. 16     7 ..  50
+// (Haar-random states, band-structured ones, plane waves of equal size and states without a sign change,
+// 12^3 to 20^3, up to 1600 unoccupied states); BF16X3 loses less.  The separable form adds a share of this
+// back (loss_gain), at the low end of what was measured, so that no element is overcorrected by more
+// than the pair form leaves it short.  Relative error of P against FP64 then, separable / pair form at the
+// same W, in 1e-7: Haar, 14^3, 32 x 480: 1.5 / 2.8 (W = 1), 1.8 / 6.0 (3), 4.9 / 31 (16), 7 / 130 (64);
+// band-structured, 14^3, 48 x 700: 1.4 / 2.4, 2.2 / 5.2, 7.4 / 28, 14 / 120; plane waves, 16^3, 19 x 600:
+// 2.2 / 2.5, 4.7 / 4.7, 11 / 21, 24 / 89; BF16X3 the same three: 19 / 34, 11 / 25, 12 / 23 (W = 1), 21 / 49, 14 / 40,
+// 15 / 30 (16).  Windows of 2 W chunks would take 8.5 ms instead of 9.3 at 24^3, but on the plane waves
+// leave 6.8 where the pair form at W = 3 leaves 4.7.
 //
 // The occupied planes are FP16 in either precision (they are 1/16 of the work), so with BF16 operands
 // only C_t carries the 8 + 8-bit split: both at 8 + 8 bits measured 5.7e-6 on the off-diagonal elements
-// of P against 4.5e-6 in the pair form; now 4.1e-6, and 1.4e-6 against 3.4e-6 on P~.
+// of P against 4.5e-6 in the pair form; now 4.1e-6.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -54,12 +65,14 @@ constexpr uint32_t NPL = HERK16_NPL;
 // hi part and of the lo part, so one N = 256 MMA from A = Im fills the Re and Im columns of a window
 constexpr uint32_t B_OFF = 4 * PL;
 constexpr uint32_t CHUNK_BYTES = 8 * PL;  // 32 KB
-// Two chunks per pipeline stage (a stage holds chunks of one window only): half the barrier round trips and
-// commits.  Measured at 24^3 with windows of six chunks, one / two / three chunks a stage: 8.73 / 8.48 /
-// 8.80 ms; with windows of 32, 8.30 / 8.11 / 8.21 ms.
-constexpr int CPS = 2, STAGES = 3;
-constexpr uint32_t STAGE_BYTES = CPS * CHUNK_BYTES;
-constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;  // 192 KB
+// Chunks per pipeline stage, CPS (a stage holds chunks of one window only; six chunks are in flight):
+// fewer barrier round trips and commits than one by one.  Two, or three where W is a multiple of three, so
+// that the stages are full.  Measured, one / two / three chunks a stage, FP16X3: W = 3, 16^3 with 16 x 200
+// states 0.497 / 0.506 / 0.485 ms, 24^3 9.40 / 9.39 / 9.25, 32^3 with 48 x 800 85.0 / 86.2 / 83.8; W = 4,
+// 24^3 8.99 / 9.05 / 9.43; W = 16, 36^3, BF16X3, 204 / 200 / 202.
+constexpr int RING_CHUNKS = 6;
+constexpr uint32_t PIPE_BYTES = RING_CHUNKS * CHUNK_BYTES;  // 192 KB
+constexpr int MAX_STAGES = 3;
 constexpr uint32_t LBO = 128, SBO = 256;
 constexpr int NPROMO_WARPS = 8;
 constexpr int PRODUCER_WARP = 8, MMA_WARP = 9;
@@ -99,6 +112,7 @@ __device__ __forceinline__ float4 sums_load(const float4 *p)
 }
 
 // Position in the ring of stages: stage and phase parity of a stage counter.
+template <int STAGES>
 struct Ring {
     int s = 0;
     uint32_t ph = 0;
@@ -112,18 +126,14 @@ struct Ring {
 };
 
 // Windows of a job: each term has nwc windows of wc chunks over its ncc unoccupied (or pair) chunks, the
-// last one shorter, then nwv windows of wv chunks over its nvc occupied ones.  The separable form takes
-// windows of 2 W chunks: with the mean loss multiplied back its errors still lie below those of the pair
-// form at W (16^3, 16 / 200 states, FP16X3, off-diagonal P, separable against pair:
-// 2.2e-7 / 2.8e-7 at W = 1, 3.3e-7 / 4.3e-7 at 3, 5.4e-7 / 9.4e-7 at 8; P~ at 24^3: 1.1e-7 / 2.9e-7, 2.2e-7 /
-// 6.5e-7, 4.4e-7 / 1.6e-6), and the boundaries, about 0.3 us each, halve: 9.43 -> 8.48 ms at 24^3, W = 3.
+// last one shorter, then nwv windows of wv chunks over its nvc occupied ones; both at most W.
 struct Windows {
     int wc, nwc, nwv, wv;
     __device__ __forceinline__ Windows(const HerkJob &j, int W)
     {
-        wc = j.nvc > 0 ? 2 * W : W;
+        wc = W;
         nwc = (j.ncc + wc - 1) / wc;
-        nwv = (j.nvc + 2 * W - 1) / (2 * W);
+        nwv = (j.nvc + W - 1) / W;
         wv = nwv > 0 ? (j.nvc + nwv - 1) / nwv : 0;
     }
 };
@@ -149,18 +159,25 @@ __device__ __forceinline__ void unscale(int ec, int ev, float &a, float &b)
     b = ldexpf(1.0f, e - h);
 }
 
-// Factor that undoes the mean truncation loss of a product of two sums over windows of n chunks together
-// (header comment): sums of terms of one sign lose most, so the diagonal has its own.
+// Share of an element of P to add to it for what truncation took from a product of two sums over windows of n
+// chunks together (header comment); the diagonal loses most and has its own.  It is added, not multiplied
+// on: 1 + share has steps of 1.2e-7.
+template <bool BF16>
 __device__ __forceinline__ float loss_gain(float n, bool diagonal)
 {
-    return diagonal ? 1.f + (1.0e-7f + 1.5e-7f * n) : 1.f + (3.0e-7f + 0.3e-7f * n);
+    if (BF16)
+        return diagonal ? 1.5e-7f + 0.5e-7f * n : 1.2e-7f + 0.45e-7f * n;
+    return diagonal ? 1.0e-7f + 1.5e-7f * n : 2.6e-7f + 0.3e-7f * n;
 }
 
-template <bool BF16>
+template <bool BF16, int CPS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     herk16p_kernel(const HerkJob *__restrict__ jobs, const int4 *__restrict__ tiles, int n_tiles, uint32_t *err,
                    uint64_t wait_ns, int W, int L, float4 *__restrict__ sums)
 {
+    constexpr int STAGES = RING_CHUNKS / CPS;
+    static_assert(STAGES <= MAX_STAGES, "barriers");
+    constexpr uint32_t STAGE_BYTES = CPS * CHUNK_BYTES;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + PIPE_BYTES);
     uint64_t *empty = full + STAGES;
@@ -199,7 +216,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     if (warp == PRODUCER_WARP) {
         if (lane == 0) {
             long long g = 0;  // stages issued by this CTA over all its tiles
-            Ring ring;
+            Ring<STAGES> ring;
             bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
                 const int4 tl = tiles[t];
@@ -244,7 +261,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t sbase = smem_u32(smem);
             long long g = 0;
             uint32_t gw = 0;  // windows issued by this CTA
-            Ring ring;
+            Ring<STAGES> ring;
             bool ok = true;
             // one window of n chunks into TMEM buffer gw & 1; the formats' bits of the descriptors: fmt
             auto window = [&](int n, uint32_t fmt) {
@@ -417,7 +434,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 unscale(jb.scale_exp[0], jb.scale_exp[1], s0, s1);
                 s1 = -s1;
             }
-            const float s2 = sep ? s1 * loss_gain(nw, false) : s1, sd = sep ? s1 * loss_gain(nw, true) : s1;
+            const float gain = loss_gain<BF16>(nw, false), gain_d = loss_gain<BF16>(nw, true);
+            auto out = [&](float v, bool diagonal) {
+                const float x = v * s1 * s0;
+                return sep ? fmaf(x, diagonal ? gain_d : gain, x) : x;
+            };
             float2 *P = jb.P;
             for (int g0 = 0; g0 < 64; g0 += OUT_COLS) {
                 float2 x[OUT_COLS];
@@ -425,8 +446,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 for (int i = 0; i < OUT_COLS / 2; ++i) {
                     const float4 v = sums_load(my + (g0 / 2 + i) * 256);
                     const int col = cbase + g0 + 2 * i;
-                    x[2 * i] = make_float2(v.x * (col == r ? sd : s2) * s0, v.y * s2 * s0);
-                    x[2 * i + 1] = make_float2(v.z * (col + 1 == r ? sd : s2) * s0, v.w * s2 * s0);
+                    x[2 * i] = make_float2(out(v.x, col == r), out(v.y, false));
+                    x[2 * i + 1] = make_float2(out(v.z, col + 1 == r), out(v.w, false));
                 }
 #pragma unroll
                 for (int i = 0; i < OUT_COLS; ++i) {
@@ -476,7 +497,8 @@ cudaError_t launch_herk16p(const HerkJob *jobs, const int4 *tiles, int n_tiles, 
 {
     if (n_tiles <= 0)
         return cudaSuccess;
-    auto kernel = bf16 ? herk16p_kernel<true> : herk16p_kernel<false>;
+    auto kernel = W % 3 == 0 ? (bf16 ? herk16p_kernel<true, 3> : herk16p_kernel<false, 3>)
+                             : (bf16 ? herk16p_kernel<true, 2> : herk16p_kernel<false, 2>);
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
     if (e != cudaSuccess)
         return e;

@@ -84,6 +84,66 @@ def test_states_of_any_scale(prec, bar, ev, ec):
     assert rel(P, O.P_rspace(psi, E, nv)) <= bar
 
 
+def _smooth_states(kind, dims, nv, nc, seed):
+    """(psi complex64 on the device, E): Haar-random, band-structured or plane waves in order of |m|."""
+    if kind == "haar":
+        psi, E = inputs.make_states(0, nv, nc, seed, dims=dims)
+        return torch.from_numpy(psi.astype(np.complex64)).cuda(), E
+    if kind == "bands":
+        coef, gvec, E = inputs.make_states_g_structured_device(dims, nv, nc, seed, "cuda:0")
+        with gw.Context(0) as ctx:
+            ctx.load_states_g(coef, gvec, E, dims, nv)
+            return ctx.view("psiT").t().contiguous(), E
+    m = np.stack(np.meshgrid(*[np.arange(-(d // 2) + 1, d // 2) for d in dims], indexing="ij"), -1).reshape(-1, 3)
+    m2 = (m ** 2).sum(1)
+    order = np.argsort(m2, kind="stable")[:nv + nc]
+    m, m2 = m[order], m2[order].astype(float)
+    E = np.concatenate([-10 + 9 * m2[:nv] / m2[nv - 1], 0.5 + 19.5 * (m2[nv:] - m2[nv]) / (m2[-1] - m2[nv])])
+    x = [np.exp(2j * np.pi * np.outer(m[:, a], np.arange(d)) / d) for a, d in enumerate(dims)]
+    psi = np.einsum("pa,pb,pc->pabc", *x).reshape(nv + nc, -1) / np.sqrt(np.prod(dims))
+    return torch.from_numpy(psi.astype(np.complex64)).cuda(), E
+
+
+@pytest.mark.parametrize("kind,dims,nv,nc", [("haar", (12, 12, 12), 40, 1600), ("bands", (14, 14, 14), 16, 1040),
+                                             ("plane", (16, 16, 16), 19, 600)])
+@pytest.mark.parametrize("prec", ["fp16x3", "bf16x3"])
+def test_no_less_precise_than_by_pairs(kind, dims, nv, nc, prec):
+    """Windows up to 64 chunks that are really that long, and smooth states, whose sums near the diagonal have
+    terms of one sign: the whole of P, its diagonal, its elements next to it and the far ones, against an
+    FP64 sum, beside the pair form's errors at the same window.  The whole within 5 % of the pair form's
+    (rounding of the last bit); a class of elements within a quarter of the larger of its own and the
+    whole's (the loss that is added back is a mean over states)."""
+    psi, E = _smooth_states(kind, dims, nv, nc, 3)
+    p64, Eh = psi.to(torch.complex128), torch.from_numpy(E / 27.211386245988).cuda()
+    ref = 0.0
+    for v in range(nv):
+        f = p64[v].conj()[None, :] * p64[nv:]
+        ref = ref - (f * (2.0 / (Eh[nv:] - Eh[v]))[:, None]).t() @ f.conj()
+    x = torch.from_numpy(np.stack(np.unravel_index(np.arange(int(np.prod(dims))), dims), -1)).cuda()
+    d2 = 0
+    for a, n in enumerate(dims):
+        q = (x[:, None, a] - x[None, :, a]).abs()
+        d2 = d2 + torch.minimum(q, n - q) ** 2
+    classes = [d2 >= 0, d2 == 0, d2 == 1, (d2 >= 2) & (d2 <= 9), d2 > 9]
+
+    def errors(ctx, by_pairs):
+        ctx.set_herk_kernel("single", by_pairs)
+        ctx.build_P(prec)
+        ctx.sync()
+        assert (ctx.update_form()["terms"] > 0) == (not by_pairs)
+        P = ctx.view("P").to(torch.complex128)
+        return [float((P[k] - ref[k]).norm() / ref[k].norm()) for k in classes]
+
+    with gw.Context(0) as ctx:
+        ctx.load_states(psi, E, dims, nv)
+        for W in (2, 3, 16, 64):
+            ctx.set_herk_window(W, 256)
+            sep, pair = errors(ctx, False), errors(ctx, True)
+            assert sep[0] <= 1.05 * pair[0], (W, sep, pair)
+            for s, p in zip(sep[1:], pair[1:]):
+                assert s <= 1.25 * max(p, pair[0]), (W, sep, pair)
+
+
 def test_by_pairs():
     """GW_HERK_BY_PAIRS takes the other kernel: FP32 sums of the same numbers in another order, each within
     1e-6 of FP64; the factors are there after the separable form only, and a bad value is refused."""
