@@ -40,6 +40,29 @@ def test_gradient(n_in, hid, B):
     assert np.linalg.norm(g - g_ref) <= 2e-5 * np.linalg.norm(g_ref)
 
 
+def test_weight_gradients_of_a_large_batch():
+    """Each layer's gradient at 8192 rows.  A truncating FP32 sum of n additions of one sign is short by n 2^-24 at
+    most and by half of that on average: 1e-6 for 35 chunks with one addition of the sum's size each, beside
+    5e-6 of the products before it (three-part splits through three layers).  Six such additions a chunk would
+    leave 6.3e-6."""
+    n_in, hid, B = 12, 256, 8192
+    X, T, rows, th = _setup(n_in, hid, B)
+    X[:, 9] = 1.0                                  # terms of one sign
+    params = M.unpack(M.to_fp16_weights(th.astype(np.float64), n_in, hid), n_in, hid)
+    _, grads = M.loss_and_grad(params, X[rows].astype(np.float64), T[rows].astype(np.float64))
+    g_ref = M.flatten(grads)
+    with gw.Mlp(n_in, hid, max_batch=B, device=0) as net:
+        net.set_params(th)
+        g = net.grad(torch.from_numpy(X).to(DEV), torch.from_numpy(T).to(DEV), torch.from_numpy(rows).to(DEV))[0]
+        net.check()
+    g = g.cpu().numpy().astype(np.float64)
+    o = 0
+    for n in (hid * n_in, hid, hid * hid, hid, hid * hid, hid, 2 * hid, 2):
+        e = np.linalg.norm(g[o:o + n] - g_ref[o:o + n]) / np.linalg.norm(g_ref[o:o + n])
+        assert e <= 6e-6, n
+        o += n
+
+
 @pytest.mark.parametrize("n_in,hid,B", [(12, 256, 300), (5, 33, 40)])
 def test_two_steps_follow_the_gradients(n_in, hid, B):
     X, T, rows, th = _setup(n_in, hid, B)
