@@ -343,8 +343,8 @@ __global__ void __launch_bounds__(256) step_finish_kernel(MlpFinish f, MlpWeight
         for (int r = 1; r < 8; ++r)
             acc += red[r][c];
         if (l == 3 && col == width - 1) {  // the loss, sum |y - t|^2 / (2B)
-            if (f.loss)
-                *f.loss += f.loss_scale * acc;
+            if (f.loss)  // the caller's, and it may collect the steps of several networks and streams
+                atomicAdd(f.loss, f.loss_scale * acc);
             return;
         }
         apply((l < 3 ? f.off_b[l] : f.off_out) + col, acc, 3, 0);

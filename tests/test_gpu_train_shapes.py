@@ -115,3 +115,25 @@ def test_pass_order_with_equal_upper_halves(n, seed):
         for t in range(4):
             b.train_step(X, T, rows[t * batch:(t + 1) * batch], 1e-3)
         assert np.array_equal(a.get_params(), b.get_params())
+
+
+def test_two_networks_add_to_one_loss():
+    """Two networks on streams of their own add their steps' losses to one accumulator."""
+    n_in, hid, B, steps = 5, 33, 40, 300
+    X, T, rows, th = _setup(n_in, hid, B)
+    Xd, Td, rd = (torch.from_numpy(a).to(DEV) for a in (X, T, rows))
+    loss = torch.zeros(1, dtype=torch.float32, device=DEV)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    nets = [gw.Mlp(n_in, hid, max_batch=B, device=0, stream=s) for s in streams]
+    for net in nets:
+        net.set_params(th)
+    one = nets[0].grad(Xd, Td, rd)[1]
+    for _ in range(steps):
+        for net in nets:
+            net.train_step(Xd, Td, rd, 1e-12, loss_accum=loss)   # the parameters stay where they are
+    for net in nets:
+        net.check()
+        net.close()
+    # FP32 sum of 2 steps terms of one sign
+    assert abs(float(loss.item()) - 2 * steps * one) <= 2 * steps * 2.0 ** -24 * 2 * steps * one
