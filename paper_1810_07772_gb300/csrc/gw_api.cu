@@ -1985,6 +1985,8 @@ gw_status batch_prepare(gw_batch &b)
         cudaFree(b.d_sums);
     b.d_sums = nullptr;
     GW_BCUDA(cudaMalloc(&b.d_sums, (size_t)b.grid * HERK16P_SUMS), "running sums");
+    // the contexts' factors and plans went up on their stream; the pass and the autotuner run on the batch's
+    GW_BCUDA(cudaStreamSynchronize(b.ctxs[0]->c.stream), "batch uploads");
     return GW_OK;
 }
 

@@ -222,3 +222,27 @@ def test_batch_of_both_forms_equals_single_instances():
                     assert torch.equal(c.view("PG"), PG)
     for c in ctxs:
         c.close()
+
+
+def test_batch_set_up_behind_queued_work():
+    """Contexts on a stream of their own with work queued on it: the factors are there when the autotuner starts
+    on the batch's stream."""
+    dims, nv, nc, gcut = (9, 10, 11), 24, 200, 5
+    loaded = [inputs.make_states(0, nv, nc, seed, dims=dims) for seed in (81, 82)]
+    s = torch.cuda.Stream()
+    refs, ctxs = [], []
+    for psi, E in loaded:
+        refs.append(build(dims, nv, nc, psi, E, window=(2, 256))[0])
+        ctx = gw.Context(0, stream=s)
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        ctxs.append(ctx)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(200_000_000)     # about 0.1 s
+    with gw.Batch(ctxs, [gcut] * 2) as b:
+        b.autotune(target_error=1e-3)
+        got = [c.view("P").clone() for c in ctxs]
+    for P, ref in zip(got, refs):
+        assert rel(P.cpu().numpy(), ref.cpu().numpy()) <= 1e-4
+    for c in ctxs:
+        c.close()
