@@ -269,7 +269,9 @@ GW_API gw_status gw_get_stats(gw_ctx *ctx, double *stats8);
  * gw_batch_create   ctxs[n] loaded contexts, gcuts[n] their sphere cuts, precision GW_PREC_FP16X3
  *                   or GW_PREC_BF16X3 (else GW_E_UNSUPPORTED).  Allocates every buffer the pass
  *                   needs, builds the sphere plans and the tile table.  The contexts must outlive
- *                   the batch and must not be reloaded while it is in use.
+ *                   the batch; one that is loaded again, or used by itself, between two passes is
+ *                   prepared again by the next one, which then runs eagerly (GW_E_INVALID if its cut
+ *                   does not fit the new grid).
  * gw_batch_run      one pass.  use_graph != 0: the first call runs eagerly, the second captures the
  *                   whole pass into a CUDA graph, later calls replay it (recaptured after
  *                   gw_batch_set_window).  Synchronises the stream and returns the first error

@@ -77,6 +77,7 @@ gw_status ensure(Ctx &c, T *&p, size_t &cap, size_t bytes, const char *what)
         return GW_OK;
     dfree(p);
     cap = 0;
+    ++c.alloc_gen;
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&p), bytes ? bytes : 16);
     if (e != cudaSuccess) {
         p = nullptr;
@@ -942,6 +943,7 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     c.loaded = c.P_ready = c.PG_ready = c.eps_ready = false;
     c.q_pairs = false;
     c.sep_known = false;
+    ++c.load_gen;
     // The sphere plan depends on the grid and the cut only (its sqrt(V) on the cell and q): states of
     // another system, k-point or step on the same grid and cell keep it.  Building it takes the host 50 us
     // at 12^3 and 130 us at 24^3, with the GPU idle.
@@ -1843,6 +1845,7 @@ struct gw_batch {
     bool own_stream = false;
     HerkJob *d_jobs = nullptr;
     std::vector<HerkJob> jobs;      // as uploaded
+    std::vector<std::array<int, 3>> gens;  // the contexts' generations when they were prepared (batch_gens)
     float4 *d_sums = nullptr;       // HERK16P_SUMS per CTA of the update
     int4 *d_tiles = nullptr;
     int n_tiles = 0, grid = 0;
@@ -1906,6 +1909,12 @@ void drop_graph(gw_batch &b)
     b.graph = nullptr;
 }
 
+// Loads, plans and buffers of a context so far.
+std::array<int, 3> batch_gens(const Ctx &c)
+{
+    return {c.load_gen, c.plan_gen, c.alloc_gen};
+}
+
 // Allocate every buffer the pass needs (graph capture must not allocate) and build the plans.
 gw_status batch_prepare(gw_batch &b)
 {
@@ -1914,6 +1923,9 @@ gw_status batch_prepare(gw_batch &b)
     std::vector<int4> tiles;
     for (size_t i = 0; i < b.ctxs.size(); ++i) {
         Ctx &c = b.ctxs[i]->c;
+        const int nmin = std::min(c.n1, std::min(c.n2, c.n3));  // the grid may be another than at gw_batch_create
+        if (4LL * b.gcut[i] >= (long long)nmin * nmin)
+            return fail(c, GW_E_INVALID, "gcut %d must satisfy 4 gcut < min(n)^2 = %d", b.gcut[i], nmin * nmin);
         const int kpad = ((c.k + HERK16_KC - 1) / HERK16_KC) * HERK16_KC;
         c.kpad = kpad;
         find_separable(c);
@@ -1987,7 +1999,30 @@ gw_status batch_prepare(gw_batch &b)
     GW_BCUDA(cudaMalloc(&b.d_sums, (size_t)b.grid * HERK16P_SUMS), "running sums");
     // the contexts' factors and plans went up on their stream; the pass and the autotuner run on the batch's
     GW_BCUDA(cudaStreamSynchronize(b.ctxs[0]->c.stream), "batch uploads");
+    b.gens.clear();
+    for (const gw_ctx *h : b.ctxs)
+        b.gens.push_back(batch_gens(h->c));
     return GW_OK;
+}
+
+// Prepare again what the contexts no longer are: one loaded anew (other energies mean other factors, even at the
+// same sizes), or used by itself with another cut or with buffers that had to grow.
+gw_status batch_refresh(gw_batch &b)
+{
+    bool same = b.gens.size() == b.ctxs.size();
+    for (size_t i = 0; same && i < b.ctxs.size(); ++i)
+        same = b.gens[i] == batch_gens(b.ctxs[i]->c) && b.gcut[i] == b.ctxs[i]->c.gcut;
+    if (same)
+        return GW_OK;
+    drop_graph(b);
+    b.runs = 0;
+    b.gens.clear();
+    const gw_status st = batch_prepare(b);
+    if (st != GW_OK)
+        for (const gw_ctx *h : b.ctxs)
+            if (b.last_error.empty())
+                b.last_error = h->c.last_error;
+    return st;
 }
 
 gw_status batch_pair_densities(gw_batch &b)
@@ -1999,9 +2034,10 @@ gw_status batch_pair_densities(gw_batch &b)
         if (sep)
             GW_CUDA(separable_planes(c, b.jobs[i], bf16, b.stream), "separable operand planes (batch)");
         else
-            GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, bf16,
-                                          c.d_small, reinterpret_cast<int *>(c.d_small + 1),
-                                          reinterpret_cast<uint16_t *>(c.d_F), b.stream),
+            GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc,
+                                          b.jobs[i].ncc * HERK16_KC, c.nr_pad, bf16, c.d_small, 
+                                          reinterpret_cast<int *>(c.d_small + 1), reinterpret_cast<uint16_t *>(c.d_F),
+                                          b.stream),
                     "pair densities (batch)");
         c.F_prec = b.precision;
         c.F_formed = !sep;
@@ -2202,6 +2238,7 @@ gw_status gw_batch_run(gw_batch *b, int use_graph)
             return bfail(bb, GW_E_NOT_READY, "a context lost its states");
     // work queued earlier on the contexts' stream comes first
     GW_BCUDA(cudaStreamSynchronize(bb.ctxs[0]->c.stream), "context stream synchronize");
+    GW_TRY(batch_refresh(bb));
     if (!use_graph || bb.runs == 0) {
         // eager pass (the first pass is always eager, so every lazy setup happens outside capture)
         const gw_status st = batch_enqueue(bb);
@@ -2250,6 +2287,11 @@ gw_status gw_batch_autotune(gw_batch *b, const char *cache_path, double target_e
         return GW_E_INVALID;
     gw_batch &bb = *b;
     cudaSetDevice(bb.device);
+    for (gw_ctx *h : bb.ctxs)
+        if (!h->c.loaded)
+            return bfail(bb, GW_E_NOT_READY, "a context lost its states");
+    GW_BCUDA(cudaStreamSynchronize(bb.ctxs[0]->c.stream), "context stream synchronize");
+    GW_TRY(batch_refresh(bb));
     // the choice depends on the error target as well as on the shapes, and on the error table
     // of the update kernel (rule2: the three-N=256 + six-N=128 form)
     char tgt[48];

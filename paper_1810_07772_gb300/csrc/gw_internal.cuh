@@ -180,6 +180,9 @@ struct Ctx {
             scal, tcw, PGsum, coef, gidx, gtw, psig, ppw;
     } cap = {};
     int tiles_nr_pad = -1, tiles_kind = -1;
+    // counters of loads and of (re)allocated buffers: what was prepared from a context and is kept elsewhere (a
+    // batch's jobs and graph) holds while these and plan_gen stay as they were
+    int load_gen = 0, alloc_gen = 0;
     // separable rank-k update (sep_factors.h, k_herk16p.cu)
     SepFactors sep;                 // factors of the loaded energies (T = 0: pair form)
     bool sep_known = false;         // sep belongs to the loaded energies

@@ -246,3 +246,49 @@ def test_batch_set_up_behind_queued_work():
         assert rel(P.cpu().numpy(), ref.cpu().numpy()) <= 1e-4
     for c in ctxs:
         c.close()
+
+
+def test_batch_after_reloading_its_contexts():
+    """Other states and energies of the same shape (graph captured before), then another shape, then a context
+    used by itself with another cut and a wider operand: the next passes equal fresh single instances."""
+    def single(dims, nv, psi, E, gcut):
+        with gw.Context(0) as ctx:
+            ctx.load_states(psi, E, dims, nv)
+            ctx.set_herk_window(2, 256)
+            ctx.build_P("fp16x3")
+            ctx.P_to_G(gcut)
+            return ctx.view("PG").clone()
+
+    def states(dims, nv, nc, seed, gap):
+        psi, E = inputs.make_states(0, nv, nc, seed, dims=dims)
+        E = np.concatenate([E[:nv], E[nv:] + gap])
+        return torch.from_numpy(psi.astype(np.complex64)).cuda(), E
+
+    gcut = 5
+    shapes = [((9, 10, 11), 24, 200), ((8, 10, 12), 3, 30)]
+    loads = [[states(*sh, 90 + i + 10 * q, gap) for i, sh in enumerate(shapes)] for q, gap in ((0, 0.0), (1, 7.0))]
+    ctxs = [gw.Context(0) for _ in shapes]
+    for c, sh, (psi, E) in zip(ctxs, shapes, loads[0]):
+        c.load_states(psi, E, sh[0], sh[1])
+    with gw.Batch(ctxs, [gcut] * 2) as b:
+        b.set_window(2, 256)
+
+        def check(data, shp):
+            for _ in range(3):
+                b.run(use_graph=True)
+                for c, sh, (psi, E) in zip(ctxs, shp, data):
+                    assert torch.equal(c.view("PG"), single(sh[0], sh[1], psi, E, gcut))
+
+        check(loads[0], shapes)
+        for c, sh, (psi, E) in zip(ctxs, shapes, loads[1]):
+            c.load_states(psi, E, sh[0], sh[1])
+        check(loads[1], shapes)
+        other = ((12, 12, 12), 33, 97)
+        data = [states(*other, 120, 1.0), loads[1][1]]
+        ctxs[0].load_states(*data[0], other[0], other[1])
+        check(data, [other, shapes[1]])
+        ctxs[1].build_P("tf32x3")
+        ctxs[1].P_to_G(3)
+        check(data, [other, shapes[1]])
+    for c in ctxs:
+        c.close()
