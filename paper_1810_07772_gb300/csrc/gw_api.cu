@@ -2115,7 +2115,8 @@ std::string batch_key(const gw_batch &b)
     for (size_t i = 0; i < b.ctxs.size(); ++i) {
         const Ctx &c = b.ctxs[i]->c;
         k += "|" + std::to_string(c.n1) + "x" + std::to_string(c.n2) + "x" + std::to_string(c.n3) + ",v" +
-             std::to_string(c.nv) + ",c" + std::to_string(c.nc) + ",g" + std::to_string(b.gcut[i]);
+             std::to_string(c.nv) + ",c" + std::to_string(c.nc) + ",g" + std::to_string(b.gcut[i]) + ",t" +
+             std::to_string(b.jobs[i].nvc > 0 ? b.jobs[i].T : 0);
     }
     return k;
 }
@@ -2292,10 +2293,10 @@ gw_status gw_batch_autotune(gw_batch *b, const char *cache_path, double target_e
             return bfail(bb, GW_E_NOT_READY, "a context lost its states");
     GW_BCUDA(cudaStreamSynchronize(bb.ctxs[0]->c.stream), "context stream synchronize");
     GW_TRY(batch_refresh(bb));
-    // the choice depends on the error target as well as on the shapes, and on the error table
-    // of the update kernel (rule2: the three-N=256 + six-N=128 form)
+    // the choice depends on the error target as well as on the shapes and on the form each update takes (its
+    // terms), and on the kernel that was timed (rule3: pair and separable form, windows of W chunks)
     char tgt[48];
-    std::snprintf(tgt, sizeof tgt, "|target%.3g|rule2", target_error);
+    std::snprintf(tgt, sizeof tgt, "|target%.3g|rule3", target_error);
     const std::string key = batch_key(bb) + tgt;
     if (cache_path) {
         if (FILE *f = std::fopen(cache_path, "r")) {

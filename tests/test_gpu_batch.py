@@ -151,3 +151,21 @@ def test_batch_rejects_mixed_or_unloaded_contexts():
     assert e.value.status == gw.GW_E_UNSUPPORTED
     ctx.close()
     empty.close()
+
+
+def test_autotune_keeps_to_entries_of_its_own_kernel(tmp_path):
+    """A window cached for the pair form of the same shapes, or by an earlier kernel, is not taken over."""
+    dims, nv, nc, gcut = (9, 10, 11), 24, 200, 5
+    psi, E = inputs.make_states(0, nv, nc, 7, dims=dims)
+    cache = tmp_path / "windows.json"
+    key = f"prec4|{dims[0]}x{dims[1]}x{dims[2]},v{nv},c{nc},g{gcut}"
+    cache.write_text("".join(f'{{"key": "{key}{form}|target0.001|{rule}", "W": 5, "L": 7}}\n'
+                             for form, rule in (("", "rule2"), ("", "rule3"), (",t0", "rule3"))))
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        with gw.Batch([ctx], [gcut]) as b:
+            W = b.autotune(str(cache), target_error=1e-3)["window_chunks"]
+            lines = cache.read_text().splitlines()
+            assert W != 5 and len(lines) == 4
+            cache.write_text(lines[-1].replace(f'"W": {W}', '"W": 9') + "\n")
+            assert b.autotune(str(cache), target_error=1e-3)["window_chunks"] == 9
