@@ -141,6 +141,9 @@ GW_API gw_status gw_load_states(gw_ctx *ctx, int n1, int n2, int n3, double cell
  *   P_out      NULL, or a device buffer of N_r x N_r complex64 that receives a copy of P.
  * P itself stays in the context (full Hermitian matrix, both triangles written, real diagonal)
  * and can be read with gw_get_buffer(GW_BUF_P).  Requires gw_load_states.
+ * The call may be captured into a CUDA graph after one call with the same sizes and settings (nothing is
+ * allocated or uploaded then).  A replay takes the states and energies loaded last, which must have the
+ * same grid, nv and nc; between the two no other call may change the context's settings.
  */
 GW_API gw_status gw_build_P(gw_ctx *ctx, int precision, void *P_out);
 

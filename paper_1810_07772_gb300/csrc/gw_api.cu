@@ -565,60 +565,98 @@ void newton_tc_record(Ctx &c)
 // 9 x 14) 1604 / 1443, 30 x 120 (225; 10 x 10) 2023 / 1329; the lines cross at 3 to 4.5 chunks a term.
 constexpr int SEP_TERM_CHUNKS = 4;
 
+constexpr int SEP_MAX_TERMS = 64;
+
+// Most terms with which the separable form contracts less.
+int sep_limit(const Ctx &c)
+{
+    const int ncc = (c.nc + HERK16_KC - 1) / HERK16_KC, nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
+    const int pair_chunks = (c.k + HERK16_KC - 1) / HERK16_KC;
+    return std::min(SEP_MAX_TERMS, (pair_chunks - 1) / (ncc + nvc + SEP_TERM_CHUNKS));
+}
+
 void find_separable(Ctx &c)
 {
     if (c.sep_known)
         return;
-    const int ncc = (c.nc + HERK16_KC - 1) / HERK16_KC, nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
-    const int pair_chunks = (c.k + HERK16_KC - 1) / HERK16_KC;
-    const int most = (pair_chunks - 1) / (ncc + nvc + SEP_TERM_CHUNKS);
+    // a captured update keeps its form whatever the energies loaded later: factors beyond the limit too
+    const int most = sep_limit(c) < 1 ? 0 : c.d_sept ? SEP_MAX_TERMS : sep_limit(c);
     c.sep = most >= 1 ? sep_factors(c.E_h.data(), c.nv, c.nc, HERK16_KC, most) : SepFactors();
     c.sep_known = true;
 }
 
 bool separable(const Ctx &c)
 {
-    return !c.by_pairs && c.sep.T > 0;
+    return !c.by_pairs && c.sep.T > 0 && c.sep.T <= sep_limit(c);
 }
 
-// The separable job of a context whose d_P and scale words exist: operand buffers, factors and job
-// table uploaded; the planes themselves are made by separable_planes.  `job` receives the job.
-gw_status prepare_separable(Ctx &c, HerkJob *job)
+// The device copy of the separable form, in this order: job record, scales of the terms, factors.
+constexpr size_t SEP_OFF_SCALE = 256, SEP_OFF_TAB = SEP_OFF_SCALE + SEP_MAX_TERMS * sizeof(float);
+static_assert(sizeof(HerkJob) <= SEP_OFF_SCALE, "job record");
+
+HerkJob separable_job(const Ctx &c)
 {
     HerkJob j = {};
     j.T = c.sep.T;
     j.ncc = (c.nc + HERK16_KC - 1) / HERK16_KC;
     j.nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
-    const size_t chunk = plane16_block(1, 0, c.nr_pad / 128, HERK16_NPL, 0) * sizeof(uint16_t);
-    GW_TRY(ensure(c, c.d_sepA, c.cap_sepA, (size_t)j.T * (j.ncc + j.nvc) * chunk, "separable operand"));
-    GW_TRY(ensure(c, c.d_sepB, c.cap_sepB, (size_t)(j.ncc + j.nvc) * chunk, "separable operand"));
-    constexpr size_t head = 256;
-    static_assert(sizeof(HerkJob) <= head, "job record");
-    const size_t off_tab = head + (j.T * sizeof(float) + 255) / 256 * 256;
-    const size_t bytes = off_tab + c.sep.tab.size() * sizeof(float);
-    GW_TRY(ensure(c, c.d_sept, c.cap_sept, bytes, "separable factors"));
-    unsigned char *dev = static_cast<unsigned char *>(c.d_sept);
     j.A = c.d_sepA;
     j.B = c.d_sepB;
     j.P = c.d_P;
     j.scale_exp = reinterpret_cast<const int *>(c.d_small + 2);
-    j.term_scale = reinterpret_cast<const float *>(dev + head);
+    j.term_scale = reinterpret_cast<const float *>(static_cast<unsigned char *>(c.d_sept) + SEP_OFF_SCALE);
     j.nr = c.nr;
     j.nr_pad = c.nr_pad;
-    c.sep_host.assign(bytes, 0);
+    return j;
+}
+
+// The loaded energies' factors and job on the device, for a context whose d_P and scale words exist: operand
+// buffers allocated, the copy queued; the planes themselves are made by separable_planes.
+gw_status upload_separable(Ctx &c)
+{
+    const size_t per_term = (c.nc + HERK16_KC - 1) / HERK16_KC + (c.nv + HERK16_KC - 1) / HERK16_KC;
+    const size_t chunk = plane16_block(1, 0, c.nr_pad / 128, HERK16_NPL, 0) * sizeof(uint16_t);
+    c.sep_up = false;
+    GW_TRY(ensure(c, c.d_sept, c.cap_sept, SEP_OFF_TAB + SEP_MAX_TERMS * per_term * HERK16_KC * sizeof(float),
+                  "separable factors"));
+    GW_TRY(ensure(c, c.d_sepA, c.cap_sepA, c.sep.T * per_term * chunk, "separable operand"));
+    GW_TRY(ensure(c, c.d_sepB, c.cap_sepB, per_term * chunk, "separable operand"));
+    const HerkJob j = separable_job(c);
+    c.sep_host.assign(SEP_OFF_TAB + c.sep.tab.size() * sizeof(float), 0);
     std::memcpy(c.sep_host.data(), &j, sizeof j);
-    std::memcpy(c.sep_host.data() + head, c.sep.scale.data(), j.T * sizeof(float));
-    std::memcpy(c.sep_host.data() + off_tab, c.sep.tab.data(), c.sep.tab.size() * sizeof(float));
-    GW_CUDA(cudaMemcpyAsync(dev, c.sep_host.data(), bytes, cudaMemcpyHostToDevice, c.stream), "separable factors");
-    c.sep_tab = reinterpret_cast<const float *>(dev + off_tab);
-    *job = j;
+    std::memcpy(c.sep_host.data() + SEP_OFF_SCALE, c.sep.scale.data(), j.T * sizeof(float));
+    std::memcpy(c.sep_host.data() + SEP_OFF_TAB, c.sep.tab.data(), c.sep.tab.size() * sizeof(float));
+    GW_CUDA(cudaMemcpyAsync(c.d_sept, c.sep_host.data(), c.sep_host.size(), cudaMemcpyHostToDevice, c.stream),
+            "separable factors");
+    c.sep_tab = reinterpret_cast<const float *>(static_cast<unsigned char *>(c.d_sept) + SEP_OFF_TAB);
+    c.sep_shape[0] = c.nr;
+    c.sep_shape[1] = c.nv;
+    c.sep_shape[2] = c.nc;
+    c.sep_up = true;
     return GW_OK;
 }
 
-cudaError_t separable_planes(Ctx &c, const HerkJob &j, bool bf16, cudaStream_t s)
+// After a load of the shape that the device copy was made for: a captured gw_build_P reads its factors, its
+// terms and its operand from there.  Where the new energies have no factors, or their operand no room, the
+// copy says so (T = 0) and a replay reports it.
+gw_status refresh_separable(Ctx &c)
 {
-    return launch_sep_planes(c.d_psiT, c.sep_tab, j.T, c.nr, c.nb, c.nv, j.ncc, j.nvc, c.nr_pad, bf16, c.d_small,
-                             reinterpret_cast<int *>(c.d_small + 2), c.d_sepA, c.d_sepB, s);
+    if (!c.d_sept || !c.d_P || c.sep_shape[0] != c.nr || c.sep_shape[1] != c.nv || c.sep_shape[2] != c.nc)
+        return GW_OK;
+    find_separable(c);
+    if (c.sep.T > 0 && upload_separable(c) == GW_OK)
+        return GW_OK;
+    cudaGetLastError();
+    if (c.d_sept)
+        GW_CUDA(cudaMemsetAsync(c.d_sept, 0, sizeof(HerkJob), c.stream), "separable job");
+    return GW_OK;
+}
+
+cudaError_t separable_planes(Ctx &c, bool bf16, cudaStream_t s)
+{
+    const HerkJob j = separable_job(c);
+    return launch_sep_planes(c.d_psiT, static_cast<const HerkJob *>(c.d_sept), c.sep_tab, c.nr, c.nb, c.nv, j.ncc, j.nvc,
+                             c.nr_pad, bf16, c.d_small, reinterpret_cast<int *>(c.d_small + 2), c.d_err, s);
 }
 
 // GW_BUF_F after a separable update, which has no pair densities: form them now.
@@ -991,8 +1029,10 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     GW_CUDA(cudaMemcpyAsync(c.d_E, Eh.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s), "copy energies");
     GW_CUDA(launch_weights(c.d_E, nv, nc, c.d_sw, s), "weights");
     c.E_h = Eh;
+    c.sep_up = false;
     if (nb <= 256)  // at most about 15 us on the host, behind the kernels above; larger sets in gw_build_P
         find_separable(c);
+    GW_TRY(refresh_separable(c));
     // Eh is a local: make sure the copy has consumed it before returning.
     GW_CUDA(cudaStreamSynchronize(s), "load sync");
     c.loaded = true;
@@ -1023,9 +1063,13 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     // CTA pairs take 256-row blocks of r: nr_pad is a multiple of 256 for every grid
     const bool pair = p16 && c.herk_kernel == GW_HERK_PAIR && c.nr_pad % 256 == 0;
     const int npl = pair ? HERK16_NPL_PAIR : HERK16_NPL;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    GW_CUDA(cudaStreamIsCapturing(s, &cs), "capture status");
     if (p16)
         find_separable(c);
-    const bool sep = p16 && separable(c);
+    // under capture nothing can be uploaded: the form whose tiles are there, with the factors that are there
+    const bool sep = p16 && (cs == cudaStreamCaptureStatusNone ? separable(c)
+                                                               : !c.by_pairs && c.sep_up && c.tiles_kind == 3);
     size_t Fbytes = 0;
     if (precision == GW_PREC_FP32_SIMT)
         Fbytes = (size_t)c.kpad * c.nr_pad * sizeof(float2);
@@ -1065,16 +1109,16 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     const uint64_t wait_ns = static_cast<uint64_t>(c.wait_limit_ms * 1e6);
     int *scale_exp = reinterpret_cast<int *>(c.d_small + 1);
 
-    HerkJob job = {};
     const int grid_sep = std::min(c.n_tiles, sm_count(c.device));
     if (sep) {
         GW_TRY(ensure(c, c.d_sums, c.cap_sums, (size_t)grid_sep * HERK16P_SUMS, "running sums"));
-        GW_TRY(prepare_separable(c, &job));
+        if (!c.sep_up)
+            GW_TRY(upload_separable(c));
     }
 
     record(c, 0);
     if (sep)
-        GW_CUDA(separable_planes(c, job, precision == GW_PREC_BF16X3, s), "separable operand planes");
+        GW_CUDA(separable_planes(c, precision == GW_PREC_BF16X3, s), "separable operand planes");
     else if (p16)
         GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad,
                                       precision == GW_PREC_BF16X3, c.d_small, scale_exp,
@@ -1959,7 +2003,9 @@ gw_status batch_prepare(gw_batch &b)
         }
         HerkJob job = {};
         if (sep) {
-            GW_TRY(prepare_separable(c, &job));
+            if (!c.sep_up)
+                GW_TRY(upload_separable(c));
+            job = separable_job(c);
         } else {
             job.A = job.B = reinterpret_cast<const uint16_t *>(c.d_F);
             job.P = c.d_P;
@@ -2032,7 +2078,7 @@ gw_status batch_pair_densities(gw_batch &b)
         Ctx &c = b.ctxs[i]->c;
         const bool sep = b.jobs[i].nvc > 0;
         if (sep)
-            GW_CUDA(separable_planes(c, b.jobs[i], bf16, b.stream), "separable operand planes (batch)");
+            GW_CUDA(separable_planes(c, bf16, b.stream), "separable operand planes (batch)");
         else
             GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc,
                                           b.jobs[i].ncc * HERK16_KC, c.nr_pad, bf16, c.d_small, 

@@ -186,6 +186,8 @@ struct Ctx {
     // separable rank-k update (sep_factors.h, k_herk16p.cu)
     SepFactors sep;                 // factors of the loaded energies (T = 0: pair form)
     bool sep_known = false;         // sep belongs to the loaded energies
+    bool sep_up = false;            // ... and so does the device copy
+    int sep_shape[3] = {0, 0, 0};   // nr, nv, nc that the device copy was made for
     std::vector<unsigned char> sep_host;  // the job, the term scales and the factors, as uploaded
     void *d_sept = nullptr;         // their device copy
     const float *sep_tab = nullptr; // the factors in it
@@ -319,9 +321,11 @@ constexpr size_t HERK16P_SUMS = 128 * 1024;  // running sums per CTA of the grid
 cudaError_t launch_herk16p(const HerkJob *jobs, const int4 *tiles, int n_tiles, int grid, bool bf16, uint32_t *err,
                            uint64_t wait_ns, int W, int L, float4 *sums, cudaStream_t s);
 // k_planes16.cu: its operands.  A: T (ncc + nvc) chunks, B: ncc + nvc chunks, both of nr_pad rows and
-// HERK16_NPL planes; tab [T][16 (ncc + nvc)] from sep_factors; bound_bits and scale_exp: two words each.
-cudaError_t launch_sep_planes(const float2 *psiT, const float *tab, int T, int nr, int nb, int nv, int ncc, int nvc,
-                              int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint16_t *A, uint16_t *B,
+// HERK16_NPL planes; tab [T][16 (ncc + nvc)] from sep_factors; bound_bits and scale_exp: two words each.  T and the
+// buffers are read from the job on the device, so that a captured launch follows the factors uploaded last; T = 0
+// (no factors for the energies loaded since) is GW_E_INVALID at SITE_INPUT.
+cudaError_t launch_sep_planes(const float2 *psiT, const HerkJob *job, const float *tab, int nr, int nb, int nv, int ncc,
+                              int nvc, int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint32_t *err,
                               cudaStream_t s);
 
 // k_mlp_tc.cu: tensor-core inference of the correction network (hidden width 256, n_in <= 16)

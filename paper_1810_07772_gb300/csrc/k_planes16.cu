@@ -275,11 +275,18 @@ __device__ __forceinline__ int state_exp(unsigned bits)
 // densities' planes take 1.70 GB.
 template <bool BF16>
 __global__ void __launch_bounds__(256)
-    sep_planes_kernel(const float2 *__restrict__ psiT, const float *__restrict__ tab, int T, int nr, int nb, int nv,
-                      int ncc, int nvc, int nr_pad, int staged, const unsigned *__restrict__ bound_bits,
-                      int *__restrict__ scale_exp, uint16_t *__restrict__ A, uint16_t *__restrict__ B)
+    sep_planes_kernel(const float2 *__restrict__ psiT, const HerkJob *__restrict__ job, const float *__restrict__ tab,
+                      int nr, int nb, int nv, int ncc, int nvc, int nr_pad, int staged,
+                      const unsigned *__restrict__ bound_bits, int *__restrict__ scale_exp, uint32_t *err)
 {
     extern __shared__ __align__(16) uint8_t smem[];
+    const int T = job->T;
+    uint16_t *const A = const_cast<uint16_t *>(job->A), *const B = const_cast<uint16_t *>(job->B);
+    if (T == 0) {
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+            record_error(err, GW_E_INVALID, SITE_INPUT, 0);
+        return;
+    }
     float2 *s_psi = reinterpret_cast<float2 *>(smem);  // [8][nb + PD_LDP_PAD] where it fits
     const int grp = blockIdx.x, nblk = nr_pad / 128;
     if (staged) {
@@ -477,8 +484,8 @@ cudaError_t launch_pair_density16(const float2 *psiT, const float *sw, float sw_
     return cudaGetLastError();
 }
 
-cudaError_t launch_sep_planes(const float2 *psiT, const float *tab, int T, int nr, int nb, int nv, int ncc, int nvc,
-                              int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint16_t *A, uint16_t *B,
+cudaError_t launch_sep_planes(const float2 *psiT, const HerkJob *job, const float *tab, int nr, int nb, int nv, int ncc,
+                              int nvc, int nr_pad, bool bf16, unsigned *bound_bits, int *scale_exp, uint32_t *err,
                               cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(bound_bits, 0, 2 * sizeof(unsigned), s);
@@ -496,8 +503,8 @@ cudaError_t launch_sep_planes(const float2 *psiT, const float *tab, int T, int n
     // parts of the chunks per row group: about four blocks per SM-resident slot, a chunk per warp at least
     const int ngrp = nr_pad / 8, nch = ncc + nvc;
     const int parts = std::max(1, std::min((nch + 7) / 8, (152 * 6 * 4 + ngrp - 1) / ngrp));
-    kernel<<<dim3(ngrp, parts), 256, smem, s>>>(psiT, tab, T, nr, nb, nv, ncc, nvc, nr_pad, staged, bound_bits,
-                                                scale_exp, A, B);
+    kernel<<<dim3(ngrp, parts), 256, smem, s>>>(psiT, job, tab, nr, nb, nv, ncc, nvc, nr_pad, staged, bound_bits,
+                                                scale_exp, err);
     count_launches(1);
     return cudaGetLastError();
 }

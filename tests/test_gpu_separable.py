@@ -292,3 +292,54 @@ def test_batch_after_reloading_its_contexts():
         check(data, [other, shapes[1]])
     for c in ctxs:
         c.close()
+
+
+def test_captured_update_follows_later_loads():
+    """gw_build_P and gw_P_to_G captured on a caller's stream: each replay takes the states and energies loaded
+    last, with fewer or more terms than at the capture, as a fresh context gives them; the third set's energies
+    crowd at the gap, so that a fresh context takes it pair by pair and the replay with all 16 terms."""
+    dims, nv, nc, gcut = (8, 8, 8), 16, 208, 5
+    nr = 512
+    loads = []
+    for seed, gap, power in ((1, 0.5, 1), (2, 30.0, 1), (3, 1e-3, 4), (1, 0.5, 1)):
+        psi, _ = inputs.make_states(0, nv, nc, seed, dims=dims)
+        E = np.concatenate([-10 * np.linspace(0, 1, nv) ** power, gap + 20 * np.linspace(0, 1, nc) ** power])
+        loads.append((torch.from_numpy(psi.astype(np.complex64)).cuda(), E))
+    want, terms = [], []
+    for psi, E in loads:
+        with gw.Context(0) as ctx:
+            ctx.load_states(psi, E, dims, nv)
+            ctx.build_P("fp16x3")
+            terms.append(ctx.update_form()["terms"])
+            ctx.P_to_G(gcut)
+            want.append((ctx.view("P").clone(), ctx.view("PG").clone()))
+    assert 0 < terms[1] < terms[0] and terms[2] == 0
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        ctx = gw.Context(0, stream=s)
+        ctx.load_states(*loads[0], dims, nv)
+        ctx.build_P("fp16x3")
+        g = ctx.P_to_G(gcut)
+        ctx.sync()
+        P = torch.empty((nr, nr), dtype=torch.complex64, device="cuda:0")
+        PG = torch.empty((len(g), len(g)), dtype=torch.complex64, device="cuda:0")
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        graph.capture_begin()
+        ctx.build_P("fp16x3", P_out=P)
+        ctx.P_to_G(gcut, PG_out=PG)
+        graph.capture_end()
+        for (psi, E), (Pw, PGw) in zip(loads, want):
+            ctx.load_states(psi, E, dims, nv)
+            graph.replay()
+            s.synchronize()
+            ctx.sync()
+            if E[nv] < 0.01:
+                assert rel(P.cpu().numpy(), Pw.cpu().numpy()) <= 2e-6
+                assert rel(PG.cpu().numpy(), PGw.cpu().numpy()) <= 2e-6
+            else:
+                assert torch.equal(P, Pw) and torch.equal(PG, PGw)
+        ctx.build_P("fp16x3")                     # and the calls by themselves as before
+        assert ctx.update_form()["terms"] == terms[-1] and torch.equal(ctx.view("P"), want[-1][0])
+        ctx.close()
