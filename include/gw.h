@@ -76,7 +76,7 @@ typedef enum gw_precision {
  * 2^-26 of every weight, so that
  *     P(r,r') = -sum_t [sum_v u_t(v) conj(psi_v(r)) psi_v(r')] [sum_c z_t(c) psi_c(r) conj(psi_c(r'))],
  * T (nv + nc) states instead of nv nc pairs (T is 8 to 13 for the gaps and band widths of Sec. 3).  The
- * library decides from nv, nc and the energies alone; GW_BUF_FACTORS is there after an update in
+ * library decides from nv, nc, the energies and the window length; GW_BUF_FACTORS is there after an update in
  * separable form.  Both forms
  * agree to the error of the precision mode; in the separable form the mean loss of the tensor cores'
  * truncating additions is multiplied back, and its error against FP64 is the smaller one.

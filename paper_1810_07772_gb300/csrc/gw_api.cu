@@ -557,37 +557,38 @@ void newton_tc_record(Ctx &c)
     c.newton_iters = static_cast<int>(c.tc_report[0]);
 }
 
-// Separable form of the 16-bit rank-k update for the loaded energies: c.sep.T terms, 0 where the pair
-// form has less to contract (or was asked for, see separable).  A term costs its ceil(nc / 16) + ceil(nv / 16) chunks of 16 states and
-// about SEP_TERM_CHUNKS more for its shorter windows and for multiplying its sums out; the pair form
-// costs ceil(nv nc / 16).  Update, pair against separable form, 20^3 grid, W = 3 (us): nv x nc =
-// 8 x 300 (150 chunks against T = 8 times 20) 1389 / 1704, 20 x 64 (80; 9 x 6) 797 / 779, 14 x 200 (175;
-// 9 x 14) 1604 / 1443, 30 x 120 (225; 10 x 10) 2023 / 1329; the lines cross at 3 to 4.5 chunks a term.
-constexpr int SEP_TERM_CHUNKS = 4;
-
+// Where the separable form of the 16-bit rank-k update pays.  A term costs its ceil(nc / 16) + ceil(nv / 16) chunks
+// of 16 states and 2.3 to 3.3 more for every window of occupied states, which is multiplied into the
+// sums over the unoccupied ones; the pair form costs ceil(nv nc / 16).  The rule counts two a window and two.  Update with its operand planes, pair against
+// separable form, 20^3 grid, W = 3 (us), nv x nc = 12 x 150 (113 chunks against T = 10 times 11) 1132 / 1377, 16 x 96
+// (96; 10 x 7) 976 / 1003, 20 x 64 (80; 9 x 6) 857 / 863, 24 x 100 (150; 10 x 9) 1452 / 1146, 30 x 120 (225; 11 x 10)
+// 2098 / 1325; W = 1, where two and three windows a term remain: 24 x 100 1897 / 1871, 40 x 40 (100; 9 x 6) 1332 / 1652
+// (W = 3: 1010 / 764).
 constexpr int SEP_MAX_TERMS = 64;
 
-// Most terms with which the separable form contracts less.
-int sep_limit(const Ctx &c)
+// Most terms with which the separable form contracts less, with windows of W chunks.
+int sep_limit(const Ctx &c, int W)
 {
     const int ncc = (c.nc + HERK16_KC - 1) / HERK16_KC, nvc = (c.nv + HERK16_KC - 1) / HERK16_KC;
     const int pair_chunks = (c.k + HERK16_KC - 1) / HERK16_KC;
-    return std::min(SEP_MAX_TERMS, (pair_chunks - 1) / (ncc + nvc + SEP_TERM_CHUNKS));
+    return std::min(SEP_MAX_TERMS, (pair_chunks - 1) / (ncc + nvc + 2 + 2 * ((nvc + W - 1) / W)));
 }
 
+// The factors of the loaded energies: c.sep.T terms, 0 where no window makes them pay.
 void find_separable(Ctx &c)
 {
     if (c.sep_known)
         return;
+    const int limit = sep_limit(c, 1 << 20);
     // a captured update keeps its form whatever the energies loaded later: factors beyond the limit too
-    const int most = sep_limit(c) < 1 ? 0 : c.d_sept ? SEP_MAX_TERMS : sep_limit(c);
+    const int most = limit < 1 ? 0 : c.d_sept ? SEP_MAX_TERMS : limit;
     c.sep = most >= 1 ? sep_factors(c.E_h.data(), c.nv, c.nc, HERK16_KC, most) : SepFactors();
     c.sep_known = true;
 }
 
-bool separable(const Ctx &c)
+bool separable(const Ctx &c, int W)
 {
-    return !c.by_pairs && c.sep.T > 0 && c.sep.T <= sep_limit(c);
+    return !c.by_pairs && c.sep.T > 0 && c.sep.T <= sep_limit(c, W);
 }
 
 // The device copy of the separable form, in this order: job record, scales of the terms, factors.
@@ -1068,7 +1069,7 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     if (p16)
         find_separable(c);
     // under capture nothing can be uploaded: the form whose tiles are there, with the factors that are there
-    const bool sep = p16 && (cs == cudaStreamCaptureStatusNone ? separable(c)
+    const bool sep = p16 && (cs == cudaStreamCaptureStatusNone ? separable(c, c.last_W)
                                                                : !c.by_pairs && c.sep_up && c.tiles_kind == 3);
     size_t Fbytes = 0;
     if (precision == GW_PREC_FP32_SIMT)
@@ -1973,7 +1974,7 @@ gw_status batch_prepare(gw_batch &b)
         const int kpad = ((c.k + HERK16_KC - 1) / HERK16_KC) * HERK16_KC;
         c.kpad = kpad;
         find_separable(c);
-        const bool sep = separable(c);
+        const bool sep = separable(c, b.W);
         const size_t Fbytes = (size_t)kpad * c.nr_pad * 2 * HERK16_NPL;
         if (!sep)
             GW_TRY(ensure(c, c.d_F, c.cap.F, Fbytes, "pair-density operand"));
@@ -2049,6 +2050,21 @@ gw_status batch_prepare(gw_batch &b)
     for (const gw_ctx *h : b.ctxs)
         b.gens.push_back(batch_gens(h->c));
     return GW_OK;
+}
+
+// Windows of W chunks from now on: the captured pass carries the old lengths, and the form of an update may
+// depend on W.
+void batch_use_window(gw_batch &b, int W, int L)
+{
+    if (b.W != W || b.L != L)
+        drop_graph(b);
+    b.W = W;
+    b.L = L;
+    for (size_t i = 0; i < b.gens.size() && i < b.jobs.size(); ++i)
+        if (separable(b.ctxs[i]->c, W) != (b.jobs[i].nvc > 0)) {
+            b.gens.clear();  // the next pass prepares
+            return;
+        }
 }
 
 // Prepare again what the contexts no longer are: one loaded anew (other energies mean other factors, even at the
@@ -2255,10 +2271,7 @@ gw_status gw_batch_set_window(gw_batch *b, int window_chunks, int flush_windows)
 {
     if (!b || window_chunks < 1 || window_chunks > 64 || flush_windows < 1 || flush_windows > 4096)
         return GW_E_INVALID;
-    if (b->W != window_chunks || b->L != flush_windows)
-        drop_graph(*b);  // the captured launch carries the old lengths
-    b->W = window_chunks;
-    b->L = flush_windows;
+    batch_use_window(*b, window_chunks, flush_windows);
     return GW_OK;
 }
 
@@ -2369,6 +2382,8 @@ gw_status gw_batch_autotune(gw_batch *b, const char *cache_path, double target_e
     };
     const Cand cands[] = {{1, 4096}, {2, 256}, {2, 4096}, {3, 4096}, {4, 4096}, {6, 4096}, {8, 4096}};
     GW_TRY(batch_pair_densities(bb));
+    // the candidates are timed in the forms of the present window
+    const int W0 = bb.W, L0 = bb.L;
     int bestW = 0, bestL = 0;
     float best = 1e30f;
     for (const Cand &cd : cands) {
@@ -2392,13 +2407,14 @@ gw_status gw_batch_autotune(gw_batch *b, const char *cache_path, double target_e
         }
     }
     const gw_status st = batch_status(bb);
+    bb.W = W0;
+    bb.L = L0;
     if (st != GW_OK)
         return st;
     if (bestW == 0)
         return bfail(bb, GW_E_UNSUPPORTED, "no window length meets error target %g", target_error);
     drop_graph(bb);
-    bb.W = bestW;
-    bb.L = bestL;
+    batch_use_window(bb, bestW, bestL);
     if (cache_path) {
         if (FILE *f = std::fopen(cache_path, "a")) {
             std::fprintf(f, "{\"key\": \"%s\", \"W\": %d, \"L\": %d, \"herk_ms\": %.4f, \"target_error\": %g}\n",

@@ -294,6 +294,29 @@ def test_batch_after_reloading_its_contexts():
         c.close()
 
 
+def test_form_follows_the_window():
+    """42 x 42 states: separable with windows of three chunks, by pairs with one (three windows a term cost more
+    than the pairs save); a batch changes over with its window, bit for bit as a single instance."""
+    dims, nv, nc, gcut = (8, 9, 8), 42, 42, 5
+    psi, E = inputs.make_states(0, nv, nc, 4, dims=dims)
+    psi = torch.from_numpy(psi.astype(np.complex64)).cuda()
+    want = {}
+    with gw.Context(0) as ctx:
+        ctx.load_states(psi, E, dims, nv)
+        for W in (1, 3):
+            ctx.set_herk_window(W, 256)
+            ctx.build_P("fp16x3")
+            assert (ctx.update_form()["terms"] > 0) == (W == 3)
+            ctx.P_to_G(gcut)
+            want[W] = ctx.view("PG").clone()
+        with gw.Batch([ctx], [gcut]) as b:
+            for W in (3, 1, 3):
+                b.set_window(W, 256)
+                for _ in range(3):
+                    b.run(use_graph=True)
+                    assert torch.equal(ctx.view("PG"), want[W])
+
+
 def test_captured_update_follows_later_loads():
     """gw_build_P and gw_P_to_G captured on a caller's stream: each replay takes the states and energies loaded
     last, with fewer or more terms than at the capture, as a fresh context gives them; the third set's energies
