@@ -7,7 +7,6 @@
 #include <algorithm>
 
 #include "gw_internal.cuh"
-#include "ptx.cuh"
 
 namespace gw {
 
@@ -390,13 +389,12 @@ __global__ void __launch_bounds__(128) chol_panel_kernel(const double2 *__restri
 }
 
 // The trailing update A -= W W^H (lower triangle) of a step, W also copied to its place in the panel, and the
-// factorisation of the next diagonal block beside it.  CTAs 0..7 update four rows each of that block; CTA 0 waits for
-// the other seven (which wait for nothing) and factors it, while the rest of the grid works on the other 16 x 16 tiles.  The
-// dynamic shared memory keeps the CTAs one per SM, so CTA 0 has its SM's FP64 units for itself.  As a launch
-// per diagonal block, panel product, copy and update, a step at N = 515 took 42 + 13 + 3 + 12..48 us,
+// factorisation of the next diagonal block beside it.  CTAs 0..7 update four rows each of that block, and the one
+// that finishes last factors it (no CTA waits for another), while the rest of the grid works on the other 16 x 16
+// tiles.  The dynamic shared memory keeps the CTAs one per SM, so that one has its SM's FP64 units for itself.  As a
+// launch per diagonal block, panel product, copy and update, a step at N = 515 took 42 + 13 + 3 + 12..48 us,
 // now 8 + 40 (every step: 9 us of update and hand-over, 31 of factorisation).
 constexpr int TRAIL_SMEM = 120 * 1024, TRAIL_HELPERS = 8;
-constexpr uint64_t TRAIL_WAIT_NS = 2000000000ull;
 
 __global__ void __launch_bounds__(256, 1)
     chol_trail_kernel(double2 *A, int lda, double2 *panel, const double2 *__restrict__ W, int rest, double2 *Linv,
@@ -432,27 +430,15 @@ __global__ void __launch_bounds__(256, 1)
                 panel[(size_t)i * lda + l] = Ws[i][l];
             }
         }
+        __shared__ int last;
         __threadfence();
+        __syncthreads();  // every row of this CTA is written before it is counted
+        if (tid == 0)
+            last = atomicAdd(arrived, 1u) == TRAIL_HELPERS - 1;
         __syncthreads();
-        if (bid > 0) {
-            if (tid == 0)
-                atomicAdd(arrived, 1u);
+        if (!last)
             return;
-        }
-        __shared__ int ready;
-        if (tid == 0) {
-            const uint64_t t0 = globaltimer_ns();
-            unsigned seen = 0;
-            do
-                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
-            while (seen < TRAIL_HELPERS - 1 && globaltimer_ns() - t0 < TRAIL_WAIT_NS);
-            ready = seen >= TRAIL_HELPERS - 1;
-            if (!ready)
-                record_error(err, GW_E_TIMEOUT, SITE_CHOL_PIVOT, (uint32_t)pivot0);
-        }
-        __syncthreads();
-        if (!ready)
-            return;
+        __threadfence();  // the other CTAs' rows, counted before this one
         DiagBlock &m = *reinterpret_cast<DiagBlock *>(trail_smem);
         for (int t = tid; t < NB * NB; t += 256) {
             const int ii = t >> 5, ll = t & 31;
