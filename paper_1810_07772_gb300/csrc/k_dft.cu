@@ -1299,7 +1299,7 @@ __global__ void __launch_bounds__(PG_WARPS * 32, 3)
         float w = 0.f;
         if (PAIR) {
             const int v = (int)row / ps.nc;
-            src = X + (size_t)(ps.c0 + (int)row - v * ps.nc) * ldx + (size_t)j1 * plane;
+            src = X + (long long)(ps.c0 + (int)row - v * ps.nc) * ldx + (size_t)j1 * plane;
             srcv = X + (size_t)v * ldx + (size_t)j1 * plane;
             w = ps.sw[row];
         } else {
@@ -1659,10 +1659,23 @@ static int planeg_warps(const DftPlan &p)
     return avail <= L.warps ? 0 : (int)std::min<size_t>(PG_WARPS, (avail - L.warps) / L.per_warp);
 }
 
+// Rows that the workspace holds.  Grids without a compiled n3, which need none with the row-block kernel, go
+// through it in slices of 1 GB, or of WS_MAX_ROWS_GENERIC rows where these are more (46 x 46 x 47, 97336 rows:
+// 12 GB in one go).  Row transforms of P in one go / in slices of 1 GB / of 256 MB: 28^3 (0.7 GB) 0.99 / 0.99 /
+// 1.07 ms, 31 x 23 x 29 with N_g = 3900 (1.5 GB) 4.14 / 4.21 / 4.44, 40 x 38 x 37 (4.1 GB) 27.6 / 28.2 / 29.3.
+constexpr size_t WS_SLICE_BYTES = (size_t)1 << 30;
+
+static int ws_rows(const DftPlan &p, int rows)
+{
+    if (p12_compiled(p.n[2]))
+        return rows;
+    const size_t most = planeg_warps(p) > 0 ? WS_SLICE_BYTES / ((size_t)p.n[0] * p.cd * sizeof(float2)) : 0;
+    return (int)std::min<size_t>(rows, std::max<size_t>(WS_MAX_ROWS_GENERIC, most));
+}
+
 size_t dft_work_bytes(const DftPlan &p, int rows)
 {
-    const int r = p12_compiled(p.n[2]) || planeg_warps(p) > 0 ? rows : std::min(rows, WS_MAX_ROWS_GENERIC);
-    return (size_t)r * p.n[0] * p.cd * sizeof(float2);
+    return (size_t)ws_rows(p, rows) * p.n[0] * p.cd * sizeof(float2);
 }
 
 template <int N3, bool PAIR>
@@ -1787,9 +1800,10 @@ static cudaError_t launch_p12(int grid, size_t smem, const float2 *X, long long 
 // The two-kernel transform of `rows` rows: of X (ps == nullptr) or of the pair densities formed
 // from the states X = psi [nb][ldx] (ps != nullptr).  Returns cudaErrorNotSupported, with nothing
 // launched, when pair rows would need the row-block kernel.
-static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, float2 *Y, long long ldy,
-                                  const DftPlan &p, float2 *work, cudaStream_t s, bool negative_exponent,
-                                  const PairSrc *ps, bool const_twiddles)
+// The rows that fit the workspace at once.
+static cudaError_t dft_two_kernel_slice(const float2 *X, long long ldx, int rows, float2 *Y, long long ldy,
+                                        const DftPlan &p, float2 *work, cudaStream_t s, bool negative_exponent,
+                                        const PairSrc *ps, bool const_twiddles)
 {
     if (rows <= 0)
         return cudaSuccess;
@@ -1883,6 +1897,37 @@ static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, floa
         dft_stage3_kernel<<<g3, 256, sm3, s>>>(work, rows, p.n[0], p.cd, p.ng, p.gmap, tw, Y, ldy);
     count_launches(2);
     return cudaGetLastError();
+}
+
+static cudaError_t dft_two_kernel(const float2 *X, long long ldx, int rows, float2 *Y, long long ldy,
+                                  const DftPlan &p, float2 *work, cudaStream_t s, bool negative_exponent,
+                                  const PairSrc *ps, bool const_twiddles)
+{
+    const int most = ws_rows(p, rows);
+    if (rows <= most || !work || !const_twiddles || planeg_warps(p) == 0)
+        return dft_two_kernel_slice(X, ldx, rows, Y, ldy, p, work, s, negative_exponent, ps, const_twiddles);
+    if (!ps) {
+        const int slices = (rows + most - 1) / most, n = (rows + slices - 1) / slices;
+        for (int r = 0; r < rows; r += n) {
+            const cudaError_t e = dft_two_kernel_slice(X + r * ldx, ldx, std::min(n, rows - r), Y + r * ldy, ldy, p, work,
+                                                       s, negative_exponent, nullptr, const_twiddles);
+            if (e != cudaSuccess)
+                return e;
+        }
+        return cudaSuccess;
+    }
+    // pair rows, v nc + c: whole occupied states at a time, or parts of one
+    const int nvs = std::max(1, most / ps->nc), ncs = std::min(ps->nc, most);
+    for (int v = 0; v < ps->nv; v += nvs)
+        for (int c = 0; c < ps->nc; c += ncs) {
+            const long long r = (long long)v * ps->nc + c;
+            const PairSrc part{ps->sw + r, std::min(nvs, ps->nv - v), std::min(ncs, ps->nc - c), ps->c0 + c - v};
+            const cudaError_t e = dft_two_kernel_slice(X + v * ldx, ldx, part.nv * part.nc, Y + r * ldy, ldy, p, work, s,
+                                                       negative_exponent, &part, const_twiddles);
+            if (e != cudaSuccess)  // not supported: at the first part, before anything is queued
+                return e;
+        }
+    return cudaSuccess;
 }
 
 cudaError_t launch_dft_rows_ws(const float2 *X, long long ldx, int rows, float2 *Y, long long ldy, const DftPlan &p,
