@@ -660,16 +660,18 @@ cudaError_t separable_planes(Ctx &c, bool bf16, cudaStream_t s)
                              c.nr_pad, bf16, c.d_small, reinterpret_cast<int *>(c.d_small + 2), c.d_err, s);
 }
 
-// GW_BUF_F after a separable update, which has no pair densities: form them now.
+// GW_BUF_F after a separable update, which has no pair densities, or after a larger operand found no room (its
+// predecessor is gone then): form them now.  k comes from the loaded states: kpad may be another precision's.
 gw_status form_pair_planes(Ctx &c)
 {
     const bool bf16 = c.F_prec == GW_PREC_BF16X3;
     GW_CUDA(cudaSetDevice(c.device), "set device");
-    c.F_bytes = (size_t)c.kpad * c.nr_pad * sizeof(uint16_t) * c.F_npl;
+    const int kpad = (c.k + HERK16_KC - 1) / HERK16_KC * HERK16_KC;
+    c.F_bytes = (size_t)kpad * c.nr_pad * sizeof(uint16_t) * c.F_npl;
     GW_TRY(ensure(c, c.d_F, c.cap.F, c.F_bytes, "pair-density operand"));
-    GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, c.kpad, c.nr_pad, bf16,
-                                  c.d_small, reinterpret_cast<int *>(c.d_small + 1),
-                                  reinterpret_cast<uint16_t *>(c.d_F), c.stream, c.F_npl),
+    GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc, kpad, c.nr_pad, bf16, c.d_small,
+                                  reinterpret_cast<int *>(c.d_small + 1), reinterpret_cast<uint16_t *>(c.d_F), c.stream,
+                                  c.F_npl),
             "pair densities (16-bit)");
     c.F_formed = true;
     return GW_OK;
@@ -1814,8 +1816,11 @@ gw_status gw_get_buffer(gw_ctx *h, int which, void **ptr, size_t *bytes)
     case GW_BUF_F:
         if (c.F_prec < 0 || !c.P_ready)
             return GW_E_NOT_READY;
-        if (!c.F_formed)
+        if (!c.F_formed || !c.d_F) {
+            if (c.F_prec != GW_PREC_FP16X3 && c.F_prec != GW_PREC_BF16X3)
+                return GW_E_NOT_READY;
             GW_TRY(form_pair_planes(c));
+        }
         *ptr = c.d_F;
         *bytes = c.F_bytes;
         return GW_OK;

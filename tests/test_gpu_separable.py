@@ -185,6 +185,39 @@ def test_kernel_setting_and_pair_densities_afterwards(kind, npl):
     assert rel(f / 2.0 ** e, O.pair_density(psi, E, nv).T) < 1e-6
 
 
+@pytest.mark.parametrize("by_pairs", [False, True])
+def test_pair_densities_after_another_operand_found_no_room(by_pairs):
+    """A TF32 build that runs out of memory leaves the earlier P; GW_BUF_F then holds that update's operand, padded
+    to 16 pairs (8021 pairs: 8032, where the TF32 operand has 8024)."""
+    from test_gpu_parity import _decode_16
+    dims, nv, nc = (16, 16, 16), 13, 617
+    psi, E = inputs.make_states(16, nv, nc, 3)
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, dims, nv)
+        ctx.set_herk_kernel("single", by_pairs)
+        ctx.build_P("fp16x3")
+        ctx.sync()
+        P = ctx.view("P").clone()
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        # 400 MB are left, with the operand that the pair form holds
+        left = (400 << 20) - (ctx.buffer("F")[1] if by_pairs else 0)
+        fill = torch.empty(torch.cuda.mem_get_info(0)[0] - left, dtype=torch.uint8, device="cuda:0")
+        with pytest.raises(gw.GwError) as e:
+            ctx.build_P("tf32x3")                # 526 MB; the 16-bit operand takes 263
+        assert e.value.status == gw.GW_E_NOMEM
+        ptr, nbytes = ctx.buffer("F")
+        torch.cuda.synchronize()
+        assert nbytes == 8032 * 4096 * 8
+        del fill
+        torch.cuda.empty_cache()
+        assert torch.equal(ctx.view("P"), P)
+        F = torch.as_tensor(gw.DeviceView(ptr, (nbytes,), "|u1"), device="cuda:0").cpu().numpy()
+        e = int(ctx.stats()["fp16_scale_exp"])
+        f, _ = _decode_16(F, 4096, 4096, nv * nc, bf16=False)
+    assert rel(f / 2.0 ** e, O.pair_density(psi, E, nv).T) < 1e-6
+
+
 def test_batch_of_both_forms_equals_single_instances():
     """One launch over a separable, a pair-form and another separable instance, replayed from the graph
     and after a change of window: bit for bit the single-instance P~."""
