@@ -72,14 +72,14 @@ typedef enum gw_precision {
 
 /*
  * How the 16-bit modes form the update.  The sum over pairs is taken either pair by pair (k = nv nc) or,
- * where that contracts less, in separable form: 2 / (E_c - E_v) = sum_{t < T} u_t(v) z_t(c) to a relative
- * 2^-26 of every weight, so that
+ * where that contracts less, in separable form: 2 / (E_c - E_v) = sum_{t < T} u_t(v) z_t(c), so that
  *     P(r,r') = -sum_t [sum_v u_t(v) conj(psi_v(r)) psi_v(r')] [sum_c z_t(c) psi_c(r) conj(psi_c(r'))],
  * T (nv + nc) states instead of nv nc pairs (T is 8 to 13 for the gaps and band widths of Sec. 3).  The
+ * elimination that gives the factors stops at 2^-26 of every weight; rounded to FP32 they give it to about 1e-7
+ * (at most 2^-26 + 2^-23 times the sum of the terms' sizes, which is 3 weights at most).  The
  * library decides from nv, nc, the energies and the window length; GW_BUF_FACTORS is there after an update in
- * separable form.  Both forms
- * agree to the error of the precision mode; in the separable form the mean loss of the tensor cores'
- * truncating additions is multiplied back, and its error against FP64 is the smaller one.
+ * separable form.  Both forms agree to the error of the precision mode; in the separable form a part of what the
+ * tensor cores' truncating additions lose is added back.
  */
 
 typedef enum gw_inv_method {

@@ -5,10 +5,29 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1810_07772_gb300 import gw, inputs
+from paper_1810_07772_gb300 import gw
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
+
+
+def two_kernel_and_tables(dims, gcut, nv, nc):
+    """P~ by both routes, each pair by the two-kernel form and by the table form."""
+    rng = np.random.default_rng(sum(dims))
+    nr = int(np.prod(dims))
+    psi = (rng.standard_normal((nv + nc, nr)) + 1j * rng.standard_normal((nv + nc, nr))) / np.sqrt(2 * nr)
+    E = np.concatenate([np.linspace(-5, -1, nv), np.linspace(1, 9, nc)])
+    out = []
+    with gw.Context(0) as ctx:
+        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(DEV), E, dims, nv)
+        for kind in ("two_kernel", "tables"):
+            ctx.set_transform_kernel(kind)
+            ctx.build_P("fp16x3")
+            ctx.P_to_G(gcut)
+            r = ctx.view("PG").cpu().numpy()
+            ctx.build_PG(gcut)
+            out.append((r, ctx.view("PG").cpu().numpy()))
+    return list(zip(*out))
 
 
 @pytest.mark.parametrize("dims,gcut,nv,nc", [
@@ -22,21 +41,7 @@ DEV = "cuda:0"
     ((6, 50, 49), 6, 1, 3),
 ])
 def test_two_kernel_matches_tables(dims, gcut, nv, nc):
-    rng = np.random.default_rng(sum(dims))
-    nr = int(np.prod(dims))
-    psi = (rng.standard_normal((nv + nc, nr)) + 1j * rng.standard_normal((nv + nc, nr))) / np.sqrt(2 * nr)
-    E = np.concatenate([np.linspace(-5, -1, nv), np.linspace(1, 9, nc)])
-    out = {}
-    with gw.Context(0) as ctx:
-        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(DEV), E, dims, nv)
-        for kind in ("two_kernel", "tables"):
-            ctx.set_transform_kernel(kind)
-            ctx.build_P("fp16x3")
-            ctx.P_to_G(gcut)
-            r = ctx.view("PG").cpu().numpy()
-            ctx.build_PG(gcut)
-            out[kind] = (r, ctx.view("PG").cpu().numpy())
-    for a, b in zip(out["two_kernel"], out["tables"]):
+    for a, b in two_kernel_and_tables(dims, gcut, nv, nc):
         # FP32 sums of the same terms in two orders: at most 50 terms a stage, three stages twice over
         assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
 

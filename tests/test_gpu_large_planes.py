@@ -3,12 +3,10 @@ table form: the widest sphere (15 columns), few and many pair rows, an odd numbe
 planes of 15, 21, 25 and 28, whose table form sums in another order."""
 import numpy as np
 import pytest
-import torch
 
-from paper_1810_07772_gb300 import gw
+from test_gpu_any_plane import two_kernel_and_tables
 
 pytestmark = pytest.mark.gpu
-DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("dims,gcut,nv,nc", [
@@ -17,42 +15,14 @@ DEV = "cuda:0"
     ((30, 12, 12), 25, 2, 5), ((32, 16, 16), 30, 2, 5), ((36, 18, 18), 30, 2, 5),
 ])
 def test_constant_form_matches_tables(dims, gcut, nv, nc):
-    rng = np.random.default_rng(sum(dims))
-    nr = int(np.prod(dims))
-    psi = (rng.standard_normal((nv + nc, nr)) + 1j * rng.standard_normal((nv + nc, nr))) / np.sqrt(2 * nr)
-    E = np.concatenate([np.linspace(-5, -1, nv), np.linspace(1, 9, nc)])
-    out = {}
-    with gw.Context(0) as ctx:
-        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(DEV), E, dims, nv)
-        for kind in ("two_kernel", "tables"):
-            ctx.set_transform_kernel(kind)
-            ctx.build_P("fp16x3")
-            ctx.P_to_G(gcut)
-            r = ctx.view("PG").cpu().numpy()
-            ctx.build_PG(gcut)
-            out[kind] = (r, ctx.view("PG").cpu().numpy())
     # the same FP32 sums in the same order; the twiddles differ only in the exact zeros
-    for a, b in zip(out["two_kernel"], out["tables"]):
+    for a, b in two_kernel_and_tables(dims, gcut, nv, nc):
         assert np.linalg.norm(a - b) <= 1e-7 * np.linalg.norm(b)
 
 
 @pytest.mark.parametrize("dims,gcut,nv,nc", [((7, 15, 15), 9, 3, 9), ((15, 21, 21), 49, 2, 5), ((9, 25, 25), 16, 5, 7),
                                              ((15, 28, 28), 49, 1, 4), ((21, 15, 15), 36, 2, 5), ((28, 25, 21), 16, 2, 3)])
 def test_sizes_without_a_compiled_table_form(dims, gcut, nv, nc):
-    rng = np.random.default_rng(sum(dims))
-    nr = int(np.prod(dims))
-    psi = (rng.standard_normal((nv + nc, nr)) + 1j * rng.standard_normal((nv + nc, nr))) / np.sqrt(2 * nr)
-    E = np.concatenate([np.linspace(-5, -1, nv), np.linspace(1, 9, nc)])
-    out = {}
-    with gw.Context(0) as ctx:
-        ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).to(DEV), E, dims, nv)
-        for kind in ("two_kernel", "tables"):
-            ctx.set_transform_kernel(kind)
-            ctx.build_P("fp16x3")
-            ctx.P_to_G(gcut)
-            r = ctx.view("PG").cpu().numpy()
-            ctx.build_PG(gcut)
-            out[kind] = (r, ctx.view("PG").cpu().numpy())
     # FP32 sums of the same terms in two orders: at most 28 terms a stage, three stages twice over
-    for a, b in zip(out["two_kernel"], out["tables"]):
+    for a, b in two_kernel_and_tables(dims, gcut, nv, nc):
         assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
