@@ -1033,7 +1033,9 @@ gw_status gw_load_states(gw_ctx *h, int n1, int n2, int n3, double cell_L, int n
     GW_CUDA(launch_weights(c.d_E, nv, nc, c.d_sw, s), "weights");
     c.E_h = Eh;
     c.sep_up = false;
-    if (nb <= 256)  // at most about 15 us on the host, behind the kernels above; larger sets in gw_build_P
+    // the factors of a context that builds P: at most about 15 us on the host, behind the kernels above; larger
+    // sets, and the first, in gw_build_P
+    if (c.built16 && nb <= 256)
         find_separable(c);
     GW_TRY(refresh_separable(c));
     // Eh is a local: make sure the copy has consumed it before returning.
@@ -1068,8 +1070,10 @@ gw_status gw_build_P(gw_ctx *h, int precision, void *P_out)
     const int npl = pair ? HERK16_NPL_PAIR : HERK16_NPL;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     GW_CUDA(cudaStreamIsCapturing(s, &cs), "capture status");
-    if (p16)
+    if (p16) {
+        c.built16 = true;
         find_separable(c);
+    }
     // under capture nothing can be uploaded: the form whose tiles are there, with the factors that are there
     const bool sep = p16 && (cs == cudaStreamCaptureStatusNone ? separable(c, c.last_W)
                                                                : !c.by_pairs && c.sep_up && c.tiles_kind == 3);

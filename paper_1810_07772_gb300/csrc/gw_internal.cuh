@@ -187,6 +187,7 @@ struct Ctx {
     SepFactors sep;                 // factors of the loaded energies (T = 0: pair form)
     bool sep_known = false;         // sep belongs to the loaded energies
     bool sep_up = false;            // ... and so does the device copy
+    bool built16 = false;           // a 16-bit gw_build_P has been made: a load looks for the factors
     int sep_shape[3] = {0, 0, 0};   // nr, nv, nc that the device copy was made for
     std::vector<unsigned char> sep_host;  // the job, the term scales and the factors, as uploaded
     void *d_sept = nullptr;         // their device copy
