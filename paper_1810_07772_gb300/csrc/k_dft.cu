@@ -1061,13 +1061,20 @@ __host__ __device__ inline size_t p12p_smem(int N, int c3, int planes)
            sizeof(float2) * ((size_t)planes * N * p12_pitch(N) + (size_t)p12p_warps(N) * 2 * c3 * (N | 1));
 }
 
-static PairTile pair_tile(int N, int c3, int nv, int nc)
+// Few pairs: fewer occupied states a tile, as long as every tile still has a CTA of its own at once (N = 36 with 4 x
+// 28 pairs on 8 planes, 24 tiles of 40 tasks 23.8 us with stage 3, 96 of 10 15.4; 12^3 with the
+// same pairs 13.2 and 11.3).
+static PairTile pair_tile(int N, int c3, int nv, int nc, int n1)
 {
     int planes = P12P_TV + p12p_warps(N);
     while (planes > 2 && p12p_smem(N, c3, planes) > (p12_ctas(N) == 2 ? 112 * 1024 : DFT_SMEM_MAX))
         --planes;
-    const int tv = std::min({nv, P12P_TV, planes / 2});
-    return {tv, std::min(nc, planes - tv)};
+    int tv = std::min({nv, P12P_TV, planes / 2});
+    const int tc = std::min(nc, planes - tv);
+    auto tiles = [&](int t) { return (long long)((nv + t - 1) / t) * ((nc + tc - 1) / tc) * n1; };
+    while (tv > 1 && tiles(tv / 2) <= 152LL * p12_ctas(N))
+        tv /= 2;
+    return {tv, tc};
 }
 
 template <int N>
@@ -1716,7 +1723,7 @@ static cudaError_t launch_p12c(int grid, const float2 *X, long long ldx, int row
                                float2 *work, const PairSrc *ps, cudaStream_t s)
 {
     if (ps) {
-        const PairTile tl = pair_tile(N, p.c3, ps->nv, ps->nc);
+        const PairTile tl = pair_tile(N, p.c3, ps->nv, ps->nc, p.n[0]);
         const size_t smem = p12p_smem(N, p.c3, tl.tv + tl.tc);
         const cudaError_t e =
             cudaFuncSetAttribute(dft_pairs12c_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
