@@ -150,14 +150,16 @@ gw_status read_device_status(Ctx &c)
                     detail == NS_DETAIL_CAP ? "; the FP16X3 steps had not converged" : "");
     if (code == GW_E_NUMERIC)
         return fail(c, GW_E_NUMERIC, "eps is not positive definite: Cholesky pivot %u <= 0", detail);
+    if (code == GW_E_INVALID && detail == INPUT_DETAIL_FACTORS)
+        return fail(c, GW_E_INVALID, "a captured update was replayed with energies that have no separable form");
     if (code == GW_E_INVALID)
         return fail(c, GW_E_INVALID, "non-finite value in the states (%s)", sname);
     return fail(c, static_cast<gw_status>(code), "device wait ran out in the %s (block %u)", sname, detail);
 }
 
-// Measured error of the FP16 split against FP64 on the 24^3 workload (k = 15360) for window
+// Measured error of the FP16 split against FP64 on the 24^3 workload (k = 15360), pair by pair, for window
 // lengths W (chunks of 16 k): the truncating TMEM sum of one window dominates and does not grow
-// with k.  BF16 keeps 8 + 8 bits (about 4e-6 at short windows); its window error is taken as
+// with k.  The separable form stays below it (1.3e-7 at W = 3; herk16p_kernel has the figures for other states).  BF16 keeps 8 + 8 bits (about 4e-6 at short windows); its window error is taken as
 // additive on top.
 double predicted_error(int precision, int W)
 {
@@ -639,7 +641,8 @@ gw_status upload_separable(Ctx &c)
 
 // After a load of the shape that the device copy was made for: a captured gw_build_P reads its factors, its
 // terms and its operand from there.  Where the new energies have no factors, or their operand no room, the
-// copy says so (T = 0) and a replay reports it.
+// copy says so (T = 0; its other fields, which herk16p_kernel reads for every tile, stay valid) and a replay
+// reports it.
 gw_status refresh_separable(Ctx &c)
 {
     if (!c.d_sept || !c.d_P || c.sep_shape[0] != c.nr || c.sep_shape[1] != c.nv || c.sep_shape[2] != c.nc)
@@ -649,7 +652,9 @@ gw_status refresh_separable(Ctx &c)
         return GW_OK;
     cudaGetLastError();
     if (c.d_sept)
-        GW_CUDA(cudaMemsetAsync(c.d_sept, 0, sizeof(HerkJob), c.stream), "separable job");
+        GW_CUDA(cudaMemsetAsync(static_cast<unsigned char *>(c.d_sept) + offsetof(HerkJob, T), 0, sizeof(HerkJob::T),
+                                c.stream),
+                "separable job");
     return GW_OK;
 }
 

@@ -22,10 +22,11 @@ enum ErrSite : uint32_t {
     SITE_HERK_EPILOGUE = 3,
     SITE_HERK_DRAIN = 4,
     SITE_CHOL_PIVOT = 5,
-    SITE_INPUT = 6,
+    SITE_INPUT = 6,             // detail INPUT_DETAIL_FACTORS: sep_planes_kernel without factors
     SITE_ZGEMM = 7,
     SITE_NS = 8,
 };
+constexpr uint32_t INPUT_DETAIL_FACTORS = 1;
 
 __device__ __forceinline__ void record_error(uint32_t *err, uint32_t code, uint32_t site, uint32_t detail)
 {

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256)
     uint16_t *const A = const_cast<uint16_t *>(job->A), *const B = const_cast<uint16_t *>(job->B);
     if (T == 0) {
         if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-            record_error(err, GW_E_INVALID, SITE_INPUT, 0);
+            record_error(err, GW_E_INVALID, SITE_INPUT, INPUT_DETAIL_FACTORS);
         return;
     }
     float2 *s_psi = reinterpret_cast<float2 *>(smem);  // [8][nb + PD_LDP_PAD] where it fits

@@ -396,6 +396,16 @@ def test_captured_update_follows_later_loads():
                 assert rel(PG.cpu().numpy(), PGw.cpu().numpy()) <= 2e-6
             else:
                 assert torch.equal(P, Pw) and torch.equal(PG, PGw)
+        # energies without factors (weights beyond the range of FP32 scales): the replay says so, once
+        ctx.load_states(loads[0][0], loads[0][1] * 1e-45, dims, nv)
+        graph.replay()
+        with pytest.raises(gw.GwError) as e:
+            ctx.sync()
+        assert e.value.status == gw.GW_E_INVALID and "separable" in str(e.value)
+        ctx.load_states(*loads[-1], dims, nv)
+        graph.replay()
+        ctx.sync()
+        assert torch.equal(P, want[-1][0])
         ctx.build_P("fp16x3")                     # and the calls by themselves as before
         assert ctx.update_form()["terms"] == terms[-1] and torch.equal(ctx.view("P"), want[-1][0])
         ctx.close()
