@@ -639,13 +639,14 @@ gw_status upload_separable(Ctx &c)
     return GW_OK;
 }
 
-// After a load of the shape that the device copy was made for: a captured gw_build_P reads its factors, its
-// terms and its operand from there.  Where the new energies have no factors, or their operand no room, the
+// After a load of the shape that the device copy was made for, with a d_P of that size (a smaller one will be
+// replaced): a captured gw_build_P reads its factors, its terms and its operand from there.  Where the new energies have no factors, or their operand no room, the
 // copy says so (T = 0; its other fields, which herk16p_kernel reads for every tile, stay valid) and a replay
 // reports it.
 gw_status refresh_separable(Ctx &c)
 {
-    if (!c.d_sept || !c.d_P || c.sep_shape[0] != c.nr || c.sep_shape[1] != c.nv || c.sep_shape[2] != c.nc)
+    const bool fits = c.d_P && c.cap.P >= (size_t)c.nr * c.nr * sizeof(float2);
+    if (!c.d_sept || !fits || c.sep_shape[0] != c.nr || c.sep_shape[1] != c.nv || c.sep_shape[2] != c.nc)
         return GW_OK;
     find_separable(c);
     if (c.sep.T > 0 && upload_separable(c) == GW_OK)
@@ -2111,7 +2112,7 @@ gw_status batch_pair_densities(gw_batch &b)
             GW_CUDA(separable_planes(c, bf16, b.stream), "separable operand planes (batch)");
         else
             GW_CUDA(launch_pair_density16(c.d_psiT, c.d_sw, c.sw_max, c.nr, c.nb, c.nv, c.nc,
-                                          b.jobs[i].ncc * HERK16_KC, c.nr_pad, bf16, c.d_small, 
+                                          b.jobs[i].ncc * HERK16_KC, c.nr_pad, bf16, c.d_small,
                                           reinterpret_cast<int *>(c.d_small + 1), reinterpret_cast<uint16_t *>(c.d_F),
                                           b.stream),
                     "pair densities (batch)");

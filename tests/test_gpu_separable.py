@@ -218,6 +218,28 @@ def test_pair_densities_after_another_operand_found_no_room(by_pairs):
     assert rel(f / 2.0 ** e, O.pair_density(psi, E, nv).T) < 1e-6
 
 
+def test_update_after_a_larger_grid_found_no_room():
+    """P(r,r') of 58^3 points (305 GB) finds no room, and the earlier buffer is gone; a smaller grid leaves one too
+    small for the first states, which are then loaded again: the update goes to the buffer that is there."""
+    systems = {n: inputs.make_states(n, nv, nc, 7) for n, nv, nc in ((16, 24, 200), (8, 2, 3))}
+    with gw.Context(0) as ctx:
+        def build(n, nv, precision):
+            psi, E = systems[n]
+            ctx.load_states(torch.from_numpy(psi.astype(np.complex64)).cuda(), E, (n, n, n), nv)
+            ctx.build_P(precision)
+            ctx.sync()
+            return ctx.view("P").clone()
+
+        first = build(16, 24, "fp16x3")
+        assert ctx.buffer("factors")[1] > 0
+        ctx.load_states(torch.zeros(2, 58 ** 3, dtype=torch.complex64, device="cuda:0"), np.array([-1.0, 1.0]), (58,) * 3, 1)
+        with pytest.raises(gw.GwError) as e:
+            ctx.build_P("fp32_simt")
+        assert e.value.status == gw.GW_E_NOMEM
+        build(8, 2, "fp32_simt")
+        assert torch.equal(build(16, 24, "fp16x3"), first)
+
+
 def test_batch_of_both_forms_equals_single_instances():
     """One launch over a separable, a pair-form and another separable instance, replayed from the graph
     and after a change of window: bit for bit the single-instance P~."""
